@@ -4,7 +4,7 @@
 // genesis constant; a seal record ends the log with the stop reason, the
 // artifacts' fingerprint and mode flags.  The configuration hash is the
 // rolling hash of the row's top stack node, carried in a hash stack parallel
-// to the LR stack and updated by k_advance at O(1) per push.
+// to the LR stack and updated by the advance at O(1) per entry pushed.
 //
 // Record layout (80 bytes, little-endian): 0 u64 step, 8 u64 config_hash,
 // 16 u8[16] mask_entry_id, 32 i32 token, 36 u32 blocked_count, 40 u32 kind,
@@ -13,7 +13,7 @@
 // Mask entry id: the mask row's words in 1,024-byte chunks (256 words, the
 // last one shorter), each hashed with BLAKE2b-128, then BLAKE2b-128 of
 // "GRIDmask" || u32 V || u32 chunks || the chunk digests: a content address
-// whose chunks the lanes of a warp hash at once.
+// whose chunks the quads of a block hash at once.
 
 #include "grid_state.cuh"
 
@@ -34,30 +34,6 @@ Digest16 genesis_digest() {
   h.update("GRID audit chain genesis", 24);
   h.final(d.b);
   return d;
-}
-
-// BLAKE2b-128 of n little-endian 32-bit words; whole 128-byte blocks are
-// packed straight from the words.
-__device__ void hash_words(const uint32_t* w, int n, uint8_t* out) {
-  uint64_t h[8];
-  for (int i = 0; i < 8; ++i) h[i] = Blake2bIV::at(i);
-  h[0] ^= 0x01010000ull ^ 16ull;
-  uint64_t m[16];
-  uint64_t t = 0;
-  int k = 0;
-  while (n - k > 32) {  // a full block that is not the last one
-    for (int j = 0; j < 16; ++j) m[j] = (uint64_t)w[k + 2 * j] | ((uint64_t)w[k + 2 * j + 1] << 32);
-    t += 128;
-    blake2b_compress(h, m, t, false);
-    k += 32;
-  }
-  for (int j = 0; j < 16; ++j) {
-    const int a = k + 2 * j, b = a + 1;
-    m[j] = (a < n ? (uint64_t)w[a] : 0ull) | (b < n ? ((uint64_t)w[b] << 32) : 0ull);
-  }
-  t += (uint64_t)(n - k) * 4;
-  blake2b_compress(h, m, t, true);
-  for (int i = 0; i < 16; ++i) out[i] = (uint8_t)(h[i >> 3] >> (8 * (i & 7)));
 }
 
 __host__ __device__ void put_le(uint8_t* p, uint64_t x, int n) {
@@ -104,39 +80,123 @@ __global__ void k_audit_init(Tables t, DevConfigs c, uint8_t* __restrict__ heads
   steps[b] = 0;
 }
 
-// One warp per row (rows whose token is negative get no record): the lanes
-// hash the mask row's chunks and count its set bits, lane 0 makes the mask
-// entry id and the record.
-__global__ void k_audit_append(Tables t, DevConfigs c, const uint32_t* __restrict__ mask,
-                               const int32_t* __restrict__ tokens, uint32_t kind, uint8_t* __restrict__ heads,
-                               uint64_t* __restrict__ steps, uint8_t* __restrict__ records, long long rec_stride,
-                               int B) {
-  extern __shared__ uint8_t s_dig[];  // chunks x 16 bytes
-  const int b = blockIdx.x, lane = threadIdx.x;
+// One block per row (rows whose token is negative get no record).  Each quad
+// of lanes hashes one chunk of the mask row at a time, a 128-byte block per
+// compression: the quad's next block is loaded into registers while it
+// compresses the one it staged in shared memory, and the set bits are counted
+// on the way.  The first warp then hashes the chunk digests into the mask
+// entry id and the record into the chain.  The chain of dependent
+// compressions bounds it (8 per chunk, one for every 8 digests, one for the
+// record: 12 at V = 151,936).  One lane per chunk with the message in local
+// memory and byte-wise records took 158 us for 32 rows of that size; an
+// audited decoding step of such rows went from 265 us to 93 us with this and
+// the deferred node hashes.
+constexpr int kAuditThreads = 128;
+__global__ void __launch_bounds__(kAuditThreads) k_audit_append(
+    Tables t, DevConfigs c, const uint32_t* __restrict__ mask, const int32_t* __restrict__ tokens, uint32_t kind,
+    uint8_t* __restrict__ heads, uint64_t* __restrict__ steps, uint8_t* __restrict__ records, long long rec_stride,
+    int B) {
+  extern __shared__ __align__(16) uint64_t s_id[];  // the id's message: "GRIDmask", V and chunks, 2 words per digest
+  __shared__ __align__(16) uint32_t s_blk[kAuditThreads / 4][34];  // each quad's block (rows on other banks)
+  __shared__ __align__(16) uint64_t s_rec[16];                     // the record
+  __shared__ int s_cnt;
+  const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = lane & 3;
   if (b >= B) return;
   const int tok = tokens[b];
   if (tok < 0) return;
+  // the row's configuration hash, step and chain head, read while the chunks are hashed
+  uint64_t cfg = 0, step = 0, h0 = 0, h1 = 0;
+  if (threadIdx.x == 0) {
+    cfg = c.hs[(size_t)b * t.D + c.depth[b] - 1];
+    step = steps[b];
+    h0 = reinterpret_cast<const uint64_t*>(heads + (size_t)b * 16)[0];
+    h1 = reinterpret_cast<const uint64_t*>(heads + (size_t)b * 16)[1];
+    s_cnt = 0;
+  }
   const int W = t.W;
   const uint32_t* row = mask + (size_t)b * W;
   const int nch = (W + kChunkWords - 1) / kChunkWords;
-  for (int ch = lane; ch < nch; ch += 32) hash_words(row + ch * kChunkWords, min(kChunkWords, W - ch * kChunkWords), s_dig + ch * 16);
+  const int id_words = 2 + 2 * nch;
+  for (int i = id_words + threadIdx.x; i < ((id_words + 15) & ~15); i += kAuditThreads) s_id[i] = 0ull;
+  __syncthreads();
+  const int quad = threadIdx.x >> 2, quads = kAuditThreads >> 2;
+  uint32_t* blk = s_blk[quad];
   int cnt = 0;
-  for (int w = lane; w < W; w += 32) cnt += __popc(row[w]);
+  for (int ch0 = 0; ch0 < nch; ch0 += quads) {  // one round at once: 32 chunks
+    if (ch0 + 8 * warp >= nch) break;           // no chunk for this warp
+    const int ch = ch0 + quad;
+    const uint32_t* p = row + (size_t)ch * kChunkWords;
+    const int n = ch < nch ? min(kChunkWords, W - ch * kChunkWords) : 0;  // words of the quad's chunk
+    const int nblk = (n + 31) >> 5;
+    const int rounds = (min(kChunkWords, W - (ch0 + 8 * warp) * kChunkWords) + 31) >> 5;  // of the warp's longest chunk
+    Blake2bQuad h;
+    h.init(lane, 16);
+    uint32_t nx[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) nx[i] = i * 4 + j < n ? p[i * 4 + j] : 0u;
+    for (int r = 0; r < rounds; ++r) {
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        blk[i * 4 + j] = nx[i];
+        cnt += __popc(nx[i]);
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int k = (r + 1) * 32 + i * 4 + j;
+        nx[i] = k < n ? p[k] : 0u;
+      }
+      __syncwarp();
+      const Blake2bQuad before = h;
+      const uint64_t* m = reinterpret_cast<const uint64_t*>(blk);
+      h.compress(lane, [&](int i) { return m[i]; }, (uint64_t)(r + 1 < nblk ? (r + 1) * 128 : n * 4), r + 1 == nblk);
+      if (r >= nblk) h = before;  // a shorter chunk beside a longer one
+    }
+    if (ch < nch && j < 2) s_id[2 + 2 * ch + j] = h.lo;
+  }
   cnt = __reduce_add_sync(0xffffffffu, cnt);
+  if (lane == 0) atomicAdd(&s_cnt, cnt);
+  if (threadIdx.x == 0) {
+    s_id[0] = 0x6B73616D44495247ull;  // "GRIDmask"
+    s_id[1] = (uint64_t)(uint32_t)t.V | ((uint64_t)nch << 32);
+  }
+  __syncthreads();
+  if (warp != 0) return;
+  // every quad of the warp computes the same from here on
+  Blake2bQuad h;
+  h.init(lane, 16);
+  for (int k = 0; k < id_words; k += 16) {
+    const bool last = k + 16 >= id_words;
+    h.compress(lane, [&](int i) { return s_id[k + i]; }, last ? (uint64_t)id_words * 8 : (uint64_t)(k + 16) * 8, last);
+  }
+  const uint64_t id0 = __shfl_sync(0xffffffffu, h.lo, 0), id1 = __shfl_sync(0xffffffffu, h.lo, 1);
+  if (lane == 0) {
+    s_rec[0] = step;
+    s_rec[1] = cfg;
+    s_rec[2] = id0;
+    s_rec[3] = id1;
+    s_rec[4] = (uint64_t)(uint32_t)tok | ((uint64_t)(uint32_t)(t.V - s_cnt) << 32);
+    s_rec[5] = (uint64_t)kind | (h0 << 32);
+    s_rec[6] = (h0 >> 32) | (h1 << 32);
+    s_rec[7] = h1 >> 32;  // and four zero bytes
+  } else if (lane >= 8 && lane < 16) {
+    s_rec[lane] = 0ull;
+  }
   __syncwarp();
-  if (lane != 0) return;
-  uint8_t id[16];
-  Blake2b h;
-  h.init(16);
-  h.update("GRIDmask", 8);
-  h.put_u32((uint32_t)t.V);
-  h.put_u32((uint32_t)nch);
-  h.update(s_dig, (size_t)nch * 16);
-  h.final(id);
-  const uint64_t cfg = c.hs[(size_t)b * t.D + c.depth[b] - 1];
-  const uint64_t step = steps[b];
-  write_record(records + (size_t)b * rec_stride, step, cfg, id, tok, (uint32_t)(t.V - cnt), kind, heads + (size_t)b * 16);
-  steps[b] = step + 1;
+  h.init(lane, 16);
+  h.compress(lane, [&](int i) { return s_rec[i]; }, 60, true);
+  const uint64_t r0 = __shfl_sync(0xffffffffu, h.lo, 0), r1 = __shfl_sync(0xffffffffu, h.lo, 1);
+  if (lane == 0) {
+    s_rec[8] = r0;
+    s_rec[9] = r1;
+    reinterpret_cast<uint64_t*>(heads + (size_t)b * 16)[0] = r0;
+    reinterpret_cast<uint64_t*>(heads + (size_t)b * 16)[1] = r1;
+    steps[b] = step + 1;
+  }
+  __syncwarp();
+  const uint8_t* r = reinterpret_cast<const uint8_t*>(s_rec);
+  uint8_t* rec = records + (size_t)b * rec_stride;
+  for (int i = lane; i < kRecBytes; i += 32) rec[i] = r[i];
 }
 
 // The seal: kind 3, the final configuration's hash, the spec's fingerprint
@@ -165,8 +225,9 @@ int audit_reset(const grid_spec* s, grid_configs* c, cudaStream_t st) {
 int audit_append(const grid_spec* s, grid_configs* c, const uint32_t* d_mask, const int32_t* d_tokens, uint32_t kind,
                  uint8_t* d_records, long long rec_stride, cudaStream_t st) {
   const int nch = (s->t.W + kChunkWords - 1) / kChunkWords;
-  k_audit_append<<<c->B, 32, (size_t)nch * 16, st>>>(s->t, c->c, d_mask, d_tokens, kind, c->heads, c->steps,
-                                                     d_records, rec_stride, c->B);
+  const size_t id_bytes = (size_t)((2 + 2 * nch + 15) & ~15) * 8;
+  k_audit_append<<<c->B, kAuditThreads, id_bytes, st>>>(s->t, c->c, d_mask, d_tokens, kind, c->heads, c->steps,
+                                                              d_records, rec_stride, c->B);
   GRID_CUDA(cudaGetLastError());
   return GRID_OK;
 }

@@ -31,13 +31,15 @@ struct Blake2bIV {
 
 // message word schedule sigma (RFC 7693, Sec. 2.7), rows 0..9; rounds 10 and
 // 11 reuse rows 0 and 1.  Row r, entry i is packed as nibble i of word r.
-GRID_HD int blake2b_sigma(int r, int i) {
+GRID_HD uint64_t blake2b_row(int r) {
   constexpr uint64_t rows[10] = {
       0xfedcba9876543210ull, 0x357b20c16df984aeull, 0x491763eadf250c8bull, 0x8f04a562ebcd1397ull,
       0xd386cb1efa427509ull, 0x91ef57d438b0a6c2ull, 0xb8293670a4def15cull, 0xa2684f05931ce7bdull,
       0x5a417d2c803b9ef6ull, 0x0dc3e9bf5167482aull};
-  return (int)((rows[r] >> (4 * i)) & 0xFu);
+  return rows[r];
 }
+
+GRID_HD int blake2b_sigma(int r, int i) { return (int)((blake2b_row(r) >> (4 * i)) & 0xFu); }
 
 GRID_HD uint64_t blake2b_rotr(uint64_t x, int n) { return (x >> n) | (x << (64 - n)); }
 
@@ -149,5 +151,67 @@ GRID_HD uint64_t node_hash(uint64_t parent, uint32_t sym) {
   for (int i = 0; i < 8; ++i) x |= (uint64_t)d[i] << (8 * i);
   return x;
 }
+
+#ifdef __CUDACC__
+// The same hash on four neighbouring lanes of a warp: lane j of the quad holds
+// column j of the working state (v[j], v[4+j], v[8+j], v[12+j]) and words j
+// and 4+j of the chained state.  What bounds a compression is its chain of
+// 24 dependent G functions (12 rounds of columns, then diagonals); one lane
+// would issue four times the instructions along it and keep the sixteen
+// message words in local memory, or pay for 12 unrolled rounds of code.
+// Between the half rounds the columns' b, c and d rotate over the quad.
+struct Blake2bQuad {
+  uint64_t lo, hi;  // words j and 4 + j of the chained state
+  __device__ __forceinline__ static uint64_t rot(uint64_t x, int from) { return __shfl_sync(0xffffffffu, x, from); }
+  __device__ __forceinline__ void init(int lane, int out_bytes) {
+    const int j = lane & 3;
+    lo = Blake2bIV::at(j) ^ (j == 0 ? 0x01010000ull ^ (uint64_t)out_bytes : 0ull);
+    hi = Blake2bIV::at(4 + j);
+  }
+  // Every lane of the warp calls it together; msg(i) is word i of the quad's block.
+  template <typename Msg>
+  __device__ __forceinline__ void compress(int lane, const Msg& msg, uint64_t t, bool last) {
+    const int j = lane & 3, q0 = lane & ~3;
+    const int l1 = q0 | ((j + 1) & 3), l2 = q0 | ((j + 2) & 3), l3 = q0 | ((j + 3) & 3);
+    uint64_t a = lo, b = hi, c = Blake2bIV::at(j), d = Blake2bIV::at(4 + j);
+    if (j == 0) d ^= t;
+    if (j == 2 && last) d = ~d;
+    auto g = [&](uint64_t x, uint64_t y) {
+      a = a + x + b;
+      d = blake2b_rotr(d ^ a, 32);
+      c = c + d;
+      b = blake2b_rotr(b ^ c, 24);
+      a = a + y + b;
+      d = blake2b_rotr(d ^ a, 16);
+      c = c + d;
+      b = blake2b_rotr(b ^ c, 63);
+    };
+#pragma unroll
+    for (int r = 0; r < 12; ++r) {
+      const uint32_t e = (uint32_t)(blake2b_row(r % 10) >> (8 * j)), f = (uint32_t)(blake2b_row(r % 10) >> (32 + 8 * j));
+      g(msg((int)(e & 15u)), msg((int)((e >> 4) & 15u)));
+      b = rot(b, l1);
+      c = rot(c, l2);
+      d = rot(d, l3);
+      g(msg((int)(f & 15u)), msg((int)((f >> 4) & 15u)));
+      b = rot(b, l3);
+      c = rot(c, l2);
+      d = rot(d, l1);
+    }
+    lo ^= a ^ c;
+    hi ^= b ^ d;
+  }
+};
+
+// node_hash on one quad, or on every quad of the warp at once (all lanes of
+// the warp call it; the result is in every lane).
+__device__ __forceinline__ uint64_t node_hash_quad(int lane, uint64_t parent, uint32_t sym) {
+  Blake2bQuad h;
+  h.init(lane, 16);
+  const uint64_t id = (uint64_t)(sym >> 16) | ((uint64_t)(sym & 0xFFFFu) << 32);
+  h.compress(lane, [&](int i) { return i == 0 ? parent : (i == 1 ? id : 0ull); }, 16, true);
+  return __shfl_sync(0xffffffffu, h.lo, lane & ~3);
+}
+#endif
 
 }  // namespace grid

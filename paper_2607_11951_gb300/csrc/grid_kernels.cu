@@ -269,7 +269,28 @@ struct AdvOut {
   int depth, q, lx, flags, status;
   uint32_t pc, wc;
   bool win;
+  int keep;  // entries below it are the incoming stack's (the node hashes from here on are new)
 };
+
+// Rolling node hashes (Sec. 6.4) of the entries keep .. depth - 1 of row b's
+// stack, by one warp: the entries' symbols are loaded together, the hashes
+// chain from the parent of entry `keep`.  Only the entries that are left are
+// hashed, once the tokens are fed, away from the chain that the mask waits
+// for: hashing each push as it was made, on the lane that feeds the tokens,
+// cost k_row 51 us of 76 at 32 rows (24 without hashes).
+__device__ __forceinline__ void hash_nodes(const Tables& t, uint64_t* __restrict__ hs, const uint16_t* stack, int keep,
+                                           int depth, int lane) {
+  if (keep >= depth) return;
+  uint64_t hp = hs[keep - 1];
+  for (int i0 = keep; i0 < depth; i0 += 32) {
+    const uint32_t sym = i0 + lane < depth ? t.acc_sym[stack[i0 + lane]] : 0u;
+    const int n = min(32, depth - i0);
+    for (int i = 0; i < n; ++i) {
+      hp = node_hash_quad(lane, hp, __shfl_sync(0xffffffffu, sym, i));
+      if (lane == 0) hs[i0 + i] = hp;
+    }
+  }
+}
 
 // Advance of row b by one warp (Sec. 3.1 parser step, Sec. 4.1 byte walk).
 // The lanes copy the row's stack for an out-of-place advance and mirror it in
@@ -350,7 +371,7 @@ __device__ __forceinline__ bool advance_warp(const Tables& t, const Tables& ts, 
   const uint32_t pc0 = __shfl_sync(0xffffffffu, cpc, 2), wc0 = __shfl_sync(0xffffffffu, cwc, 2);
   __syncwarp();
   if (lane != 0) return false;
-  int depth = depth0, q = q0, lx = lx0, flags = flags0;
+  int depth = depth0, q = q0, lx = lx0, flags = flags0, keep = depth0;
   uint32_t pc = pc0, wcat = wc0;
   int status = GRID_ST_OK;
   const int mc = max_chain_of(t);
@@ -399,14 +420,7 @@ __device__ __forceinline__ bool advance_warp(const Tables& t, const Tables& ts, 
       break;
     }
     for (int i = 0; i < w.m; ++i) stack[w.keep + i] = w.ovl[i];
-    if (cout.hs) {  // rolling hash of every pushed node: O(1) per push
-      uint64_t* hrow = cout.hs + (size_t)b * t.D;
-      uint64_t hp = hrow[w.keep - 1];
-      for (int i = 0; i < w.m; ++i) {
-        hp = node_hash(hp, t.acc_sym[w.ovl[i]]);
-        hrow[w.keep + i] = hp;
-      }
-    }
+    if (w.m > 0) keep = min(keep, w.keep);
     if (use_win && w.keep + w.m <= kStackWin) {
       for (int i = 0; i < w.m; ++i) win[w.keep + i] = w.ovl[i];
     } else {
@@ -431,6 +445,7 @@ __device__ __forceinline__ bool advance_warp(const Tables& t, const Tables& ts, 
   out.pc = pc;
   out.wc = wcat;
   out.win = use_win;
+  out.keep = keep;
   return true;
 }
 
@@ -471,7 +486,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_row(Tables t, DevConfigs c, 
   __shared__ uint32_t s_A0[4], s_A1[4], s_keep[8], s_kill[8];
   __shared__ int s_row[8];  // complete, depth, q, lx, emit_ok, keep1, m1, eos_ok
   __shared__ uint32_t s_pc[2];
-  __shared__ int s_status, s_total0, s_nrng, s_adv[2];
+  __shared__ int s_status, s_total0, s_nrng, s_adv[3];
   if ((int)blockIdx.x >= B) {
     // clearing blocks: zero both verdict bitmaps and the verdict-class bits of every row
     pdl_wait();
@@ -513,6 +528,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_row(Tables t, DevConfigs c, 
       s_pc[1] = o.wc;
       s_adv[0] = o.status;
       s_adv[1] = o.win ? 1 : 0;
+      s_adv[2] = o.keep;
       s_status = GRID_ST_OK;
       s_total0 = 0;
       s_nrng = 0;
@@ -569,6 +585,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_row(Tables t, DevConfigs c, 
       const uint32_t word = __ballot_sync(0xffffffffu, kill);
       if (lane == 0) s_kill[b0 >> 5] = word;
     }
+    if (ADV && c.hs) hash_nodes(t, c.hs + (size_t)b * t.D, base, s_adv[2], depth, lane);
   } else if (warp == 1) {
     // the forced emission of the pending lexeme (sigma -> sigma'), and the
     // EOS gate (Sec. 3.2) on the stack it leaves
@@ -1373,8 +1390,14 @@ __global__ void __launch_bounds__(kAdvWarps * 32) k_advance(Tables t, DevConfigs
   const int b = blockIdx.x * kAdvWarps + warp;
   if (b >= B) return;
   AdvOut out;
+  out.depth = out.keep = 0;
   advance_warp(t, ts, cin, cout, tokens, n_steps, d_status, b, copy, lane, s_stk[warp], LArr{s_lo[warp], 1},
                LArr{s_ls[warp], 1}, out);
+  if (cout.hs) {
+    __syncwarp();
+    hash_nodes(t, cout.hs + (size_t)b * t.D, cout.stack + (size_t)b * t.D, __shfl_sync(0xffffffffu, out.keep, 0),
+               __shfl_sync(0xffffffffu, out.depth, 0), lane);
+  }
 }
 
 // In-place -inf fill, grid = (blocks per row, B): threads stride over a row's
