@@ -85,7 +85,7 @@ struct Tables {
   Bits4 ign;  // ignored terminals (the set I)
   Bits4 cm;   // category terminals
   int cat_term[32];
-  // staged block: these eight arrays live contiguously in `blob`
+  // staged block: these arrays (and live_any) live contiguously in `blob`
   const uint8_t* blob;
   int blob_bytes;  // 0 = too large to stage in shared memory
   const uint8_t* byte_class;
@@ -144,6 +144,12 @@ struct Tables {
   const uint32_t* cls_sets;   // ncls * 4: terminal set of every class id
   const uint32_t* cls_mask;   // T1 * nselw: bit c of row tau = tau is in class c's set
   const uint32_t* acc_sym;    // S: the symbol entering each state (audit node hash)
+  // a chain on a stack of d entries takes at most (d + 1) * chain_rate + chain_base steps, and pushes fewer
+  // entries than a walk's scratch holds (chain_bounds; chain_rate 0: not shown, tokens are fed by one lane)
+  int chain_rate, chain_base;
+  // per lexer state q and category bits c, at q << n_cat | c (lexeme_tables):
+  const uint64_t* ev_list;  // the emission's candidates (LexBatch::ev; 0: none, count 0x7F: more than it holds)
+  const uint32_t* live_any; // bit set: a lexeme there is live
 };
 
 // Work counters of a walk, kept in the lane's registers when the walk is
@@ -215,6 +221,7 @@ __device__ __forceinline__ void stage_tables(const Tables& t, Tables& ts, uint8_
       ts.red_off = reinterpret_cast<const uint32_t*>(rebase(t.red_off));
       ts.red_p = reinterpret_cast<const uint16_t*>(rebase(t.red_p));
       ts.red_mask = reinterpret_cast<const uint32_t*>(rebase(t.red_mask));
+      ts.live_any = reinterpret_cast<const uint32_t*>(rebase(t.live_any));
     }
   }
   __syncthreads();
@@ -597,6 +604,283 @@ __device__ __forceinline__ int walk_bytes(const Tables& t, Walker& w, const Spel
     if (!any) return 0;
   }
   return trailing_live(t, w, max_chain);
+}
+
+// ---- feeding tokens with a warp (grid_advance, the decoding step)
+//
+// The lexer does not look at the parser: where a lexeme ends, and which
+// terminals it can be, follows from the bytes alone, because an emission
+// always takes the whole lexeme.  So a warp lexes up to 32 tokens at once
+// (lex_batch) and leaves the candidate list of each lexeme that ends in them,
+// and the parser (parse_batch) only has to go through the lists: its lanes run
+// the reduce chains of a list's candidates side by side, and the first in
+// priority order that reaches SHIFT is shifted.
+constexpr int kLexBytes = 384;  // bytes of one batch, at most
+constexpr int kLexCand = 7;     // candidates of one lexeme, at most (more: the lane-serial feed)
+constexpr int kChainNs = 8;     // entries that a chain pushes, at most
+
+struct LexState {
+  int q, lx;
+  uint32_t pc, wc;
+};
+
+// What lex_batch leaves about its tokens.
+struct LexBatch {
+  uint64_t ev[kLexBytes];  // per lexeme end: candidates in priority order, a byte each; top byte: their count,
+                           // | 0x80 if an ignored terminal follows them; 0: the stack stays as it is
+  LexState in, out[32], end;     // the lexer's state before the batch, after each token, after the batch
+  uint16_t q[kLexBytes];         // per byte: the DFA state after it
+  uint16_t start[kLexBytes + 1]; // per lexeme: its first byte in the batch
+  uint16_t evo[33];              // per token: the lexeme ends before it
+  uint8_t cls[kLexBytes], byte[kLexBytes];
+  uint8_t last[kLexBytes];       // token + 1 if the byte is its last
+  uint8_t st[32];                // 0: no token, 1: lexed, 2: for the lane-serial feed (EOS, refused, too long)
+  int next;                      // the first token after the batch
+};
+
+// The lane's token of the batch that starts at token k, loaded ahead of lexing it.
+struct LexToken {
+  int st;  // as LexBatch::st
+  Spell sp;
+};
+
+__device__ __forceinline__ LexToken lex_fetch(const Tables& t, const int32_t* tokens, int k, int n_steps, int lane) {
+  const int tok = k + lane < n_steps ? tokens[k + lane] : -1;
+  LexToken x;
+  x.st = tok < 0 ? 0 : 2;
+  x.sp.len = 0;
+  if (tok >= 0 && tok < t.V && tok != t.eos) {
+    const int s = t.spell_of_id[tok];
+    if (s >= 0) {
+      x.sp = load_spell(t, s);
+      x.st = 1;
+    }
+  }
+  return x;
+}
+
+// Lex the next tokens, from number k on, from state `carry`.  The DFA's chain
+// through the bytes (two shared-memory look-ups a byte) is all that is serial;
+// the walks through the identifier trie (a dependent L2 access a byte) run a
+// lexeme per lane, once the DFA has found where the lexemes start.
+__device__ __forceinline__ void lex_batch(const Tables& t, const Tables& ts, const LexToken& own, int k, int n_steps,
+                                          int lane, LexState& carry, LexBatch& L) {
+  const Spell& sp = own.sp;
+  int st = own.st;
+  int at = sp.len;
+  for (int d = 1; d < 32 && d < n_steps - k; d <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, at, d);
+    if (lane >= d) at += v;
+  }
+  const uint32_t over = __ballot_sync(0xffffffffu, at > kLexBytes);
+  int n = min(32, n_steps - k);  // tokens of the batch: as many as fit, at least one
+  if (over) n = min(n, max(1, __ffs(over) - 1));
+  if (lane >= n) st = 0;
+  if (at > kLexBytes && st == 1) st = 2;  // (lane 0: a token that never fits)
+  const uint32_t act = __ballot_sync(0xffffffffu, st == 1);
+  at -= sp.len;
+  if (st == 1) {
+    for (int i = 0; i < sp.len; ++i) {
+      const int b = sp.at(i);
+      L.byte[at + i] = (uint8_t)b;
+      L.cls[at + i] = ts.byte_class[b];
+      L.last[at + i] = i + 1 == sp.len ? (uint8_t)(lane + 1) : (uint8_t)0;
+    }
+  }
+  const int total = act ? __shfl_sync(0xffffffffu, at + sp.len, 31 - __clz(act)) : 0;
+  __syncwarp();
+  // the DFA, the same in every lane
+  int q = carry.q, kills = 0, bad = total;  // bad: the first byte that a token is refused at
+  if (lane == 0) L.start[0] = 0;
+  const int row0 = kStart * ts.C;
+  for (int i = 0; i < total; ++i) {
+    const int c = L.cls[i];
+    int nq = ts.next[q * ts.C + c];
+    if (nq == kDead) {
+      if (q != kStart) nq = ts.next[row0 + c];
+      if (nq == kDead) {
+        bad = i;
+        break;
+      }
+      ++kills;
+      if (lane == 0) L.start[kills] = (uint16_t)i;
+    }
+    q = nq;
+    if (lane == 0) {
+      L.q[i] = (uint16_t)q;
+      if (L.last[i]) L.evo[L.last[i]] = (uint16_t)kills;
+    }
+  }
+  __syncwarp();
+  // the lexemes, one per lane: the trie, the lexeme's liveness, its candidates
+  for (int j = lane; j <= kills; j += 32) {
+    const int a = L.start[j], z = j < kills ? L.start[j + 1] : bad;
+    LexState s = j == 0 ? carry : LexState{kStart, 0, t.root_pc, t.root_wc};
+    int i = a;
+    for (; i < z; ++i) {
+      s.q = L.q[i];
+      s.lx = lex_step(ts, s.lx, L.byte[i], s.pc, s.wc);
+      const int id = (s.q << ts.n_cat) | (int)s.pc;
+      if (!((ts.live_any[id >> 5] >> (id & 31)) & 1u)) break;
+      if (L.last[i]) L.out[L.last[i] - 1] = s;
+    }
+    if (i < z) {
+      bad = min(bad, i);
+    } else if (j < kills) {
+      uint64_t list = __ldg(&t.ev_list[(s.q << t.n_cat) | (int)s.wc]);
+      const int cnt = (int)(list >> 56) & 0x7F;
+      if (list == 0 || cnt > kLexCand) bad = min(bad, z);
+      if (cnt == 0) list = 0;  // an ignored terminal first
+      L.ev[j] = list;
+    }
+  }
+  bad = __reduce_min_sync(0xffffffffu, bad);
+  if (st == 1 && at + sp.len > bad) st = 2;
+  L.st[lane] = (uint8_t)st;
+  __syncwarp();
+  const uint32_t good = __ballot_sync(0xffffffffu, st == 1);
+  const LexState was = carry;
+  if (good) carry = L.out[31 - __clz(good)];
+  if (lane == 0) {
+    L.in = was;
+    L.end = carry;
+    L.next = k + n;
+  }
+  __syncwarp();
+}
+
+// The parser's side, the same in every lane of the warp.  win[0:depth) is the
+// stack.  Tokens before `tok` are accepted; the state at the start of token
+// `tok` is (s_depth, s), and undo[low:s_depth) holds what its emissions took
+// off the stack.
+struct Feed {
+  uint16_t* win;
+  uint16_t* undo;
+  uint16_t* scr;  // kChainNs * 32
+  int cap;        // entries of win
+  int depth, low, s_depth, tok;
+  int wlow;  // entries below it were never written
+  bool any;  // a token was fed
+  LexState s;
+};
+
+// Reduce chain of tau on win[0:depth): simulate() for a stack without overlay.
+__device__ __forceinline__ int chain(const Tables& t, const uint16_t* win, int depth, int tau, uint16_t* scr,
+                                     int& keep_o, int& ns_o, int max_chain) {
+  int k = depth, ns = 0, bk = depth;
+  int top = win[k - 1], bv = top;  // bv = win[bk - 1]
+  for (int it = 0; it < max_chain; ++it) {
+    if (top >= t.S) return 0;
+    const int a = t.action[top * t.T1 + tau];
+    if (a >= 0) {
+      keep_o = k;
+      ns_o = ns;
+      return a;
+    }
+    const int code = -a - 1;  // plen << 10 | lhs
+    const int n = code >> 10, x = min(n, ns);
+    ns -= x;
+    k -= n - x;
+    if (k < 1) return 0;
+    if (k != bk) {
+      bk = k;
+      bv = win[k - 1];
+    }
+    const int top2 = ns ? scr[(ns - 1) * 32] : bv;
+    if (top2 >= t.S) return 0;
+    if (ns >= kChainNs) return -1;
+    top = t.go[top2 * t.NNT + (code & 1023)];
+    scr[ns * 32] = (uint16_t)top;
+    ++ns;
+  }
+  return -1;
+}
+
+// Def. 2 trailing liveness of lexer state (q, pc) on win[0:depth), 32 terminals at a time.  1 / 0 / -1.
+__device__ __forceinline__ int feed_live(const Tables& t, const Feed& f, int q, uint32_t pc, int lane, int max_chain) {
+  const Bits4 Lv = live_prime(t, q, pc);
+  if ((Lv & t.ign).any()) return 1;
+  bool ok = false, bound = false;
+  for (int w = 0; w < 4; ++w) {
+    const uint32_t word = Lv.word(w);
+    if (!word) continue;
+    int a = 0, k, ns;
+    if ((word >> lane) & 1u) a = chain(t, f.win, f.depth, 32 * w + lane, f.scr + lane, k, ns, max_chain);
+    ok |= __any_sync(0xffffffffu, a > 0 && a != kAccept);
+    bound |= __any_sync(0xffffffffu, a < 0);
+  }
+  return bound ? -1 : (ok ? 1 : 0);
+}
+
+// Go through a batch's lists (its token k is number k0 + k).  True if
+// every token was fed; false if the feed has to go on lane-serially at token
+// f.tok, in the state at its start (the stack is put back by feed_back).
+//
+// A token is accepted when its own emissions succeed and the lexeme it leaves
+// can still become an allowed terminal.  That test is not made where the next
+// emission makes it: if the lexeme's emission shifts tau (or an ignored
+// terminal), tau was live in the lexeme all along, on the same stack.  What is
+// left is the test after the last token, and, where a chain could run into its
+// bound (deep stacks of grammars with long chains), the test of every token,
+// which would report that bound.
+__device__ __forceinline__ bool parse_batch(const Tables& t, Feed& f, const LexBatch& L, int k0, int lane,
+                                            int max_chain) {
+  const int own = L.st[lane];
+  uint32_t todo = __ballot_sync(0xffffffffu, own != 0);
+  const uint32_t good = __ballot_sync(0xffffffffu, own == 1);
+  f.any |= todo != 0u;
+  while (todo) {
+    const int k = __ffs(todo) - 1;
+    todo &= todo - 1u;
+    if (!((good >> k) & 1u)) return false;
+    const uint32_t before = good & ((1u << k) - 1u);
+    const int prev = before ? 31 - __clz(before) : -1;  // the token before it
+    const int e1 = L.evo[k + 1];
+    for (int e = prev < 0 ? 0 : L.evo[prev + 1]; e < e1; ++e) {
+      const uint64_t ev = L.ev[e];
+      if (ev == 0) continue;
+      const int n = (int)(ev >> 56) & 0x7F;
+      int a = 0, ko = 0, ns = 0;
+      if (lane < n) a = chain(t, f.win, f.depth, (int)(ev >> (8 * lane)) & 0xFF, f.scr + lane, ko, ns, max_chain);
+      if (__any_sync(0xffffffffu, a < 0)) return false;
+      const uint32_t win = __ballot_sync(0xffffffffu, a > 0 && a != kAccept);
+      if (!win && !(ev >> 63)) return false;
+      if (k0 + k != f.tok) {  // the tokens before this one are accepted
+        if (f.depth > t.D) return false;
+        f.tok = k0 + k;
+        f.s = prev < 0 ? L.in : L.out[prev];
+        f.s_depth = f.low = f.depth;
+      }
+      if (!win) continue;  // ignored
+      const int l = __ffs(win) - 1;
+      ko = __shfl_sync(0xffffffffu, ko, l);
+      ns = __shfl_sync(0xffffffffu, ns, l);
+      a = __shfl_sync(0xffffffffu, a, l);
+      const int low = min(f.low, ko), nd = ko + ns + 1;
+      if (nd - low > kMaxOvl || nd > f.cap) return false;
+      for (int i = low + lane; i < f.low; i += 32) f.undo[i] = f.win[i];
+      __syncwarp();
+      if (lane < ns) f.win[ko + lane] = f.scr[lane * 32 + l];
+      if (lane == 0) f.win[ko + ns] = (uint16_t)(a - 1);
+      __syncwarp();
+      f.low = low;
+      f.wlow = min(f.wlow, low);
+      f.depth = nd;
+    }
+    if ((f.depth + 1) * t.chain_rate + t.chain_base > max_chain &&
+        feed_live(t, f, L.out[k].q, L.out[k].pc, lane, max_chain) != 1)
+      return false;
+  }
+  return true;
+}
+
+// The stack at the start of token f.tok.
+__device__ __forceinline__ void feed_back(Feed& f, int lane) {
+  __syncwarp();
+  for (int i = f.low + lane; i < f.s_depth; i += 32) f.win[i] = f.undo[i];
+  f.depth = f.s_depth;
+  f.low = f.s_depth;
+  __syncwarp();
 }
 
 // EOS gate (Sec. 3.2).  1 / 0 / -1.

@@ -65,7 +65,6 @@ namespace {
 
 constexpr int kWalkWarps = 8;    // warps per k_walk block
 constexpr int kSpan = 32;        // CD list entries per walk item (one warp batch)
-constexpr int kAdvWarps = 4;     // rows per k_advance block
 constexpr int kStackWin = 1024;  // stacks up to this depth are copied to shared memory in k_row/k_advance
 constexpr int kFilterPer = 4;    // records per k_filter thread
 constexpr int kRangeSpan = 32;   // continuing first-byte ranges are walked in items of (up to) this many spellings
@@ -292,30 +291,43 @@ __device__ __forceinline__ void hash_nodes(const Tables& t, uint64_t* __restrict
   }
 }
 
-// Advance of row b by one warp (Sec. 3.1 parser step, Sec. 4.1 byte walk).
-// The lanes copy the row's stack for an out-of-place advance and mirror it in
-// `win` (kStackWin entries, 16-byte accesses when the row stride allows them);
-// lane 0 then feeds the tokens, with its overlay and simulation scratch in
-// `lo` / `ls`, and writes the configuration it leaves (and the row's status
-// when d_status is given).  The loads that start a row are issued as two
-// independent chains: the configuration and then its stack (the first 256
-// entries are read before the depth is known), and the first token with its
-// spelling.  Returns in lane 0 only; the other lanes return once the copy is
-// done.
+// Advance of row b (Sec. 3.1 parser step, Sec. 4.1 byte walk) by one warp, in
+// three parts.  advance_load: the lanes copy the row's stack for an
+// out-of-place advance and mirror it in `win` (kStackWin entries, 16-byte
+// accesses when the row stride allows them); the first 256 entries are read
+// before the depth is known.  parse_batch, over the batches that lex_batch
+// made, feeds the tokens while the stack fits the window and the grammar's
+// chains have a bound (Tables::chain_rate).  advance_rest feeds what is left
+// on lane 0 (a token that is refused, EOS, a stack beyond the window) and
+// writes the configuration it leaves, and the row's status when d_status is
+// given.
+//
+// A token that is fed costs the chain of its table look-ups, so nothing but
+// the stack's own steps stays serial: feeding every byte on lane 0, with the
+// token's spelling loaded when its turn came and each reduce chain run twice
+// (once for a set of terminals, once for the one that shifts), took 3.9 us a
+// token (2,000 tokens, 32 SQL rows: 7.8 ms; 1.9 ms this way).
 constexpr int kAdvSpec = 32;  // 16-byte stack accesses issued per lane before the depth is known
-__device__ __forceinline__ bool advance_warp(const Tables& t, const Tables& ts, const DevConfigs& cin,
-                                             const DevConfigs& cout, const int32_t* __restrict__ tokens,
-                                             int n_steps, int32_t* __restrict__ d_status, int b, int copy,
-                                             int lane, uint16_t* win, LArr lo, LArr ls, AdvOut& out) {
-  // chain 1: the row's configuration (lanes 0-3), the speculative stack read
-  const uint16_t* src = (copy ? cin.stack : cout.stack) + (size_t)b * t.D;
-  uint16_t* stack = cout.stack + (size_t)b * t.D;
+
+// What the parts share, in shared memory.
+struct AdvShared {
+  LexBatch lex;
+  uint16_t undo[kStackWin];
+  uint16_t scr[kChainNs * 32];
+  uint16_t lo[kMaxOvl], ls[kMaxOvl];  // lane 0's overlay and scratch
+};
+
+struct AdvRow {
+  int depth, flags;
+  LexState s;
+  bool win;
+};
+
+// The row's configuration (every lane gets it) and its pending lexeme's categories.
+__device__ __forceinline__ AdvRow advance_config(const Tables& t, const DevConfigs& c, int b, int lane) {
   int cf = 0;
   if (lane < 4) {
-    const int32_t* f = lane == 0 ? (copy ? cin.depth : cout.depth)
-                     : lane == 1 ? (copy ? cin.q : cout.q)
-                     : lane == 2 ? (copy ? cin.lx : cout.lx)
-                                 : (copy ? cin.flags : cout.flags);
+    const int32_t* f = lane == 0 ? c.depth : lane == 1 ? c.q : lane == 2 ? c.lx : c.flags;
     cf = f[b];
   }
   uint32_t cpc = 0u, cwc = 0u;  // category bits of the pending lexeme's trie node (lane 2)
@@ -323,60 +335,98 @@ __device__ __forceinline__ bool advance_warp(const Tables& t, const Tables& ts, 
     cpc = t.lx_pcats[cf];
     cwc = t.lx_wcats[cf];
   }
+  AdvRow r;
+  r.depth = __shfl_sync(0xffffffffu, cf, 0);
+  r.s.q = __shfl_sync(0xffffffffu, cf, 1);
+  r.s.lx = __shfl_sync(0xffffffffu, cf, 2);
+  r.flags = __shfl_sync(0xffffffffu, cf, 3);
+  r.s.pc = __shfl_sync(0xffffffffu, cpc, 2);
+  r.s.wc = __shfl_sync(0xffffffffu, cwc, 2);
+  r.win = r.depth <= kStackWin;
+  return r;
+}
+
+__device__ __forceinline__ AdvRow advance_load(const Tables& t, const DevConfigs& cin, const DevConfigs& cout, int b,
+                                               int copy, int lane, uint16_t* win) {
+  const uint16_t* src = (copy ? cin.stack : cout.stack) + (size_t)b * t.D;
+  uint16_t* stack = cout.stack + (size_t)b * t.D;
   const bool vec = t.D % 8 == 0;  // rows start on 16-byte boundaries: 8 entries per access
   const uint4* s4 = reinterpret_cast<const uint4*>(src);
   uint4 sv = make_uint4(0u, 0u, 0u, 0u);
   if (vec && lane < kAdvSpec && lane * 8 < t.D) sv = s4[lane];
-  // chain 2: the first token and its spelling (lane 0)
-  int tok0 = -1, sp0 = -1;
-  Spell spl0;
-  spl0.len = 0;
-  if (lane == 0 && n_steps > 0) {
-    tok0 = tokens[(size_t)b * n_steps];
-    if (tok0 >= 0 && tok0 < t.V && tok0 != t.eos) {
-      sp0 = t.spell_of_id[tok0];
-      if (sp0 >= 0) spl0 = load_spell(t, sp0);
-    }
-  }
-  const int depth0 = __shfl_sync(0xffffffffu, cf, 0);
-  bool use_win = depth0 <= kStackWin;
+  const AdvRow r = advance_config(t, copy ? cin : cout, b, lane);
   if (vec) {
-    const int n8 = (depth0 + 7) >> 3;  // (n8 * 8 <= D: the last access stays inside the row)
+    const int n8 = (r.depth + 7) >> 3;  // (n8 * 8 <= D: the last access stays inside the row)
     uint4* d4 = reinterpret_cast<uint4*>(stack);
     uint4* w4 = reinterpret_cast<uint4*>(win);
     if (lane < n8) {
       if (copy) d4[lane] = sv;
-      if (use_win) w4[lane] = sv;
+      if (r.win) w4[lane] = sv;
     }
     for (int i = lane + kAdvSpec; i < n8; i += 32) {
       const uint4 v = s4[i];
       if (copy) d4[i] = v;
-      if (use_win) w4[i] = v;
+      if (r.win) w4[i] = v;
     }
   } else {
-    for (int i = lane; i < depth0; i += 32) {
+    for (int i = lane; i < r.depth; i += 32) {
       const uint16_t v = src[i];
       if (copy) stack[i] = v;
-      if (use_win) win[i] = v;
+      if (r.win) win[i] = v;
     }
   }
   if (copy && cout.hs) {  // the node hashes travel with the stack
     const uint64_t* hsrc = cin.hs + (size_t)b * t.D;
     uint64_t* hdst = cout.hs + (size_t)b * t.D;
-    for (int i = lane; i < depth0; i += 32) hdst[i] = hsrc[i];
+    for (int i = lane; i < r.depth; i += 32) hdst[i] = hsrc[i];
   }
-  const int q0 = __shfl_sync(0xffffffffu, cf, 1);
-  const int lx0 = __shfl_sync(0xffffffffu, cf, 2);
-  const int flags0 = __shfl_sync(0xffffffffu, cf, 3);
-  const uint32_t pc0 = __shfl_sync(0xffffffffu, cpc, 2), wc0 = __shfl_sync(0xffffffffu, cwc, 2);
   __syncwarp();
-  if (lane != 0) return false;
-  int depth = depth0, q = q0, lx = lx0, flags = flags0, keep = depth0;
-  uint32_t pc = pc0, wcat = wc0;
+  return r;
+}
+
+// Whether the warp feeds the row's tokens (else all are advance_rest's).  A
+// single token is lane 0's: with one token there is little to lex side by
+// side, and setting the batch up costs a step of one expression row 0.8 us of
+// 31 (SQL rows: no difference).
+__device__ __forceinline__ bool feed_fits(const Tables& t, const AdvRow& r, int n_steps) {
+  return n_steps > 1 && t.chain_rate > 0 && r.win && !(r.flags & 1);
+}
+
+__device__ __forceinline__ Feed feed_begin(const AdvRow& r, uint16_t* win, AdvShared& sh) {
+  return Feed{win, sh.undo, sh.scr, kStackWin, r.depth, r.depth, r.depth, 0, r.depth, false, r.s};
+}
+
+// After the last batch (`fed`: parse_batch went through all of them, `end` is
+// the lexer's state there): the test of the last token, the stack written
+// back, and the row as advance_rest goes on with it at token f.tok.
+__device__ __forceinline__ void feed_end(const Tables& ts, Feed& f, bool fed, const LexState& end, int n_steps,
+                                         AdvRow& r, uint16_t* stack, int lane, int max_chain) {
+  if (fed && (!f.any || (f.depth <= ts.D && feed_live(ts, f, end.q, end.pc, lane, max_chain) == 1))) {
+    f.tok = n_steps;
+    f.s = end;
+  } else {
+    feed_back(f, lane);
+  }
+  for (int i = f.wlow + lane; i < f.depth; i += 32) stack[i] = f.win[i];
+  r.depth = f.depth;
+  r.s = f.s;
+  __syncwarp();
+}
+
+// Lane 0 only: tokens k0 .. n_steps - 1, one after the other (`first`: token 0, loaded ahead).
+__device__ __forceinline__ void advance_rest(const Tables& t, const Tables& ts, const DevConfigs& cout,
+                                             const int32_t* __restrict__ tokens, int k0, int n_steps,
+                                             int32_t* __restrict__ d_status, int b, uint16_t* win, AdvShared& sh,
+                                             const AdvRow& r, int keep, const LexToken& first, AdvOut& out) {
+  uint16_t* stack = cout.stack + (size_t)b * t.D;
+  const LArr lo{sh.lo, 1}, ls{sh.ls, 1};
+  int depth = r.depth, q = r.s.q, lx = r.s.lx, flags = r.flags;
+  uint32_t pc = r.s.pc, wcat = r.s.wc;
+  bool use_win = r.win;
   int status = GRID_ST_OK;
   const int mc = max_chain_of(t);
   Walker w;
-  for (int k = 0; k < n_steps; ++k) {
+  for (int k = k0; k < n_steps; ++k) {
     const int tok = tokens[(size_t)b * n_steps + k];
     if (tok < 0) continue;
     if (flags & 1) {
@@ -401,17 +451,17 @@ __device__ __forceinline__ bool advance_warp(const Tables& t, const Tables& ts, 
       flags |= 1;
       continue;
     }
-    const int s = k == 0 ? sp0 : t.spell_of_id[tok];
-    if (s < 0) {
+    const LexToken x = k == 0 ? first : lex_fetch(t, &tokens[(size_t)b * n_steps + k], 0, 1, 0);
+    if (x.st != 1) {
       status = GRID_ST_TOKEN_NOT_ALLOWED;
       break;
     }
-    const int r = walk_bytes(ts, w, k == 0 ? spl0 : load_spell(t, s), mc);
-    if (r < 0) {
+    const int e = walk_bytes(ts, w, x.sp, mc);
+    if (e < 0) {
       status = GRID_ST_BOUND;
       break;
     }
-    if (r == 0) {
+    if (e == 0) {
       status = GRID_ST_TOKEN_NOT_ALLOWED;
       break;
     }
@@ -446,7 +496,6 @@ __device__ __forceinline__ bool advance_warp(const Tables& t, const Tables& ts, 
   out.wc = wcat;
   out.win = use_win;
   out.keep = keep;
-  return true;
 }
 
 // One block per row (kRowWarps warps), plus clearing blocks after the rows.
@@ -465,13 +514,15 @@ __device__ __forceinline__ bool advance_warp(const Tables& t, const Tables& ts, 
 // cache, looks the row's key up (k_pack reads a ready entry) or claims an
 // empty slot for it (k_pack fills it).
 // Clearing blocks zero both verdict bitmaps and the verdict-class bits.
-// With ADV the row's tokens are fed first (advance_warp on warp 0, from
+// With ADV the row's tokens are fed first (by warp 0, from
 // adv.cin into c), and the row is masked in the configuration that leaves:
 // the advance of one row and the mask preparation of another overlap, and
 // the stack window is taken from the advance.  The row's status is then the
 // advance's error, if its token was refused, else the mask step's.
-template <bool ADV>
-__global__ void __launch_bounds__(kRowWarps * 32) k_row(Tables t, DevConfigs c, RowCtx* __restrict__ ctx,
+// ADV: 0 no tokens, 1 one token per row, 2 several (its own instance, so that
+// the usual step does not carry the batch feed's code).
+template <int ADV>
+__global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(Tables t, DevConfigs c, RowCtx* __restrict__ ctx,
                                                         RowRanges* __restrict__ rng, uint32_t* __restrict__ A2,
                                                         uint32_t* __restrict__ sel, uint32_t* __restrict__ verd0,
                                                         uint32_t* __restrict__ verd1, uint32_t* __restrict__ vcbits,
@@ -481,7 +532,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_row(Tables t, DevConfigs c, 
   __shared__ Tables ts;
   __shared__ __align__(16) uint16_t s_stk[kStackWin];
   __shared__ uint16_t s_ovl1[kMaxOvl];
-  __shared__ uint16_t s_ovl2[kRowJobWarps][kMaxOvl * 32];
+  __shared__ __align__(16) uint16_t s_ovl2[kRowJobWarps][kMaxOvl * 32];
   __shared__ uint16_t s_scr[kRowJobWarps][kMaxOvl * 32];
   __shared__ uint32_t s_A0[4], s_A1[4], s_keep[8], s_kill[8];
   __shared__ int s_row[8];  // complete, depth, q, lx, emit_ok, keep1, m1, eos_ok
@@ -512,14 +563,40 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_row(Tables t, DevConfigs c, 
   const int b = blockIdx.x;
   RowCtx& r = ctx[b];
   const uint16_t* base = c.stack + (size_t)b * t.D;
-  const bool vec = !ADV && t.D % 8 == 0 && kStackWin / 8 <= kRowWarps * 32;
+  const bool vec = ADV == 0 && t.D % 8 == 0 && kStackWin / 8 <= kRowWarps * 32;
   uint4 sv = make_uint4(0u, 0u, 0u, 0u);
   if (ADV) {
-    // the row's tokens, on warp 0 (overlay and scratch in job warp 0's area,
+    // the row's tokens, on warp 0 (its shared state in the job warps' area,
     // which phase 1 uses only after the barrier below)
     AdvOut o;
-    if (warp == 0 && advance_warp(t, ts, adv.cin, c, adv.tokens, adv.n_steps, nullptr, b, adv.copy, lane, s_stk,
-                                  LArr{s_scr[0], 1}, LArr{s_scr[0] + kMaxOvl, 1}, o)) {
+    AdvShared& sh = *reinterpret_cast<AdvShared*>(s_ovl2);
+    static_assert(sizeof(AdvShared) <= sizeof(s_ovl2), "the advance's shared state overlays the job warps' area");
+    int k0 = 0, keep = 0;
+    AdvRow row;
+    LexToken own;
+    if (warp == 0) {
+      // (the first tokens with their spellings, and the configuration with its stack: two chains of loads)
+      const int32_t* toks = adv.tokens + (size_t)b * adv.n_steps;
+      own = lex_fetch(t, toks, 0, adv.n_steps, lane);
+      row = advance_load(t, adv.cin, c, b, adv.copy, lane, s_stk);
+      keep = row.depth;
+      if (ADV == 2 && feed_fits(t, row, adv.n_steps)) {
+        Feed f = feed_begin(row, s_stk, sh);
+        LexState carry = row.s;
+        bool fed = true;
+        for (int k = 0; k < adv.n_steps && fed; k = sh.lex.next) {
+          const LexToken mine = k == 0 ? own : lex_fetch(t, toks, k, adv.n_steps, lane);
+          lex_batch(t, ts, mine, k, adv.n_steps, lane, carry, sh.lex);
+          fed = parse_batch(ts, f, sh.lex, k, lane, max_chain_of(t));
+          __syncwarp();
+        }
+        feed_end(ts, f, fed, carry, adv.n_steps, row, c.stack + (size_t)b * t.D, lane, max_chain_of(t));
+        k0 = f.tok;
+        keep = f.wlow;
+      }
+    }
+    if (threadIdx.x == 0) {
+      advance_rest(t, ts, c, adv.tokens, k0, adv.n_steps, nullptr, b, s_stk, sh, row, keep, own, o);
       s_row[0] = o.flags & 1;
       s_row[1] = o.depth;
       s_row[2] = o.q;
@@ -1376,23 +1453,65 @@ __global__ void __launch_bounds__(kPackWords) k_pack(Tables t, RowCtx* __restric
   }
 }
 
-// One warp per row (advance_warp).
-__global__ void __launch_bounds__(kAdvWarps * 32) k_advance(Tables t, DevConfigs cin, DevConfigs cout,
-                                                             const int32_t* __restrict__ tokens, int n_steps,
-                                                             int32_t* __restrict__ d_status, int B, int copy) {
+// One block of two warps per row: warp 1 lexes the next batch of tokens while
+// warp 0 parses the last one.
+__global__ void __launch_bounds__(64, 3) k_advance(Tables t, DevConfigs cin, DevConfigs cout,
+                                                const int32_t* __restrict__ tokens, int n_steps,
+                                                int32_t* __restrict__ d_status, int B, int copy) {
   extern __shared__ __align__(16) uint8_t smem[];
   __shared__ Tables ts;
-  __shared__ __align__(16) uint16_t s_stk[kAdvWarps][kStackWin];
-  __shared__ uint16_t s_lo[kAdvWarps][kMaxOvl], s_ls[kAdvWarps][kMaxOvl];
+  __shared__ __align__(16) uint16_t s_stk[kStackWin];
+  __shared__ AdvShared sh;
+  __shared__ LexBatch s_lex1;  // with sh.lex: the batch being parsed and the one being made
+  __shared__ int s_stop[2];    // set while batch j is parsed, read before batch j + 1 is: j odd, j even
   stage_tables(t, ts, smem);
   pdl_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int b = blockIdx.x * kAdvWarps + warp;
-  if (b >= B) return;
+  const int b = blockIdx.x;
+  const int mc = max_chain_of(t);
+  const int32_t* toks = tokens + (size_t)b * n_steps;
+  AdvRow row;
+  Feed f;
+  LexToken own;
+  bool fed = true;
+  own = lex_fetch(t, toks, 0, n_steps, lane);
+  if (warp == 0) {
+    row = advance_load(t, cin, cout, b, copy, lane, s_stk);
+    f = feed_begin(row, s_stk, sh);
+    if (lane == 0) {
+      s_stop[0] = 0;
+      s_stop[1] = feed_fits(t, row, n_steps) ? 0 : 1;
+    }
+    fed = feed_fits(t, row, n_steps);
+  } else {
+    row = advance_config(t, copy ? cin : cout, b, lane);
+  }
+  LexState carry = row.s;
+  for (int k = 0, j = 0, next; k < n_steps; k = next, ++j) {
+    LexBatch& L = j & 1 ? s_lex1 : sh.lex;
+    if (warp == 1 && feed_fits(t, row, n_steps)) {
+      const LexToken mine = k == 0 ? own : lex_fetch(t, toks, k, n_steps, lane);
+      lex_batch(t, ts, mine, k, n_steps, lane, carry, L);
+    }
+    __syncthreads();
+    next = L.next;
+    if (((volatile int*)s_stop)[(j + 1) & 1]) break;
+    if (warp == 0) {
+      fed = parse_batch(ts, f, L, k, lane, mc);
+      carry = L.end;
+      if (lane == 0) s_stop[j & 1] = fed ? 0 : 1;
+    }
+  }
+  if (warp != 0) return;
+  int k0 = 0, keep = row.depth;
+  if (feed_fits(t, row, n_steps)) {
+    feed_end(ts, f, fed, carry, n_steps, row, cout.stack + (size_t)b * t.D, lane, mc);
+    k0 = f.tok;
+    keep = f.wlow;
+  }
   AdvOut out;
   out.depth = out.keep = 0;
-  advance_warp(t, ts, cin, cout, tokens, n_steps, d_status, b, copy, lane, s_stk[warp], LArr{s_lo[warp], 1},
-               LArr{s_ls[warp], 1}, out);
+  if (lane == 0) advance_rest(t, ts, cout, tokens, k0, n_steps, d_status, b, s_stk, sh, row, keep, own, out);
   if (cout.hs) {
     __syncwarp();
     hash_nodes(t, cout.hs + (size_t)b * t.D, cout.stack + (size_t)b * t.D, __shfl_sync(0xffffffffu, out.keep, 0),
@@ -1527,12 +1646,125 @@ static int set_smem_limits() {
   GRID_CUDA(cudaFuncSetAttribute(k_pack<0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
   GRID_CUDA(cudaFuncSetAttribute(k_pack<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
   GRID_CUDA(cudaFuncSetAttribute(k_pack<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-  GRID_CUDA(cudaFuncSetAttribute(k_row<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-  GRID_CUDA(cudaFuncSetAttribute(k_row<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
+  GRID_CUDA(cudaFuncSetAttribute(k_row<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
+  GRID_CUDA(cudaFuncSetAttribute(k_row<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
+  GRID_CUDA(cudaFuncSetAttribute(k_row<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
   GRID_CUDA(cudaFuncSetAttribute(k_walk<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
   GRID_CUDA(cudaFuncSetAttribute(k_walk<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
   GRID_CUDA(cudaFuncSetAttribute(k_advance, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
   return GRID_OK;
+}
+
+// Bounds of the reduce chains under one lookahead (Tables::chain_rate,
+// chain_base), 0 where none is shown.  A chain's reductions are the nodes of
+// parse trees: nodes of empty yield; nodes over one symbol that is not empty
+// beside empty ones; and nodes over two or more such symbols, each of which
+// leaves fewer of them on the stack (at most one per stack entry).  Between
+// two of the last kind, at one place of the stack, no nonterminal comes twice
+// (the grammar would be ambiguous, and its tables would conflict), so a run of
+// the second kind is a path in the graph of its productions.  What a chain
+// pushes is one symbol and empty ones on top of it: a path in the goto graph
+// over nullable nonterminals.
+static void chain_bounds(const HostGrammar& h, Tables& t) {
+  t.chain_rate = t.chain_base = 0;
+  const int T1 = h.T1, N = h.NNT;
+  constexpr int kBig = 1 << 12;
+  // eps[A]: the most nodes of an empty tree of A (-1: A is not nullable)
+  std::vector<int> eps(N, -1);
+  for (int round = 0; round <= N + 1; ++round) {
+    bool changed = false;
+    for (int p = 0; p < h.P; ++p) {
+      int sum = 1;
+      for (int j = h.prod_off[p]; j < h.prod_off[p + 1] && sum > 0; ++j) {
+        const int X = h.prod_rhs[j];
+        sum = X < T1 || eps[X - T1] < 0 ? 0 : std::min(kBig, sum + eps[X - T1]);
+      }
+      if (sum > eps[h.plhs[p]] && sum > 0) {
+        eps[h.plhs[p]] = sum;
+        changed = true;
+      }
+    }
+    if (!changed) break;
+    if (round == N + 1) return;  // empty trees without a bound
+  }
+  // up[A]: the most steps of a run of second-kind nodes (and their empty parts) that ends in A
+  std::vector<int> up(N, 0);
+  int emax = 0, longest = 0;
+  for (int round = 0; round <= N + 1; ++round) {
+    bool changed = false;
+    for (int p = 0; p < h.P; ++p) {
+      int sum = 0, solid = 0;
+      for (int j = h.prod_off[p]; j < h.prod_off[p + 1]; ++j) {
+        const int X = h.prod_rhs[j];
+        if (X >= T1 && eps[X - T1] > 0)
+          sum = std::min(kBig, sum + eps[X - T1]);
+        else
+          ++solid;
+      }
+      emax = std::max(emax, sum);
+      if (solid > 1) continue;
+      for (int j = h.prod_off[p]; j < h.prod_off[p + 1]; ++j) {  // the symbol that is not empty
+        const int X = h.prod_rhs[j];
+        if (solid == 1 && X >= T1 && eps[X - T1] > 0) continue;
+        const int v = std::min(kBig, (X < T1 ? 0 : up[X - T1]) + 1 + sum);
+        if (v > up[h.plhs[p]]) {
+          up[h.plhs[p]] = v;
+          changed = true;
+        }
+      }
+    }
+    if (!changed) break;
+    if (round == N + 1) return;
+  }
+  for (int A = 0; A < N; ++A) longest = std::max(longest, up[A]);
+  // the longest path over nullable gotos
+  std::vector<int> len(h.S, 0);
+  int path = 0;
+  for (int round = 0; round <= h.S + 1; ++round) {
+    bool changed = false;
+    for (int s = 0; s < h.S; ++s)
+      for (int A = 0; A < N; ++A) {
+        const int g = h.go[(size_t)s * N + A];
+        if (eps[A] < 0 || g >= h.S || len[g] + 1 <= len[s]) continue;
+        len[s] = len[g] + 1;
+        path = std::max(path, len[s]);
+        changed = true;
+      }
+    if (!changed) break;
+    if (path + 2 >= kLaneOvl || round == h.S + 1) return;
+  }
+  const int rate = 1 + emax + longest + 1, base = (path + 1) * (emax + 1);
+  if (path + 2 >= kLaneOvl || emax >= kBig || longest >= kBig) return;
+  t.chain_rate = rate;
+  t.chain_base = base;
+}
+
+// Tables::ev_list and Tables::live_any.
+static void lexeme_tables(const HostGrammar& h, std::vector<uint64_t>& ev, std::vector<uint32_t>& live) {
+  const int sets = 1 << h.n_cat;
+  ev.assign((size_t)h.Q * sets, 0);
+  live.assign(((size_t)h.Q * sets + 31) / 32, 0u);
+  for (int q = 0; q < h.Q; ++q)
+    for (int c = 0; c < sets; ++c) {
+      auto has = [&](const std::vector<uint32_t>& set, int tau) {
+        if (!((set[q * 4 + (tau >> 5)] >> (tau & 31)) & 1u)) return false;
+        if (!((h.catmask[tau >> 5] >> (tau & 31)) & 1u)) return true;
+        for (int k = 0; k < h.n_cat; ++k)
+          if (h.cat_term[k] == tau && ((c >> k) & 1)) return true;
+        return false;
+      };
+      uint64_t list = 0;
+      int n = 0;
+      bool ign = false;
+      for (int tau = 0; tau < h.n_term; ++tau) {
+        if (has(h.live, tau)) live[((size_t)q * sets + c) >> 5] |= 1u << ((q * sets + c) & 31);
+        if (ign || !has(h.acc, tau)) continue;
+        ign = (h.ignored[tau >> 5] >> (tau & 31)) & 1u;
+        if (!ign && n < kLexCand) list |= (uint64_t)tau << (8 * n);
+        n += ign ? 0 : 1;
+      }
+      ev[(size_t)q * sets + c] = n > kLexCand ? (uint64_t)0x7F << 56 : list | ((uint64_t)(n | (ign ? 0x80 : 0)) << 56);
+    }
 }
 
 extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void* stream, grid_spec** out) {
@@ -1560,6 +1792,7 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   t.eos = hv.eos;
   t.W = (hv.V + 31) / 32;
   t.D = h.max_depth;
+  chain_bounds(h, t);
   t.ign = Bits4{h.ignored[0], h.ignored[1], h.ignored[2], h.ignored[3]};
   t.cm = Bits4{h.catmask[0], h.catmask[1], h.catmask[2], h.catmask[3]};
   for (int c = 0; c < h.n_cat; ++c) t.cat_term[c] = h.cat_term[c];
@@ -1607,16 +1840,23 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
     }
     red_off[st + 1] = (uint32_t)red_p.size();
   }
+  // lexeme tables, where the class ids fit (the bound of ci_on below)
+  std::vector<uint64_t> ev_list;
+  std::vector<uint32_t> live_any;
+  if (((long)(2 * h.Q) << h.n_cat) < (long)kClsFirstCode)
+    lexeme_tables(h, ev_list, live_any);
+  else
+    t.chain_rate = 0;
   // staged block: byte classes, DFA, acc/live, ACTION, GOTO, production
-  // tables, shift masks and reduce groups
-  constexpr int kSec = 12;
+  // tables, shift masks and reduce groups, live lexemes
+  constexpr int kSec = 13;
   std::vector<size_t> off(kSec + 1, 0);
   const size_t sizes[kSec] = {256, h.next.size() * 2, h.acc.size() * 4, h.live.size() * 4, h.action.size() * 2,
                               h.go.size() * 2, h.plen.size(), h.plhs.size() * 2, shift_mask.size() * 4,
-                              red_off.size() * 4, red_p.size() * 2, red_mask.size() * 4};
+                              red_off.size() * 4, red_p.size() * 2, red_mask.size() * 4, live_any.size() * 4};
   const void* srcs[kSec] = {h.byte_class, h.next.data(), h.acc.data(), h.live.data(), action16.data(),
                             h.go.data(), h.plen.data(), h.plhs.data(), shift_mask.data(), red_off.data(),
-                            red_p.data(), red_mask.data()};
+                            red_p.data(), red_mask.data(), live_any.data()};
   for (int k = 0; k < kSec; ++k) off[k + 1] = align16(off[k] + sizes[k]);
   std::vector<uint8_t> blob(off[kSec], 0);
   for (int k = 0; k < kSec; ++k)
@@ -1638,7 +1878,9 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   t.red_off = reinterpret_cast<const uint32_t*>(dblob + off[9]);
   t.red_p = reinterpret_cast<const uint16_t*>(dblob + off[10]);
   t.red_mask = reinterpret_cast<const uint32_t*>(dblob + off[11]);
+  t.live_any = reinterpret_cast<const uint32_t*>(dblob + off[12]);
   Arena& a = s->mem;
+  if ((rc = a.upload(ev_list, &t.ev_list))) return fail(rc);
   {
     // identifier-trie edges -> open-addressing hash (load factor <= 1/2)
     const size_t edges = h.lx_cbyte.size();
@@ -2000,7 +2242,7 @@ extern "C" int grid_configs_reset(const grid_spec* s, grid_configs* c, void* str
 
 int grid::launch_advance(const grid_spec* s, const DevConfigs& in, const DevConfigs& out, int B,
                          const int32_t* d_tokens, int32_t n_steps, int32_t* d_status, int copy, cudaStream_t st) {
-  GRID_CUDA(launch_pdl(k_advance, dim3((B + kAdvWarps - 1) / kAdvWarps), dim3(kAdvWarps * 32), s->t.blob_bytes, st,
+  GRID_CUDA(launch_pdl(k_advance, dim3(B), dim3(64), s->t.blob_bytes, st,
                        s->t, in, out, d_tokens, n_steps, d_status, B, copy));
   GRID_CUDA(cudaGetLastError());
   return GRID_OK;
@@ -2027,13 +2269,11 @@ int grid::launch_masks(const grid_spec* s, const DevConfigs& c, const MaskScratc
   const size_t zero_words = (size_t)B * m.words_v * 2 + n_vcbits;
   const int zero_blocks = std::min(128, (int)((zero_words / 8 + kRowWarps * 32 * 4 - 1) / (kRowWarps * 32 * 4)) + 1);
   if (ev) GRID_CUDA(cudaEventRecord(ev[0], st));
-  if (adv)
-    GRID_CUDA(launch_pdl(k_row<true>, dim3(B + zero_blocks), dim3(kRowWarps * 32), t.blob_bytes, st, t, c, m.ctx,
-                         m.rng, m.A2, m.sel, m.verd0, m.verd1, m.vcbits, n_vcbits, B, m.words_v, m.cache, *adv));
-  else
-    GRID_CUDA(launch_pdl(k_row<false>, dim3(B + zero_blocks), dim3(kRowWarps * 32), t.blob_bytes, st, t, c, m.ctx,
-                         m.rng, m.A2, m.sel, m.verd0, m.verd1, m.vcbits, n_vcbits, B, m.words_v, m.cache,
-                         AdvArgs{}));
+  auto row = [&](auto kern) {
+    return launch_pdl(kern, dim3(B + zero_blocks), dim3(kRowWarps * 32), t.blob_bytes, st, t, c, m.ctx, m.rng, m.A2,
+                      m.sel, m.verd0, m.verd1, m.vcbits, n_vcbits, B, m.words_v, m.cache, adv ? *adv : AdvArgs{});
+  };
+  GRID_CUDA(!adv ? row(k_row<0>) : adv->n_steps <= 1 ? row(k_row<1>) : row(k_row<2>));
   if (ev) GRID_CUDA(cudaEventRecord(ev[1], st));
   const int cd_blocks = (s->max_cd + 256 * kFilterPer - 1) / (256 * kFilterPer);
   const int vc_blocks = (s->max_vc + 256 * kFilterPer - 1) / (256 * kFilterPer);
