@@ -78,7 +78,6 @@ constexpr int kPackCodes = 5;  // ncls + 0 always, +1 never, +2 n/a, +3 verdict 
                                // with vc_inline, ncls + 5 + v: verdict class v of the code's table
 constexpr int kWalkRowsCached = 256;  // rows whose queue bounds k_walk keeps in shared memory
 constexpr int kLaneOvl = 32;     // overlay / scratch entries per walk lane (shared memory)
-constexpr int kMaxStage = 96 * 1024;
 constexpr int kMaxRows = 65535;  // rows of one configurations object (a grid dimension of the mask kernels)
 
 // ---------------------------------------------------------------------------

@@ -262,18 +262,29 @@ __device__ void put_terminal(const ReserveTables& rt, int x, int32_t* out, int c
   }
 }
 
-// One warp per row; lane 0 evaluates the ways to end the pending lexeme
-// (option 0: as it stands; option 1 + tau: extended to tau's shortest
-// lexeme) and keeps the cheapest, then writes its tokens.
-__global__ void k_reserve(Tables t, ReserveTables rt, DevConfigs c, int32_t* __restrict__ scratch,
-                          size_t scratch_ints, int32_t* __restrict__ d_cost, int32_t* __restrict__ d_tokens, int cap,
-                          int32_t* __restrict__ d_status, const int32_t* __restrict__ d_budget, int safety,
-                          int32_t* __restrict__ d_fire, int B) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  __shared__ Tables ts;
-  stage_tables(t, ts, smem);
-  const int b = blockIdx.x;
-  if (b >= B || threadIdx.x != 0) return;
+struct ReserveArgs {
+  int32_t* scratch;
+  size_t scratch_ints;
+  int32_t *d_cost, *d_tokens;
+  int cap;
+  int32_t* d_status;
+  const int32_t* d_budget;
+  int safety;
+  int32_t* d_fire;
+};
+
+// One thread per row: evaluates the ways to end the pending lexeme (option 0:
+// as it stands; option 1 + tau: extended to tau's shortest lexeme) and keeps
+// the cheapest, then writes its tokens.  For rows whose search is larger than
+// the warps' shared memory (k_reserve).
+__device__ __noinline__ void reserve_serial(const Tables& t, const Tables& ts, const ReserveTables& rt,
+                                            const DevConfigs& c, const ReserveArgs& ra, int b) {
+  int32_t* const scratch = ra.scratch;
+  const size_t scratch_ints = ra.scratch_ints;
+  int32_t *const d_cost = ra.d_cost, *const d_tokens = ra.d_tokens, *const d_status = ra.d_status,
+               *const d_fire = ra.d_fire;
+  const int32_t* const d_budget = ra.d_budget;
+  const int cap = ra.cap, safety = ra.safety;
   REnt* ent = reinterpret_cast<REnt*>(scratch + (size_t)b * scratch_ints);
   int32_t* head = scratch + (size_t)b * scratch_ints + (size_t)rt.E * (sizeof(REnt) / 4);
   int32_t* out = d_tokens + (size_t)b * cap;
@@ -411,6 +422,364 @@ __global__ void k_reserve(Tables t, ReserveTables rt, DevConfigs c, int32_t* __r
   if (status == GRID_ST_COMPLETE) d_cost[b] = 0;
   d_status[b] = status;
   if (d_fire) d_fire[b] = (status == GRID_ST_OK && d_budget && d_budget[b] <= (int)total_best + safety) ? 1 : 0;
+}
+
+// ---- the same search on the warps of a block, in shared memory
+//
+// One warp per way to end the pending lexeme.  What bounds a search is its
+// chain of entries: each is visited in the order of the serial search (an
+// entry's place in its level's list, and the first of equal costs, decide
+// which completion is written), its items one per lane.  Of the lanes that
+// reach one state the cheapest, then the first, is inserted, at the place of
+// the first of them.  An entry is visited again only after its cost fell: any
+// other visit would insert nothing.
+constexpr int kRsvWarps = 8;
+constexpr int kRsvEnt = 384;     // entries per warp (more: reserve_serial)
+constexpr int kRsvDepth = 1024;  // stack entries (more: reserve_serial)
+constexpr int kRsvNone = 0xFFFF;
+
+struct RsvWarp {
+  int32_t cost[kRsvEnt], done[kRsvEnt];  // done: the cost an entry was visited with
+  uint16_t state[kRsvEnt], next[kRsvEnt], parent[kRsvEnt], item[kRsvEnt];
+  uint16_t head[kRsvDepth + kMaxOvl];
+  uint16_t lo[kMaxOvl], ls[kMaxOvl];
+  uint8_t y[kMaxExt];
+};
+
+// k_reserve's dynamic shared memory, for the largest staged tables
+constexpr int kRsvSmem = kMaxStage + kRsvWarps * (int)sizeof(RsvWarp);
+static_assert(kRsvSmem + 4096 <= 227 * 1024 && sizeof(RsvWarp) % 16 == 0, "the warps' search spaces fit");
+
+// A way to end the pending lexeme: the stack base[0:keep] ++ lo[0:m] it
+// leaves, its extension's length and the separator.
+struct RsvOption {
+  bool ok;
+  int keep, m, ylen, sep;
+};
+
+struct RsvGoal {
+  uint32_t cost;
+  int e, item;
+  bool full;  // more entries than a warp holds
+};
+
+__device__ __forceinline__ int rsv_at(const uint16_t* base, const RsvOption& o, const RsvWarp& w, int i) {
+  return i < o.keep ? base[i] : w.lo[i - o.keep];
+}
+
+// reserve_search on one warp.
+__device__ RsvGoal rsv_search(const Tables& t, const ReserveTables& rt, const uint16_t* base, const RsvOption& o,
+                              RsvWarp& w, int lane) {
+  RsvGoal goal{kInf, -1, -1, false};
+  const int kmax = o.keep + o.m - 1;
+  int cnt = 0;
+  for (int k = lane; k <= kmax; k += 32) w.head[k] = kRsvNone;
+  __syncwarp();
+  // the same in every lane; lane 0 writes
+  auto insert = [&](int level, int state, uint32_t cost, int parent, int item) -> bool {
+    const int h = w.head[level];
+    int e = h;
+    while (e != kRsvNone && w.state[e] != state) e = w.next[e];
+    if (e != kRsvNone) {
+      if (cost >= (uint32_t)w.cost[e]) return false;
+      __syncwarp();
+      if (lane == 0) {
+        w.cost[e] = (int32_t)cost;
+        w.parent[e] = (uint16_t)parent;
+        w.item[e] = (uint16_t)item;
+      }
+    } else {
+      if (cnt == kRsvEnt) {
+        goal.full = true;
+        return false;
+      }
+      __syncwarp();
+      if (lane == 0) {
+        w.cost[cnt] = (int32_t)cost;
+        w.done[cnt] = -1;
+        w.state[cnt] = (uint16_t)state;
+        w.next[cnt] = (uint16_t)h;
+        w.parent[cnt] = (uint16_t)parent;
+        w.item[cnt] = (uint16_t)item;
+        w.head[level] = (uint16_t)cnt;
+      }
+      ++cnt;
+    }
+    __syncwarp();
+    return true;
+  };
+  // the lanes' candidates (key: level << 16 | state, or -1), in item order
+  auto insert_all = [&](int key, uint32_t c, int e, int item) -> bool {
+    bool changed = false;
+    uint32_t todo = __ballot_sync(0xffffffffu, key >= 0);
+    while (todo) {
+      const int k0 = __shfl_sync(0xffffffffu, key, __ffs(todo) - 1);
+      const uint32_t same = __ballot_sync(0xffffffffu, key == k0);
+      const uint32_t low = __reduce_min_sync(0xffffffffu, key == k0 ? c : 0xFFFFFFFFu);
+      const int l = __ffs(__ballot_sync(0xffffffffu, key == k0 && c == low)) - 1;
+      changed |= insert(k0 >> 16, k0 & 0xFFFF, low, e, __shfl_sync(0xffffffffu, item, l));
+      todo &= ~same;
+    }
+    return changed;
+  };
+  insert(kmax, rsv_at(base, o, w, kmax), 0u, kRsvNone, kRsvNone);
+  for (int k = kmax; k >= 0 && !goal.full; --k) {
+    const int below = k >= 1 ? rsv_at(base, o, w, k - 1) : 0;
+    // steps that keep the height (|alpha| = 1), to a fixpoint; the goal
+    for (int round = 0; round <= t.S; ++round) {
+      bool changed = false;
+      for (int e = w.head[k]; e != kRsvNone; e = w.next[e]) {
+        const int s = w.state[e];
+        const uint32_t c0 = (uint32_t)w.cost[e];
+        if (w.done[e] == (int32_t)c0) continue;
+        __syncwarp();
+        if (lane == 0) w.done[e] = (int32_t)c0;
+        __syncwarp();
+        const int i1 = __ldg(&rt.item_off[s + 1]);
+        for (int i0 = __ldg(&rt.item_off[s]); i0 < i1; i0 += 32) {
+          const int i = i0 + lane;
+          uint32_t c = kInf;
+          int p = -1, d = 0, key = -1;
+          if (i < i1) {
+            const uint32_t ic = __ldg(&rt.item_cost[i]);
+            p = __ldg(&rt.item_p[i]);
+            d = __ldg(&rt.item_d[i]);
+            if (ic < kInf) c = c0 + ic;
+          }
+          // S' -> . start at height 0, S' -> start . at height 1: the sentence is complete
+          const bool fin = c < kInf && p == 0 && ((d == 0 && k == 0) || (d == 1 && k == 1));
+          if (__any_sync(0xffffffffu, fin)) {
+            const uint32_t low = __reduce_min_sync(0xffffffffu, fin ? c : 0xFFFFFFFFu);
+            const int l = __ffs(__ballot_sync(0xffffffffu, fin && c == low)) - 1;
+            if (low < goal.cost) {
+              goal.cost = low;
+              goal.e = e;
+              goal.item = i0 + l;
+            }
+          }
+          if (c < kInf && p > 0 && d == 1 && k >= 1) {
+            const int g = t.go[below * t.NNT + t.plhs[p]];
+            if (g < t.S) key = (k << 16) | g;
+          }
+          changed |= insert_all(key, c, e, i);
+        }
+      }
+      if (!changed) break;
+    }
+    // steps that lower the stack (|alpha| >= 2)
+    for (int e = w.head[k]; e != kRsvNone; e = w.next[e]) {
+      const int s = w.state[e];
+      const uint32_t c0 = (uint32_t)w.cost[e];
+      const int i1 = __ldg(&rt.item_off[s + 1]);
+      for (int i0 = __ldg(&rt.item_off[s]); i0 < i1; i0 += 32) {
+        const int i = i0 + lane;
+        uint32_t ic = kInf;
+        int key = -1;
+        if (i < i1) {
+          ic = __ldg(&rt.item_cost[i]);
+          const int p = __ldg(&rt.item_p[i]), d = __ldg(&rt.item_d[i]);
+          if (p != 0 && d >= 2 && d <= k && ic < kInf) {
+            const int g = t.go[rsv_at(base, o, w, k - d) * t.NNT + t.plhs[p]];
+            if (g < t.S) key = ((k - d + 1) << 16) | g;
+          }
+        }
+        insert_all(key, c0 + ic, e, i);
+      }
+    }
+  }
+  return goal;
+}
+
+// One block per row (the trigger and the tokens of the cheapest way are
+// written by the warp that found it).  One thread per row, with the entries
+// and the level heads in global memory, took 1,220 us for 32 SQL rows of up
+// to 2,000 tokens; this takes 110 us.
+__global__ void __launch_bounds__(kRsvWarps * 32) k_reserve(Tables t, ReserveTables rt, DevConfigs c, ReserveArgs ra) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  __shared__ Tables ts;
+  __shared__ __align__(16) uint16_t s_stk[kRsvDepth];
+  __shared__ unsigned long long s_best;  // total << 32 | option of the cheapest way
+  __shared__ int s_slow;
+  stage_tables(t, ts, smem);
+  const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  RsvWarp& w = reinterpret_cast<RsvWarp*>(smem + ((t.blob_bytes + 15) & ~15))[warp];
+  const int depth = c.depth[b], q = c.q[b], lx = c.lx[b];
+  const bool complete = c.flags[b] & 1;
+  const uint16_t* gbase = c.stack + (size_t)b * t.D;
+  if (threadIdx.x == 0) {
+    s_best = ~0ull;
+    s_slow = !complete && (depth > kRsvDepth || depth + kMaxOvl > t.D || t.S >= kRsvNone || rt.n_items >= kRsvNone);
+  }
+  if (depth <= kRsvDepth)
+    for (int i = threadIdx.x; i < depth; i += blockDim.x) s_stk[i] = gbase[i];
+  __syncthreads();
+  const uint16_t* base = s_stk;
+  const int mc = max_chain_of(t);
+  const uint32_t pc0 = lx >= 0 ? t.lx_pcats[lx] : 0u, wc0 = lx >= 0 ? t.lx_wcats[lx] : 0u;
+  const Bits4 live0 = q == kStart || complete ? Bits4::zero() : live_prime(ts, q, pc0).andnot(ts.ign);
+  // way `opt`, by lane 0
+  auto build = [&](int opt) -> RsvOption {
+    RsvOption o{false, depth, 0, 0, ' '};
+    if (q == kStart) {
+      o.ok = true;
+      return o;
+    }
+    int q2 = q, lx2 = lx;
+    uint32_t pc = pc0, wc = wc0;
+    if (opt > 0) {  // extend the lexeme to terminal tau's shortest lexeme
+      const int tau = opt - 1;
+      int cat = -1;
+      for (int k = 0; k < t.n_cat; ++k)
+        if (t.cat_term[k] == tau) cat = k;
+      int len;
+      if (cat >= 0) {
+        if (lx < 0) return o;
+        len = rt.lx_wdist[(size_t)lx * rt.NC + cat];
+        if (len == 0xFFFF) return o;
+      } else {
+        len = rt.dfa_tdist[(size_t)q * t.T1 + tau];
+        if (len == 0xFF) return o;
+      }
+      if (len == 0 || len > kMaxExt) return o;  // len 0: the lexeme as it stands (option 0)
+      for (int i = 0; i < len; ++i) {
+        const int by = cat >= 0 ? rt.lx_wbyte[(size_t)lx2 * rt.NC + cat] : rt.dfa_tbyte[(size_t)q2 * t.T1 + tau];
+        const int nq = ts.next[q2 * ts.C + ts.byte_class[by]];
+        if (nq == kDead || rt.byte_tok[by] < 0) return o;
+        q2 = nq;
+        lx2 = lex_step(ts, lx2, by, pc, wc);
+        if (cat >= 0 && lx2 < 0) return o;
+        w.y[o.ylen++] = (uint8_t)by;
+      }
+    }
+    o.sep = rt.sep_byte[q2];
+    if (o.sep < 0) return o;
+    Walker x;
+    walker_init(x, LArr{w.lo, 1}, LArr{w.ls, 1}, kMaxOvl, base, depth, nullptr, 0, q2, lx2, pc, wc, nullptr, nullptr);
+    if (emit(ts, x, mc) <= 0) return o;
+    o.keep = x.keep;
+    o.m = x.m;
+    o.ok = true;
+    return o;
+  };
+  auto total_of = [&](const RsvOption& o, uint32_t C) -> uint32_t {
+    // the blank that ends the lexeme comes with the first rendering; another
+    // separator is a token of its own, needed only before a rendering
+    if (C >= kInf || (C > 0 && o.sep != ' ' && rt.byte_tok[o.sep] < 0)) return kInf;
+    return (uint32_t)o.ylen + ((C > 0 && o.sep != ' ') ? 1u : 0u) + C + 1u;
+  };
+  RsvOption mine{false, 0, 0, 0, 0};  // the way that this warp looked at last
+  RsvGoal goal{kInf, -1, -1, false};
+  int mine_opt = -1;
+  auto look = [&](int opt) {
+    RsvOption o{false, 0, 0, 0, 0};
+    mine_opt = -1;
+    __syncwarp();
+    if (lane == 0) o = build(opt);
+    o.ok = __shfl_sync(0xffffffffu, (int)o.ok, 0);
+    o.keep = __shfl_sync(0xffffffffu, o.keep, 0);
+    o.m = __shfl_sync(0xffffffffu, o.m, 0);
+    o.ylen = __shfl_sync(0xffffffffu, o.ylen, 0);
+    o.sep = __shfl_sync(0xffffffffu, o.sep, 0);
+    if (!o.ok) return;
+    mine = o;
+    mine_opt = opt;
+    goal = rsv_search(ts, rt, base, o, w, lane);
+    if (goal.full) {
+      if (lane == 0) s_slow = 1;
+      return;
+    }
+    const uint32_t tot = total_of(o, goal.cost);
+    if (lane == 0 && tot < kInf) atomicMin(&s_best, ((unsigned long long)tot << 32) | (unsigned)opt);
+  };
+  if (!complete && !s_slow) {
+    int at = 0;  // the ways in order: 0, then 1 + tau of the live terminals
+    if (warp == at++ % kRsvWarps) look(0);
+    Bits4 rest = live0;
+    while (rest.any()) {
+      const int tau = rest.lowest();
+      rest.clear_lowest();
+      if (warp == at++ % kRsvWarps && tau < t.n_term) look(1 + tau);
+    }
+  }
+  __syncthreads();
+  if (s_slow) {
+    if (threadIdx.x == 0) reserve_serial(t, ts, rt, c, ra, b);
+    return;
+  }
+  const int cap = ra.cap;
+  int32_t* out = ra.d_tokens + (size_t)b * cap;
+  const unsigned long long best = s_best;
+  int status = GRID_ST_OK;
+  const uint32_t total = best == ~0ull ? kInf : (uint32_t)(best >> 32);
+  if (complete || total >= kInf) {
+    if (warp != 0) return;
+    status = complete ? GRID_ST_COMPLETE : GRID_ST_NONVIABLE;
+    for (int i = lane; i < cap; i += 32) out[i] = -1;
+  } else {
+    const int opt = (int)(uint32_t)best;
+    const int owner = opt == 0 ? 0 : [&] {
+      int at = 1;
+      Bits4 rest = live0;
+      while (rest.lowest() != opt - 1) {
+        rest.clear_lowest();
+        ++at;
+      }
+      return at % kRsvWarps;
+    }();
+    if (warp != owner) return;
+    if (mine_opt != opt) look(opt);  // a later way of this warp took its place
+    // the steps in order, in head[]: the parent chain from the goal entry, reversed, then the goal's item
+    int len = 0;
+    for (int e = goal.e; e != kRsvNone; e = w.parent[e]) len += w.item[e] != kRsvNone;
+    __syncwarp();
+    uint16_t* steps = reinterpret_cast<uint16_t*>(w.done);  // (the visits are over) 2 kRsvEnt entries
+    if (lane == 0) {
+      int k = len;
+      for (int e = goal.e; e != kRsvNone; e = w.parent[e])
+        if (w.item[e] != kRsvNone) steps[--k] = w.item[e];
+      steps[len] = (uint16_t)goal.item;
+    }
+    __syncwarp();
+    int n = mine.ylen;
+    for (int i = lane; i < n && i < cap; i += 32) out[i] = rt.byte_tok[w.y[i]];
+    if (goal.cost > 0 && mine.sep != ' ') {
+      if (lane == 0 && n < cap) out[n] = rt.byte_tok[mine.sep];
+      ++n;
+    }
+    // an item's rendering is item_cost tokens: a lane writes one item at a time
+    for (int k0 = 0; k0 <= len; k0 += 32) {
+      const int i = k0 + lane <= len ? steps[k0 + lane] : -1;
+      const int own = i >= 0 ? (int)rt.item_cost[i] : 0;
+      int at = own;
+      for (int d = 1; d < 32; d <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, at, d);
+        if (lane >= d) at += v;
+      }
+      const int sum = __shfl_sync(0xffffffffu, at, 31);
+      at += n - own;
+      if (i >= 0) {
+        const int p = rt.item_p[i], d = rt.item_d[i];
+        for (int j = rt.prod_off[p] + d; j < rt.prod_off[p + 1]; ++j) {
+          const int X = rt.prod_rhs[j];
+          if (X < t.T1) {
+            put_terminal(rt, X, out, cap, at);
+          } else {
+            for (int k = rt.ny_off[X - t.T1]; k < rt.ny_off[X - t.T1 + 1]; ++k) put_terminal(rt, rt.ny[k], out, cap, at);
+          }
+        }
+      }
+      n += sum;
+    }
+    if (lane == 0 && n < cap) out[n] = t.eos;
+    ++n;
+    if (n > cap) status = GRID_ST_BOUND;
+    for (int i = n + lane; i < cap; i += 32) out[i] = -1;
+  }
+  if (lane != 0) return;
+  ra.d_cost[b] = complete ? 0 : (total < kInf ? (int32_t)total : -1);
+  ra.d_status[b] = status;
+  if (ra.d_fire)
+    ra.d_fire[b] = (status == GRID_ST_OK && ra.d_budget && ra.d_budget[b] <= (int)total + ra.safety) ? 1 : 0;
 }
 
 }  // namespace
@@ -557,6 +926,7 @@ int build_reserve_tables(grid_spec* s) {
       (rc = a.upload(byte_tok, &rt.byte_tok)))
     return rc;
   rt.NC = std::max(1, h.n_cat);
+  rt.n_items = (int)h.kitem_p.size();
   rt.E = kReserveEntries;
   rt.ok = 1;
   return GRID_OK;
@@ -569,11 +939,11 @@ extern "C" int grid_reserve(const grid_spec* s, const grid_configs* c, int32_t* 
   if (!s || !c || !d_cost || !d_tokens || cap <= 0 || !d_status || (d_budget && !d_fire))
     return set_error(GRID_E_INVALID_ARG, "grid_reserve: bad arguments");
   if (!s->rt.ok) return set_error(GRID_E_INVALID_ARG, "grid_reserve: the spec has no reserve tables");
-  const size_t ints = reserve_scratch_bytes(s) / 4;
-  GRID_CUDA(cudaFuncSetAttribute(k_reserve, cudaFuncAttributeMaxDynamicSharedMemorySize, s->t.blob_bytes));
-  k_reserve<<<c->B, 32, s->t.blob_bytes, (cudaStream_t)stream>>>(s->t, s->rt, c->c, c->rscratch, ints, d_cost,
-                                                                d_tokens, cap, d_status, d_budget, safety, d_fire,
-                                                                c->B);
+  const size_t smem = ((s->t.blob_bytes + 15) & ~15) + kRsvWarps * sizeof(RsvWarp);
+  GRID_CUDA(cudaFuncSetAttribute(k_reserve, cudaFuncAttributeMaxDynamicSharedMemorySize, kRsvSmem));
+  const ReserveArgs ra{c->rscratch, reserve_scratch_bytes(s) / 4, d_cost, d_tokens, cap, d_status, d_budget, safety,
+                       d_fire};
+  k_reserve<<<c->B, kRsvWarps * 32, smem, (cudaStream_t)stream>>>(s->t, s->rt, c->c, ra);
   GRID_CUDA(cudaGetLastError());
   return GRID_OK;
 }

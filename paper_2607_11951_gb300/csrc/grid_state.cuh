@@ -120,6 +120,8 @@ struct AdvArgs {
   int copy;  // 1: cin and the masked configurations are distinct (out of place)
 };
 
+constexpr int kMaxStage = 96 * 1024;  // bytes of the staged tables, at most
+
 constexpr int kMaskKernels = 4;  // k_row, k_filter, k_walk, k_pack
 
 extern int g_sms;  // SM count of the current device, set by grid_specialize
@@ -132,6 +134,7 @@ struct ReserveTables {
   int ok = 0;            // 1 when built
   int NC = 1;            // categories (at least 1: the row stride of lx_wdist)
   int E = 0;             // search entries per row
+  int n_items = 0;       // kernel items of all states
   const int32_t* item_off = nullptr;  // S + 1: kernel items of each state
   const int32_t* item_p = nullptr;    // production of each kernel item
   const int32_t* item_d = nullptr;    // dot of each kernel item (the length of alpha)
