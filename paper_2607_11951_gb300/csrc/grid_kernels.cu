@@ -561,6 +561,10 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(Tables t, DevConfigs 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int b = blockIdx.x;
   RowCtx& r = ctx[b];
+  if (ADV && adv.skip && adv.skip[b]) {  // a row that is done with: its mask and status stay as they are
+    if (threadIdx.x == 0) r.complete = 2;
+    return;
+  }
   const uint16_t* base = c.stack + (size_t)b * t.D;
   const bool vec = ADV == 0 && t.D % 8 == 0 && kStackWin / 8 <= kRowWarps * 32;
   uint4 sv = make_uint4(0u, 0u, 0u, 0u);
@@ -901,6 +905,8 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(Tables t, DevConfigs 
     r.nvs[0] = 0;
     r.nvs[1] = 0;
     r.nrng = s_nrng;
+    r.fcnt = 0;
+    r.fid = 0x7FFFFFFF;
   }
   for (int i = threadIdx.x; i < m1; i += blockDim.x) r.ovl1[i] = s_ovl1[i];
   if (threadIdx.x == 0) r.status = s_adv[0] != GRID_ST_OK ? s_adv[0] : (complete ? GRID_ST_COMPLETE : s_status);
@@ -1243,16 +1249,21 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 2) k_walk(Tables t, RowCtx* _
 // whose ids are all rejected is written with -inf without being read, a mixed
 // sector is read, blended and written, an accepted sector is not touched.
 constexpr int kPackWords = 256;
-template <int APPLY, bool CACHE>
+//
+// With FORCE (a step of grid_forced_span) the last block of a row also finds
+// the row's forced token: where the step's status is OK and the mask holds
+// exactly one bit, that id is appended to the span and is the next step's
+// token; any other row stops.  Rows that stopped before are left alone.
+template <int APPLY, bool CACHE, bool FORCE = false>
 __global__ void __launch_bounds__(kPackWords) k_pack(Tables t, RowCtx* __restrict__ ctx, const uint32_t* __restrict__ sel,
                                                      const uint32_t* __restrict__ vcbits, int vcw,
                                                      const uint32_t* __restrict__ verd0,
                                                      const uint32_t* __restrict__ verd1, int words_v,
                                                      uint32_t* __restrict__ mask, int32_t* __restrict__ d_status,
                                                      void* __restrict__ logits, long long stride, int vec_ok,
-                                                     CacheDev cache) {
+                                                     CacheDev cache, ForceArgs force) {
   extern __shared__ __align__(16) uint32_t s_dyn[];  // class selections (2 nselw) | verdict-class bits (2 vcw)
-  __shared__ int s_fl, s_tb, s_any, s_hit, s_fill, s_q;
+  __shared__ int s_fl, s_tb, s_any, s_hit, s_fill, s_q, s_cnt, s_id;
   const int b = blockIdx.y;
   const int wi = blockIdx.x * kPackWords + threadIdx.x;
   const bool have = wi < t.W;
@@ -1272,8 +1283,12 @@ __global__ void __launch_bounds__(kPackWords) k_pack(Tables t, RowCtx* __restric
   const RowCtx& rc = ctx[b];
   if (threadIdx.x == 0) {
     s_tb = rc.tbl0;
-    s_fl = (rc.emit_ok ? 1 : 0) | (rc.eos_ok ? 2 : 0) | (rc.complete ? 4 : 0);
+    s_fl = (rc.emit_ok ? 1 : 0) | (rc.eos_ok ? 2 : 0) | (rc.complete ? 4 : 0) | (rc.complete == 2 ? 8 : 0);
     s_any = 0;
+    if (FORCE) {
+      s_cnt = 0;
+      s_id = 0x7FFFFFFF;
+    }
     s_hit = CACHE ? rc.chit : -1;
     s_fill = CACHE ? rc.cfill : -1;
     s_q = rc.q;
@@ -1287,6 +1302,7 @@ __global__ void __launch_bounds__(kPackWords) k_pack(Tables t, RowCtx* __restric
   }
   __syncthreads();
   const int fl = s_fl, tb = s_tb, hit = CACHE ? s_hit : -1, fill = CACHE ? s_fill : -1;
+  if (fl & 8) return;
   // a context that k_row did not select for (a completed row, sigma' without
   // a forced emission, sigma without a table) selects no class
   const uint32_t v0 = (t.ci_on && !(fl & 4) && tb >= 0) ? 1u : 0u, v1 = (t.ci_on && !(fl & 4) && (fl & 1)) ? 1u : 0u;
@@ -1386,6 +1402,10 @@ __global__ void __launch_bounds__(kPackWords) k_pack(Tables t, RowCtx* __restric
   if (have) {
     mask[(size_t)b * t.W + wi] = m;
     if (m) s_any = 1;
+    if (FORCE && m) {
+      atomicAdd(&s_cnt, __popc(m));
+      atomicMin(&s_id, 32 * wi + __ffs(m) - 1);
+    }
   }
   if (APPLY && have) {
     using T = typename std::conditional<APPLY == 1, uint32_t, uint16_t>::type;
@@ -1439,11 +1459,27 @@ __global__ void __launch_bounds__(kPackWords) k_pack(Tables t, RowCtx* __restric
   // set a bit; the row's last block writes the status (and marks a cache
   // entry the row filled ready: all blocks have written their words)
   if (threadIdx.x == 0) {
+    if (FORCE && s_cnt) {
+      atomicAdd(&ctx[b].fcnt, s_cnt);
+      atomicMin(&ctx[b].fid, s_id);
+      __threadfence();
+    }
     const unsigned long long old = atomicAdd(&ctx[b].pack_done, 1ull + (s_any ? (1ull << 32) : 0ull));
     if ((uint32_t)old == gridDim.x - 1) {
       int st = atomicAdd(&ctx[b].status, 0);
       if (st == GRID_ST_OK && (old >> 32) == 0ull && !s_any) st = GRID_ST_EMPTY_MASK;
       d_status[b] = st;
+      if (FORCE) {
+        __threadfence();
+        const bool one = st == GRID_ST_OK && atomicAdd(&ctx[b].fcnt, 0) == 1;
+        const int id = atomicMin(&ctx[b].fid, 0x7FFFFFFF);
+        if (one) {
+          force.span[(size_t)b * force.max_span + force.pos] = id;
+          force.span_len[b] = force.pos + 1;
+        }
+        force.tok[b] = one ? id : -1;
+        force.stop[b] = one ? 0 : 1;
+      }
       if (CACHE && fill >= 0) {
         __threadfence();
         atomicExch(cache.hdr + (size_t)fill * 16, 2u);
@@ -1640,6 +1676,7 @@ static int set_smem_limits() {
   GRID_CUDA(cudaFuncSetAttribute(k_events, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
   // k_pack: one row's class selections and verdict-class bits, two contexts
   GRID_CUDA(cudaFuncSetAttribute(k_pack<0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
+  GRID_CUDA(cudaFuncSetAttribute(k_pack<0, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
   GRID_CUDA(cudaFuncSetAttribute(k_pack<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
   GRID_CUDA(cudaFuncSetAttribute(k_pack<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
   GRID_CUDA(cudaFuncSetAttribute(k_pack<0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
@@ -2211,7 +2248,7 @@ extern "C" int grid_configs_create(const grid_spec* s, int32_t B, grid_configs**
       (rc = a.alloc((size_t)B * 2 * std::max(1, s->vcw) * 4, (void**)&c->vcbits)) ||
       (rc = a.alloc((size_t)B * 2 * std::max(1, s->max_cd) * 4, (void**)&c->surv)) ||
       (rc = a.alloc((size_t)B * 2 * c->vcap * 4, (void**)&c->vsurv)) ||
-      (rc = a.alloc((size_t)B * 4 * 4, (void**)&c->aux)) ||
+      (rc = a.alloc((size_t)B * 2 * 4, (void**)&c->aux)) ||
       (rc = a.alloc((size_t)B * reserve_scratch_bytes(s), (void**)&c->rscratch))) {
     grid_configs_free(c);
     return rc;
@@ -2261,7 +2298,7 @@ extern "C" int grid_advance(const grid_spec* s, const grid_configs* in, grid_con
 // recorded before the first kernel and after each.
 int grid::launch_masks(const grid_spec* s, const DevConfigs& c, const MaskScratch& m, int B, uint32_t* d_mask,
                        int32_t* d_status, cudaStream_t st, const cudaEvent_t* ev, const FusedLogits& lg,
-                       const AdvArgs* adv) {
+                       const AdvArgs* adv, const ForceArgs* force) {
   const Tables& t = s->t;
   const int vcw = std::max(1, s->vcw);
   const int n_vcbits = B * 2 * vcw;
@@ -2297,12 +2334,15 @@ int grid::launch_masks(const grid_spec* s, const DevConfigs& c, const MaskScratc
   auto pack = [&](auto kern) {
     return launch_pdl(kern, pgrid, dim3(kPackWords), psmem, st, t, m.ctx, (const uint32_t*)m.sel,
                       (const uint32_t*)m.vcbits, vcw, (const uint32_t*)m.verd0, (const uint32_t*)m.verd1, m.words_v,
-                      d_mask, d_status, lg.p, (long long)lg.stride, lg.p ? vec_ok : 0, m.cache);
+                      d_mask, d_status, lg.p, (long long)lg.stride, lg.p ? vec_ok : 0, m.cache,
+                      force ? *force : ForceArgs{});
   };
   const bool cached = m.cache.n > 0;
   const int mode = !lg.p ? 0 : (lg.dtype == GRID_DTYPE_F32 ? 1 : 2);
   cudaError_t pe;
-  if (mode == 0)
+  if (force)  // (a span's step has neither logits nor a cache)
+    pe = pack(k_pack<0, false, true>);
+  else if (mode == 0)
     pe = cached ? pack(k_pack<0, true>) : pack(k_pack<0, false>);
   else if (mode == 1)
     pe = cached ? pack(k_pack<1, true>) : pack(k_pack<1, false>);
@@ -2435,7 +2475,7 @@ extern "C" int grid_advance_masks(const grid_spec* s, const grid_configs* in, gr
   lg.p = d_logits;
   lg.dtype = dtype;
   lg.stride = row_stride;
-  const AdvArgs adv{in->c, d_tokens, n_steps, in != out ? 1 : 0};
+  const AdvArgs adv{in->c, d_tokens, n_steps, in != out ? 1 : 0, nullptr};
   return launch_masks(s, out->c, m, out->B, d_mask, d_status, (cudaStream_t)stream, out->ev[0] ? out->ev : nullptr,
                       lg, &adv);
 }

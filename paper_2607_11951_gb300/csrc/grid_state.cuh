@@ -27,7 +27,7 @@ struct RowCtx {
   uint32_t A1[4];   // allowed terminals at sigma' (after the forced emission)
   int32_t q, lx, depth, tbl0;
   uint32_t pc0, wc0;  // category bits of the pending lexeme's trie node
-  int32_t emit_ok, eos_ok, status, complete;
+  int32_t emit_ok, eos_ok, status, complete;  // complete: 2 = the row is left out of the step
   unsigned long long pack_done;  // k_pack blocks done with the row (low half) and with a set bit (high half)
   int32_t keep1, m1;
   int32_t work0;          // next item of the row's walk queue
@@ -35,6 +35,7 @@ struct RowCtx {
   int32_t nsurv[2];       // CD spellings that survived k_filter, per context (0: sigma, 1: sigma')
   int32_t nvs[2];         // verdict classes that survived k_filter, per context
   int32_t nrng;
+  int32_t fcnt, fid;    // a span's step: bits set in the mask, the lowest
   int32_t chit, cfill;  // mask-cache entry this row reads (hit) or fills (miss), or -1
   uint32_t kill[8];  // bit b: first byte b ends the pending lexeme
   uint16_t ovl1[kMaxOvl];
@@ -118,6 +119,13 @@ struct AdvArgs {
   const int32_t* tokens;
   int n_steps;
   int copy;  // 1: cin and the masked configurations are distinct (out of place)
+  const int32_t* skip;  // rows to leave out of the step (their masks and statuses stay), or NULL
+};
+
+// The forced tokens that a step of grid_forced_span finds, for position `pos`.
+struct ForceArgs {
+  int32_t *span, *span_len, *tok, *stop;
+  int pos, max_span;
 };
 
 constexpr int kMaxStage = 96 * 1024;  // bytes of the staged tables, at most
@@ -184,7 +192,7 @@ struct grid_configs {
   int32_t* surv = nullptr;
   int32_t* vsurv = nullptr;
   int cap = 0, vcap = 0;
-  int32_t* aux = nullptr;  // 4 x B ints of per-row working state for forced spans and reserves
+  int32_t* aux = nullptr;  // 2 x B ints of per-row working state for forced spans
   int32_t* rscratch = nullptr;  // per-row search space of grid_reserve (entries and level heads)
   // audit chain (grid_configs_enable_audit): node hashes (c.hs), per-row
   // chain heads (16 bytes) and record counters
@@ -199,10 +207,11 @@ namespace grid {
 // The four kernels of one mask step (k_row, k_filter, k_walk, k_pack) on
 // `st`; `ev` (5 events or NULL) is recorded before the first kernel and after
 // each.  With lg.p set, k_pack also masks the logits; with adv set, k_row
-// first feeds adv's tokens into c.
+// first feeds adv's tokens into c; with force set, k_pack also finds the rows'
+// forced tokens.
 int launch_masks(const grid_spec* s, const DevConfigs& c, const MaskScratch& m, int B, uint32_t* d_mask,
                  int32_t* d_status, cudaStream_t st, const cudaEvent_t* ev, const FusedLogits& lg = FusedLogits(),
-                 const AdvArgs* adv = nullptr);
+                 const AdvArgs* adv = nullptr, const ForceArgs* force = nullptr);
 
 // The parser step (k_advance) of B rows from `in` into `out` (copy = 1: out
 // of place) on `st`.
