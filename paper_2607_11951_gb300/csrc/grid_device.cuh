@@ -45,7 +45,11 @@ constexpr int kMaxEv = kRecLen - 2;
 struct Bits4 {
   uint32_t x, y, z, w;
   __host__ __device__ __forceinline__ static Bits4 zero() { return Bits4{0u, 0u, 0u, 0u}; }
-  __device__ __forceinline__ static Bits4 load(const uint32_t* p) { return Bits4{p[0], p[1], p[2], p[3]}; }
+  // (p is 16-byte aligned)
+  __device__ __forceinline__ static Bits4 load(const uint32_t* p) {
+    const uint4 v = *reinterpret_cast<const uint4*>(p);
+    return Bits4{v.x, v.y, v.z, v.w};
+  }
   __device__ __forceinline__ uint32_t word(int i) const { return i == 0 ? x : (i == 1 ? y : (i == 2 ? z : w)); }
   __device__ __forceinline__ bool has(int t) const { return (word(t >> 5) >> (t & 31)) & 1u; }
   __device__ __forceinline__ void set(int t) {
@@ -150,6 +154,42 @@ struct Tables {
   // per lexer state q and category bits c, at q << n_cat | c (lexeme_tables):
   const uint64_t* ev_list;  // the emission's candidates (LexBatch::ev; 0: none, count 0x7F: more than it holds)
   const uint32_t* live_any; // bit set: a lexeme there is live
+  // byte offsets of the staged block's arrays in it
+  int o_class, o_next, o_acc, o_live, o_action, o_go, o_lhs, o_shift, o_roff, o_rp, o_red, o_lany;
+};
+
+extern __shared__ __align__(16) uint8_t smem[];
+
+// The tables as a kernel's parameter reads them: where the block is staged,
+// from its place in dynamic shared memory.  The parameter stays in constant
+// memory and the offsets are operands of the address arithmetic, with 32-bit
+// shared-memory loads; a descriptor in shared memory, rebased onto the block,
+// cost a look-up of the pointer and a generic 64-bit load per access, and its
+// copying by each block.
+template <bool STAGED>
+struct TabT : Tables {
+  TabT() = default;
+  explicit TabT(const Tables& t) : Tables(t) {}
+  template <typename E>
+  __device__ __forceinline__ E get(const E* p, int o, int i) const {
+    return STAGED ? reinterpret_cast<const E*>(smem + o)[i] : p[i];
+  }
+  __device__ __forceinline__ Bits4 get4(const uint32_t* p, int o, int i) const {
+    const uint4 v = STAGED ? reinterpret_cast<const uint4*>(smem + o)[i] : reinterpret_cast<const uint4*>(p)[i];
+    return Bits4{v.x, v.y, v.z, v.w};
+  }
+  __device__ __forceinline__ int cls(int b) const { return get(byte_class, o_class, b); }
+  __device__ __forceinline__ int nxt(int i) const { return get(next, o_next, i); }
+  __device__ __forceinline__ int act(int i) const { return get(action, o_action, i); }
+  __device__ __forceinline__ int gto(int i) const { return get(go, o_go, i); }
+  __device__ __forceinline__ int lhs(int p) const { return get(plhs, o_lhs, p); }
+  __device__ __forceinline__ uint32_t roff(int s) const { return get(red_off, o_roff, s); }
+  __device__ __forceinline__ int rp(int e) const { return get(red_p, o_rp, e); }
+  __device__ __forceinline__ Bits4 acc4(int q) const { return get4(acc, o_acc, q); }
+  __device__ __forceinline__ Bits4 live4(int q) const { return get4(live, o_live, q); }
+  __device__ __forceinline__ Bits4 shift4(int s) const { return get4(shift_mask, o_shift, s); }
+  __device__ __forceinline__ Bits4 red4(int e) const { return get4(red_mask, o_red, e); }
+  __device__ __forceinline__ bool live_any_at(int i) const { return (get(live_any, o_lany, i >> 5) >> (i & 31)) & 1u; }
 };
 
 // Work counters of a walk, kept in the lane's registers when the walk is
@@ -164,18 +204,17 @@ __device__ __forceinline__ void count_work(uint32_t* ctr, int k) {
 // Membership test in a 4-word set stored in memory.
 __device__ __forceinline__ bool bit4(const uint32_t* m, int t) { return (m[t >> 5] >> (t & 31)) & 1u; }
 
-// Copy the staged block into shared memory and publish one block-wide copy of
-// the table descriptor, rebased onto it, in shared memory (`ts`).  Every thread
-// of the block must call this.
-// Copy the staged block into shared memory with one bulk asynchronous copy
-// (the block is 16-byte aligned and a multiple of 16 bytes), completion
+// Copy the staged block into shared memory (at the start of the kernel's
+// dynamic shared memory, where TabT<true> reads it) with one bulk asynchronous
+// copy (the block is 16-byte aligned and a multiple of 16 bytes), completion
 // tracked by an mbarrier.  The wait is bounded; if it gives up, the block is
 // copied again with plain loads (same bytes), so the result never depends on
-// the bulk copy finishing.
-__device__ __forceinline__ void stage_tables(const Tables& t, Tables& ts, uint8_t* smem) {
-  __shared__ __align__(8) uint64_t s_bar;
-  __shared__ int s_late;
-  if (t.blob_bytes) {
+// the bulk copy finishing.  Every thread of the block must call this.
+template <bool STAGED>
+__device__ __forceinline__ void stage_tables(const TabT<STAGED>& t) {
+  if constexpr (STAGED) {
+    __shared__ __align__(8) uint64_t s_bar;
+    __shared__ int s_late;
     const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&s_bar);
     if (threadIdx.x == 0) {
       s_late = 0;
@@ -203,28 +242,9 @@ __device__ __forceinline__ void stage_tables(const Tables& t, Tables& ts, uint8_
       const uint4* src = reinterpret_cast<const uint4*>(t.blob);
       uint4* dst = reinterpret_cast<uint4*>(smem);
       for (int i = threadIdx.x; i < (t.blob_bytes >> 4); i += blockDim.x) dst[i] = src[i];
+      __syncthreads();
     }
   }
-  if (threadIdx.x == 0) {
-    ts = t;
-    if (t.blob_bytes) {
-      auto rebase = [&](const void* p) { return smem + ((const uint8_t*)p - t.blob); };
-      ts.byte_class = rebase(t.byte_class);
-      ts.next = reinterpret_cast<const uint16_t*>(rebase(t.next));
-      ts.acc = reinterpret_cast<const uint32_t*>(rebase(t.acc));
-      ts.live = reinterpret_cast<const uint32_t*>(rebase(t.live));
-      ts.action = reinterpret_cast<const int16_t*>(rebase(t.action));
-      ts.go = reinterpret_cast<const uint16_t*>(rebase(t.go));
-      ts.plen = rebase(t.plen);
-      ts.plhs = reinterpret_cast<const uint16_t*>(rebase(t.plhs));
-      ts.shift_mask = reinterpret_cast<const uint32_t*>(rebase(t.shift_mask));
-      ts.red_off = reinterpret_cast<const uint32_t*>(rebase(t.red_off));
-      ts.red_p = reinterpret_cast<const uint16_t*>(rebase(t.red_p));
-      ts.red_mask = reinterpret_cast<const uint32_t*>(rebase(t.red_mask));
-      ts.live_any = reinterpret_cast<const uint32_t*>(rebase(t.live_any));
-    }
-  }
-  __syncthreads();
 }
 
 // Programmatic dependent launch: the step's kernels are launched so that each
@@ -237,7 +257,8 @@ constexpr uint32_t kHashEmpty = 0xFFFFFFFFu;
 // Child of identifier-trie node lx on byte b (-1 if none), with the child's
 // prefix / word category bits (0 when there is no child).  One 16-byte load
 // per probe; the table is at most half full, so probing ends at an empty slot.
-__device__ __forceinline__ int lex_step(const Tables& t, int lx, int b, uint32_t& pc, uint32_t& wc) {
+template <class T>
+__device__ __forceinline__ int lex_step(const T& t, int lx, int b, uint32_t& pc, uint32_t& wc) {
   pc = 0u;
   wc = 0u;
   if (lx < 0) return -1;
@@ -258,8 +279,8 @@ __device__ __forceinline__ int lex_step(const Tables& t, int lx, int b, uint32_t
 
 // Terminal set of DFA state q filtered by the lexicon: non-category terminals
 // pass, category terminal c passes iff bit c of `cats` is set.
-__device__ __forceinline__ Bits4 lex_filter(const Tables& t, const uint32_t* src, int q, uint32_t cats) {
-  const Bits4 v = Bits4::load(src + q * 4);
+template <class T>
+__device__ __forceinline__ Bits4 lex_filter(const T& t, const Bits4 v, uint32_t cats) {
   Bits4 out = v.andnot(t.cm);
   while (cats) {
     const int c = __ffs(cats) - 1;
@@ -272,13 +293,16 @@ __device__ __forceinline__ Bits4 lex_filter(const Tables& t, const uint32_t* src
 
 // live'(q, r): terminals live at q, category terminals only while r is a
 // prefix of one of their words (pc = prefix category bits of r's trie node).
-__device__ __forceinline__ Bits4 live_prime(const Tables& t, int q, uint32_t pc) { return lex_filter(t, t.live, q, pc); }
+template <class T>
+__device__ __forceinline__ Bits4 live_prime(const T& t, int q, uint32_t pc) { return lex_filter(t, t.live4(q), pc); }
 
 // Emission candidates of r: terminals accepting at q, category terminals only
 // if r is one of their words (wc = word category bits of r's trie node).
-__device__ __forceinline__ Bits4 cands(const Tables& t, int q, uint32_t wc) { return lex_filter(t, t.acc, q, wc); }
+template <class T>
+__device__ __forceinline__ Bits4 cands(const T& t, int q, uint32_t wc) { return lex_filter(t, t.acc4(q), wc); }
 
-__device__ __forceinline__ int max_chain_of(const Tables& t) { return 2 * t.D + 256; }
+template <class T>
+__device__ __forceinline__ int max_chain_of(const T& t) { return 2 * t.D + 256; }
 
 // A lane's small array: element i lives at p[i * s].  Walk lanes keep their
 // overlays in shared memory interleaved across the warp (s = 32, no bank
@@ -293,8 +317,8 @@ struct LArr {
 // (Sec. 3.2, "allowed terminals by simulation").  Returns the ACTION code that
 // ends it (> 0: shift to code-1, or kAccept), 0 on error, -1 on a bound.  On
 // shift/accept, (keep_o, m_o, scr[0:ns]) is the stack under the pushed state.
-template <typename OV>
-__device__ __forceinline__ int simulate(const Tables& t, const uint16_t* base, int keep, OV ovl, int m, int tau,
+template <class T, typename OV>
+__device__ __forceinline__ int simulate(const T& t, const uint16_t* base, int keep, OV ovl, int m, int tau,
                                         LArr scr, int cap, int& keep_o, int& m_o, int& ns, int max_chain,
                                         uint32_t* ctr = nullptr) {
   int k = keep, mm = m;
@@ -303,7 +327,7 @@ __device__ __forceinline__ int simulate(const Tables& t, const uint16_t* base, i
   for (int it = 0; it < max_chain; ++it) {
     if (top >= t.S) return 0;
     count_work(ctr, 1);
-    const int a = t.action[top * t.T1 + tau];
+    const int a = t.act(top * t.T1 + tau);
     if (a == 0) return 0;
     if (a > 0) {
       keep_o = k;
@@ -324,7 +348,7 @@ __device__ __forceinline__ int simulate(const Tables& t, const uint16_t* base, i
     if (top2 >= t.S) return 0;
     if (ns >= cap) return -1;
     count_work(ctr, 2);
-    top = t.go[top2 * t.NNT + (code & 1023)];
+    top = t.gto(top2 * t.NNT + (code & 1023));
     scr[ns++] = (uint16_t)top;
   }
   return -1;
@@ -339,8 +363,8 @@ __device__ __forceinline__ int simulate(const Tables& t, const uint16_t* base, i
 // rest is simulated one terminal at a time.  `bound` is set on a bound.
 constexpr int kSetRounds = 8;
 
-template <typename OV>
-__device__ __forceinline__ Bits4 simulate_set(const Tables& t, const uint16_t* base, int keep, OV ovl, int m, Bits4 G,
+template <class T, typename OV>
+__device__ __forceinline__ Bits4 simulate_set(const T& t, const uint16_t* base, int keep, OV ovl, int m, Bits4 G,
                                               LArr scr, int cap, int max_chain, bool& bound,
                                               uint32_t* ctr = nullptr) {
   Bits4 res = Bits4::zero();
@@ -354,17 +378,17 @@ __device__ __forceinline__ Bits4 simulate_set(const Tables& t, const uint16_t* b
     for (; it < max_chain && g.any(); ++it) {
       if (top >= t.S) break;
       count_work(ctr, 1);
-      const Bits4 sh = Bits4::load(t.shift_mask + top * 4);
+      const Bits4 sh = t.shift4(top);
       res = res | (g & sh);
       g = g.andnot(sh);
       if (!g.any()) break;
       int p = -1;
       Bits4 gp = Bits4::zero();
-      for (uint32_t e = t.red_off[top]; e < t.red_off[top + 1]; ++e) {
-        const Bits4 x = g & Bits4::load(t.red_mask + e * 4);
+      for (uint32_t e = t.roff(top); e < t.roff(top + 1); ++e) {
+        const Bits4 x = g & t.red4(e);
         if (!x.any()) continue;
         if (p < 0) {
-          p = t.red_p[e];
+          p = t.rp(e);
           gp = x;
         } else {
           todo = todo | x;
@@ -388,7 +412,7 @@ __device__ __forceinline__ Bits4 simulate_set(const Tables& t, const uint16_t* b
         return res;
       }
       count_work(ctr, 2);
-      top = t.go[top2 * t.NNT + (p & 1023)];
+      top = t.gto(top2 * t.NNT + (p & 1023));
       scr[ns++] = (uint16_t)top;
     }
     if (it == max_chain && g.any()) {
@@ -464,7 +488,8 @@ __device__ __forceinline__ bool commit(Walker& w, int keep_o, int m_o, int ns, i
 
 // Apply a deferred first shift to the overlay.  The terminal is in the
 // allowed set of the stack it was deferred at, so it reaches SHIFT.
-__device__ __forceinline__ bool materialize(const Tables& t, Walker& w, int max_chain) {
+template <class T>
+__device__ __forceinline__ bool materialize(const T& t, Walker& w, int max_chain) {
   int keep_o, m_o, ns;
   const int a = simulate(t, w.base, w.keep, w.ovl, w.m, w.pend, w.scr, w.cap, keep_o, m_o, ns, max_chain, w.ctr);
   w.pend = -1;
@@ -478,7 +503,8 @@ __device__ __forceinline__ bool materialize(const Tables& t, Walker& w, int max_
 // pick is a set test; a first shift whose successor allowed set is known (A2)
 // is only recorded, and applied to the overlay when a later step needs the
 // stack itself.  Returns 1 ok, 0 reject, -1 bound.
-__device__ __forceinline__ int emit_set(const Tables& t, Walker& w, Bits4 K, int max_chain) {
+template <class T>
+__device__ __forceinline__ int emit_set(const T& t, Walker& w, Bits4 K, int max_chain) {
   while (K.any()) {
     const int tau = K.lowest();
     K.clear_lowest();
@@ -527,12 +553,14 @@ __device__ __forceinline__ int emit_set(const Tables& t, Walker& w, Bits4 K, int
   return 0;
 }
 
-__device__ __forceinline__ int emit(const Tables& t, Walker& w, int max_chain) {
+template <class T>
+__device__ __forceinline__ int emit(const T& t, Walker& w, int max_chain) {
   return emit_set(t, w, cands(t, w.q, w.wc), max_chain);
 }
 
 // Def. 2 trailing liveness for live set L.  1 / 0 / -1.
-__device__ __forceinline__ int trailing_set(const Tables& t, Walker& w, Bits4 L, int max_chain) {
+template <class T>
+__device__ __forceinline__ int trailing_set(const T& t, Walker& w, Bits4 L, int max_chain) {
   if ((L & t.ign).any()) return 1;
   if (const uint32_t* A = w.Acur) return (L & Bits4::load(A)).any() ? 1 : 0;
   if (w.pend >= 0 && !materialize(t, w, max_chain)) return -1;
@@ -549,7 +577,8 @@ __device__ __forceinline__ int trailing_set(const Tables& t, Walker& w, Bits4 L,
   return ok.any() ? 1 : 0;
 }
 
-__device__ __forceinline__ int trailing_live(const Tables& t, Walker& w, int max_chain) {
+template <class T>
+__device__ __forceinline__ int trailing_live(const T& t, Walker& w, int max_chain) {
   return trailing_set(t, w, live_prime(t, w.q, w.pc), max_chain);
 }
 
@@ -568,7 +597,8 @@ struct Spell {
   }
 };
 
-__device__ __forceinline__ Spell load_spell(const Tables& t, int s) {
+template <class T>
+__device__ __forceinline__ Spell load_spell(const T& t, int s) {
   Spell sp;
   const int off = t.spell_off[s];
   sp.len = t.spell_off[s + 1] - off;
@@ -579,13 +609,14 @@ __device__ __forceinline__ Spell load_spell(const Tables& t, int s) {
 
 // Walk one token's bytes (Sec. 4.1).  1 = the output stays a viable prefix,
 // 0 = rejected, -1 = bound.
-__device__ __forceinline__ int walk_bytes(const Tables& t, Walker& w, const Spell& sp, int max_chain) {
+template <class T>
+__device__ __forceinline__ int walk_bytes(const T& t, Walker& w, const Spell& sp, int max_chain) {
   const int len = sp.len;
   for (int i = 0; i < len; ++i) {
     count_work(w.ctr, 0);
     const int b = sp.at(i);
-    const int c = t.byte_class[b];
-    int nq = t.next[w.q * t.C + c];
+    const int c = t.cls(b);
+    int nq = t.nxt(w.q * t.C + c);
     if (nq == kDead) {
       if (w.q == kStart) return 0;
       const int e = emit(t, w, max_chain);
@@ -594,7 +625,7 @@ __device__ __forceinline__ int walk_bytes(const Tables& t, Walker& w, const Spel
       w.lx = 0;
       w.pc = t.root_pc;
       w.wc = t.root_wc;
-      nq = t.next[kStart * t.C + c];
+      nq = t.nxt(kStart * t.C + c);
       if (nq == kDead) return 0;
     }
     w.q = nq;
@@ -644,7 +675,8 @@ struct LexToken {
   Spell sp;
 };
 
-__device__ __forceinline__ LexToken lex_fetch(const Tables& t, const int32_t* tokens, int k, int n_steps, int lane) {
+template <class T>
+__device__ __forceinline__ LexToken lex_fetch(const T& t, const int32_t* tokens, int k, int n_steps, int lane) {
   const int tok = k + lane < n_steps ? tokens[k + lane] : -1;
   LexToken x;
   x.st = tok < 0 ? 0 : 2;
@@ -663,7 +695,8 @@ __device__ __forceinline__ LexToken lex_fetch(const Tables& t, const int32_t* to
 // through the bytes (two shared-memory look-ups a byte) is all that is serial;
 // the walks through the identifier trie (a dependent L2 access a byte) run a
 // lexeme per lane, once the DFA has found where the lexemes start.
-__device__ __forceinline__ void lex_batch(const Tables& t, const Tables& ts, const LexToken& own, int k, int n_steps,
+template <class T>
+__device__ __forceinline__ void lex_batch(const T& t, const T& ts, const LexToken& own, int k, int n_steps,
                                           int lane, LexState& carry, LexBatch& L) {
   const Spell& sp = own.sp;
   int st = own.st;
@@ -683,7 +716,7 @@ __device__ __forceinline__ void lex_batch(const Tables& t, const Tables& ts, con
     for (int i = 0; i < sp.len; ++i) {
       const int b = sp.at(i);
       L.byte[at + i] = (uint8_t)b;
-      L.cls[at + i] = ts.byte_class[b];
+      L.cls[at + i] = ts.cls(b);
       L.last[at + i] = i + 1 == sp.len ? (uint8_t)(lane + 1) : (uint8_t)0;
     }
   }
@@ -695,9 +728,9 @@ __device__ __forceinline__ void lex_batch(const Tables& t, const Tables& ts, con
   const int row0 = kStart * ts.C;
   for (int i = 0; i < total; ++i) {
     const int c = L.cls[i];
-    int nq = ts.next[q * ts.C + c];
+    int nq = ts.nxt(q * ts.C + c);
     if (nq == kDead) {
-      if (q != kStart) nq = ts.next[row0 + c];
+      if (q != kStart) nq = ts.nxt(row0 + c);
       if (nq == kDead) {
         bad = i;
         break;
@@ -721,7 +754,7 @@ __device__ __forceinline__ void lex_batch(const Tables& t, const Tables& ts, con
       s.q = L.q[i];
       s.lx = lex_step(ts, s.lx, L.byte[i], s.pc, s.wc);
       const int id = (s.q << ts.n_cat) | (int)s.pc;
-      if (!((ts.live_any[id >> 5] >> (id & 31)) & 1u)) break;
+      if (!ts.live_any_at(id)) break;
       if (L.last[i]) L.out[L.last[i] - 1] = s;
     }
     if (i < z) {
@@ -765,13 +798,14 @@ struct Feed {
 };
 
 // Reduce chain of tau on win[0:depth): simulate() for a stack without overlay.
-__device__ __forceinline__ int chain(const Tables& t, const uint16_t* win, int depth, int tau, uint16_t* scr,
+template <class T>
+__device__ __forceinline__ int chain(const T& t, const uint16_t* win, int depth, int tau, uint16_t* scr,
                                      int& keep_o, int& ns_o, int max_chain) {
   int k = depth, ns = 0, bk = depth;
   int top = win[k - 1], bv = top;  // bv = win[bk - 1]
   for (int it = 0; it < max_chain; ++it) {
     if (top >= t.S) return 0;
-    const int a = t.action[top * t.T1 + tau];
+    const int a = t.act(top * t.T1 + tau);
     if (a >= 0) {
       keep_o = k;
       ns_o = ns;
@@ -789,7 +823,7 @@ __device__ __forceinline__ int chain(const Tables& t, const uint16_t* win, int d
     const int top2 = ns ? scr[(ns - 1) * 32] : bv;
     if (top2 >= t.S) return 0;
     if (ns >= kChainNs) return -1;
-    top = t.go[top2 * t.NNT + (code & 1023)];
+    top = t.gto(top2 * t.NNT + (code & 1023));
     scr[ns * 32] = (uint16_t)top;
     ++ns;
   }
@@ -797,7 +831,8 @@ __device__ __forceinline__ int chain(const Tables& t, const uint16_t* win, int d
 }
 
 // Def. 2 trailing liveness of lexer state (q, pc) on win[0:depth), 32 terminals at a time.  1 / 0 / -1.
-__device__ __forceinline__ int feed_live(const Tables& t, const Feed& f, int q, uint32_t pc, int lane, int max_chain) {
+template <class T>
+__device__ __forceinline__ int feed_live(const T& t, const Feed& f, int q, uint32_t pc, int lane, int max_chain) {
   const Bits4 Lv = live_prime(t, q, pc);
   if ((Lv & t.ign).any()) return 1;
   bool ok = false, bound = false;
@@ -823,7 +858,8 @@ __device__ __forceinline__ int feed_live(const Tables& t, const Feed& f, int q, 
 // left is the test after the last token, and, where a chain could run into its
 // bound (deep stacks of grammars with long chains), the test of every token,
 // which would report that bound.
-__device__ __forceinline__ bool parse_batch(const Tables& t, Feed& f, const LexBatch& L, int k0, int lane,
+template <class T>
+__device__ __forceinline__ bool parse_batch(const T& t, Feed& f, const LexBatch& L, int k0, int lane,
                                             int max_chain) {
   const int own = L.st[lane];
   uint32_t todo = __ballot_sync(0xffffffffu, own != 0);
@@ -884,7 +920,8 @@ __device__ __forceinline__ void feed_back(Feed& f, int lane) {
 }
 
 // EOS gate (Sec. 3.2).  1 / 0 / -1.
-__device__ __forceinline__ int eos_gate(const Tables& t, Walker& w, int max_chain) {
+template <class T>
+__device__ __forceinline__ int eos_gate(const T& t, Walker& w, int max_chain) {
   if (w.q != kStart) {
     int e = emit(t, w, max_chain);
     if (e <= 0) return e;
@@ -896,20 +933,23 @@ __device__ __forceinline__ int eos_gate(const Tables& t, Walker& w, int max_chai
   return a == kAccept ? 1 : 0;
 }
 
-__device__ __forceinline__ int class_id(const Tables& t, int kind, int q, uint32_t cats) {
+template <class T>
+__device__ __forceinline__ int class_id(const T& t, int kind, int q, uint32_t cats) {
   return ((kind * t.Q + q) << t.n_cat) | (int)(cats & ((1u << t.n_cat) - 1u));
 }
 
 // Terminal set of a class id, computed from the lexer tables.
-__device__ __forceinline__ Bits4 class_terms(const Tables& t, int cls) {
+template <class T>
+__device__ __forceinline__ Bits4 class_terms(const T& t, int cls) {
   const int hi = cls >> t.n_cat;
   const uint32_t cats = (uint32_t)cls & ((1u << t.n_cat) - 1u);
   const int kind = hi / t.Q, q = hi - kind * t.Q;
-  return lex_filter(t, kind ? t.acc : t.live, q, cats);
+  return lex_filter(t, kind ? t.acc4(q) : t.live4(q), cats);
 }
 
 // The same, from the table of all class ids' sets built at specialization.
-__device__ __forceinline__ Bits4 class_set(const Tables& t, int cls) { return Bits4::load(t.cls_sets + cls * 4); }
+template <class T>
+__device__ __forceinline__ Bits4 class_set(const T& t, int cls) { return Bits4::load(t.cls_sets + cls * 4); }
 
 // Sec. 4.2 CI/CD classification of one spelling from lexer state (q, lx),
 // with the stack abstracted away.  Emissions whose first candidate is ignored
@@ -922,7 +962,8 @@ __device__ __forceinline__ Bits4 class_set(const Tables& t, int cls) { return Bi
 //                                       emissions; then `first_key` is the
 //                                       class of the first one, 0xFFFF if that
 //                                       emission always succeeds)
-__device__ __forceinline__ uint16_t classify(const Tables& t, int q, int lx, const uint8_t* bytes, int len,
+template <class T>
+__device__ __forceinline__ uint16_t classify(const T& t, int q, int lx, const uint8_t* bytes, int len,
                                              uint16_t& first_key, uint16_t* rec) {
   first_key = 0xFFFF;
   uint32_t pc = lx == 0 ? t.root_pc : 0u, wc = lx == 0 ? t.root_wc : 0u;
@@ -930,8 +971,8 @@ __device__ __forceinline__ uint16_t classify(const Tables& t, int q, int lx, con
   bool first_ign = false, overflow = false;
   for (int i = 0; i < len; ++i) {
     const int b = bytes[i];
-    const int c = t.byte_class[b];
-    int nq = t.next[q * t.C + c];
+    const int c = t.cls(b);
+    int nq = t.nxt(q * t.C + c);
     if (nq == kDead) {
       if (q == kStart) return kClsRej;
       const Bits4 K = cands(t, q, wc);
@@ -949,7 +990,7 @@ __device__ __forceinline__ uint16_t classify(const Tables& t, int q, int lx, con
       lx = 0;
       pc = t.root_pc;
       wc = t.root_wc;
-      nq = t.next[kStart * t.C + c];
+      nq = t.nxt(kStart * t.C + c);
       if (nq == kDead) return kClsRej;
     }
     q = nq;
@@ -971,7 +1012,8 @@ __device__ __forceinline__ uint16_t classify(const Tables& t, int q, int lx, con
 
 // Verdict of an event record at the walker's stack: each event is an emission
 // with the recorded candidate set, then the final liveness test.  1 / 0 / -1.
-__device__ __forceinline__ int eval_record(const Tables& t, Walker& w, const uint16_t* rec, int max_chain) {
+template <class T>
+__device__ __forceinline__ int eval_record(const T& t, Walker& w, const uint16_t* rec, int max_chain) {
   const int n = rec[0];
   for (int i = 0; i < n; ++i) {
     count_work(w.ctr, 3);

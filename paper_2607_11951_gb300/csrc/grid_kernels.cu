@@ -93,11 +93,11 @@ __global__ void k_reset(DevConfigs c, int B, int D) {
 }
 
 // ---------------- specialization ----------------
-__global__ void k_classify(Tables t, uint16_t* __restrict__ cls_sp, uint16_t* __restrict__ key_sp,
+template <bool ST>
+__global__ void k_classify(TabT<ST> t, uint16_t* __restrict__ cls_sp, uint16_t* __restrict__ key_sp,
                            int32_t* __restrict__ counts) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  __shared__ Tables ts;
-  stage_tables(t, ts, smem);
+  stage_tables(t);
+  const auto& ts = t;
   const int tbl = blockIdx.y;
   const int q0 = t.tbl_q[tbl];
   const int lx0 = q0 == kStart ? 0 : -1;
@@ -110,7 +110,7 @@ __global__ void k_classify(Tables t, uint16_t* __restrict__ cls_sp, uint16_t* __
     uint16_t code, key = 0xFFFF;
     if (!t.ci_on)
       code = kClsCD;
-    else if (q0 != kStart && ts.next[q0 * ts.C + ts.byte_class[by[0]]] == kDead)
+    else if (q0 != kStart && ts.nxt(q0 * ts.C + ts.cls(by[0])) == kDead)
       code = kClsNA;
     else
       code = classify(ts, q0, lx0, by, len, key, rec);
@@ -129,12 +129,12 @@ __global__ void k_classify(Tables t, uint16_t* __restrict__ cls_sp, uint16_t* __
 
 // Event records of the kClsVC spellings, appended per table in any order:
 // slot -> (table, spelling, record).
-__global__ void k_events(Tables t, const uint16_t* __restrict__ cls_sp, const int32_t* __restrict__ vc_base,
+template <bool ST>
+__global__ void k_events(TabT<ST> t, const uint16_t* __restrict__ cls_sp, const int32_t* __restrict__ vc_base,
                          int32_t* __restrict__ fill, int32_t* __restrict__ slot_tbl, int32_t* __restrict__ slot_sp,
                          uint16_t* __restrict__ slot_rec) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  __shared__ Tables ts;
-  stage_tables(t, ts, smem);
+  stage_tables(t);
+  const auto& ts = t;
   const int tbl = blockIdx.y;
   const int q0 = t.tbl_q[tbl];
   const int lx0 = q0 == kStart ? 0 : -1;
@@ -170,7 +170,7 @@ __global__ void k_killw(Tables t, uint32_t* __restrict__ out) {
 
 // Terminal set of every class id (events and final tests of the verdict
 // classes use nothing else of a class).
-__global__ void k_class_sets(Tables t, uint4* __restrict__ out) {
+__global__ void k_class_sets(TabT<false> t, uint4* __restrict__ out) {
   const int cls = blockIdx.x * blockDim.x + threadIdx.x;
   if (cls >= t.ncls) return;
   const Bits4 v = class_terms(t, cls);
@@ -240,7 +240,8 @@ __global__ void k_permute(Tables t, const uint16_t* __restrict__ cls_sp, const u
 // are loaded kSelBatch at a time, so that a word costs |A u I| / kSelBatch
 // memory round trips instead of |A u I|.
 constexpr int kSelBatch = 16;
-__device__ __forceinline__ uint32_t select_word(const Tables& t, const Bits4 AI, int w0) {
+template <class T>
+__device__ __forceinline__ uint32_t select_word(const T& t, const Bits4 AI, int w0) {
   uint32_t acc = 0u;
   Bits4 r = AI;
   while (r.any()) {
@@ -276,7 +277,8 @@ struct AdvOut {
 // hashed, once the tokens are fed, away from the chain that the mask waits
 // for: hashing each push as it was made, on the lane that feeds the tokens,
 // cost k_row 51 us of 76 at 32 rows (24 without hashes).
-__device__ __forceinline__ void hash_nodes(const Tables& t, uint64_t* __restrict__ hs, const uint16_t* stack, int keep,
+template <class T>
+__device__ __forceinline__ void hash_nodes(const T& t, uint64_t* __restrict__ hs, const uint16_t* stack, int keep,
                                            int depth, int lane) {
   if (keep >= depth) return;
   uint64_t hp = hs[keep - 1];
@@ -323,7 +325,8 @@ struct AdvRow {
 };
 
 // The row's configuration (every lane gets it) and its pending lexeme's categories.
-__device__ __forceinline__ AdvRow advance_config(const Tables& t, const DevConfigs& c, int b, int lane) {
+template <class T>
+__device__ __forceinline__ AdvRow advance_config(const T& t, const DevConfigs& c, int b, int lane) {
   int cf = 0;
   if (lane < 4) {
     const int32_t* f = lane == 0 ? c.depth : lane == 1 ? c.q : lane == 2 ? c.lx : c.flags;
@@ -345,7 +348,8 @@ __device__ __forceinline__ AdvRow advance_config(const Tables& t, const DevConfi
   return r;
 }
 
-__device__ __forceinline__ AdvRow advance_load(const Tables& t, const DevConfigs& cin, const DevConfigs& cout, int b,
+template <class T>
+__device__ __forceinline__ AdvRow advance_load(const T& t, const DevConfigs& cin, const DevConfigs& cout, int b,
                                                int copy, int lane, uint16_t* win) {
   const uint16_t* src = (copy ? cin.stack : cout.stack) + (size_t)b * t.D;
   uint16_t* stack = cout.stack + (size_t)b * t.D;
@@ -387,7 +391,8 @@ __device__ __forceinline__ AdvRow advance_load(const Tables& t, const DevConfigs
 // single token is lane 0's: with one token there is little to lex side by
 // side, and setting the batch up costs a step of one expression row 0.8 us of
 // 31 (SQL rows: no difference).
-__device__ __forceinline__ bool feed_fits(const Tables& t, const AdvRow& r, int n_steps) {
+template <class T>
+__device__ __forceinline__ bool feed_fits(const T& t, const AdvRow& r, int n_steps) {
   return n_steps > 1 && t.chain_rate > 0 && r.win && !(r.flags & 1);
 }
 
@@ -398,7 +403,8 @@ __device__ __forceinline__ Feed feed_begin(const AdvRow& r, uint16_t* win, AdvSh
 // After the last batch (`fed`: parse_batch went through all of them, `end` is
 // the lexer's state there): the test of the last token, the stack written
 // back, and the row as advance_rest goes on with it at token f.tok.
-__device__ __forceinline__ void feed_end(const Tables& ts, Feed& f, bool fed, const LexState& end, int n_steps,
+template <class T>
+__device__ __forceinline__ void feed_end(const T& ts, Feed& f, bool fed, const LexState& end, int n_steps,
                                          AdvRow& r, uint16_t* stack, int lane, int max_chain) {
   if (fed && (!f.any || (f.depth <= ts.D && feed_live(ts, f, end.q, end.pc, lane, max_chain) == 1))) {
     f.tok = n_steps;
@@ -413,7 +419,8 @@ __device__ __forceinline__ void feed_end(const Tables& ts, Feed& f, bool fed, co
 }
 
 // Lane 0 only: tokens k0 .. n_steps - 1, one after the other (`first`: token 0, loaded ahead).
-__device__ __forceinline__ void advance_rest(const Tables& t, const Tables& ts, const DevConfigs& cout,
+template <class T>
+__device__ __forceinline__ void advance_rest(const T& t, const T& ts, const DevConfigs& cout,
                                              const int32_t* __restrict__ tokens, int k0, int n_steps,
                                              int32_t* __restrict__ d_status, int b, uint16_t* win, AdvShared& sh,
                                              const AdvRow& r, int keep, const LexToken& first, AdvOut& out) {
@@ -520,20 +527,19 @@ __device__ __forceinline__ void advance_rest(const Tables& t, const Tables& ts, 
 // advance's error, if its token was refused, else the mask step's.
 // ADV: 0 no tokens, 1 one token per row, 2 several (its own instance, so that
 // the usual step does not carry the batch feed's code).
-template <int ADV>
-__global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(Tables t, DevConfigs c, RowCtx* __restrict__ ctx,
+template <int ADV, bool ST>
+__global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfigs c, RowCtx* __restrict__ ctx,
                                                         RowRanges* __restrict__ rng, uint32_t* __restrict__ A2,
                                                         uint32_t* __restrict__ sel, uint32_t* __restrict__ verd0,
                                                         uint32_t* __restrict__ verd1, uint32_t* __restrict__ vcbits,
                                                         int n_vcbits, int B, int words_v, CacheDev cache,
                                                         AdvArgs adv) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  __shared__ Tables ts;
   __shared__ __align__(16) uint16_t s_stk[kStackWin];
   __shared__ uint16_t s_ovl1[kMaxOvl];
   __shared__ __align__(16) uint16_t s_ovl2[kRowJobWarps][kMaxOvl * 32];
   __shared__ uint16_t s_scr[kRowJobWarps][kMaxOvl * 32];
-  __shared__ uint32_t s_A0[4], s_A1[4], s_keep[8], s_kill[8];
+  __shared__ __align__(16) uint32_t s_A0[4], s_A1[4];
+  __shared__ uint32_t s_keep[8], s_kill[8];
   __shared__ int s_row[8];  // complete, depth, q, lx, emit_ok, keep1, m1, eos_ok
   __shared__ uint32_t s_pc[2];
   __shared__ int s_status, s_total0, s_nrng, s_adv[3];
@@ -556,7 +562,8 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(Tables t, DevConfigs 
     for (size_t i = first; i < (size_t)n_vcbits; i += stride) vcbits[i] = 0u;
     return;
   }
-  stage_tables(t, ts, smem);
+  stage_tables(t);
+  const auto& ts = t;
   pdl_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int b = blockIdx.x;
@@ -661,7 +668,7 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(Tables t, DevConfigs 
     // first bytes that end the pending lexeme (every byte when it is empty)
     for (int b0 = 0; b0 < 256; b0 += 32) {
       const int by = b0 + lane;
-      const bool kill = q == kStart || ts.next[q * ts.C + ts.byte_class[by]] == kDead;
+      const bool kill = q == kStart || ts.nxt(q * ts.C + ts.cls(by)) == kDead;
       const uint32_t word = __ballot_sync(0xffffffffu, kill);
       if (lane == 0) s_kill[b0 >> 5] = word;
     }
@@ -784,7 +791,7 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(Tables t, DevConfigs 
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const int by = j * 32 + lane;
-        cw[j] = __ballot_sync(0xffffffffu, hi_r[j] > lo_r[j] && ts.next[q * ts.C + ts.byte_class[by]] != kDead);
+        cw[j] = __ballot_sync(0xffffffffu, hi_r[j] > lo_r[j] && ts.nxt(q * ts.C + ts.cls(by)) != kDead);
         nc += __popc(cw[j]);
       }
       for (int i0 = 0; i0 < nc; i0 += 32) {  // the live test of the continuing bytes, one per lane
@@ -800,7 +807,7 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(Tables t, DevConfigs 
         if (by >= 0) {
           uint32_t pc2 = 0u, wc2 = 0u;
           if (lx >= 0) lex_step(ts, lx, by, pc2, wc2);
-          const int q2 = ts.next[q * ts.C + ts.byte_class[by]];
+          const int q2 = ts.nxt(q * ts.C + ts.cls(by));
           if ((live_prime(ts, q2, pc2) & AI).any()) atomicOr(&s_keep[by >> 5], 1u << (by & 31));
         }
       }
@@ -1037,8 +1044,8 @@ __device__ __forceinline__ int4 row_queue(const Tables& t, const RowCtx& x) {
 // lookups, verdict-class events) in registers and adds the totals to
 // work[0..3] when it is done (and the records and spellings it evaluated to
 // work[4..5]); the plain instance has no counting code.
-template <bool COUNT>
-__global__ void __launch_bounds__(kWalkWarps * 32, 2) k_walk(Tables t, RowCtx* __restrict__ ctx,
+template <bool COUNT, bool ST>
+__global__ void __launch_bounds__(kWalkWarps * 32, 2) k_walk(TabT<ST> t, RowCtx* __restrict__ ctx,
                                                              const RowRanges* __restrict__ rng, const uint16_t* stacks,
                                                              const int32_t* __restrict__ surv, int cap,
                                                              const uint32_t* __restrict__ A2,
@@ -1047,14 +1054,13 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 2) k_walk(Tables t, RowCtx* _
                                                              int vcw, const int32_t* __restrict__ vsurv, int vcap,
                                                              int words_v, int B,
                                                              unsigned long long* __restrict__ work) {
-  extern __shared__ __align__(16) uint8_t smem[];
   __shared__ uint16_t s_ovl[kWalkWarps][kMaxOvl];
   __shared__ uint16_t s_win[kWalkWarps][kWalkWin];
   __shared__ uint16_t s_lane[kWalkWarps][2 * kLaneOvl * 32];
-  __shared__ uint32_t s_A[kWalkWarps][2][4];  // the cached row's A0 and A1
+  __shared__ __align__(16) uint32_t s_A[kWalkWarps][2][4];  // the cached row's A0 and A1
   __shared__ int4 s_seg[kWalkRowsCached];
-  __shared__ Tables ts;
-  stage_tables(t, ts, smem);
+  stage_tables(t);
+  const auto& ts = t;
   pdl_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int gw = blockIdx.x * kWalkWarps + warp;
@@ -1490,16 +1496,16 @@ __global__ void __launch_bounds__(kPackWords) k_pack(Tables t, RowCtx* __restric
 
 // One block of two warps per row: warp 1 lexes the next batch of tokens while
 // warp 0 parses the last one.
-__global__ void __launch_bounds__(64, 3) k_advance(Tables t, DevConfigs cin, DevConfigs cout,
+template <bool ST>
+__global__ void __launch_bounds__(64, 3) k_advance(TabT<ST> t, DevConfigs cin, DevConfigs cout,
                                                 const int32_t* __restrict__ tokens, int n_steps,
                                                 int32_t* __restrict__ d_status, int B, int copy) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  __shared__ Tables ts;
   __shared__ __align__(16) uint16_t s_stk[kStackWin];
   __shared__ AdvShared sh;
   __shared__ LexBatch s_lex1;  // with sh.lex: the batch being parsed and the one being made
   __shared__ int s_stop[2];    // set while batch j is parsed, read before batch j + 1 is: j odd, j even
-  stage_tables(t, ts, smem);
+  stage_tables(t);
+  const auto& ts = t;
   pdl_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int b = blockIdx.x;
@@ -1672,22 +1678,15 @@ int grid::g_sms = 152;  // SM count of the current device, set by grid_specializ
 // allowed instead of to this spec's size.
 static int set_smem_limits() {
   const int dyn = kMaxStage;
-  GRID_CUDA(cudaFuncSetAttribute(k_classify, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-  GRID_CUDA(cudaFuncSetAttribute(k_events, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-  // k_pack: one row's class selections and verdict-class bits, two contexts
-  GRID_CUDA(cudaFuncSetAttribute(k_pack<0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-  GRID_CUDA(cudaFuncSetAttribute(k_pack<0, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-  GRID_CUDA(cudaFuncSetAttribute(k_pack<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-  GRID_CUDA(cudaFuncSetAttribute(k_pack<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-  GRID_CUDA(cudaFuncSetAttribute(k_pack<0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-  GRID_CUDA(cudaFuncSetAttribute(k_pack<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-  GRID_CUDA(cudaFuncSetAttribute(k_pack<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-  GRID_CUDA(cudaFuncSetAttribute(k_row<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-  GRID_CUDA(cudaFuncSetAttribute(k_row<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-  GRID_CUDA(cudaFuncSetAttribute(k_row<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-  GRID_CUDA(cudaFuncSetAttribute(k_walk<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-  GRID_CUDA(cudaFuncSetAttribute(k_walk<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-  GRID_CUDA(cudaFuncSetAttribute(k_advance, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
+  const void* kernels[] = {
+      (const void*)k_classify<true>, (const void*)k_events<true>, (const void*)k_advance<true>,
+      (const void*)k_row<0, true>, (const void*)k_row<1, true>, (const void*)k_row<2, true>,
+      (const void*)k_walk<false, true>, (const void*)k_walk<true, true>,
+      // k_pack: one row's class selections and verdict-class bits, two contexts
+      (const void*)k_pack<0, false>, (const void*)k_pack<1, false>, (const void*)k_pack<2, false>,
+      (const void*)k_pack<0, true>, (const void*)k_pack<1, true>, (const void*)k_pack<2, true>,
+      (const void*)k_pack<0, false, true>};
+  for (const void* k : kernels) GRID_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
   return GRID_OK;
 }
 
@@ -1902,6 +1901,18 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   if (rc) return fail(rc);
   t.blob = dblob;
   t.blob_bytes = off[kSec] <= (size_t)kMaxStage ? (int)off[kSec] : 0;
+  t.o_class = (int)off[0];
+  t.o_next = (int)off[1];
+  t.o_acc = (int)off[2];
+  t.o_live = (int)off[3];
+  t.o_action = (int)off[4];
+  t.o_go = (int)off[5];
+  t.o_lhs = (int)off[7];
+  t.o_shift = (int)off[8];
+  t.o_roff = (int)off[9];
+  t.o_rp = (int)off[10];
+  t.o_red = (int)off[11];
+  t.o_lany = (int)off[12];
   t.byte_class = dblob + off[0];
   t.next = reinterpret_cast<const uint16_t*>(dblob + off[1]);
   t.acc = reinterpret_cast<const uint32_t*>(dblob + off[2]);
@@ -2039,7 +2050,10 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   t.first_byte_by_id = fb;
   GRID_CUDA(cudaMemsetAsync(counts_d, 0, (size_t)t.n_tbl * 8, st));
   const dim3 cgrid(std::max(1, std::min((t.NS + 255) / 256, 4 * s->sms)), t.n_tbl);
-  k_classify<<<cgrid, 256, t.blob_bytes, st>>>(t, cls_sp, key_sp, counts_d);
+  if (t.blob_bytes)
+    k_classify<true><<<cgrid, 256, t.blob_bytes, st>>>(TabT<true>(t), cls_sp, key_sp, counts_d);
+  else
+    k_classify<false><<<cgrid, 256, 0, st>>>(TabT<false>(t), cls_sp, key_sp, counts_d);
   std::vector<int32_t> counts2(2 * t.n_tbl);
   GRID_CUDA(cudaMemcpyAsync(counts2.data(), counts_d, t.n_tbl * 8, cudaMemcpyDeviceToHost, st));
   GRID_CUDA(cudaStreamSynchronize(st));
@@ -2070,7 +2084,10 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
       (rc = tmp.alloc((size_t)t.n_tbl * t.NS * 4, (void**)&vc_sp)))
     return fail_tmp(rc);
   GRID_CUDA(cudaMemsetAsync(fill, 0, (size_t)t.n_tbl * 4, st));
-  if (nslot > 0) k_events<<<cgrid, 256, t.blob_bytes, st>>>(t, cls_sp, vcbase_d, fill, slot_tbl, slot_sp, slot_rec);
+  if (nslot > 0 && t.blob_bytes)
+    k_events<true><<<cgrid, 256, t.blob_bytes, st>>>(TabT<true>(t), cls_sp, vcbase_d, fill, slot_tbl, slot_sp, slot_rec);
+  else if (nslot > 0)
+    k_events<false><<<cgrid, 256, 0, st>>>(TabT<false>(t), cls_sp, vcbase_d, fill, slot_tbl, slot_sp, slot_rec);
   std::vector<int32_t> h_tbl(nslot);
   std::vector<uint16_t> h_rec((size_t)nslot * kRecLen);
   if (nslot > 0) {
@@ -2086,7 +2103,7 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
     // classes whose set holds it (the class selection ORs these)
     uint4* sets_d = nullptr;
     if ((rc = a.alloc((size_t)t.ncls * 16, (void**)&sets_d))) return fail_tmp(rc);
-    k_class_sets<<<(t.ncls + 255) / 256, 256, 0, st>>>(t, sets_d);
+    k_class_sets<<<(t.ncls + 255) / 256, 256, 0, st>>>(TabT<false>(t), sets_d);
     std::vector<uint4> sets(t.ncls);
     GRID_CUDA(cudaMemcpyAsync(sets.data(), sets_d, (size_t)t.ncls * 16, cudaMemcpyDeviceToHost, st));
     GRID_CUDA(cudaStreamSynchronize(st));
@@ -2194,7 +2211,11 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   s->n1 = (counts[0] + kSpan - 1) / kSpan;
   s->max_cd = *std::max_element(counts.begin(), counts.end());
   int per_sm = 0;
-  GRID_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_walk<false>, kWalkWarps * 32, t.blob_bytes));
+  if (t.blob_bytes)
+    GRID_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_walk<false, true>, kWalkWarps * 32,
+                                                            t.blob_bytes));
+  else
+    GRID_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_walk<false, false>, kWalkWarps * 32, 0));
   s->walk_blocks = std::max(1, per_sm) * s->sms;
   if ((rc = build_reserve_tables(s))) return fail(rc);
   *out = s;
@@ -2278,8 +2299,10 @@ extern "C" int grid_configs_reset(const grid_spec* s, grid_configs* c, void* str
 
 int grid::launch_advance(const grid_spec* s, const DevConfigs& in, const DevConfigs& out, int B,
                          const int32_t* d_tokens, int32_t n_steps, int32_t* d_status, int copy, cudaStream_t st) {
-  GRID_CUDA(launch_pdl(k_advance, dim3(B), dim3(64), s->t.blob_bytes, st,
-                       s->t, in, out, d_tokens, n_steps, d_status, B, copy));
+  auto advance = [&](auto kern, const auto& t) {
+    return launch_pdl(kern, dim3(B), dim3(64), t.blob_bytes, st, t, in, out, d_tokens, n_steps, d_status, B, copy);
+  };
+  GRID_CUDA(s->t.blob_bytes ? advance(k_advance<true>, TabT<true>(s->t)) : advance(k_advance<false>, TabT<false>(s->t)));
   GRID_CUDA(cudaGetLastError());
   return GRID_OK;
 }
@@ -2305,27 +2328,34 @@ int grid::launch_masks(const grid_spec* s, const DevConfigs& c, const MaskScratc
   const size_t zero_words = (size_t)B * m.words_v * 2 + n_vcbits;
   const int zero_blocks = std::min(128, (int)((zero_words / 8 + kRowWarps * 32 * 4 - 1) / (kRowWarps * 32 * 4)) + 1);
   if (ev) GRID_CUDA(cudaEventRecord(ev[0], st));
-  auto row = [&](auto kern) {
-    return launch_pdl(kern, dim3(B + zero_blocks), dim3(kRowWarps * 32), t.blob_bytes, st, t, c, m.ctx, m.rng, m.A2,
-                      m.sel, m.verd0, m.verd1, m.vcbits, n_vcbits, B, m.words_v, m.cache, adv ? *adv : AdvArgs{});
+  const TabT<true> ts(t);  // the tables as the kernels that stage them take them, or
+  const TabT<false> tg(t);  // that read a block too large to stage from global memory
+  const bool staged = t.blob_bytes > 0;
+  auto row = [&](auto kern, const auto& tab) {
+    return launch_pdl(kern, dim3(B + zero_blocks), dim3(kRowWarps * 32), tab.blob_bytes, st, tab, c, m.ctx, m.rng,
+                      m.A2, m.sel, m.verd0, m.verd1, m.vcbits, n_vcbits, B, m.words_v, m.cache,
+                      adv ? *adv : AdvArgs{});
   };
-  GRID_CUDA(!adv ? row(k_row<0>) : adv->n_steps <= 1 ? row(k_row<1>) : row(k_row<2>));
+  if (staged)
+    GRID_CUDA(!adv ? row(k_row<0, true>, ts) : adv->n_steps <= 1 ? row(k_row<1, true>, ts) : row(k_row<2, true>, ts));
+  else
+    GRID_CUDA(!adv ? row(k_row<0, false>, tg) : adv->n_steps <= 1 ? row(k_row<1, false>, tg) : row(k_row<2, false>, tg));
   if (ev) GRID_CUDA(cudaEventRecord(ev[1], st));
   const int cd_blocks = (s->max_cd + 256 * kFilterPer - 1) / (256 * kFilterPer);
   const int vc_blocks = (s->max_vc + 256 * kFilterPer - 1) / (256 * kFilterPer);
   GRID_CUDA(launch_pdl(k_filter, dim3(std::max(1, cd_blocks + vc_blocks), B, 2), dim3(256), 0, st, t, m.ctx,
                        (const uint32_t*)m.sel, m.surv, m.cap, m.vsurv, m.vcap, cd_blocks));
   if (ev) GRID_CUDA(cudaEventRecord(ev[2], st));
+  auto walk = [&](auto kern, const auto& tab) {
+    return launch_pdl(kern, dim3(s->walk_blocks), dim3(kWalkWarps * 32), tab.blob_bytes, st, tab, m.ctx,
+                      (const RowRanges*)m.rng, (const uint16_t*)c.stack, (const int32_t*)m.surv, m.cap,
+                      (const uint32_t*)m.A2, m.verd0, m.verd1, m.vcbits, vcw, (const int32_t*)m.vsurv, m.vcap,
+                      m.words_v, B, s->walk_work);
+  };
   if (s->walk_work)  // the measured instance, which counts its work
-    GRID_CUDA(launch_pdl(k_walk<true>, dim3(s->walk_blocks), dim3(kWalkWarps * 32), t.blob_bytes, st, t, m.ctx,
-                         (const RowRanges*)m.rng, (const uint16_t*)c.stack, (const int32_t*)m.surv, m.cap,
-                         (const uint32_t*)m.A2, m.verd0, m.verd1, m.vcbits, vcw, (const int32_t*)m.vsurv, m.vcap,
-                         m.words_v, B, s->walk_work));
+    GRID_CUDA(staged ? walk(k_walk<true, true>, ts) : walk(k_walk<true, false>, tg));
   else
-    GRID_CUDA(launch_pdl(k_walk<false>, dim3(s->walk_blocks), dim3(kWalkWarps * 32), t.blob_bytes, st, t, m.ctx,
-                         (const RowRanges*)m.rng, (const uint16_t*)c.stack, (const int32_t*)m.surv, m.cap,
-                         (const uint32_t*)m.A2, m.verd0, m.verd1, m.vcbits, vcw, (const int32_t*)m.vsurv, m.vcap,
-                         m.words_v, B, (unsigned long long*)nullptr));
+    GRID_CUDA(staged ? walk(k_walk<false, true>, ts) : walk(k_walk<false, false>, tg));
   if (ev) GRID_CUDA(cudaEventRecord(ev[3], st));
   const dim3 pgrid((t.W + kPackWords - 1) / kPackWords, B);
   const size_t psmem = (size_t)(2 * std::max(1, t.nselw) + 2 * vcw) * 4;

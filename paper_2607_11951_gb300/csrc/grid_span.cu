@@ -109,7 +109,8 @@ struct VStack {
 
 // The cheapest terminal completion of `vs` (in rendering tokens), or kInf;
 // on success goal_e / goal_item name its last step.
-__device__ uint32_t reserve_search(const Tables& t, const ReserveTables& rt, const VStack& vs, REnt* ent,
+template <class T>
+__device__ uint32_t reserve_search(const T& t, const ReserveTables& rt, const VStack& vs, REnt* ent,
                                    int32_t* head, int& goal_e, int& goal_item, bool& overflow) {
   const int kmax = vs.size() - 1;
   goal_e = goal_item = -1;
@@ -161,7 +162,7 @@ __device__ uint32_t reserve_search(const Tables& t, const ReserveTables& rt, con
             continue;
           }
           if (d != 1 || k < 1) continue;
-          const int g = t.go[vs.at(k - 1) * t.NNT + t.plhs[p]];
+          const int g = t.gto(vs.at(k - 1) * t.NNT + t.lhs(p));
           if (g >= t.S) continue;
           if (insert(k, g, c, e, i)) changed = true;
         }
@@ -176,7 +177,7 @@ __device__ uint32_t reserve_search(const Tables& t, const ReserveTables& rt, con
         const int p = rt.item_p[i], d = rt.item_d[i];
         const uint32_t ic = rt.item_cost[i];
         if (p == 0 || d < 2 || d > k || ic >= kInf) continue;
-        const int g = t.go[vs.at(k - d) * t.NNT + t.plhs[p]];
+        const int g = t.gto(vs.at(k - d) * t.NNT + t.lhs(p));
         if (g >= t.S) continue;
         insert(k - d + 1, g, c0 + ic, e, i);
       }
@@ -208,7 +209,8 @@ struct ReserveArgs {
 // as it stands; option 1 + tau: extended to tau's shortest lexeme) and keeps
 // the cheapest, then writes its tokens.  For rows whose search is larger than
 // the warps' shared memory (k_reserve).
-__device__ __noinline__ void reserve_serial(const Tables& t, const Tables& ts, const ReserveTables& rt,
+template <class T>
+__device__ __noinline__ void reserve_serial(const T& t, const T& ts, const ReserveTables& rt,
                                             const DevConfigs& c, const ReserveArgs& ra, int b) {
   int32_t* const scratch = ra.scratch;
   const size_t scratch_ints = ra.scratch_ints;
@@ -262,7 +264,7 @@ __device__ __noinline__ void reserve_serial(const Tables& t, const Tables& ts, c
         if (len == 0 || len > kMaxExt) return false;  // len 0: the lexeme as it stands (option 0)
         for (int i = 0; i < len; ++i) {
           const int by = cat >= 0 ? rt.lx_wbyte[(size_t)lx2 * rt.NC + cat] : rt.dfa_tbyte[(size_t)q2 * t.T1 + tau];
-          const int nq = ts.next[q2 * ts.C + ts.byte_class[by]];
+          const int nq = ts.nxt(q2 * ts.C + ts.cls(by));
           if (nq == kDead) return false;
           q2 = nq;
           lx2 = lex_step(ts, lx2, by, pc, wc);
@@ -399,7 +401,8 @@ __device__ __forceinline__ int rsv_at(const uint16_t* base, const RsvOption& o, 
 }
 
 // reserve_search on one warp.
-__device__ RsvGoal rsv_search(const Tables& t, const ReserveTables& rt, const uint16_t* base, const RsvOption& o,
+template <class T>
+__device__ RsvGoal rsv_search(const T& t, const ReserveTables& rt, const uint16_t* base, const RsvOption& o,
                               RsvWarp& w, int lane) {
   RsvGoal goal{kInf, -1, -1, false};
   const int kmax = o.keep + o.m - 1;
@@ -489,7 +492,7 @@ __device__ RsvGoal rsv_search(const Tables& t, const ReserveTables& rt, const ui
             }
           }
           if (c < kInf && p > 0 && d == 1 && k >= 1) {
-            const int g = t.go[below * t.NNT + t.plhs[p]];
+            const int g = t.gto(below * t.NNT + t.lhs(p));
             if (g < t.S) key = (k << 16) | g;
           }
           changed |= insert_all(key, c, e, i);
@@ -510,7 +513,7 @@ __device__ RsvGoal rsv_search(const Tables& t, const ReserveTables& rt, const ui
           ic = __ldg(&rt.item_cost[i]);
           const int p = __ldg(&rt.item_p[i]), d = __ldg(&rt.item_d[i]);
           if (p != 0 && d >= 2 && d <= k && ic < kInf) {
-            const int g = t.go[rsv_at(base, o, w, k - d) * t.NNT + t.plhs[p]];
+            const int g = t.gto(rsv_at(base, o, w, k - d) * t.NNT + t.lhs(p));
             if (g < t.S) key = ((k - d + 1) << 16) | g;
           }
         }
@@ -525,13 +528,13 @@ __device__ RsvGoal rsv_search(const Tables& t, const ReserveTables& rt, const ui
 // written by the warp that found it).  One thread per row, with the entries
 // and the level heads in global memory, took 1,220 us for 32 SQL rows of up
 // to 2,000 tokens; this takes 110 us.
-__global__ void __launch_bounds__(kRsvWarps * 32) k_reserve(Tables t, ReserveTables rt, DevConfigs c, ReserveArgs ra) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  __shared__ Tables ts;
+template <bool ST>
+__global__ void __launch_bounds__(kRsvWarps * 32) k_reserve(TabT<ST> t, ReserveTables rt, DevConfigs c, ReserveArgs ra) {
   __shared__ __align__(16) uint16_t s_stk[kRsvDepth];
   __shared__ unsigned long long s_best;  // total << 32 | option of the cheapest way
   __shared__ int s_slow;
-  stage_tables(t, ts, smem);
+  stage_tables(t);
+  const auto& ts = t;
   const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   RsvWarp& w = reinterpret_cast<RsvWarp*>(smem + ((t.blob_bytes + 15) & ~15))[warp];
   const int depth = c.depth[b], q = c.q[b], lx = c.lx[b];
@@ -574,7 +577,7 @@ __global__ void __launch_bounds__(kRsvWarps * 32) k_reserve(Tables t, ReserveTab
       if (len == 0 || len > kMaxExt) return o;  // len 0: the lexeme as it stands (option 0)
       for (int i = 0; i < len; ++i) {
         const int by = cat >= 0 ? rt.lx_wbyte[(size_t)lx2 * rt.NC + cat] : rt.dfa_tbyte[(size_t)q2 * t.T1 + tau];
-        const int nq = ts.next[q2 * ts.C + ts.byte_class[by]];
+        const int nq = ts.nxt(q2 * ts.C + ts.cls(by));
         if (nq == kDead || rt.byte_tok[by] < 0) return o;
         q2 = nq;
         lx2 = lex_step(ts, lx2, by, pc, wc);
@@ -870,11 +873,16 @@ extern "C" int grid_reserve(const grid_spec* s, const grid_configs* c, int32_t* 
   if (!s || !c || !d_cost || !d_tokens || cap <= 0 || !d_status || (d_budget && !d_fire))
     return set_error(GRID_E_INVALID_ARG, "grid_reserve: bad arguments");
   if (!s->rt.ok) return set_error(GRID_E_INVALID_ARG, "grid_reserve: the spec has no reserve tables");
-  const size_t smem = ((s->t.blob_bytes + 15) & ~15) + kRsvWarps * sizeof(RsvWarp);
-  GRID_CUDA(cudaFuncSetAttribute(k_reserve, cudaFuncAttributeMaxDynamicSharedMemorySize, kRsvSmem));
+  const size_t dyn = ((s->t.blob_bytes + 15) & ~15) + kRsvWarps * sizeof(RsvWarp);
   const ReserveArgs ra{c->rscratch, reserve_scratch_bytes(s) / 4, d_cost, d_tokens, cap, d_status, d_budget, safety,
                        d_fire};
-  k_reserve<<<c->B, kRsvWarps * 32, smem, (cudaStream_t)stream>>>(s->t, s->rt, c->c, ra);
+  auto launch = [&](auto kern, const auto& t) -> int {
+    GRID_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kRsvSmem));
+    kern<<<c->B, kRsvWarps * 32, dyn, (cudaStream_t)stream>>>(t, s->rt, c->c, ra);
+    return GRID_OK;
+  };
+  if (int rc = s->t.blob_bytes ? launch(k_reserve<true>, TabT<true>(s->t)) : launch(k_reserve<false>, TabT<false>(s->t)))
+    return rc;
   GRID_CUDA(cudaGetLastError());
   return GRID_OK;
 }
