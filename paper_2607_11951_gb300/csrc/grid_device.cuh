@@ -105,9 +105,6 @@ struct Tables {
   const uint16_t* red_p;       // each reduce group's production as plen << 10 | lhs
   const uint32_t* red_mask;    // 4 per reduce group: its lookahead terminals
   // identifier trie
-  const int32_t* lx_cstart;
-  const uint8_t* lx_cbyte;
-  const int32_t* lx_cnode;
   const uint32_t* lx_pcats;
   const uint32_t* lx_wcats;
   // open-addressing hash of the identifier-trie edges: key = node * 256 + byte,
@@ -130,7 +127,7 @@ struct Tables {
   // CI tables (one per lexer state in the precomputed set; table 0 = start state)
   int ci_on;
   int n_tbl;
-  int ncls;
+  int ncls;                   // distinct terminal sets of the CI class ids: the classes that the step works with
   int nselw;
   const int16_t* tbl_of_q;
   const int32_t* tbl_q;
@@ -145,8 +142,8 @@ struct Tables {
   const uint32_t* vc_by_id;   // n_tbl * V: verdict class (within its table) of kClsVC spellings, or NULL
                               // when the class codes carry it (vc_inline)
   int vc_inline;              // 1: a verdict-class id's code is ncls + kPackCodes + its class index
-  const uint32_t* cls_sets;   // ncls * 4: terminal set of every class id
-  const uint32_t* cls_mask;   // T1 * nselw: bit c of row tau = tau is in class c's set
+  const uint32_t* cls_sets;   // ncls * 4: terminal set of every class (staged too where o_sets >= 0)
+  const uint16_t* cls_map;    // class of every CI class id
   const uint32_t* acc_sym;    // S: the symbol entering each state (audit node hash)
   // a chain on a stack of d entries takes at most (d + 1) * chain_rate + chain_base steps, and pushes fewer
   // entries than a walk's scratch holds (chain_bounds; chain_rate 0: not shown, tokens are fed by one lane)
@@ -155,7 +152,7 @@ struct Tables {
   const uint64_t* ev_list;  // the emission's candidates (LexBatch::ev; 0: none, count 0x7F: more than it holds)
   const uint32_t* live_any; // bit set: a lexeme there is live
   // byte offsets of the staged block's arrays in it
-  int o_class, o_next, o_acc, o_live, o_action, o_go, o_lhs, o_shift, o_roff, o_rp, o_red, o_lany;
+  int o_class, o_next, o_acc, o_live, o_action, o_go, o_lhs, o_shift, o_roff, o_rp, o_red, o_lany, o_sets;
 };
 
 extern __shared__ __align__(16) uint8_t smem[];
@@ -189,6 +186,13 @@ struct TabT : Tables {
   __device__ __forceinline__ Bits4 live4(int q) const { return get4(live, o_live, q); }
   __device__ __forceinline__ Bits4 shift4(int s) const { return get4(shift_mask, o_shift, s); }
   __device__ __forceinline__ Bits4 red4(int e) const { return get4(red_mask, o_red, e); }
+  __device__ __forceinline__ Bits4 set4(int c) const {
+    if (STAGED && o_sets >= 0) {
+      const uint4 v = reinterpret_cast<const uint4*>(smem + o_sets)[c];
+      return Bits4{v.x, v.y, v.z, v.w};
+    }
+    return Bits4::load(cls_sets + c * 4);
+  }
   __device__ __forceinline__ bool live_any_at(int i) const { return (get(live_any, o_lany, i >> 5) >> (i & 31)) & 1u; }
 };
 
@@ -938,19 +942,6 @@ __device__ __forceinline__ int class_id(const T& t, int kind, int q, uint32_t ca
   return ((kind * t.Q + q) << t.n_cat) | (int)(cats & ((1u << t.n_cat) - 1u));
 }
 
-// Terminal set of a class id, computed from the lexer tables.
-template <class T>
-__device__ __forceinline__ Bits4 class_terms(const T& t, int cls) {
-  const int hi = cls >> t.n_cat;
-  const uint32_t cats = (uint32_t)cls & ((1u << t.n_cat) - 1u);
-  const int kind = hi / t.Q, q = hi - kind * t.Q;
-  return lex_filter(t, kind ? t.acc4(q) : t.live4(q), cats);
-}
-
-// The same, from the table of all class ids' sets built at specialization.
-template <class T>
-__device__ __forceinline__ Bits4 class_set(const T& t, int cls) { return Bits4::load(t.cls_sets + cls * 4); }
-
 // Sec. 4.2 CI/CD classification of one spelling from lexer state (q, lx),
 // with the stack abstracted away.  Emissions whose first candidate is ignored
 // leave the stack alone and are dropped; every other emission, and the final
@@ -1017,12 +1008,12 @@ __device__ __forceinline__ int eval_record(const T& t, Walker& w, const uint16_t
   const int n = rec[0];
   for (int i = 0; i < n; ++i) {
     count_work(w.ctr, 3);
-    const int e = emit_set(t, w, class_set(t, rec[2 + i]), max_chain);
+    const int e = emit_set(t, w, t.set4(rec[2 + i]), max_chain);
     if (e <= 0) return e;
   }
   const uint16_t f = rec[1];
   if (f == kClsAcc) return 1;
-  return trailing_set(t, w, class_set(t, f), max_chain);
+  return trailing_set(t, w, t.set4(f), max_chain);
 }
 
 }  // namespace grid

@@ -4,14 +4,17 @@
 // Specialization (grid_specialize, Sec. 4.2 / cold-schema specialization), for
 // every precomputed lexer state (the start state and each state where no
 // lexicon category is live) and every distinct spelling:
+//   k_lex_hash, k_ids, k_spell16   the identifier trie's hash, the alias lists,
+//                 the spellings' first bytes
 //   k_classify    the spelling's class: a CI class id (its verdict is a
 //                 function of the allowed set alone), always / never viable,
 //                 a verdict class (its stack-dependent events fit one record),
 //                 or byte-walked CD (more events than a record holds)
-//   k_events      the event records of the verdict-class spellings; the host
-//                 merges equal records (after rewriting class ids with equal
-//                 terminal sets to one id) into the table's verdict classes
-//   k_compact     per lexer state: the ascending list of its byte-walked spellings
+//   k_events      the event records of the verdict-class spellings, class ids
+//                 with equal terminal sets rewritten to one class
+//   k_vc_merge, k_vc_gather, k_vc_rank, k_vc_place   equal records become the
+//                 table's verdict classes, in the order of their events
+//   k_compact     per lexer state: the list of its byte-walked spellings
 //   k_scatter_vc, k_permute   class codes and verdict-class indices re-indexed
 //                 by token id (coalesced in k_pack)
 //
@@ -77,6 +80,7 @@ constexpr int kRowJobWarps = 4;  // k_row: warps 2 .. 5 compute the allowed sets
 constexpr int kPackCodes = 5;  // ncls + 0 always, +1 never, +2 n/a, +3 verdict class, +4 walked;
                                // with vc_inline, ncls + 5 + v: verdict class v of the code's table
 constexpr int kWalkRowsCached = 256;  // rows whose queue bounds k_walk keeps in shared memory
+constexpr int kStagedSets = 512; // classes whose terminal sets are staged with the tables, at most
 constexpr int kLaneOvl = 32;     // overlay / scratch entries per walk lane (shared memory)
 constexpr int kMaxRows = 65535;  // rows of one configurations object (a grid dimension of the mask kernels)
 
@@ -148,7 +152,8 @@ __global__ void k_events(TabT<ST> t, const uint16_t* __restrict__ cls_sp, const 
     const int slot = vc_base[tbl] + atomicAdd(&fill[tbl], 1);
     slot_tbl[slot] = tbl;
     slot_sp[slot] = s;
-    for (int k = 0; k < kRecLen; ++k) slot_rec[(size_t)slot * kRecLen + k] = rec[k];
+    for (int k = 0; k < kRecLen; ++k)  // class ids of equal terminal sets become one class
+      slot_rec[(size_t)slot * kRecLen + k] = k > 0 && k < 2 + rec[0] && rec[k] < kClsFirstCode ? t.cls_map[rec[k]] : rec[k];
   }
 }
 
@@ -168,51 +173,203 @@ __global__ void k_killw(Tables t, uint32_t* __restrict__ out) {
   out[(size_t)q * t.W + wi] = w;
 }
 
-// Terminal set of every class id (events and final tests of the verdict
-// classes use nothing else of a class).
-__global__ void k_class_sets(TabT<false> t, uint4* __restrict__ out) {
-  const int cls = blockIdx.x * blockDim.x + threadIdx.x;
-  if (cls >= t.ncls) return;
-  const Bits4 v = class_terms(t, cls);
-  out[cls] = make_uint4(v.x, v.y, v.z, v.w);
+// ---- tables made on the device from what was uploaded: each replaces a host
+// loop over the vocabulary or the identifier trie (50,000 identifiers and
+// V = 151,936: the trie's hash 5.9 ms, the merge of the event records 10.3 ms,
+// the sixteen-byte heads and the alias lists 0.8 ms of 22 ms).
+
+// Identifier-trie edges into the open-addressing hash (entries cleared to
+// 0xFF bytes, load factor <= 1/2), a node per thread.
+__global__ void k_lex_hash(const int32_t* __restrict__ cstart, const uint8_t* __restrict__ cbyte,
+                           const int32_t* __restrict__ cnode, const uint32_t* __restrict__ pcats,
+                           const uint32_t* __restrict__ wcats, int LN, uint4* __restrict__ tab, uint32_t mask,
+                           int shift) {
+  const int n = blockIdx.x * blockDim.x + threadIdx.x;
+  if (n >= LN) return;
+  for (int e = cstart[n]; e < cstart[n + 1]; ++e) {
+    const uint32_t key = (uint32_t)n * 256u + cbyte[e];
+    const int child = cnode[e];
+    uint32_t h = (key * 0x9E3779B1u) >> shift;
+    for (uint32_t i = 0; i <= mask; ++i) {
+      if (atomicCAS(&tab[h].x, kHashEmpty, key) == kHashEmpty) {
+        tab[h].y = (uint32_t)child;
+        tab[h].z = pcats[child];
+        tab[h].w = wcats[child];
+        break;
+      }
+      h = (h + 1u) & mask;
+    }
+  }
+}
+
+// Per token id: the list of each spelling's ids (aliases, in any order) and
+// the ids with a spelling (not EOS, special or padding); Vp is a multiple of 32.
+__global__ void k_ids(const int32_t* __restrict__ spell_of_id, int Vp, int32_t* __restrict__ id_of_spell,
+                      int32_t* __restrict__ next_alias, uint32_t* __restrict__ valid) {
+  const int id = blockIdx.x * blockDim.x + threadIdx.x;
+  if (id >= Vp) return;
+  const int sp = spell_of_id[id];
+  next_alias[id] = sp >= 0 ? atomicExch(&id_of_spell[sp], id) : -1;
+  const uint32_t word = __ballot_sync(0xffffffffu, sp >= 0);
+  if ((id & 31) == 0) valid[id >> 5] = word;
+}
+
+// The first 16 bytes of each spelling, zero padded.
+__global__ void k_spell16(const int32_t* __restrict__ spell_off, const uint8_t* __restrict__ bytes, int NS,
+                          uint4* __restrict__ out) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= NS) return;
+  const int off = spell_off[s], len = min(16, spell_off[s + 1] - off);
+  uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+  for (int i = 0; i < 16; ++i)
+    if (i < len) w[i >> 2] |= (uint32_t)bytes[off + i] << (8 * (i & 3));
+  out[s] = make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// ---- the event records' merge into verdict classes
+struct Rec {
+  uint4 a, b;
+  __device__ __forceinline__ bool operator==(const Rec& o) const {
+    return a.x == o.a.x && a.y == o.a.y && a.z == o.a.z && a.w == o.a.w && b.x == o.b.x && b.y == o.b.y &&
+           b.z == o.b.z && b.w == o.b.w;
+  }
+};
+static_assert(sizeof(Rec) == kRecLen * 2, "an event record is two 16-byte words");
+
+// A record's place in its table's order: the events one after the other (each
+// + 1; 0 after the last, so that a record comes before those it starts), then
+// the final class.
+struct RecKey {
+  unsigned long long k[4];
+  __device__ __forceinline__ bool operator<(const RecKey& o) const {
+    if (k[0] != o.k[0]) return k[0] < o.k[0];
+    if (k[1] != o.k[1]) return k[1] < o.k[1];
+    if (k[2] != o.k[2]) return k[2] < o.k[2];
+    return k[3] < o.k[3];
+  }
+};
+
+__device__ __forceinline__ RecKey rec_key(const uint16_t* r) {
+  RecKey x;
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+    unsigned long long v = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int e = 4 * w + j;
+      const unsigned long long f = e < kMaxEv ? (e < r[0] ? r[2 + e] + 1ull : 0ull) : (e == kMaxEv ? r[1] : 0ull);
+      v = (v << 16) | f;
+    }
+    x.k[w] = v;
+  }
+  return x;
+}
+
+// Equal records of one table find one slot (rep): an open-addressing table of
+// slots (cleared to -1, at least twice as large), the first to claim an entry
+// stands for its record and takes the next place in its table.
+__global__ void k_vc_merge(const int32_t* __restrict__ slot_tbl, const Rec* __restrict__ rec, int nslot,
+                           int32_t* __restrict__ tab, uint32_t mask, int32_t* __restrict__ rep,
+                           int32_t* __restrict__ place, int32_t* __restrict__ count) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nslot) return;
+  const Rec r = rec[i];
+  const int tbl = slot_tbl[i];
+  uint32_t h = (uint32_t)tbl;
+  const uint32_t w[8] = {r.a.x, r.a.y, r.a.z, r.a.w, r.b.x, r.b.y, r.b.z, r.b.w};
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    h = (h ^ w[k]) * 0x9E3779B1u;
+    h ^= h >> 15;
+  }
+  h &= mask;
+  for (uint32_t n = 0; n <= mask; ++n) {
+    const int cur = atomicCAS(&tab[h], -1, i);
+    if (cur == -1) {
+      rep[i] = i;
+      place[i] = atomicAdd(&count[tbl], 1);
+      return;
+    }
+    if (slot_tbl[cur] == tbl && rec[cur] == r) {
+      rep[i] = cur;
+      return;
+    }
+    h = (h + 1u) & mask;
+  }
+}
+
+// The distinct records, table by table (in any order within it), with their keys.
+__global__ void k_vc_gather(const int32_t* __restrict__ slot_tbl, const Rec* __restrict__ rec, int nslot,
+                            const int32_t* __restrict__ rep, const int32_t* __restrict__ place,
+                            const int32_t* __restrict__ vc_off, int32_t* __restrict__ src, RecKey* __restrict__ key,
+                            int32_t* __restrict__ rank) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nslot || rep[i] != i) return;
+  const int at = vc_off[slot_tbl[i]] + place[i];
+  src[at] = i;
+  key[at] = rec_key(reinterpret_cast<const uint16_t*>(rec + i));
+  rank[at] = 0;
+}
+
+// Each record's rank in its table: the number of smaller keys, counted over
+// the table's keys in tiles; grid (records / 256, tables, parts of the tiles).
+__global__ void __launch_bounds__(256) k_vc_rank(const RecKey* __restrict__ key, const int32_t* __restrict__ vc_off,
+                                                 int32_t* __restrict__ rank) {
+  __shared__ RecKey s_key[256];
+  const int a = vc_off[blockIdx.y], n = vc_off[blockIdx.y + 1] - a;
+  const int p = blockIdx.x * 256 + threadIdx.x;
+  if ((int)blockIdx.x * 256 >= n) return;
+  const RecKey own = key[a + min(p, n - 1)];
+  int less = 0;
+  for (int t0 = blockIdx.z * 256; t0 < n; t0 += gridDim.z * 256) {
+    __syncthreads();
+    if (t0 + (int)threadIdx.x < n) s_key[threadIdx.x] = key[a + t0 + threadIdx.x];
+    __syncthreads();
+    const int m = min(256, n - t0);
+    for (int j = 0; j < m; ++j) less += s_key[j] < own ? 1 : 0;
+  }
+  if (p < n && less) atomicAdd(&rank[a + p], less);
+}
+
+// The records in their order, and each one's index for its slots (place, reused).
+__global__ void k_vc_place(const Rec* __restrict__ rec, const int32_t* __restrict__ slot_tbl,
+                           const int32_t* __restrict__ src, const int32_t* __restrict__ rank, int n,
+                           const int32_t* __restrict__ vc_off, Rec* __restrict__ out, uint16_t* __restrict__ first,
+                           int32_t* __restrict__ place) {
+  const int at = blockIdx.x * blockDim.x + threadIdx.x;
+  if (at >= n) return;
+  const int i = src[at], to = vc_off[slot_tbl[i]] + rank[at];
+  const Rec r = rec[i];
+  out[to] = r;
+  first[to] = (uint16_t)(r.a.y & 0xFFFFu);
+  place[i] = rank[at];
 }
 
 __global__ void k_scatter_vc(const int32_t* __restrict__ slot_tbl, const int32_t* __restrict__ slot_sp,
-                             const int32_t* __restrict__ slot_vc, int nslot, int NS, uint32_t* __restrict__ vc_sp) {
+                             const int32_t* __restrict__ rep, const int32_t* __restrict__ place, int nslot, int NS,
+                             uint32_t* __restrict__ vc_sp) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < nslot) vc_sp[(size_t)slot_tbl[i] * NS + slot_sp[i]] = (uint32_t)slot_vc[i];
+  if (i < nslot) vc_sp[(size_t)slot_tbl[i] * NS + slot_sp[i]] = (uint32_t)place[rep[i]];
 }
 
-// One block per table: ordered stream compaction of the CD spellings.
+// Per table the list of its byte-walked spellings and their keys (runs of
+// neighbours in any order; grid.y: tables).
 __global__ void k_compact(const uint16_t* __restrict__ cls_sp, const uint16_t* __restrict__ key_sp, int NS,
-                          const int32_t* __restrict__ cd_off, int32_t* __restrict__ cd_list,
-                          uint16_t* __restrict__ cd_key) {
-  __shared__ int32_t warp_tot[32];
-  __shared__ int32_t base;
-  const int tbl = blockIdx.x;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if (threadIdx.x == 0) base = cd_off[tbl];
-  __syncthreads();
-  for (int s0 = 0; s0 < NS; s0 += blockDim.x) {
-    const int s = s0 + threadIdx.x;
-    const bool f = s < NS && cls_sp[(size_t)tbl * NS + s] == kClsCD;
-    const uint32_t bal = __ballot_sync(0xffffffffu, f);
-    if (lane == 0) warp_tot[warp] = __popc(bal);
-    __syncthreads();
-    int before = 0;
-    for (int k = 0; k < warp; ++k) before += warp_tot[k];
-    if (f) {
-      const int at = base + before + __popc(bal & ((1u << lane) - 1u));
-      cd_list[at] = s;
-      cd_key[at] = key_sp[(size_t)tbl * NS + s];
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int tot = 0;
-      for (int k = 0; k < nw; ++k) tot += warp_tot[k];
-      base += tot;
-    }
-    __syncthreads();
+                          const int32_t* __restrict__ cd_off, const uint16_t* __restrict__ cls_map,
+                          int32_t* __restrict__ fill, int32_t* __restrict__ cd_list, uint16_t* __restrict__ cd_key) {
+  const int tbl = blockIdx.y, lane = threadIdx.x & 31;
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  const bool f = s < NS && cls_sp[(size_t)tbl * NS + s] == kClsCD;
+  const uint32_t bal = __ballot_sync(0xffffffffu, f);
+  if (!bal) return;
+  int at = 0;
+  if (lane == 0) at = cd_off[tbl] + atomicAdd(&fill[tbl], __popc(bal));
+  at = __shfl_sync(0xffffffffu, at, 0) + __popc(bal & ((1u << lane) - 1u));
+  if (f) {
+    const uint16_t k = key_sp[(size_t)tbl * NS + s];
+    cd_list[at] = s;
+    cd_key[at] = k == 0xFFFF ? k : cls_map[k];
   }
 }
 
@@ -225,7 +382,7 @@ __global__ void k_permute(Tables t, const uint16_t* __restrict__ cls_sp, const u
   fb_by_id[id] = s >= 0 ? t.spell_bytes[t.spell_off[s]] : 0;
   for (int k = 0; k < t.n_tbl; ++k) {
     const uint16_t c = s >= 0 ? cls_sp[(size_t)k * t.NS + s] : kClsNA;
-    uint16_t code = c;  // the k_pack code of c
+    uint16_t code = c < kClsFirstCode ? t.cls_map[c] : c;  // the k_pack code of c
     if (c >= kClsFirstCode)
       code = (uint16_t)(t.ncls + (c == kClsAcc ? 0 : c == kClsRej ? 1 : c == kClsNA ? 2 : c == kClsVC ? 3 : 4));
     if (c == kClsVC && t.vc_inline) code = (uint16_t)(t.ncls + kPackCodes + vc_sp[(size_t)k * t.NS + s]);
@@ -235,31 +392,17 @@ __global__ void k_permute(Tables t, const uint16_t* __restrict__ cls_sp, const u
 }
 
 // ---------------- mask step ----------------
-// Class selection for allowed set A, word w0: bit c = set(c) meets A u I,
-// the OR of the class masks of the terminals in A u I.  The terminals' words
-// are loaded kSelBatch at a time, so that a word costs |A u I| / kSelBatch
-// memory round trips instead of |A u I|.
-constexpr int kSelBatch = 16;
+// Class selections for the allowed sets AI0 and AI1 (with the ignored
+// terminals), word w0, by a warp: bit c = the set of class c meets them.
 template <class T>
-__device__ __forceinline__ uint32_t select_word(const T& t, const Bits4 AI, int w0) {
-  uint32_t acc = 0u;
-  Bits4 r = AI;
-  while (r.any()) {
-    uint32_t v[kSelBatch];
-#pragma unroll
-    for (int k = 0; k < kSelBatch; ++k) {
-      const int tau = r.lowest();
-      v[k] = 0u;
-      if (tau >= 0) {
-        r.clear_lowest();
-        v[k] = __ldg(&t.cls_mask[(size_t)tau * t.nselw + w0]);
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < kSelBatch; ++k) acc |= v[k];
-  }
-  if (w0 == (t.ncls >> 5)) acc |= 1u << (t.ncls & 31);  // the code "always"
-  return acc;
+__device__ __forceinline__ void select_word(const T& t, const Bits4 AI0, const Bits4 AI1, int w0, int lane,
+                                            uint32_t& v0, uint32_t& v1) {
+  const int c = w0 * 32 + lane;
+  Bits4 set = Bits4::zero();
+  if (c < t.ncls) set = t.set4(c);
+  const bool all = c == t.ncls;  // the code "always"
+  v0 = __ballot_sync(0xffffffffu, all || (set & AI0).any());
+  v1 = __ballot_sync(0xffffffffu, all || (set & AI1).any());
 }
 
 // The configuration one warp leaves after feeding its row's tokens (lane 0's
@@ -837,13 +980,14 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfig
         s_nrng = nrng;
       }
     } else if (warp >= 1 && t.ci_on) {
-      // both contexts' selection words, one per lane of warps 1 ..
+      // both contexts' selection words, one at a time per warp 1 ..
       const Bits4 AI0 = A0 | ts.ign, AI1 = A1 | ts.ign;
       const int nw = t.nselw;
-      for (int i = (warp - 1) * 32 + lane; i < 2 * nw; i += (kRowWarps - 1) * 32) {
-        const int cx = i >= nw ? 1 : 0, w0 = i - cx * nw;
-        if (cx ? !emit_ok : tbl0 < 0) continue;
-        sel[((size_t)b * 2 + cx) * nw + w0] = select_word(ts, cx ? AI1 : AI0, w0);
+      for (int w0 = warp - 1; w0 < nw; w0 += kRowWarps - 1) {
+        uint32_t v0, v1;
+        select_word(ts, AI0, AI1, w0, lane, v0, v1);
+        if (lane == 0 && tbl0 >= 0) sel[(size_t)b * 2 * nw + w0] = v0;
+        if (lane == 0 && emit_ok) sel[((size_t)b * 2 + 1) * nw + w0] = v1;
       }
     }
   }
@@ -1774,6 +1918,28 @@ static void chain_bounds(const HostGrammar& h, Tables& t) {
   t.chain_base = base;
 }
 
+// The distinct terminal sets of the CI class ids (four words each, in the order
+// of their first id) and each id's set: events and final tests use nothing else
+// of a class, so that ids with equal sets are one class from there on.
+static void class_sets(const HostGrammar& h, std::vector<uint32_t>& sets, std::vector<uint16_t>& map) {
+  const int n = (2 * h.Q) << h.n_cat;
+  map.resize(n);
+  std::unordered_map<std::string, uint16_t> seen;
+  for (int c = 0; c < n; ++c) {
+    const int hi = c >> h.n_cat, kind = hi / h.Q, q = hi - kind * h.Q;
+    const uint32_t* v = (kind ? h.acc : h.live).data() + (size_t)q * 4;
+    uint32_t w[4];
+    for (int k = 0; k < 4; ++k) w[k] = v[k] & ~h.catmask[k];
+    for (int k = 0; k < h.n_cat; ++k) {
+      const int tau = h.cat_term[k];
+      if ((c >> k) & 1) w[tau >> 5] |= v[tau >> 5] & (1u << (tau & 31));
+    }
+    const auto it = seen.emplace(std::string(reinterpret_cast<const char*>(w), 16), (uint16_t)(sets.size() / 4));
+    if (it.second) sets.insert(sets.end(), w, w + 4);
+    map[c] = it.first->second;
+  }
+}
+
 // Tables::ev_list and Tables::live_any.
 static void lexeme_tables(const HostGrammar& h, std::vector<uint64_t>& ev, std::vector<uint32_t>& live) {
   const int sets = 1 << h.n_cat;
@@ -1878,27 +2044,110 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   // lexeme tables, where the class ids fit (the bound of ci_on below)
   std::vector<uint64_t> ev_list;
   std::vector<uint32_t> live_any;
-  if (((long)(2 * h.Q) << h.n_cat) < (long)kClsFirstCode)
+  const long n_ids = (long)(2 * h.Q) << h.n_cat;  // CI class ids
+  t.ci_on = n_ids < (long)kClsFirstCode ? 1 : 0;
+  std::vector<uint32_t> sets;
+  std::vector<uint16_t> cls_map;
+  if (t.ci_on) {
     lexeme_tables(h, ev_list, live_any);
-  else
+    class_sets(h, sets, cls_map);
+  } else {
     t.chain_rate = 0;
+  }
+  s->n_classes = t.ci_on ? (int)n_ids : 0;
+  t.ncls = (int)(sets.size() / 4);
+  t.nselw = (t.ncls + kPackCodes + 31) / 32;
+  const std::vector<uint32_t> no_sets;
+  const std::vector<uint32_t>& staged_sets = t.ncls <= kStagedSets ? sets : no_sets;
   // staged block: byte classes, DFA, acc/live, ACTION, GOTO, production
-  // tables, shift masks and reduce groups, live lexemes
-  constexpr int kSec = 13;
+  // tables, shift masks and reduce groups, live lexemes, class sets
+  constexpr int kSec = 14;
   std::vector<size_t> off(kSec + 1, 0);
   const size_t sizes[kSec] = {256, h.next.size() * 2, h.acc.size() * 4, h.live.size() * 4, h.action.size() * 2,
                               h.go.size() * 2, h.plen.size(), h.plhs.size() * 2, shift_mask.size() * 4,
-                              red_off.size() * 4, red_p.size() * 2, red_mask.size() * 4, live_any.size() * 4};
+                              red_off.size() * 4, red_p.size() * 2, red_mask.size() * 4, live_any.size() * 4,
+                              staged_sets.size() * 4};
   const void* srcs[kSec] = {h.byte_class, h.next.data(), h.acc.data(), h.live.data(), action16.data(),
                             h.go.data(), h.plen.data(), h.plhs.data(), shift_mask.data(), red_off.data(),
-                            red_p.data(), red_mask.data(), live_any.data()};
+                            red_p.data(), red_mask.data(), live_any.data(), staged_sets.data()};
   for (int k = 0; k < kSec; ++k) off[k + 1] = align16(off[k] + sizes[k]);
   std::vector<uint8_t> blob(off[kSec], 0);
   for (int k = 0; k < kSec; ++k)
     if (sizes[k]) std::memcpy(blob.data() + off[k], srcs[k], sizes[k]);
+  Arena& a = s->mem;
+  int rc;
+  // id-indexed tables are padded to Vp ids (a multiple of 32), so that the
+  // ids of one mask word are read with 16-byte loads
+  t.Vp = (hv.V + 31) & ~31;
+  std::vector<int32_t> spell_of_id_p(hv.spell_of_id);
+  spell_of_id_p.resize(t.Vp, -1);
+  // precomputed lexer states: the start state and every state at which no
+  // lexicon category is live (there the lexicon node cannot matter)
+  std::vector<int32_t> tq{kStart};
+  std::vector<int16_t> tbl_of_q(h.Q, -1);
+  tbl_of_q[kStart] = 0;
+  if (t.ci_on) {
+    for (int q = 2; q < h.Q; ++q) {
+      bool catlive = false;
+      for (int w = 0; w < 4; ++w)
+        if (h.live[q * 4 + w] & h.catmask[w]) catlive = true;
+      if (!catlive && tq.size() < 4096) {
+        tbl_of_q[q] = (int16_t)tq.size();
+        tq.push_back(q);
+      }
+    }
+  }
+  t.n_tbl = (int)tq.size();
+  // identifier-trie edges -> open-addressing hash (load factor <= 1/2)
+  int hash_bits = 4;
+  while ((size_t(1) << hash_bits) < 2 * h.lx_cbyte.size() + 2) ++hash_bits;
+  t.lx_hmask = (1u << hash_bits) - 1u;
+  t.lx_hshift = 32 - hash_bits;
+  t.root_pc = h.LN > 0 ? h.lx_pcats[0] : 0u;
+  t.root_wc = h.LN > 0 ? h.lx_wcats[0] : 0u;
   const uint8_t* dblob = nullptr;
-  int rc = s->mem.upload(blob, &dblob);
-  if (rc) return fail(rc);
+  const int32_t *lx_cstart = nullptr, *lx_cnode = nullptr;
+  const uint8_t* lx_cbyte = nullptr;
+  uint4 *lx_hash = nullptr, *spell16 = nullptr;
+  int32_t *id_of_spell = nullptr, *next_alias = nullptr;
+  uint32_t* id_valid = nullptr;
+  Arena tmp;  // what only the specialization needs
+  std::vector<std::vector<uint8_t>> keep;  // host buffers of copies in flight
+  auto fail_tmp = [&](int code) {
+    cudaStreamSynchronize(st);
+    tmp.release();
+    return fail(code);
+  };
+  {
+    Upload up, up_tmp;
+    up.add(blob, &dblob);
+    up.add(ev_list, &t.ev_list);
+    up.add(sets, &t.cls_sets);
+    up.add(cls_map, &t.cls_map);
+    up.add(tq, &t.tbl_q);
+    up.add(tbl_of_q, &t.tbl_of_q);
+    up.add(h.acc_sym, &t.acc_sym);
+    up.add(hv.first_of_byte, &t.first_of_byte);
+    up.add(h.lx_pcats, &t.lx_pcats);
+    up.add(h.lx_wcats, &t.lx_wcats);
+    up.add(hv.spell_off, &t.spell_off);
+    up.add(hv.spell_bytes, &t.spell_bytes);
+    up.add(spell_of_id_p, &t.spell_of_id);
+    up.reserve((size_t)t.lx_hmask + 1, &lx_hash);
+    up.reserve(std::max(1, t.NS), &spell16);
+    up.reserve(std::max(1, t.NS), &id_of_spell);
+    up.reserve(t.Vp, &next_alias);
+    up.reserve(t.W, &id_valid);
+    up_tmp.add(h.lx_cstart, &lx_cstart);
+    up_tmp.add(h.lx_cbyte, &lx_cbyte);
+    up_tmp.add(h.lx_cnode, &lx_cnode);
+    if ((rc = up.commit(a, st, keep)) || (rc = up_tmp.commit(tmp, st, keep))) return fail_tmp(rc);
+  }
+  t.lx_hash = lx_hash;
+  t.spell16 = spell16;
+  t.id_of_spell = id_of_spell;
+  t.next_alias = next_alias;
+  t.id_valid = id_valid;
   t.blob = dblob;
   t.blob_bytes = off[kSec] <= (size_t)kMaxStage ? (int)off[kSec] : 0;
   t.o_class = (int)off[0];
@@ -1913,6 +2162,7 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   t.o_rp = (int)off[10];
   t.o_red = (int)off[11];
   t.o_lany = (int)off[12];
+  t.o_sets = staged_sets.empty() ? -1 : (int)off[13];
   t.byte_class = dblob + off[0];
   t.next = reinterpret_cast<const uint16_t*>(dblob + off[1]);
   t.acc = reinterpret_cast<const uint32_t*>(dblob + off[2]);
@@ -1926,95 +2176,12 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   t.red_p = reinterpret_cast<const uint16_t*>(dblob + off[10]);
   t.red_mask = reinterpret_cast<const uint32_t*>(dblob + off[11]);
   t.live_any = reinterpret_cast<const uint32_t*>(dblob + off[12]);
-  Arena& a = s->mem;
-  if ((rc = a.upload(ev_list, &t.ev_list))) return fail(rc);
-  {
-    // identifier-trie edges -> open-addressing hash (load factor <= 1/2)
-    const size_t edges = h.lx_cbyte.size();
-    int bits = 4;
-    while ((size_t(1) << bits) < 2 * edges + 2) ++bits;
-    std::vector<uint32_t> hv4((size_t(4) << bits), 0u);
-    for (size_t i = 0; i < (size_t(1) << bits); ++i) hv4[4 * i] = kHashEmpty;
-    const uint32_t mask = (1u << bits) - 1u;
-    for (int n = 0; n < h.LN; ++n)
-      for (int e = h.lx_cstart[n]; e < h.lx_cstart[n + 1]; ++e) {
-        const uint32_t key = (uint32_t)n * 256u + h.lx_cbyte[e];
-        uint32_t hh = (key * 0x9E3779B1u) >> (32 - bits);
-        while (hv4[4 * hh] != kHashEmpty) hh = (hh + 1u) & mask;
-        const int child = h.lx_cnode[e];
-        hv4[4 * hh] = key;
-        hv4[4 * hh + 1] = (uint32_t)child;
-        hv4[4 * hh + 2] = h.lx_pcats[child];
-        hv4[4 * hh + 3] = h.lx_wcats[child];
-      }
-    const uint32_t* dh = nullptr;
-    if ((rc = a.upload(hv4, &dh))) return fail(rc);
-    t.lx_hash = reinterpret_cast<const uint4*>(dh);
-    t.lx_hmask = mask;
-    t.lx_hshift = 32 - bits;
-    t.root_pc = h.LN > 0 ? h.lx_pcats[0] : 0u;
-    t.root_wc = h.LN > 0 ? h.lx_wcats[0] : 0u;
-  }
-  // id-indexed tables are padded to Vp ids (a multiple of 32), so that the
-  // ids of one mask word are read with 16-byte loads
-  t.Vp = (hv.V + 31) & ~31;
-  std::vector<int32_t> spell_of_id_p(hv.spell_of_id);
-  spell_of_id_p.resize(t.Vp, -1);
-  {
-    std::vector<uint32_t> valid(t.W, 0u);  // ids with a spelling: not EOS, special or padding
-    for (int id = 0; id < hv.V; ++id)
-      if (spell_of_id_p[id] >= 0) valid[id >> 5] |= 1u << (id & 31);
-    int rcv = s->mem.upload(valid, &t.id_valid);
-    if (rcv) return fail(rcv);
-  }
-  // the ids of each spelling (aliases), for the walks' id-indexed verdicts
-  std::vector<int32_t> id_of_spell(std::max(1, t.NS), -1), next_alias(t.Vp, -1);
-  for (int id = t.Vp - 1; id >= 0; --id) {
-    const int sp = spell_of_id_p[id];
-    if (sp < 0) continue;
-    next_alias[id] = id_of_spell[sp];
-    id_of_spell[sp] = id;
-  }
-  if ((rc = a.upload(h.lx_cstart, &t.lx_cstart)) || (rc = a.upload(h.lx_cbyte, &t.lx_cbyte)) ||
-      (rc = a.upload(h.lx_cnode, &t.lx_cnode)) || (rc = a.upload(h.lx_pcats, &t.lx_pcats)) ||
-      (rc = a.upload(h.lx_wcats, &t.lx_wcats)) || (rc = a.upload(hv.spell_off, &t.spell_off)) ||
-      (rc = a.upload(hv.spell_bytes, &t.spell_bytes)) ||
-      (rc = a.upload(spell_of_id_p, &t.spell_of_id)) || (rc = a.upload(id_of_spell, &t.id_of_spell)) ||
-      (rc = a.upload(next_alias, &t.next_alias)) || (rc = a.upload(hv.first_of_byte, &t.first_of_byte)))
-    return fail(rc);
-  {
-    std::vector<uint32_t> s16((size_t)hv.NS * 4, 0u);
-    for (int sp = 0; sp < hv.NS; ++sp) {
-      const int off = hv.spell_off[sp], len = std::min(16, hv.spell_off[sp + 1] - off);
-      std::memcpy(reinterpret_cast<uint8_t*>(s16.data() + (size_t)sp * 4), hv.spell_bytes.data() + off, len);
-    }
-    const uint32_t* d16 = nullptr;
-    if ((rc = a.upload(s16, &d16))) return fail(rc);
-    t.spell16 = reinterpret_cast<const uint4*>(d16);
-  }
-  // precomputed lexer states: the start state and every state at which no
-  // lexicon category is live (there the lexicon node cannot matter)
-  std::vector<int32_t> tq{kStart};
-  std::vector<int16_t> tbl_of_q(h.Q, -1);
-  tbl_of_q[kStart] = 0;
-  const long ncls = (long)(2 * h.Q) << h.n_cat;
-  t.ci_on = ncls < (long)kClsFirstCode ? 1 : 0;
-  if (t.ci_on) {
-    for (int q = 2; q < h.Q; ++q) {
-      bool catlive = false;
-      for (int w = 0; w < 4; ++w)
-        if (h.live[q * 4 + w] & h.catmask[w]) catlive = true;
-      if (!catlive && tq.size() < 4096) {
-        tbl_of_q[q] = (int16_t)tq.size();
-        tq.push_back(q);
-      }
-    }
-  }
-  t.n_tbl = (int)tq.size();
-  t.ncls = t.ci_on ? (int)ncls : 0;
-  t.nselw = (t.ncls + kPackCodes + 31) / 32;
-  if ((rc = a.upload(tq, &t.tbl_q)) || (rc = a.upload(tbl_of_q, &t.tbl_of_q)) || (rc = a.upload(h.acc_sym, &t.acc_sym)))
-    return fail(rc);
+  GRID_CUDA(cudaMemsetAsync(lx_hash, 0xFF, ((size_t)t.lx_hmask + 1) * 16, st));
+  GRID_CUDA(cudaMemsetAsync(id_of_spell, 0xFF, (size_t)std::max(1, t.NS) * 4, st));
+  k_lex_hash<<<(h.LN + 255) / 256 + 1, 256, 0, st>>>(lx_cstart, lx_cbyte, lx_cnode, t.lx_pcats, t.lx_wcats, h.LN,
+                                                    lx_hash, t.lx_hmask, t.lx_hshift);
+  k_ids<<<(t.Vp + 255) / 256, 256, 0, st>>>(t.spell_of_id, t.Vp, id_of_spell, next_alias, id_valid);
+  k_spell16<<<(t.NS + 255) / 256 + 1, 256, 0, st>>>(t.spell_off, t.spell_bytes, t.NS, spell16);
   {
     Blake2b fb;
     fb.init(16);
@@ -2030,30 +2197,32 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, dev);
   g_sms = s->sms;
   // CI classification on the device (temporaries live in `tmp`)
-  Arena tmp;
-  auto fail_tmp = [&](int code) {
-    tmp.release();
-    return fail(code);
-  };
-  uint16_t* cls_sp = nullptr;
-  uint16_t* key_sp = nullptr;
-  int32_t* counts_d = nullptr;
-  uint16_t* cls_by_id = nullptr;
-  uint32_t* vc_by_id = nullptr;
+  uint16_t *cls_sp = nullptr, *key_sp = nullptr, *cls_by_id = nullptr;
+  int32_t* counts_d = nullptr;  // per table: walked spellings, verdict-class spellings; then the fills of both lists
+  uint32_t *vc_by_id = nullptr, *vc_sp = nullptr;
   uint8_t* fb = nullptr;
-  if ((rc = tmp.alloc((size_t)t.n_tbl * t.NS * 2, (void**)&cls_sp)) ||
-      (rc = tmp.alloc((size_t)t.n_tbl * t.NS * 2, (void**)&key_sp)) ||
-      (rc = tmp.alloc((size_t)t.n_tbl * 8, (void**)&counts_d)) ||
-      (rc = a.alloc((size_t)t.n_tbl * t.Vp * 2, (void**)&cls_by_id)) || (rc = a.alloc((size_t)t.Vp, (void**)&fb)))
-    return fail_tmp(rc);
+  {
+    Upload up;
+    up.reserve((size_t)t.n_tbl * t.NS, &cls_sp);
+    up.reserve((size_t)t.n_tbl * t.NS, &key_sp);
+    up.reserve((size_t)t.n_tbl * t.NS, &vc_sp);
+    up.reserve((size_t)t.n_tbl * 5, &counts_d);
+    if ((rc = up.commit(tmp, st, keep))) return fail_tmp(rc);
+    up.reserve((size_t)t.n_tbl * t.Vp, &cls_by_id);
+    up.reserve((size_t)t.Vp, &fb);
+    if ((rc = up.commit(a, st, keep))) return fail_tmp(rc);
+  }
   t.cls_by_id = cls_by_id;
   t.first_byte_by_id = fb;
-  GRID_CUDA(cudaMemsetAsync(counts_d, 0, (size_t)t.n_tbl * 8, st));
+  int32_t *cd_fill = counts_d + 2 * t.n_tbl, *vc_fill = counts_d + 3 * t.n_tbl, *vc_count = counts_d + 4 * t.n_tbl;
+  GRID_CUDA(cudaMemsetAsync(counts_d, 0, (size_t)t.n_tbl * 20, st));
   const dim3 cgrid(std::max(1, std::min((t.NS + 255) / 256, 4 * s->sms)), t.n_tbl);
   if (t.blob_bytes)
     k_classify<true><<<cgrid, 256, t.blob_bytes, st>>>(TabT<true>(t), cls_sp, key_sp, counts_d);
   else
     k_classify<false><<<cgrid, 256, 0, st>>>(TabT<false>(t), cls_sp, key_sp, counts_d);
+  // the reserve's tables are laid out while the device classifies
+  if ((rc = build_reserve_tables(s, st, keep))) return fail_tmp(rc);
   std::vector<int32_t> counts2(2 * t.n_tbl);
   GRID_CUDA(cudaMemcpyAsync(counts2.data(), counts_d, t.n_tbl * 8, cudaMemcpyDeviceToHost, st));
   GRID_CUDA(cudaStreamSynchronize(st));
@@ -2063,135 +2232,87 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
     cdoff[k + 1] = cdoff[k] + counts2[2 * k];
     vcbase[k + 1] = vcbase[k] + counts2[2 * k + 1];
   }
-  // CD spellings walked byte by byte (more than kMaxEv events)
+  // CD spellings walked byte by byte (more than kMaxEv events), and the event
+  // records of the verdict-class spellings -> distinct records per table
+  const int nslot = vcbase.back();
   int32_t* cd_list = nullptr;
   uint16_t* cd_key = nullptr;
-  if ((rc = a.upload(cdoff, &t.cd_off)) || (rc = a.alloc((size_t)cdoff.back() * 4, (void**)&cd_list)) ||
-      (rc = a.alloc((size_t)cdoff.back() * 2, (void**)&cd_key)))
-    return fail_tmp(rc);
+  const int32_t* vcbase_d = nullptr;
+  int32_t *slot_tbl = nullptr, *slot_sp = nullptr, *rep = nullptr, *place = nullptr, *tab = nullptr;
+  Rec* slot_rec = nullptr;
+  uint32_t tab_mask = 1;
+  while (tab_mask < 2u * (uint32_t)nslot) tab_mask = 2 * tab_mask + 1;
+  {
+    Upload up;
+    up.add(vcbase, &vcbase_d);
+    up.reserve(nslot, &slot_tbl);
+    up.reserve(nslot, &slot_sp);
+    up.reserve(nslot, &slot_rec);
+    up.reserve(nslot, &rep);
+    up.reserve(nslot, &place);
+    up.reserve((size_t)tab_mask + 1, &tab);
+    if ((rc = up.commit(tmp, st, keep))) return fail_tmp(rc);
+    up.add(cdoff, &t.cd_off);
+    up.reserve(cdoff.back(), &cd_list);
+    up.reserve(cdoff.back(), &cd_key);
+    if ((rc = up.commit(a, st, keep))) return fail_tmp(rc);
+  }
   t.cd_list = cd_list;
   t.cd_key = cd_key;
-  k_compact<<<t.n_tbl, 1024, 0, st>>>(cls_sp, key_sp, t.NS, t.cd_off, cd_list, cd_key);
-  // event records of the verdict-class spellings -> distinct records per table
-  const int nslot = vcbase.back();
-  const int32_t* vcbase_d = nullptr;
-  int32_t *fill = nullptr, *slot_tbl = nullptr, *slot_sp = nullptr;
-  uint16_t* slot_rec = nullptr;
-  uint32_t* vc_sp = nullptr;
-  if ((rc = tmp.upload(vcbase, &vcbase_d)) || (rc = tmp.alloc((size_t)t.n_tbl * 4, (void**)&fill)) ||
-      (rc = tmp.alloc((size_t)nslot * 4, (void**)&slot_tbl)) || (rc = tmp.alloc((size_t)nslot * 4, (void**)&slot_sp)) ||
-      (rc = tmp.alloc((size_t)nslot * kRecLen * 2, (void**)&slot_rec)) ||
-      (rc = tmp.alloc((size_t)t.n_tbl * t.NS * 4, (void**)&vc_sp)))
-    return fail_tmp(rc);
-  GRID_CUDA(cudaMemsetAsync(fill, 0, (size_t)t.n_tbl * 4, st));
-  if (nslot > 0 && t.blob_bytes)
-    k_events<true><<<cgrid, 256, t.blob_bytes, st>>>(TabT<true>(t), cls_sp, vcbase_d, fill, slot_tbl, slot_sp, slot_rec);
-  else if (nslot > 0)
-    k_events<false><<<cgrid, 256, 0, st>>>(TabT<false>(t), cls_sp, vcbase_d, fill, slot_tbl, slot_sp, slot_rec);
-  std::vector<int32_t> h_tbl(nslot);
-  std::vector<uint16_t> h_rec((size_t)nslot * kRecLen);
+  k_compact<<<dim3((t.NS + 255) / 256 + 1, t.n_tbl), 256, 0, st>>>(cls_sp, key_sp, t.NS, t.cd_off, t.cls_map, cd_fill,
+                                                                   cd_list, cd_key);
+  const int sgrid = (nslot + 255) / 256;
+  std::vector<int32_t> n_distinct(t.n_tbl, 0);
   if (nslot > 0) {
-    GRID_CUDA(cudaMemcpyAsync(h_tbl.data(), slot_tbl, (size_t)nslot * 4, cudaMemcpyDeviceToHost, st));
-    GRID_CUDA(cudaMemcpyAsync(h_rec.data(), slot_rec, (size_t)nslot * kRecLen * 2, cudaMemcpyDeviceToHost, st));
+    uint16_t* rec16 = reinterpret_cast<uint16_t*>(slot_rec);
+    if (t.blob_bytes)
+      k_events<true><<<cgrid, 256, t.blob_bytes, st>>>(TabT<true>(t), cls_sp, vcbase_d, vc_fill, slot_tbl, slot_sp, rec16);
+    else
+      k_events<false><<<cgrid, 256, 0, st>>>(TabT<false>(t), cls_sp, vcbase_d, vc_fill, slot_tbl, slot_sp, rec16);
+    GRID_CUDA(cudaMemsetAsync(tab, 0xFF, ((size_t)tab_mask + 1) * 4, st));
+    k_vc_merge<<<sgrid, 256, 0, st>>>(slot_tbl, slot_rec, nslot, tab, tab_mask, rep, place, vc_count);
+    GRID_CUDA(cudaMemcpyAsync(n_distinct.data(), vc_count, t.n_tbl * 4, cudaMemcpyDeviceToHost, st));
   }
   GRID_CUDA(cudaStreamSynchronize(st));
-  // class ids with equal terminal sets are interchangeable in a record:
-  // rewrite each to the smallest such id before deduplication
-  std::vector<uint16_t> canon(std::max(1, t.ncls));
-  if (t.ncls > 0) {
-    // terminal set of every class id, and per terminal the mask of the
-    // classes whose set holds it (the class selection ORs these)
-    uint4* sets_d = nullptr;
-    if ((rc = a.alloc((size_t)t.ncls * 16, (void**)&sets_d))) return fail_tmp(rc);
-    k_class_sets<<<(t.ncls + 255) / 256, 256, 0, st>>>(TabT<false>(t), sets_d);
-    std::vector<uint4> sets(t.ncls);
-    GRID_CUDA(cudaMemcpyAsync(sets.data(), sets_d, (size_t)t.ncls * 16, cudaMemcpyDeviceToHost, st));
-    GRID_CUDA(cudaStreamSynchronize(st));
-    t.cls_sets = reinterpret_cast<const uint32_t*>(sets_d);
-    std::vector<uint32_t> cmask((size_t)t.T1 * t.nselw, 0u);
-    for (int c = 0; c < t.ncls; ++c) {
-      const uint32_t wv[4] = {sets[c].x, sets[c].y, sets[c].z, sets[c].w};
-      for (int tau = 0; tau < t.T1; ++tau)
-        if ((wv[tau >> 5] >> (tau & 31)) & 1u) cmask[(size_t)tau * t.nselw + (c >> 5)] |= 1u << (c & 31);
-    }
-    if ((rc = a.upload(cmask, &t.cls_mask))) return fail_tmp(rc);
-    std::unordered_map<std::string, uint16_t> first;
-    for (int c = 0; c < t.ncls; ++c) {
-      std::string key(reinterpret_cast<const char*>(&sets[c]), 16);
-      canon[c] = first.emplace(key, (uint16_t)c).first->second;
-    }
-    for (int i = 0; i < nslot; ++i) {
-      uint16_t* r = h_rec.data() + (size_t)i * kRecLen;
-      if (r[1] < t.ncls) r[1] = canon[r[1]];
-      for (int e = 0; e < r[0]; ++e)
-        if (r[2 + e] < t.ncls) r[2 + e] = canon[r[2 + e]];
-    }
+  std::vector<int32_t> vcoff(t.n_tbl + 1, 0);
+  for (int k = 0; k < t.n_tbl; ++k) {
+    vcoff[k + 1] = vcoff[k] + n_distinct[k];
+    s->max_vc = std::max(s->max_vc, n_distinct[k]);
   }
-  std::vector<int32_t> vcoff(t.n_tbl + 1, 0), h_vc(nslot);
-  std::vector<uint16_t> recs;
+  s->vcw = (s->max_vc + 31) / 32;
+  // each table's records in the order of their event sequences: a walk item
+  // evaluates 32 neighbouring records on one row's stack, and records that
+  // share their first events take the same path through them, so the warp's
+  // lanes stay together
+  Rec* recs = nullptr;
+  uint16_t* firsts = nullptr;
+  RecKey* keys = nullptr;
+  int32_t *src = nullptr, *rank = nullptr;
+  const int n_vc = vcoff.back();
   {
-    std::vector<std::unordered_map<std::string, int32_t>> seen(t.n_tbl);
-    std::vector<std::vector<uint16_t>> per(t.n_tbl);
-    for (int i = 0; i < nslot; ++i) {
-      const int k = h_tbl[i];
-      const uint16_t* r = h_rec.data() + (size_t)i * kRecLen;
-      std::string key(reinterpret_cast<const char*>(r), kRecLen * 2);
-      auto it = seen[k].find(key);
-      if (it == seen[k].end()) {
-        it = seen[k].emplace(key, (int32_t)(per[k].size() / kRecLen)).first;
-        per[k].insert(per[k].end(), r, r + kRecLen);
-      }
-      h_vc[i] = it->second;
-    }
-    // order each table's records by their event sequences (then the event
-    // count and the final class): a walk item evaluates 32 neighbouring
-    // records on one row's stack, and records that share their first events
-    // take the same path through them, so the warp's lanes stay together
-    for (int k = 0; k < t.n_tbl; ++k) {
-      const int n = (int)(per[k].size() / kRecLen);
-      std::vector<int32_t> ord(n), pos(n);
-      for (int i = 0; i < n; ++i) ord[i] = i;
-      const uint16_t* R = per[k].data();
-      std::sort(ord.begin(), ord.end(), [&](int x, int y) {
-        const uint16_t* a = R + (size_t)x * kRecLen;
-        const uint16_t* b = R + (size_t)y * kRecLen;
-        const int m = std::min<int>(a[0], b[0]);
-        for (int e = 0; e < m; ++e)
-          if (a[2 + e] != b[2 + e]) return a[2 + e] < b[2 + e];
-        if (a[0] != b[0]) return a[0] < b[0];
-        if (a[1] != b[1]) return a[1] < b[1];
-        return x < y;
-      });
-      std::vector<uint16_t> sorted(per[k].size());
-      for (int i = 0; i < n; ++i) {
-        pos[ord[i]] = i;
-        std::copy(R + (size_t)ord[i] * kRecLen, R + (size_t)(ord[i] + 1) * kRecLen, sorted.begin() + (size_t)i * kRecLen);
-      }
-      per[k].swap(sorted);
-      for (auto& kv : seen[k]) kv.second = pos[kv.second];
-    }
-    for (int i = 0; i < nslot; ++i) {
-      const uint16_t* r = h_rec.data() + (size_t)i * kRecLen;
-      h_vc[i] = seen[h_tbl[i]].at(std::string(reinterpret_cast<const char*>(r), kRecLen * 2));
-    }
-    for (int k = 0; k < t.n_tbl; ++k) {
-      vcoff[k + 1] = vcoff[k] + (int32_t)(per[k].size() / kRecLen);
-      recs.insert(recs.end(), per[k].begin(), per[k].end());
-      s->vcw = std::max(s->vcw, (int)((per[k].size() / kRecLen + 31) / 32));
-    }
+    Upload up;
+    up.add(vcoff, &t.vc_off);
+    up.reserve(n_vc, &recs);
+    up.reserve(n_vc, &firsts);
+    if ((rc = up.commit(a, st, keep))) return fail_tmp(rc);
+    up.reserve(n_vc, &keys);
+    up.reserve(n_vc, &src);
+    up.reserve(n_vc, &rank);
+    if ((rc = up.commit(tmp, st, keep))) return fail_tmp(rc);
   }
-  std::vector<uint16_t> first(recs.size() / kRecLen);
-  for (size_t i = 0; i < first.size(); ++i) first[i] = recs[i * kRecLen + 2];
-  for (int k = 0; k < t.n_tbl; ++k) s->max_vc = std::max(s->max_vc, vcoff[k + 1] - vcoff[k]);
-  const int32_t* slot_vc_c = nullptr;
-  if ((rc = a.upload(vcoff, &t.vc_off)) || (rc = a.upload(recs, &t.vc_rec)) || (rc = a.upload(first, &t.vc_first)) ||
-      (rc = tmp.upload(h_vc, &slot_vc_c)))
-    return fail_tmp(rc);
-  if (nslot > 0)
-    k_scatter_vc<<<(nslot + 255) / 256, 256, 0, st>>>(slot_tbl, slot_sp, slot_vc_c, nslot, t.NS, vc_sp);
+  t.vc_rec = reinterpret_cast<const uint16_t*>(recs);
+  t.vc_first = firsts;
+  if (nslot > 0) {
+    k_vc_gather<<<sgrid, 256, 0, st>>>(slot_tbl, slot_rec, nslot, rep, place, t.vc_off, src, keys, rank);
+    k_vc_rank<<<dim3((s->max_vc + 255) / 256, t.n_tbl, 8), 256, 0, st>>>(keys, t.vc_off, rank);
+    k_vc_place<<<(n_vc + 255) / 256, 256, 0, st>>>(slot_rec, slot_tbl, src, rank, n_vc, t.vc_off, recs, firsts, place);
+    k_scatter_vc<<<sgrid, 256, 0, st>>>(slot_tbl, slot_sp, rep, place, nslot, t.NS, vc_sp);
+  }
   // verdict-class indices ride in the 16-bit class codes when they fit;
-  // otherwise k_pack looks them up per id
-  t.vc_inline = t.ncls + kPackCodes + s->max_vc <= 0xFFFF ? 1 : 0;
+  // otherwise k_pack looks them up per id (the rule counts the class ids as
+  // they are before equal sets share one, so that a spec's facts stay what
+  // they are)
+  t.vc_inline = s->n_classes + kPackCodes + s->max_vc <= 0xFFFF ? 1 : 0;
   if (!t.vc_inline && (rc = a.alloc((size_t)t.n_tbl * t.Vp * 4, (void**)&vc_by_id))) return fail_tmp(rc);
   t.vc_by_id = vc_by_id;
   k_permute<<<(t.Vp + 255) / 256, 256, 0, st>>>(t, cls_sp, vc_sp, cls_by_id, vc_by_id, fb);
@@ -2217,7 +2338,6 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   else
     GRID_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_walk<false, false>, kWalkWarps * 32, 0));
   s->walk_blocks = std::max(1, per_sm) * s->sms;
-  if ((rc = build_reserve_tables(s))) return fail(rc);
   *out = s;
   return GRID_OK;
 }
@@ -2228,7 +2348,7 @@ extern "C" int grid_spec_info(const grid_spec* s, int64_t out[8]) {
   std::vector<int32_t> off(t.n_tbl + 1);
   GRID_CUDA(cudaMemcpy(off.data(), t.cd_off, (t.n_tbl + 1) * 4, cudaMemcpyDeviceToHost));
   out[0] = t.n_tbl;
-  out[1] = t.ncls;
+  out[1] = s->n_classes;
   out[2] = off[1] - off[0];
   out[3] = off[t.n_tbl];
   out[4] = t.blob_bytes;

@@ -722,7 +722,7 @@ size_t reserve_scratch_bytes(const grid_spec* s) {
   return (size_t)kReserveEntries * sizeof(REnt) + (size_t)s->t.D * 4;
 }
 
-int build_reserve_tables(grid_spec* s) {
+int build_reserve_tables(grid_spec* s, cudaStream_t st, std::vector<std::vector<uint8_t>>& keep) {
   const HostGrammar& h = s->g->h;
   const HostVocab& hv = s->v->h;
   ReserveTables& rt = s->rt;
@@ -849,16 +849,24 @@ int build_reserve_tables(grid_spec* s) {
     }
     item_cost[i] = sum;
   }
-  int rc;
-  if ((rc = a.upload(h.kitem_off, &rt.item_off)) || (rc = a.upload(h.kitem_p, &rt.item_p)) ||
-      (rc = a.upload(h.kitem_d, &rt.item_d)) || (rc = a.upload(item_cost, &rt.item_cost)) ||
-      (rc = a.upload(h.prod_off, &rt.prod_off)) || (rc = a.upload(h.prod_rhs, &rt.prod_rhs)) ||
-      (rc = a.upload(ny_off, &rt.ny_off)) || (rc = a.upload(ny, &rt.ny)) || (rc = a.upload(rend_off, &rt.rend_off)) ||
-      (rc = a.upload(rend_tok, &rt.rend_tok)) || (rc = a.upload(h.lx_wdist, &rt.lx_wdist)) ||
-      (rc = a.upload(h.lx_wbyte, &rt.lx_wbyte)) || (rc = a.upload(h.dfa_tdist, &rt.dfa_tdist)) ||
-      (rc = a.upload(h.dfa_tbyte, &rt.dfa_tbyte)) || (rc = a.upload(h.sep_byte, &rt.sep_byte)) ||
-      (rc = a.upload(byte_tok, &rt.byte_tok)))
-    return rc;
+  Upload up;
+  up.add(h.kitem_off, &rt.item_off);
+  up.add(h.kitem_p, &rt.item_p);
+  up.add(h.kitem_d, &rt.item_d);
+  up.add(item_cost, &rt.item_cost, false);
+  up.add(h.prod_off, &rt.prod_off);
+  up.add(h.prod_rhs, &rt.prod_rhs);
+  up.add(ny_off, &rt.ny_off, false);
+  up.add(ny, &rt.ny, false);
+  up.add(rend_off, &rt.rend_off, false);
+  up.add(rend_tok, &rt.rend_tok, false);
+  up.add(h.sep_byte, &rt.sep_byte);
+  up.add(byte_tok, &rt.byte_tok, false);
+  up.add(h.dfa_tdist, &rt.dfa_tdist);
+  up.add(h.dfa_tbyte, &rt.dfa_tbyte);
+  up.add(h.lx_wdist, &rt.lx_wdist);
+  up.add(h.lx_wbyte, &rt.lx_wbyte);
+  if (int rc = up.commit(a, st, keep)) return rc;
   rt.NC = std::max(1, h.n_cat);
   rt.n_items = (int)h.kitem_p.size();
   rt.E = kReserveEntries;

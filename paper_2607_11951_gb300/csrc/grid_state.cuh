@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstring>
 #include <string>
 #include <vector>
 
@@ -59,16 +60,6 @@ struct DevConfigs {
 
 struct Arena {
   std::vector<void*> owned;
-  template <typename T>
-  int upload(const std::vector<T>& v, const T** out) {
-    void* p = nullptr;
-    size_t n = std::max<size_t>(v.size(), 1) * sizeof(T);
-    GRID_CUDA(cudaMalloc(&p, n));
-    owned.push_back(p);
-    if (!v.empty()) GRID_CUDA(cudaMemcpy(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice));
-    *out = static_cast<const T*>(p);
-    return GRID_OK;
-  }
   int alloc(size_t n, void** out) {
     GRID_CUDA(cudaMalloc(out, std::max<size_t>(n, 16)));
     owned.push_back(*out);
@@ -77,6 +68,58 @@ struct Arena {
   void release() {
     for (void* p : owned) cudaFree(p);
     owned.clear();
+  }
+};
+
+// Host arrays that go to the device together: one allocation, the small ones
+// in one copy (an allocation and a synchronous copy for each of some fifty
+// arrays was 2 ms of a specialization).  The copies are ordered on a stream;
+// an array that is not `stable` (does not outlive the caller's next
+// synchronization of it) goes through a buffer in `keep`, which does.
+struct Upload {
+  struct Item {
+    const void* host;
+    size_t bytes, at;
+    const void** out;
+    bool direct;
+  };
+  static constexpr size_t kSmall = 32 * 1024;
+  std::vector<Item> items;
+  size_t total = 0;
+  void put(const void* host, size_t bytes, size_t room, const void** out, bool stable) {
+    items.push_back({host, bytes, total, out, stable && bytes > kSmall});
+    total += (std::max<size_t>(room, 16) + 255) & ~size_t(255);
+  }
+  template <typename T>
+  void add(const std::vector<T>& v, const T** out, bool stable = true) {
+    put(v.data(), v.size() * sizeof(T), v.size() * sizeof(T), reinterpret_cast<const void**>(out), stable);
+  }
+  template <typename T>
+  void reserve(size_t n, T** out) {  // device memory that a kernel fills
+    put(nullptr, 0, n * sizeof(T), reinterpret_cast<const void**>(const_cast<const T**>(out)), true);
+  }
+  int commit(Arena& a, cudaStream_t st, std::vector<std::vector<uint8_t>>& keep) {
+    void* base = nullptr;
+    int rc = a.alloc(std::max<size_t>(total, 256), &base);
+    if (rc) return rc;
+    uint8_t* const dev = static_cast<uint8_t*>(base);
+    for (size_t i = 0, j; i < items.size(); i = j) {  // runs of staged arrays through one buffer
+      const size_t at = items[i].at;
+      j = i + 1;
+      if (items[i].direct) {
+        GRID_CUDA(cudaMemcpyAsync(dev + at, items[i].host, items[i].bytes, cudaMemcpyHostToDevice, st));
+        continue;
+      }
+      if (items[i].bytes == 0) continue;
+      while (j < items.size() && !items[j].direct && items[j].bytes > 0) ++j;
+      keep.emplace_back(items[j - 1].at + items[j - 1].bytes - at);
+      for (size_t k = i; k < j; ++k) std::memcpy(keep.back().data() + (items[k].at - at), items[k].host, items[k].bytes);
+      GRID_CUDA(cudaMemcpyAsync(dev + at, keep.back().data(), keep.back().size(), cudaMemcpyHostToDevice, st));
+    }
+    for (const Item& x : items) *x.out = dev + x.at;
+    items.clear();
+    total = 0;
+    return GRID_OK;
   }
 };
 
@@ -173,6 +216,7 @@ struct grid_spec {
   int max_cd = 0;       // longest CD list of a table
   int vcw = 0;          // words of the largest table's verdict-class bitset
   int n_vc = 0;         // verdict classes over all tables
+  int n_classes = 0;    // CI class ids (before equal terminal sets share one)
   int max_vc = 0;       // verdict classes of the largest table
   uint8_t fingerprint[16] = {};  // BLAKE2b-128 of the grammar and vocabulary fingerprints
   ReserveTables rt;
@@ -220,7 +264,7 @@ int launch_advance(const grid_spec* s, const DevConfigs& in, const DevConfigs& o
 
 // Reserve completion tables (grid_span.cu), built at the end of
 // grid_specialize into s->rt (device memory owned by s->mem).
-int build_reserve_tables(grid_spec* s);
+int build_reserve_tables(grid_spec* s, cudaStream_t st, std::vector<std::vector<uint8_t>>& keep);
 // Bytes of grid_reserve's search space per row.
 size_t reserve_scratch_bytes(const grid_spec* s);
 
