@@ -1001,17 +1001,30 @@ __device__ __forceinline__ uint16_t classify(const T& t, int q, int lx, const ui
   return kClsVC;
 }
 
+// An event record in registers: two 16-byte loads, issued together.
+struct RecRegs {
+  uint4 a, b;
+  __device__ __forceinline__ int at(int i) const {
+    const uint32_t w = i < 8 ? (i < 4 ? (i < 2 ? a.x : a.y) : (i < 6 ? a.z : a.w))
+                             : (i < 12 ? (i < 10 ? b.x : b.y) : (i < 14 ? b.z : b.w));
+    return (int)((w >> ((i & 1) * 16)) & 0xFFFFu);
+  }
+};
+
 // Verdict of an event record at the walker's stack: each event is an emission
 // with the recorded candidate set, then the final liveness test.  1 / 0 / -1.
 template <class T>
 __device__ __forceinline__ int eval_record(const T& t, Walker& w, const uint16_t* rec, int max_chain) {
-  const int n = rec[0];
+  RecRegs r;
+  r.a = __ldg(reinterpret_cast<const uint4*>(rec));
+  r.b = __ldg(reinterpret_cast<const uint4*>(rec) + 1);
+  const int n = r.at(0);
   for (int i = 0; i < n; ++i) {
     count_work(w.ctr, 3);
-    const int e = emit_set(t, w, t.set4(rec[2 + i]), max_chain);
+    const int e = emit_set(t, w, t.set4(r.at(2 + i)), max_chain);
     if (e <= 0) return e;
   }
-  const uint16_t f = rec[1];
+  const int f = r.at(1);
   if (f == kClsAcc) return 1;
   return trailing_set(t, w, t.set4(f), max_chain);
 }

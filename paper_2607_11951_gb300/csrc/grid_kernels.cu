@@ -66,7 +66,7 @@
 namespace grid {
 namespace {
 
-constexpr int kWalkWarps = 8;    // warps per k_walk block
+constexpr int kWalkWarps = 24;   // warps per k_walk block, at most (one block per SM)
 constexpr int kSpan = 32;        // CD list entries per walk item (one warp batch)
 constexpr int kStackWin = 1024;  // stacks up to this depth are copied to shared memory in k_row/k_advance
 constexpr int kFilterPer = 4;    // records per k_filter thread
@@ -1188,8 +1188,17 @@ __device__ __forceinline__ int4 row_queue(const Tables& t, const RowCtx& x) {
 // lookups, verdict-class events) in registers and adds the totals to
 // work[0..3] when it is done (and the records and spellings it evaluated to
 // work[4..5]); the plain instance has no counting code.
+struct WalkWarp {
+  uint32_t A[2][4];                 // the cached row's A0 and A1
+  uint16_t lane[2 * kLaneOvl * 32];  // the lanes' overlays and scratch
+  uint16_t win[kWalkWin];           // the row's stack
+  uint16_t ovl[kMaxOvl];            // sigma's overlay
+};
+static_assert(sizeof(WalkWarp) % 16 == 0, "the warps' parts start on 16-byte boundaries");
+constexpr int kWalkSmem = kWalkWarps * (int)sizeof(WalkWarp);  // k_walk's dynamic shared memory beside the tables
+
 template <bool COUNT, bool ST>
-__global__ void __launch_bounds__(kWalkWarps * 32, 2) k_walk(TabT<ST> t, RowCtx* __restrict__ ctx,
+__global__ void __launch_bounds__(kWalkWarps * 32, 1) k_walk(TabT<ST> t, RowCtx* __restrict__ ctx,
                                                              const RowRanges* __restrict__ rng, const uint16_t* stacks,
                                                              const int32_t* __restrict__ surv, int cap,
                                                              const uint32_t* __restrict__ A2,
@@ -1198,18 +1207,15 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 2) k_walk(TabT<ST> t, RowCtx*
                                                              int vcw, const int32_t* __restrict__ vsurv, int vcap,
                                                              int words_v, int B,
                                                              unsigned long long* __restrict__ work) {
-  __shared__ uint16_t s_ovl[kWalkWarps][kMaxOvl];
-  __shared__ uint16_t s_win[kWalkWarps][kWalkWin];
-  __shared__ uint16_t s_lane[kWalkWarps][2 * kLaneOvl * 32];
-  __shared__ __align__(16) uint32_t s_A[kWalkWarps][2][4];  // the cached row's A0 and A1
+  WalkWarp& sw = reinterpret_cast<WalkWarp*>(smem + t.blob_bytes)[threadIdx.x >> 5];
   __shared__ int4 s_seg[kWalkRowsCached];
   stage_tables(t);
   const auto& ts = t;
   pdl_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int gw = blockIdx.x * kWalkWarps + warp;
+  const int gw = blockIdx.x * (blockDim.x >> 5) + warp;
   const int mc = max_chain_of(t);
-  const LArr lo{s_lane[warp] + lane, 32}, ls{s_lane[warp] + kLaneOvl * 32 + lane, 32};
+  const LArr lo{sw.lane + lane, 32}, ls{sw.lane + kLaneOvl * 32 + lane, 32};
   uint32_t cnt[6] = {0u, 0u, 0u, 0u, 0u, 0u};  // the walk's work units, then records and spellings evaluated
   uint32_t* const ctr = COUNT ? cnt : nullptr;
   // queue length and segment ends of every row
@@ -1285,14 +1291,14 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 2) k_walk(TabT<ST> t, RowCtx*
       nrng = r.nrng;
       __syncwarp();
       if (lane < 4) {
-        s_A[warp][0][lane] = r.A0[lane];
-        s_A[warp][1][lane] = r.A1[lane];
+        sw.A[0][lane] = r.A0[lane];
+        sw.A[1][lane] = r.A1[lane];
       }
-      for (int i = lane; i < m1 && i < kMaxOvl; i += 32) s_ovl[warp][i] = r.ovl1[i];
+      for (int i = lane; i < m1 && i < kMaxOvl; i += 32) sw.ovl[i] = r.ovl1[i];
       base = stacks + (size_t)row * t.D;
       if (depth <= kWalkWin) {  // mirror the row's stack: reduce chains read its top repeatedly
-        for (int i = lane; i < depth; i += 32) s_win[warp][i] = base[i];
-        base = s_win[warp];
+        for (int i = lane; i < depth; i += 32) sw.win[i] = base[i];
+        base = sw.win;
       }
       __syncwarp();
     }
@@ -1303,7 +1309,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 2) k_walk(TabT<ST> t, RowCtx*
       bound_row = bound_row < 0 ? row : bound_row;
       continue;
     }
-    const uint32_t* Ac = s_A[warp][c1 ? 1 : 0];
+    const uint32_t* Ac = sw.A[c1 ? 1 : 0];
     const uint32_t* A2row = A2 + ((size_t)row * 2 + (c1 ? 1 : 0)) * t.T1 * 4;
     const int ckeep = c1 ? keep1 : depth, cm = c1 ? m1 : 0;
     const int cq = c1 ? kStart : q, clx = c1 ? 0 : lx;
@@ -1318,7 +1324,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 2) k_walk(TabT<ST> t, RowCtx*
         if (COUNT) ++cnt[4];
         v = vsurv[((size_t)row * 2 + cxi) * vcap + k];
         Walker w;
-        walker_init(w, lo, ls, kLaneOvl, base, ckeep, s_ovl[warp], cm, cq, clx, cpc, cwc, Ac, A2row, ctr);
+        walker_init(w, lo, ls, kLaneOvl, base, ckeep, sw.ovl, cm, cq, clx, cpc, cwc, Ac, A2row, ctr);
         res = eval_record(ts, w, ts.vc_rec + (size_t)(t.vc_off[tb] + v) * kRecLen, mc);
         if (res < 0 && bound_row < 0) bound_row = row;
       }
@@ -1368,7 +1374,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 2) k_walk(TabT<ST> t, RowCtx*
         if (COUNT) ++cnt[5];
         const Spell sp = load_spell(ts, sp_i);
         Walker w;
-        walker_init(w, lo, ls, kLaneOvl, base, ckeep, s_ovl[warp], cm, cq, clx, cpc, cwc, Ac, A2row, ctr);
+        walker_init(w, lo, ls, kLaneOvl, base, ckeep, sw.ovl, cm, cq, clx, cpc, cwc, Ac, A2row, ctr);
         const int res = walk_bytes(ts, w, sp, mc);
         if (res < 0 && bound_row < 0) bound_row = row;
         if (res > 0)  // the verdict of every id with this spelling, in the mask's layout
@@ -1825,12 +1831,15 @@ static int set_smem_limits() {
   const void* kernels[] = {
       (const void*)k_classify<true>, (const void*)k_events<true>, (const void*)k_advance<true>,
       (const void*)k_row<0, true>, (const void*)k_row<1, true>, (const void*)k_row<2, true>,
-      (const void*)k_walk<false, true>, (const void*)k_walk<true, true>,
       // k_pack: one row's class selections and verdict-class bits, two contexts
       (const void*)k_pack<0, false>, (const void*)k_pack<1, false>, (const void*)k_pack<2, false>,
       (const void*)k_pack<0, true>, (const void*)k_pack<1, true>, (const void*)k_pack<2, true>,
       (const void*)k_pack<0, false, true>};
   for (const void* k : kernels) GRID_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
+  const void* walks[] = {(const void*)k_walk<false, true>, (const void*)k_walk<true, true>,
+                         (const void*)k_walk<false, false>, (const void*)k_walk<true, false>};
+  for (const void* k : walks)
+    GRID_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn + kWalkSmem));
   return GRID_OK;
 }
 
@@ -2331,13 +2340,6 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
                                             "row exceed the packing kernel's shared memory"));
   s->n1 = (counts[0] + kSpan - 1) / kSpan;
   s->max_cd = *std::max_element(counts.begin(), counts.end());
-  int per_sm = 0;
-  if (t.blob_bytes)
-    GRID_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_walk<false, true>, kWalkWarps * 32,
-                                                            t.blob_bytes));
-  else
-    GRID_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_walk<false, false>, kWalkWarps * 32, 0));
-  s->walk_blocks = std::max(1, per_sm) * s->sms;
   *out = s;
   return GRID_OK;
 }
@@ -2437,6 +2439,18 @@ extern "C" int grid_advance(const grid_spec* s, const grid_configs* in, grid_con
                         (cudaStream_t)stream);
 }
 
+// Warps per k_walk block.  A walk waits for its look-ups, so a large batch
+// wants every warp that fits (24, by shared memory and 80 registers: 256 SQL
+// rows 291 us a step, 514 us with 8 warps, 337 us with 16), a small one the
+// shortest start, and room for the next kernel's blocks beside it (one
+// expression row 24.4 us with 4 warps, 27.8 us with 24; one SQL row 49.2 and
+// 53.1).  Between them by the items that may come up, about one per 1,024
+// spellings of the vocabulary and row (8 SQL rows: 12 warps, 16 rows: 16).
+static int walk_warps(const grid_spec* s, int B) {
+  const long per_sm = (long)B * ((s->t.NS + 1023) / 1024) / s->sms;
+  return per_sm < 2 ? 4 : per_sm < 4 ? 8 : per_sm < 10 ? 12 : per_sm < 20 ? 16 : kWalkWarps;
+}
+
 // The four kernels of one mask step on `st`; `ev` (5 events or NULL) is
 // recorded before the first kernel and after each.
 int grid::launch_masks(const grid_spec* s, const DevConfigs& c, const MaskScratch& m, int B, uint32_t* d_mask,
@@ -2466,8 +2480,9 @@ int grid::launch_masks(const grid_spec* s, const DevConfigs& c, const MaskScratc
   GRID_CUDA(launch_pdl(k_filter, dim3(std::max(1, cd_blocks + vc_blocks), B, 2), dim3(256), 0, st, t, m.ctx,
                        (const uint32_t*)m.sel, m.surv, m.cap, m.vsurv, m.vcap, cd_blocks));
   if (ev) GRID_CUDA(cudaEventRecord(ev[2], st));
+  const int ww = walk_warps(s, B);
   auto walk = [&](auto kern, const auto& tab) {
-    return launch_pdl(kern, dim3(s->walk_blocks), dim3(kWalkWarps * 32), tab.blob_bytes, st, tab, m.ctx,
+    return launch_pdl(kern, dim3(s->sms), dim3(ww * 32), tab.blob_bytes + ww * sizeof(WalkWarp), st, tab, m.ctx,
                       (const RowRanges*)m.rng, (const uint16_t*)c.stack, (const int32_t*)m.surv, m.cap,
                       (const uint32_t*)m.A2, m.verd0, m.verd1, m.vcbits, vcw, (const int32_t*)m.vsurv, m.vcap,
                       m.words_v, B, s->walk_work);

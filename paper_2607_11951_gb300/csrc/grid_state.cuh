@@ -212,7 +212,6 @@ struct grid_spec {
   int device = 0;
   int sms = 152;
   int n1 = 0;  // walk chunks of the start state's CD list
-  int walk_blocks = 0;  // persistent k_walk grid: resident blocks per SM x SMs
   int max_cd = 0;       // longest CD list of a table
   int vcw = 0;          // words of the largest table's verdict-class bitset
   int n_vc = 0;         // verdict classes over all tables
