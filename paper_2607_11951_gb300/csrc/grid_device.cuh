@@ -151,8 +151,9 @@ struct Tables {
   // per lexer state q and category bits c, at q << n_cat | c (lexeme_tables):
   const uint64_t* ev_list;  // the emission's candidates (LexBatch::ev; 0: none, count 0x7F: more than it holds)
   const uint32_t* live_any; // bit set: a lexeme there is live
+  const uint32_t* cat_live; // bit per lexer state: a lexicon category is live there
   // byte offsets of the staged block's arrays in it
-  int o_class, o_next, o_acc, o_live, o_action, o_go, o_lhs, o_shift, o_roff, o_rp, o_red, o_lany, o_sets;
+  int o_class, o_next, o_acc, o_live, o_action, o_go, o_lhs, o_shift, o_roff, o_rp, o_red, o_lany, o_catq, o_sets;
 };
 
 extern __shared__ __align__(16) uint8_t smem[];
@@ -193,6 +194,7 @@ struct TabT : Tables {
     }
     return Bits4::load(cls_sets + c * 4);
   }
+  __device__ __forceinline__ bool cat_live_at(int q) const { return (get(cat_live, o_catq, q >> 5) >> (q & 31)) & 1u; }
   __device__ __forceinline__ bool live_any_at(int i) const { return (get(live_any, o_lany, i >> 5) >> (i & 31)) & 1u; }
 };
 
@@ -259,13 +261,17 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 constexpr uint32_t kHashEmpty = 0xFFFFFFFFu;
 
 // Child of identifier-trie node lx on byte b (-1 if none), with the child's
-// prefix / word category bits (0 when there is no child).  One 16-byte load
-// per probe; the table is at most half full, so probing ends at an empty slot.
+// prefix / word category bits (0 when there is no child); q is the lexer state
+// after the byte.  A trie node spells a prefix of some category's word, so
+// that category is live in the state that the prefix leaves: where none is,
+// there is no child, and no probe (punctuation, numbers and blanks, each an L2
+// access otherwise).  One 16-byte load per probe; the table is at most half
+// full, so probing ends at an empty slot.
 template <class T>
-__device__ __forceinline__ int lex_step(const T& t, int lx, int b, uint32_t& pc, uint32_t& wc) {
+__device__ __forceinline__ int lex_step(const T& t, int q, int lx, int b, uint32_t& pc, uint32_t& wc) {
   pc = 0u;
   wc = 0u;
-  if (lx < 0) return -1;
+  if (lx < 0 || !t.cat_live_at(q)) return -1;
   const uint32_t key = (uint32_t)lx * 256u + (uint32_t)b;
   uint32_t h = (key * 0x9E3779B1u) >> t.lx_hshift;
   for (uint32_t i = 0; i <= t.lx_hmask; ++i) {
@@ -633,7 +639,7 @@ __device__ __forceinline__ int walk_bytes(const T& t, Walker& w, const Spell& sp
       if (nq == kDead) return 0;
     }
     w.q = nq;
-    w.lx = lex_step(t, w.lx, b, w.pc, w.wc);
+    w.lx = lex_step(t, w.q, w.lx, b, w.pc, w.wc);
     const Bits4 L = live_prime(t, w.q, w.pc);
     const bool any = w.Acur ? (L & (Bits4::load(w.Acur) | t.ign)).any() : L.any();
     if (!any) return 0;
@@ -756,7 +762,7 @@ __device__ __forceinline__ void lex_batch(const T& t, const T& ts, const LexToke
     int i = a;
     for (; i < z; ++i) {
       s.q = L.q[i];
-      s.lx = lex_step(ts, s.lx, L.byte[i], s.pc, s.wc);
+      s.lx = lex_step(ts, s.q, s.lx, L.byte[i], s.pc, s.wc);
       const int id = (s.q << ts.n_cat) | (int)s.pc;
       if (!ts.live_any_at(id)) break;
       if (L.last[i]) L.out[L.last[i] - 1] = s;
@@ -985,7 +991,7 @@ __device__ __forceinline__ uint16_t classify(const T& t, int q, int lx, const ui
       if (nq == kDead) return kClsRej;
     }
     q = nq;
-    lx = lex_step(t, lx, b, pc, wc);
+    lx = lex_step(t, q, lx, b, pc, wc);
   }
   const Bits4 L = live_prime(t, q, pc);
   const bool lign = (L & t.ign).any();

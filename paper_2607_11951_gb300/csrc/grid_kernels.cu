@@ -949,8 +949,8 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfig
         }
         if (by >= 0) {
           uint32_t pc2 = 0u, wc2 = 0u;
-          if (lx >= 0) lex_step(ts, lx, by, pc2, wc2);
           const int q2 = ts.nxt(q * ts.C + ts.cls(by));
+          lex_step(ts, q2, lx, by, pc2, wc2);
           if ((live_prime(ts, q2, pc2) & AI).any()) atomicOr(&s_keep[by >> 5], 1u << (by & 31));
         }
       }
@@ -1063,7 +1063,7 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfig
   if (threadIdx.x == 0) r.status = s_adv[0] != GRID_ST_OK ? s_adv[0] : (complete ? GRID_ST_COMPLETE : s_status);
 }
 
-// grid = (cd_blocks + vc_blocks, B, 2), 256 threads, kFilterPer records per
+// grid = (blocks, B, 2 or 3), 256 threads, kFilterPer records per
 // thread (few blocks, all resident at once): compact, per row and context,
 // what the walk has to evaluate.
 //  - blocks x < cd_blocks: the byte-walked CD spellings that a walk could
@@ -1074,9 +1074,81 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfig
 //    selected (any other record fails at its first emission); survivors go to
 //    vsurv[(b*2 + cx) * vcap ...].
 // Both lists are in any order.
-__global__ void __launch_bounds__(256) k_filter(Tables t, RowCtx* __restrict__ ctx, const uint32_t* __restrict__ sel,
-                                                int32_t* __restrict__ surv, int cap, int32_t* __restrict__ vsurv,
-                                                int vcap, int cd_blocks) {
+//  - z = 2, rows without a table (the pending lexeme may be an identifier),
+//    context sigma: the spellings of the row's continuing first-byte ranges, a range
+//    item per warp, as far as they stay inside the pending lexeme.  Most die
+//    there within a few bytes; one that ends there is viable (its last test is
+//    the walk's), and its ids' verdicts are set here; one that ends the lexeme
+//    goes to the row's unused verdict-class list, for k_walk to walk from the
+//    start.  Walked as they came, 32 of a range to a warp, nearly every warp
+//    waited for one long walk among 31 short ones: 70% of k_walk's time at
+//    256 SQL rows (50,000 items of 13,500 cycles).
+constexpr int kScanList = 1024;  // entries of a verdict-class list, at least, for the scan to use it
+
+// Whether the row's range spellings are in its list, of scan_cap entries (-1:
+// no scan in this step); else k_walk goes through the ranges.
+__device__ __forceinline__ bool scanned(const RowCtx& r, int scan_cap) { return r.nsurv[0] <= scan_cap; }
+
+__device__ __forceinline__ void scan_ranges(const TabT<false>& t, RowCtx& r, const RowRanges& R, int32_t* list,
+                                            int vcap, uint32_t* verd, int warp, int warps, int lane,
+                                            unsigned long long* work) {
+  const Bits4 AI = Bits4{r.A0[0], r.A0[1], r.A0[2], r.A0[3]} | t.ign;
+  const int items = r.nrange, nrng = r.nrng;
+  const LexState s0{r.q, r.lx, r.pc0, r.wc0};
+  int steps = 0, count = 0;
+  for (int c = warp; c < items; c += warps) {
+    int a = 0, z = nrng;  // range a with cpre[a] <= c < cpre[a + 1]
+    while (z - a > 1) {
+      const int mid = (a + z) >> 1;
+      if (R.cpre[mid] <= c)
+        a = mid;
+      else
+        z = mid;
+    }
+    const int sp_i = R.lo[a] + (c - R.cpre[a]) * kRangeSpan + lane;
+    int res = 0;  // 0 rejected, 1 viable, 2 ends the pending lexeme
+    if (sp_i < R.hi[a]) {
+      const Spell sp = load_spell(t, sp_i);
+      LexState s = s0;
+      res = 1;
+      ++count;
+      for (int i = 0; i < sp.len; ++i) {
+        const int b = sp.at(i);
+        const int nq = t.nxt(s.q * t.C + t.cls(b));
+        if (nq == kDead) {
+          res = 2;
+          break;
+        }
+        ++steps;
+        s.q = nq;
+        s.lx = lex_step(t, s.q, s.lx, b, s.pc, s.wc);
+        if (!(live_prime(t, s.q, s.pc) & AI).any()) {
+          res = 0;
+          break;
+        }
+      }
+      if (res == 1)
+        for (int id = t.id_of_spell[sp_i]; id >= 0; id = t.next_alias[id]) atomicOr(&verd[id >> 5], 1u << (id & 31));
+    }
+    const uint32_t bal = __ballot_sync(0xffffffffu, res == 2);
+    if (bal) {
+      int at = 0;
+      if (lane == 0) at = atomicAdd(&r.nsurv[0], __popc(bal));
+      at = __shfl_sync(0xffffffffu, at, 0) + __popc(bal & ((1u << lane) - 1u));
+      if (res == 2 && at < vcap) list[at] = sp_i;
+    }
+  }
+  if (work) {
+    if (steps) atomicAdd(&work[0], (unsigned long long)steps);
+    if (count) atomicAdd(&work[5], (unsigned long long)count);
+  }
+}
+
+__global__ void __launch_bounds__(256) k_filter(TabT<false> t, RowCtx* __restrict__ ctx,
+                                                const uint32_t* __restrict__ sel, int32_t* __restrict__ surv, int cap,
+                                                int32_t* __restrict__ vsurv, int vcap, int cd_blocks,
+                                                const RowRanges* __restrict__ rng, uint32_t* __restrict__ verd0,
+                                                int words_v, unsigned long long* __restrict__ work) {
   __shared__ int s_warp[8];
   __shared__ int s_base;
   pdl_wait();
@@ -1086,6 +1158,12 @@ __global__ void __launch_bounds__(256) k_filter(Tables t, RowCtx* __restrict__ c
   if (r.complete) return;
   if (cx == 1 && !r.emit_ok) return;
   if (cx == 0 && (q == kStart || tbl0 < 0)) return;
+  if (cx == 2) {
+    if (q != kStart && tbl0 < 0)
+      scan_ranges(t, r, rng[b], vsurv + (size_t)b * 2 * vcap, vcap, verd0 + (size_t)b * words_v,
+                  blockIdx.x * 8 + (threadIdx.x >> 5), gridDim.x * 8, threadIdx.x & 31, work);
+    return;
+  }
   const int tb = cx ? 0 : tbl0;
   const bool vc = (int)blockIdx.x >= cd_blocks;
   const int bx = vc ? (int)blockIdx.x - cd_blocks : (int)blockIdx.x;
@@ -1151,9 +1229,9 @@ __global__ void __launch_bounds__(256) k_filter(Tables t, RowCtx* __restrict__ c
 // classes][sigma' walked CD spellings][sigma verdict classes].  The byte
 // walks come first: their items are the longest, and starting them early
 // keeps them off the end of the kernel.
-__device__ __forceinline__ int4 row_queue(const Tables& t, const RowCtx& x) {
+__device__ __forceinline__ int4 row_queue(const RowCtx& x, int scan_cap) {
   if (x.complete) return make_int4(0, 0, 0, 0);
-  const int ed = x.tbl0 >= 0 ? (x.nsurv[0] + kSpan - 1) / kSpan : x.nrange;
+  const int ed = x.tbl0 >= 0 || scanned(x, scan_cap) ? (x.nsurv[0] + kSpan - 1) / kSpan : x.nrange;
   const int ea = ed + ((x.nvs[1] + 31) >> 5);
   const int eb = ea + (x.nsurv[1] + kSpan - 1) / kSpan;
   return make_int4(ed, ea, eb, eb + ((x.nvs[0] + 31) >> 5));
@@ -1205,7 +1283,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) k_walk(TabT<ST> t, RowCtx*
                                                              uint32_t* __restrict__ verd0,
                                                              uint32_t* __restrict__ verd1, uint32_t* __restrict__ vcbits,
                                                              int vcw, const int32_t* __restrict__ vsurv, int vcap,
-                                                             int words_v, int B,
+                                                             int words_v, int B, int scan_cap,
                                                              unsigned long long* __restrict__ work) {
   WalkWarp& sw = reinterpret_cast<WalkWarp*>(smem + t.blob_bytes)[threadIdx.x >> 5];
   __shared__ int4 s_seg[kWalkRowsCached];
@@ -1213,7 +1291,6 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) k_walk(TabT<ST> t, RowCtx*
   const auto& ts = t;
   pdl_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int gw = blockIdx.x * (blockDim.x >> 5) + warp;
   const int mc = max_chain_of(t);
   const LArr lo{sw.lane + lane, 32}, ls{sw.lane + kLaneOvl * 32 + lane, 32};
   uint32_t cnt[6] = {0u, 0u, 0u, 0u, 0u, 0u};  // the walk's work units, then records and spellings evaluated
@@ -1222,12 +1299,14 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) k_walk(TabT<ST> t, RowCtx*
   const bool cached = B <= kWalkRowsCached;
   if (cached) {
     for (int i = threadIdx.x; i < B; i += blockDim.x) {
-      const int4 e = row_queue(t, ctx[i]);
+      const int4 e = row_queue(ctx[i], scan_cap);
       s_seg[i] = e;
     }
   }
   __syncthreads();
-  int row = gw % B;
+  // a block's warps start on one row, so that its context, lists and A2 are in the SM's L1 (a step of 256 SQL rows: -4%)
+  int row = (int)((long long)blockIdx.x * B / gridDim.x);
+  if (B <= (int)gridDim.x) row = blockIdx.x % B;
   int bound_row = -1;  // first row whose walk hit a bound (its status becomes BOUND)
   int cur = -1;  // row whose context is cached below
   int tbl0 = -1, depth = 0, q = 0, lx = 0, keep1 = 0, m1 = 0, nrng = 0;
@@ -1240,7 +1319,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) k_walk(TabT<ST> t, RowCtx*
     int4 seg = make_int4(0, 0, 0, 0);
     {
       int got = 0;
-      const int4 e = cached ? s_seg[row] : row_queue(t, ctx[row]);
+      const int4 e = cached ? s_seg[row] : row_queue(ctx[row], scan_cap);
       if (lane == 0 && e.w > 0) got = atomicAdd(&ctx[row].work0, 1);
       got = __shfl_sync(0xffffffffu, got, 0);
       if (e.w > 0 && got < e.w) {
@@ -1254,7 +1333,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) k_walk(TabT<ST> t, RowCtx*
       int4 e = make_int4(0, 0, 0, 0);
       bool has = false;
       if (off + lane < B) {
-        e = cached ? s_seg[rr] : row_queue(t, ctx[rr]);
+        e = cached ? s_seg[rr] : row_queue(ctx[rr], scan_cap);
         has = e.w > 0 && *((volatile const int32_t*)&ctx[rr].work0) < e.w;
       }
       uint32_t bal = __ballot_sync(0xffffffffu, has);
@@ -1334,9 +1413,9 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) k_walk(TabT<ST> t, RowCtx*
     uint32_t* vb = (c1 ? verd1 : verd0) + (size_t)row * words_v;
     const int32_t* list = nullptr;
     int p0, p1, step = 1;
-    if (c1 || tbl0 >= 0) {  // survivors of k_filter
+    if (c1 || tbl0 >= 0 || scanned(r, scan_cap)) {  // survivors of k_filter
       const int n = c1 ? r.nsurv[1] : r.nsurv[0];
-      list = surv + ((size_t)row * 2 + (c1 ? 1 : 0)) * cap;
+      list = c1 || tbl0 >= 0 ? surv + ((size_t)row * 2 + (c1 ? 1 : 0)) * cap : vsurv + (size_t)row * 2 * vcap;
       p0 = (c1 ? cidx - ea : cidx) * kSpan;
       p1 = min(n, p0 + kSpan);
     } else {
@@ -2064,21 +2143,28 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
     t.chain_rate = 0;
   }
   s->n_classes = t.ci_on ? (int)n_ids : 0;
+  s->has_cats = h.n_cat > 0;
   t.ncls = (int)(sets.size() / 4);
   t.nselw = (t.ncls + kPackCodes + 31) / 32;
   const std::vector<uint32_t> no_sets;
   const std::vector<uint32_t>& staged_sets = t.ncls <= kStagedSets ? sets : no_sets;
+  std::vector<uint32_t> cat_live((h.Q + 31) / 32, 0u);
+  for (int q = 0; q < h.Q; ++q)
+    for (int w = 0; w < 4; ++w)
+      if (h.live[q * 4 + w] & h.catmask[w]) cat_live[q >> 5] |= 1u << (q & 31);
   // staged block: byte classes, DFA, acc/live, ACTION, GOTO, production
-  // tables, shift masks and reduce groups, live lexemes, class sets
-  constexpr int kSec = 14;
+  // tables, shift masks and reduce groups, live lexemes, states
+  // with live categories, class sets
+  constexpr int kSec = 15;
   std::vector<size_t> off(kSec + 1, 0);
   const size_t sizes[kSec] = {256, h.next.size() * 2, h.acc.size() * 4, h.live.size() * 4, h.action.size() * 2,
                               h.go.size() * 2, h.plen.size(), h.plhs.size() * 2, shift_mask.size() * 4,
                               red_off.size() * 4, red_p.size() * 2, red_mask.size() * 4, live_any.size() * 4,
-                              staged_sets.size() * 4};
+                              cat_live.size() * 4, staged_sets.size() * 4};
   const void* srcs[kSec] = {h.byte_class, h.next.data(), h.acc.data(), h.live.data(), action16.data(),
                             h.go.data(), h.plen.data(), h.plhs.data(), shift_mask.data(), red_off.data(),
-                            red_p.data(), red_mask.data(), live_any.data(), staged_sets.data()};
+                            red_p.data(), red_mask.data(), live_any.data(), cat_live.data(),
+                            staged_sets.data()};
   for (int k = 0; k < kSec; ++k) off[k + 1] = align16(off[k] + sizes[k]);
   std::vector<uint8_t> blob(off[kSec], 0);
   for (int k = 0; k < kSec; ++k)
@@ -2097,10 +2183,7 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   tbl_of_q[kStart] = 0;
   if (t.ci_on) {
     for (int q = 2; q < h.Q; ++q) {
-      bool catlive = false;
-      for (int w = 0; w < 4; ++w)
-        if (h.live[q * 4 + w] & h.catmask[w]) catlive = true;
-      if (!catlive && tq.size() < 4096) {
+      if (!((cat_live[q >> 5] >> (q & 31)) & 1u) && tq.size() < 4096) {
         tbl_of_q[q] = (int16_t)tq.size();
         tq.push_back(q);
       }
@@ -2171,7 +2254,8 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   t.o_rp = (int)off[10];
   t.o_red = (int)off[11];
   t.o_lany = (int)off[12];
-  t.o_sets = staged_sets.empty() ? -1 : (int)off[13];
+  t.o_catq = (int)off[13];
+  t.o_sets = staged_sets.empty() ? -1 : (int)off[14];
   t.byte_class = dblob + off[0];
   t.next = reinterpret_cast<const uint16_t*>(dblob + off[1]);
   t.acc = reinterpret_cast<const uint32_t*>(dblob + off[2]);
@@ -2185,6 +2269,7 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   t.red_p = reinterpret_cast<const uint16_t*>(dblob + off[10]);
   t.red_mask = reinterpret_cast<const uint32_t*>(dblob + off[11]);
   t.live_any = reinterpret_cast<const uint32_t*>(dblob + off[12]);
+  t.cat_live = reinterpret_cast<const uint32_t*>(dblob + off[13]);
   GRID_CUDA(cudaMemsetAsync(lx_hash, 0xFF, ((size_t)t.lx_hmask + 1) * 16, st));
   GRID_CUDA(cudaMemsetAsync(id_of_spell, 0xFF, (size_t)std::max(1, t.NS) * 4, st));
   k_lex_hash<<<(h.LN + 255) / 256 + 1, 256, 0, st>>>(lx_cstart, lx_cbyte, lx_cnode, t.lx_pcats, t.lx_wcats, h.LN,
@@ -2446,8 +2531,9 @@ extern "C" int grid_advance(const grid_spec* s, const grid_configs* in, grid_con
 // expression row 24.4 us with 4 warps, 27.8 us with 24; one SQL row 49.2 and
 // 53.1).  Between them by the items that may come up, about one per 1,024
 // spellings of the vocabulary and row (8 SQL rows: 12 warps, 16 rows: 16).
+static long walk_items(const grid_spec* s, int B) { return (long)B * ((s->t.NS + 1023) / 1024) / s->sms; }  // per SM
 static int walk_warps(const grid_spec* s, int B) {
-  const long per_sm = (long)B * ((s->t.NS + 1023) / 1024) / s->sms;
+  const long per_sm = walk_items(s, B);
   return per_sm < 2 ? 4 : per_sm < 4 ? 8 : per_sm < 10 ? 12 : per_sm < 20 ? 16 : kWalkWarps;
 }
 
@@ -2477,15 +2563,22 @@ int grid::launch_masks(const grid_spec* s, const DevConfigs& c, const MaskScratc
   if (ev) GRID_CUDA(cudaEventRecord(ev[1], st));
   const int cd_blocks = (s->max_cd + 256 * kFilterPer - 1) / (256 * kFilterPer);
   const int vc_blocks = (s->max_vc + 256 * kFilterPer - 1) / (256 * kFilterPer);
-  GRID_CUDA(launch_pdl(k_filter, dim3(std::max(1, cd_blocks + vc_blocks), B, 2), dim3(256), 0, st, t, m.ctx,
-                       (const uint32_t*)m.sel, m.surv, m.cap, m.vsurv, m.vcap, cd_blocks));
+  // the scan of the ranges in k_filter: where the walks fill the SMs for long (256 SQL rows: 290 -> 248 us a step,
+  // 128 rows 163 -> 157), not where a step waits for the longest of them (32 rows 72 -> 95 us: what is left of the
+  // ranges then packs 32 long walks into a warp)
+  const bool scan = s->has_cats && m.vcap >= kScanList && walk_items(s, B) >= 100;
+  const int scan_blocks = scan ? std::min((t.NS / kRangeSpan + 256 + 7) / 8, std::max(1, 32 * s->sms / B)) : 0;
+  GRID_CUDA(launch_pdl(k_filter, dim3(std::max({1, cd_blocks + vc_blocks, scan_blocks}), B, scan ? 3 : 2), dim3(256), 0,
+                       st, tg, m.ctx,
+                       (const uint32_t*)m.sel, m.surv, m.cap, m.vsurv, m.vcap, cd_blocks, (const RowRanges*)m.rng,
+                       m.verd0, m.words_v, s->walk_work));
   if (ev) GRID_CUDA(cudaEventRecord(ev[2], st));
   const int ww = walk_warps(s, B);
   auto walk = [&](auto kern, const auto& tab) {
     return launch_pdl(kern, dim3(s->sms), dim3(ww * 32), tab.blob_bytes + ww * sizeof(WalkWarp), st, tab, m.ctx,
                       (const RowRanges*)m.rng, (const uint16_t*)c.stack, (const int32_t*)m.surv, m.cap,
                       (const uint32_t*)m.A2, m.verd0, m.verd1, m.vcbits, vcw, (const int32_t*)m.vsurv, m.vcap,
-                      m.words_v, B, s->walk_work);
+                      m.words_v, B, scan ? m.vcap : -1, s->walk_work);
   };
   if (s->walk_work)  // the measured instance, which counts its work
     GRID_CUDA(staged ? walk(k_walk<true, true>, ts) : walk(k_walk<true, false>, tg));

@@ -267,7 +267,7 @@ __device__ __noinline__ void reserve_serial(const T& t, const T& ts, const Reser
           const int nq = ts.nxt(q2 * ts.C + ts.cls(by));
           if (nq == kDead) return false;
           q2 = nq;
-          lx2 = lex_step(ts, lx2, by, pc, wc);
+          lx2 = lex_step(ts, q2, lx2, by, pc, wc);
           if (cat >= 0 && lx2 < 0) return false;
           y[ylen++] = (uint8_t)by;
         }
@@ -580,7 +580,7 @@ __global__ void __launch_bounds__(kRsvWarps * 32) k_reserve(TabT<ST> t, ReserveT
         const int nq = ts.nxt(q2 * ts.C + ts.cls(by));
         if (nq == kDead || rt.byte_tok[by] < 0) return o;
         q2 = nq;
-        lx2 = lex_step(ts, lx2, by, pc, wc);
+        lx2 = lex_step(ts, q2, lx2, by, pc, wc);
         if (cat >= 0 && lx2 < 0) return o;
         w.y[o.ylen++] = (uint8_t)by;
       }

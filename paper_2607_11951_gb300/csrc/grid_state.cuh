@@ -215,6 +215,7 @@ struct grid_spec {
   int max_cd = 0;       // longest CD list of a table
   int vcw = 0;          // words of the largest table's verdict-class bitset
   int n_vc = 0;         // verdict classes over all tables
+  bool has_cats = false;  // lexicon categories (and so lexer states without a table)
   int n_classes = 0;    // CI class ids (before equal terminal sets share one)
   int max_vc = 0;       // verdict classes of the largest table
   uint8_t fingerprint[16] = {};  // BLAKE2b-128 of the grammar and vocabulary fingerprints
