@@ -88,6 +88,7 @@ struct Tables {
   int Vp;     // V rounded up to a multiple of 32: the row length of the id-indexed tables
   Bits4 ign;  // ignored terminals (the set I)
   Bits4 cm;   // category terminals
+  Bits4 par;  // the terminals that the parser sees (not ignored, without $end)
   int cat_term[32];
   // staged block: these arrays (and live_any) live contiguously in `blob`
   const uint8_t* blob;
@@ -153,7 +154,7 @@ struct Tables {
   const uint32_t* live_any; // bit set: a lexeme there is live
   const uint32_t* cat_live; // bit per lexer state: a lexicon category is live there
   // byte offsets of the staged block's arrays in it
-  int o_class, o_next, o_acc, o_live, o_action, o_go, o_lhs, o_shift, o_roff, o_rp, o_red, o_lany, o_catq, o_sets;
+  int o_class, o_next, o_acc, o_live, o_action, o_go, o_lhs, o_shift, o_roff, o_rp, o_red, o_lany, o_catq, o_tblq, o_sets;
 };
 
 extern __shared__ __align__(16) uint8_t smem[];
@@ -194,6 +195,7 @@ struct TabT : Tables {
     }
     return Bits4::load(cls_sets + c * 4);
   }
+  __device__ __forceinline__ int tblq(int q) const { return get(tbl_of_q, o_tblq, q); }
   __device__ __forceinline__ bool cat_live_at(int q) const { return (get(cat_live, o_catq, q >> 5) >> (q & 31)) & 1u; }
   __device__ __forceinline__ bool live_any_at(int i) const { return (get(live_any, o_lany, i >> 5) >> (i & 31)) & 1u; }
 };

@@ -73,7 +73,7 @@ constexpr int kFilterPer = 4;    // records per k_filter thread
 constexpr int kRangeSpan = 32;   // continuing first-byte ranges are walked in items of (up to) this many spellings
 constexpr int kWalkWin = 512;    // k_walk mirrors row stacks up to this depth per warp
 constexpr int kRowWarps = 6;     // k_row: warps per row block
-constexpr int kRowJobWarps = 4;  // k_row: warps 2 .. 5 compute the allowed sets after one shift
+constexpr int kRowJobWarps = kRowWarps - 1;  // k_row: warps 1 .. compute the allowed sets
 // Class codes as k_pack reads them: CI class ids 0..ncls-1, then these five
 // (so that one bit test of the row's class selection covers CI, always and
 // never, and only verdict-class and walked tokens need a second lookup).
@@ -648,17 +648,15 @@ __device__ __forceinline__ void advance_rest(const T& t, const T& ts, const DevC
 }
 
 // One block per row (kRowWarps warps), plus clearing blocks after the rows.
-// Phase 1, every warp at once: warp 0 finds the first bytes that end the
-// pending lexeme; warp 1 makes the forced emission of the pending lexeme
-// (sigma -> sigma', what every token whose first byte ends the lexeme must go
-// through) and the EOS gate (Sec. 3.2) on the stack it leaves; lanes of the
-// job warps take one terminal tau each, in sigma (first half) or sigma'
-// (second half, each lane making the same forced emission itself): tau is
-// allowed iff its reduce chain reaches SHIFT (A0 and A1 are the warps'
-// ballots), and then the allowed set after that shift is A2 (walks and verdict
+// Phase 1, every warp at once: warp 0 finds the first bytes that continue the
+// pending lexeme and what can follow each (rows without a CI table); the job
+// warps make the forced emission of the pending lexeme (sigma -> sigma', what
+// every token whose first byte ends the lexeme must go through), the allowed
+// sets of both contexts (A0 and A1), the EOS gate (Sec. 3.2) and, for every
+// allowed terminal, the allowed set after its shift (A2: walks and verdict
 // classes simulate nothing before their second shift).  Phase 2: warp 0 lays
-// out the live first-byte ranges that continue the lexeme (rows without a CI
-// table; they need A0), warps 1 .. 5 select the contexts' CI classes.  Then
+// out the live ones of the continuing first-byte ranges, warps 1 .. 5 select
+// the contexts' CI classes.  Then
 // thread 0 writes the row's context for the later kernels and, with a mask
 // cache, looks the row's key up (k_pack reads a ready entry) or claims an
 // empty slot for it (k_pack fills it).
@@ -681,8 +679,11 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfig
   __shared__ uint16_t s_ovl1[kMaxOvl];
   __shared__ __align__(16) uint16_t s_ovl2[kRowJobWarps][kMaxOvl * 32];
   __shared__ uint16_t s_scr[kRowJobWarps][kMaxOvl * 32];
+  __shared__ uint16_t s_em[kRowJobWarps][kMaxOvl];
   __shared__ __align__(16) uint32_t s_A0[4], s_A1[4];
-  __shared__ uint32_t s_keep[8], s_kill[8];
+  __shared__ LexToken s_own;
+  __shared__ uint4 s_lv[256];   // rows without a table: live' after each continuing byte
+  __shared__ uint8_t s_by[256]; // the continuing bytes
   __shared__ int s_row[8];  // complete, depth, q, lx, emit_ok, keep1, m1, eos_ok
   __shared__ uint32_t s_pc[2];
   __shared__ int s_status, s_total0, s_nrng, s_adv[3];
@@ -727,10 +728,13 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfig
     int k0 = 0, keep = 0;
     AdvRow row;
     LexToken own;
-    if (warp == 0) {
-      // (the first tokens with their spellings, and the configuration with its stack: two chains of loads)
-      const int32_t* toks = adv.tokens + (size_t)b * adv.n_steps;
+    const int32_t* toks = adv.tokens + (size_t)b * adv.n_steps;
+    if (ADV == 1 && warp == 1) {  // the token with its spelling, beside the configuration with its stack: two chains of loads
       own = lex_fetch(t, toks, 0, adv.n_steps, lane);
+      if (lane == 0) s_own = own;
+    }
+    if (warp == 0) {
+      if (ADV == 2) own = lex_fetch(t, toks, 0, adv.n_steps, lane);
       row = advance_load(t, adv.cin, c, b, adv.copy, lane, s_stk);
       keep = row.depth;
       if (ADV == 2 && feed_fits(t, row, adv.n_steps)) {
@@ -748,7 +752,9 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfig
         keep = f.wlow;
       }
     }
+    if (ADV == 1) __syncthreads();
     if (threadIdx.x == 0) {
+      if (ADV == 1) own = s_own;
       advance_rest(t, ts, c, adv.tokens, k0, adv.n_steps, nullptr, b, s_stk, sh, row, keep, own, o);
       s_row[0] = o.flags & 1;
       s_row[1] = o.depth;
@@ -783,6 +789,7 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfig
       s_nrng = 0;
     }
   }
+  if (threadIdx.x < 4) s_A0[threadIdx.x] = s_A1[threadIdx.x] = 0u;
   __syncthreads();
   const int complete = s_row[0], depth = s_row[1], q = s_row[2], lx = s_row[3];
   const uint32_t pc0 = s_pc[0], wc0 = s_pc[1];
@@ -796,115 +803,147 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfig
     }
     base = s_stk;
   }
-  __syncthreads();
+  if (!ADV || !s_adv[1]) __syncthreads();
   const int mc = max_chain_of(t);
-  const int tbl0 = (q != kStart && t.ci_on) ? t.tbl_of_q[q] : -1;
+  const int tbl0 = (q != kStart && t.ci_on) ? ts.tblq(q) : -1;
   int status = GRID_ST_OK;
   // ---- phase 1: all at once
-  if (threadIdx.x < 8) s_keep[threadIdx.x] = 0u;
-  if (threadIdx.x < 4) {
-    s_A0[threadIdx.x] = 0u;
-    s_A1[threadIdx.x] = 0u;
-  }
-  __syncthreads();
+  const bool ranged = q != kStart && tbl0 < 0 && !complete;  // the spellings that go on are those of first-byte ranges
+  int lo_r[8], hi_r[8];  // warp 0, a ranged row: spellings by first byte 32 j + lane
+  uint32_t cw[8];        // and which of the bytes continue the lexeme
   if (warp == 0) {
-    // first bytes that end the pending lexeme (every byte when it is empty)
-    for (int b0 = 0; b0 < 256; b0 += 32) {
-      const int by = b0 + lane;
-      const bool kill = q == kStart || ts.nxt(q * ts.C + ts.cls(by)) == kDead;
-      const uint32_t word = __ballot_sync(0xffffffffu, kill);
-      if (lane == 0) s_kill[b0 >> 5] = word;
+    if (ranged) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        lo_r[j] = t.first_of_byte[j * 32 + lane];
+        hi_r[j] = t.first_of_byte[j * 32 + lane + 1];
+      }
+      // what can follow the lexeme on each continuing byte that starts a
+      // spelling, a byte per lane: known before the allowed set is
+      int nc = 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const bool go = hi_r[j] > lo_r[j] && ts.nxt(q * ts.C + ts.cls(j * 32 + lane)) != kDead;
+        cw[j] = __ballot_sync(0xffffffffu, go);
+        if (go) s_by[nc + __popc(cw[j] & ((1u << lane) - 1u))] = (uint8_t)(j * 32 + lane);
+        nc += __popc(cw[j]);
+      }
+      __syncwarp();
+      for (int i = lane; i < nc; i += 32) {
+        const int by = s_by[i];
+        uint32_t pc2 = 0u, wc2 = 0u;
+        const int q2 = ts.nxt(q * ts.C + ts.cls(by));
+        lex_step(ts, q2, lx, by, pc2, wc2);
+        const Bits4 L = live_prime(ts, q2, pc2);
+        s_lv[by] = make_uint4(L.x, L.y, L.z, L.w);
+      }
+      __syncwarp();
     }
     if (ADV && c.hs) hash_nodes(t, c.hs + (size_t)b * t.D, base, s_adv[2], depth, lane);
-  } else if (warp == 1) {
-    // the forced emission of the pending lexeme (sigma -> sigma'), and the
-    // EOS gate (Sec. 3.2) on the stack it leaves
-    int emit_ok = 0, keep1 = depth, m1 = 0, eos = 0;
-    if (lane == 0 && !complete) {
-      Walker w;
-      uint16_t lo[kMaxOvl], ls[kMaxOvl];
-      walker_init(w, LArr{lo, 1}, LArr{ls, 1}, kMaxOvl, base, depth, nullptr, 0, q, lx, pc0, wc0, nullptr, nullptr);
-      if (q == kStart) {
-        emit_ok = 1;
-      } else {
-        const int e = emit(ts, w, mc);
-        if (e < 0) status = GRID_ST_BOUND;
-        emit_ok = e > 0;
-        keep1 = w.keep;
-        m1 = w.m;
-        for (int i = 0; i < m1; ++i) s_ovl1[i] = w.ovl[i];
-      }
-      if (emit_ok) {
-        int keep_o, m_o, ns;
-        const int a = simulate(ts, base, keep1, (const uint16_t*)s_ovl1, m1, t.n_term, LArr{ls, 1}, kMaxOvl, keep_o, m_o,
-                               ns, mc);
-        if (a < 0) status = GRID_ST_BOUND;
-        eos = a == kAccept;
-      }
-      s_row[4] = emit_ok;
-      s_row[5] = keep1;
-      s_row[6] = m1;
-      s_row[7] = eos;
-    }
   } else if (!complete) {
-    // job warps: lane l of job warp jw takes terminal tau = 32 jw + l (and
-    // tau + 32 * half, ...) in one context: tau is allowed iff its reduce
-    // chain reaches SHIFT (A0 / A1 are the ballots), and then the allowed set
-    // after that shift (A2) comes from one set simulation.  sigma' lanes make
-    // the forced emission themselves (the same pick as warp 1), so that both
-    // contexts start at once.
-    const int half = kRowJobWarps / 2;
-    const int cx = warp - 2 >= half ? 1 : 0;
-    const int jw = warp - 2 - cx * half;
-    const LArr scr{s_scr[warp - 2] + lane, 32}, ovl{s_ovl2[warp - 2] + lane, 32};
-    int keep = depth, m = 0;
-    bool has_ctx = cx == 0 ? q != kStart : true;
-    if (cx == 1 && q != kStart) {
-      Walker w;
-      walker_init(w, ovl, scr, kMaxOvl, base, depth, nullptr, 0, q, lx, pc0, wc0, nullptr, nullptr);
-      const int e = emit(ts, w, mc);
-      if (e < 0) status = GRID_ST_BOUND;
-      has_ctx = e > 0;
-      keep = w.keep;
-      m = w.m;  // sigma' is base[0:keep] ++ ovl[0:m]
-    }
-    Bits4 G = Bits4::zero();
-    for (int k = 0; k < t.n_term; ++k) G.set(k);
-    G = G.andnot(ts.ign);
-    for (int tau0 = jw * 32; has_ctx && tau0 < t.n_term; tau0 += 32 * half) {
-      const int tau = tau0 + lane;
-      bool allowed = false;
-      Bits4 An = Bits4::zero();
-      if (tau < t.n_term && !ts.ign.has(tau)) {
-        int keep_o, m_o, ns;
-        const int a = simulate(ts, base, keep, ovl, m, tau, scr, kMaxOvl, keep_o, m_o, ns, mc);
-        if (a < 0) status = GRID_ST_BOUND;
-        allowed = a > 0 && a != kAccept;
-        if (allowed) {
-          if (m_o + ns + 1 <= kMaxOvl) {
-            // the stack after the shift, built in place: base[0:keep_o] ++
-            // ovl[0:m_o] ++ scr[0:ns] ++ (a-1); sigma' itself is rebuilt for
-            // the next terminal of this lane
-            uint16_t saved[kMaxOvl];
-            for (int i = 0; i < m; ++i) saved[i] = ovl[i];
-            for (int i = 0; i < ns; ++i) ovl[m_o + i] = scr[i];
-            ovl[m_o + ns] = (uint16_t)(a - 1);
-            bool bound = false;
-            An = simulate_set(ts, base, keep_o, ovl, m_o + ns + 1, G, scr, kMaxOvl, mc, bound);
-            if (bound) status = GRID_ST_BOUND;
-            for (int i = 0; i < m; ++i) ovl[i] = saved[i];
-          } else {
-            status = GRID_ST_BOUND;
-          }
-          uint32_t* out = A2 + (((size_t)b * 2 + cx) * t.T1 + tau) * 4;
-          out[0] = An.x;
-          out[1] = An.y;
-          out[2] = An.z;
-          out[3] = An.w;
+    // job warps: 32 terminals of one context each, one per lane: tau is
+    // allowed iff its reduce chain reaches SHIFT (A0 / A1 are the ballots),
+    // and then the allowed set after that shift (A2) comes from one set
+    // simulation.  In sigma' (first: its jobs are the longer ones) a warp
+    // begins with the forced emission of the pending lexeme, what every token
+    // whose first byte ends the lexeme must go through: its candidates' chains
+    // run on the lanes, and the first in priority order that reaches SHIFT (or
+    // is ignored) is shifted; and $end's lane finds the EOS gate (Sec. 3.2).
+    // Emission and terminals share one copy of the chain's code: a third of
+    // the issue slots of this kernel went by waiting for instructions.
+    const int nw = (t.T1 + 31) >> 5;
+    uint16_t* const em = s_em[warp - 1];
+    const LArr scr{s_scr[warp - 1] + lane, 32}, ovl{s_ovl2[warp - 1] + lane, 32};
+    for (int job = warp - 1; job < 2 * nw; job += kRowJobWarps) {
+      const int cx = job < nw ? 1 : 0, w0 = cx ? job : job - nw;
+      bool has = cx == 1 || q != kStart;
+      int keep = depth, m = 0;  // the context: base[0:keep] ++ em[0:m]
+      int pick_keep = depth, pick_m = 0;
+      bool emitting = cx == 1 && q != kStart, picked = false, bound = false;
+      Bits4 K = Bits4::zero();
+      if (emitting) {
+        K = cands(ts, q, wc0);
+        if (K.any() && ts.ign.has(K.lowest())) {
+          emitting = false;  // an ignored lexeme: the stack stays
+        } else if (!K.any()) {
+          emitting = has = false;
         }
       }
+      int tau = 32 * w0 + lane, a = 0, ko = 0, mo = 0, ns = 0;
+      for (;;) {
+        const int kw = K.x ? 0 : (K.y ? 1 : (K.z ? 2 : 3));
+        const bool run = emitting ? ((K.word(kw) >> lane) & 1u) && !ts.ign.has(32 * kw + lane)
+                                  : has && tau < (cx ? t.T1 : t.n_term) && !ts.ign.has(tau);
+        a = 0;
+        if (run)
+          a = simulate(ts, base, keep, (const uint16_t*)em, m, emitting ? 32 * kw + lane : tau, scr, kMaxOvl, ko, mo,
+                       ns, mc);
+        if (!emitting) break;
+        bound |= __any_sync(0xffffffffu, a < 0);
+        const uint32_t ok = __ballot_sync(0xffffffffu, a > 0 && a != kAccept), ig = K.word(kw) & ts.ign.word(kw);
+        if (!picked && (ok | ig)) {
+          picked = true;
+          const int l = __ffs(ok | ig) - 1;
+          if ((ok >> l) & 1u) {
+            pick_keep = __shfl_sync(0xffffffffu, ko, l);
+            const int pns = __shfl_sync(0xffffffffu, ns, l);
+            pick_m = pns + 1;
+            if (pick_m > kMaxOvl) {
+              bound = true;
+              pick_m = 0;
+            } else if (lane == l) {
+              for (int i = 0; i < pns; ++i) em[i] = scr[i];
+              em[pns] = (uint16_t)(a - 1);
+            }
+            __syncwarp();
+          }
+        }
+        if (kw == 0) K.x = 0u;
+        else if (kw == 1) K.y = 0u;
+        else if (kw == 2) K.z = 0u;
+        else K.w = 0u;
+        if (!K.any()) {
+          emitting = false;
+          has = picked && !bound;
+          if (bound) status = GRID_ST_BOUND;
+          if (has) {
+            keep = pick_keep;
+            m = pick_m;
+          }
+        }
+      }
+      if (a < 0) status = GRID_ST_BOUND;
+      const bool allowed = a > 0 && a != kAccept;
+      if (cx == 1 && (t.n_term >> 5) == w0) {
+        const bool eos = __any_sync(0xffffffffu, tau == t.n_term && a == kAccept);
+        if (lane == 0) s_row[7] = eos;
+      }
+      if (allowed) {
+        Bits4 An = Bits4::zero();
+        if (mo + ns + 1 <= kMaxOvl) {
+          // the stack after the shift: base[0:ko] ++ em[0:mo] ++ scr[0:ns] ++ (a-1)
+          for (int i = 0; i < mo; ++i) ovl[i] = em[i];
+          for (int i = 0; i < ns; ++i) ovl[mo + i] = scr[i];
+          ovl[mo + ns] = (uint16_t)(a - 1);
+          bool over = false;
+          An = simulate_set(ts, base, ko, ovl, mo + ns + 1, t.par, scr, kMaxOvl, mc, over);
+          if (over) status = GRID_ST_BOUND;
+        } else {
+          status = GRID_ST_BOUND;
+        }
+        reinterpret_cast<uint4*>(A2)[((size_t)b * 2 + cx) * t.T1 + tau] = make_uint4(An.x, An.y, An.z, An.w);
+      }
       const uint32_t word = __ballot_sync(0xffffffffu, allowed);
-      if (lane == 0 && word) atomicOr(cx ? &s_A1[tau0 >> 5] : &s_A0[tau0 >> 5], word);
+      if (lane == 0) (cx ? s_A1 : s_A0)[w0] = word;
+      if (cx == 1 && w0 == 0) {
+        if (lane == 0) {
+          s_row[4] = has;
+          s_row[5] = keep;
+          s_row[6] = m;
+        }
+        for (int i = lane; i < m; i += 32) s_ovl1[i] = em[i];
+      }
+      __syncwarp();
     }
   }
   status = __reduce_max_sync(0xffffffffu, status);
@@ -914,7 +953,7 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfig
   const Bits4 A0 = Bits4::load(s_A0), A1 = Bits4::load(s_A1);
   // ---- phase 2: ranges (warp 0), class selections (warps 1, 2)
   if (!complete) {
-    if (warp == 0 && q != kStart && tbl0 < 0) {
+    if (warp == 0 && ranged) {
       // continuing first-byte ranges (rows without a CI table for q).  A first
       // byte whose lexeme has no live terminal in A0 u I (category terminals
       // counted only while the lexeme is a prefix of one of their words)
@@ -923,41 +962,14 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfig
       int total0 = 0, nrng = 0;
       RowRanges& R = rng[b];
       const Bits4 AI = A0 | ts.ign;
-      int lo_r[8], hi_r[8];
-      uint32_t cw[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        lo_r[j] = t.first_of_byte[j * 32 + lane];
-        hi_r[j] = t.first_of_byte[j * 32 + lane + 1];
-      }
-      int nc = 0;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int by = j * 32 + lane;
-        cw[j] = __ballot_sync(0xffffffffu, hi_r[j] > lo_r[j] && ts.nxt(q * ts.C + ts.cls(by)) != kDead);
-        nc += __popc(cw[j]);
-      }
-      for (int i0 = 0; i0 < nc; i0 += 32) {  // the live test of the continuing bytes, one per lane
-        int idx = i0 + lane, by = -1;
-        if (idx < nc) {
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const int cnt = __popc(cw[j]);
-            if (by < 0 && idx < cnt) by = j * 32 + (int)__fns(cw[j], 0u, idx + 1);
-            if (by < 0) idx -= cnt;
-          }
+        if (!cw[j]) continue;
+        bool cont = (cw[j] >> lane) & 1u;
+        if (cont) {
+          const uint4 v = s_lv[j * 32 + lane];
+          cont = (Bits4{v.x, v.y, v.z, v.w} & AI).any();
         }
-        if (by >= 0) {
-          uint32_t pc2 = 0u, wc2 = 0u;
-          const int q2 = ts.nxt(q * ts.C + ts.cls(by));
-          lex_step(ts, q2, lx, by, pc2, wc2);
-          if ((live_prime(ts, q2, pc2) & AI).any()) atomicOr(&s_keep[by >> 5], 1u << (by & 31));
-        }
-      }
-      __syncwarp();
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const bool cont = (s_keep[j] >> lane) & 1u;
         const int chunks = cont ? (hi_r[j] - lo_r[j] + kRangeSpan - 1) / kRangeSpan : 0;
         const uint32_t bal = __ballot_sync(0xffffffffu, cont);
         int incl = chunks;
@@ -1036,7 +1048,6 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfig
       r.A0[k] = s_A0[k];
       r.A1[k] = emit_ok ? s_A1[k] : 0u;
     }
-    for (int k = 0; k < 8; ++k) r.kill[k] = s_kill[k];
     r.q = q;
     r.lx = lx;
     r.pc0 = pc0;
@@ -2085,6 +2096,9 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   t.ign = Bits4{h.ignored[0], h.ignored[1], h.ignored[2], h.ignored[3]};
   t.cm = Bits4{h.catmask[0], h.catmask[1], h.catmask[2], h.catmask[3]};
   for (int c = 0; c < h.n_cat; ++c) t.cat_term[c] = h.cat_term[c];
+  uint32_t par[4] = {0u, 0u, 0u, 0u};
+  for (int tau = 0; tau < h.n_term; ++tau) par[tau >> 5] |= 1u << (tau & 31);
+  t.par = Bits4{par[0] & ~h.ignored[0], par[1] & ~h.ignored[1], par[2] & ~h.ignored[2], par[3] & ~h.ignored[3]};
   auto fail = [&](int rc) {
     s->mem.release();
     delete s;
@@ -2152,30 +2166,6 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   for (int q = 0; q < h.Q; ++q)
     for (int w = 0; w < 4; ++w)
       if (h.live[q * 4 + w] & h.catmask[w]) cat_live[q >> 5] |= 1u << (q & 31);
-  // staged block: byte classes, DFA, acc/live, ACTION, GOTO, production
-  // tables, shift masks and reduce groups, live lexemes, states
-  // with live categories, class sets
-  constexpr int kSec = 15;
-  std::vector<size_t> off(kSec + 1, 0);
-  const size_t sizes[kSec] = {256, h.next.size() * 2, h.acc.size() * 4, h.live.size() * 4, h.action.size() * 2,
-                              h.go.size() * 2, h.plen.size(), h.plhs.size() * 2, shift_mask.size() * 4,
-                              red_off.size() * 4, red_p.size() * 2, red_mask.size() * 4, live_any.size() * 4,
-                              cat_live.size() * 4, staged_sets.size() * 4};
-  const void* srcs[kSec] = {h.byte_class, h.next.data(), h.acc.data(), h.live.data(), action16.data(),
-                            h.go.data(), h.plen.data(), h.plhs.data(), shift_mask.data(), red_off.data(),
-                            red_p.data(), red_mask.data(), live_any.data(), cat_live.data(),
-                            staged_sets.data()};
-  for (int k = 0; k < kSec; ++k) off[k + 1] = align16(off[k] + sizes[k]);
-  std::vector<uint8_t> blob(off[kSec], 0);
-  for (int k = 0; k < kSec; ++k)
-    if (sizes[k]) std::memcpy(blob.data() + off[k], srcs[k], sizes[k]);
-  Arena& a = s->mem;
-  int rc;
-  // id-indexed tables are padded to Vp ids (a multiple of 32), so that the
-  // ids of one mask word are read with 16-byte loads
-  t.Vp = (hv.V + 31) & ~31;
-  std::vector<int32_t> spell_of_id_p(hv.spell_of_id);
-  spell_of_id_p.resize(t.Vp, -1);
   // precomputed lexer states: the start state and every state at which no
   // lexicon category is live (there the lexicon node cannot matter)
   std::vector<int32_t> tq{kStart};
@@ -2190,6 +2180,31 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
     }
   }
   t.n_tbl = (int)tq.size();
+  // staged block: byte classes, DFA, acc/live, ACTION, GOTO, production
+  // tables, shift masks and reduce groups, live lexemes, states
+  // with live categories, tables of states, class sets
+  constexpr int kSec = 16;
+  std::vector<size_t> off(kSec + 1, 0);
+  const size_t sizes[kSec] = {256, h.next.size() * 2, h.acc.size() * 4, h.live.size() * 4, h.action.size() * 2,
+                              h.go.size() * 2, h.plen.size(), h.plhs.size() * 2, shift_mask.size() * 4,
+                              red_off.size() * 4, red_p.size() * 2, red_mask.size() * 4, live_any.size() * 4,
+                              cat_live.size() * 4, tbl_of_q.size() * 2,
+                              staged_sets.size() * 4};
+  const void* srcs[kSec] = {h.byte_class, h.next.data(), h.acc.data(), h.live.data(), action16.data(),
+                            h.go.data(), h.plen.data(), h.plhs.data(), shift_mask.data(), red_off.data(),
+                            red_p.data(), red_mask.data(), live_any.data(), cat_live.data(),
+                            tbl_of_q.data(), staged_sets.data()};
+  for (int k = 0; k < kSec; ++k) off[k + 1] = align16(off[k] + sizes[k]);
+  std::vector<uint8_t> blob(off[kSec], 0);
+  for (int k = 0; k < kSec; ++k)
+    if (sizes[k]) std::memcpy(blob.data() + off[k], srcs[k], sizes[k]);
+  Arena& a = s->mem;
+  int rc;
+  // id-indexed tables are padded to Vp ids (a multiple of 32), so that the
+  // ids of one mask word are read with 16-byte loads
+  t.Vp = (hv.V + 31) & ~31;
+  std::vector<int32_t> spell_of_id_p(hv.spell_of_id);
+  spell_of_id_p.resize(t.Vp, -1);
   // identifier-trie edges -> open-addressing hash (load factor <= 1/2)
   int hash_bits = 4;
   while ((size_t(1) << hash_bits) < 2 * h.lx_cbyte.size() + 2) ++hash_bits;
@@ -2217,7 +2232,6 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
     up.add(sets, &t.cls_sets);
     up.add(cls_map, &t.cls_map);
     up.add(tq, &t.tbl_q);
-    up.add(tbl_of_q, &t.tbl_of_q);
     up.add(h.acc_sym, &t.acc_sym);
     up.add(hv.first_of_byte, &t.first_of_byte);
     up.add(h.lx_pcats, &t.lx_pcats);
@@ -2255,7 +2269,8 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   t.o_red = (int)off[11];
   t.o_lany = (int)off[12];
   t.o_catq = (int)off[13];
-  t.o_sets = staged_sets.empty() ? -1 : (int)off[14];
+  t.o_tblq = (int)off[14];
+  t.o_sets = staged_sets.empty() ? -1 : (int)off[15];
   t.byte_class = dblob + off[0];
   t.next = reinterpret_cast<const uint16_t*>(dblob + off[1]);
   t.acc = reinterpret_cast<const uint32_t*>(dblob + off[2]);
@@ -2270,6 +2285,7 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   t.red_mask = reinterpret_cast<const uint32_t*>(dblob + off[11]);
   t.live_any = reinterpret_cast<const uint32_t*>(dblob + off[12]);
   t.cat_live = reinterpret_cast<const uint32_t*>(dblob + off[13]);
+  t.tbl_of_q = reinterpret_cast<const int16_t*>(dblob + off[14]);
   GRID_CUDA(cudaMemsetAsync(lx_hash, 0xFF, ((size_t)t.lx_hmask + 1) * 16, st));
   GRID_CUDA(cudaMemsetAsync(id_of_spell, 0xFF, (size_t)std::max(1, t.NS) * 4, st));
   k_lex_hash<<<(h.LN + 255) / 256 + 1, 256, 0, st>>>(lx_cstart, lx_cbyte, lx_cnode, t.lx_pcats, t.lx_wcats, h.LN,

@@ -38,7 +38,6 @@ struct RowCtx {
   int32_t nrng;
   int32_t fcnt, fid;    // a span's step: bits set in the mask, the lowest
   int32_t chit, cfill;  // mask-cache entry this row reads (hit) or fills (miss), or -1
-  uint32_t kill[8];  // bit b: first byte b ends the pending lexeme
   uint16_t ovl1[kMaxOvl];
 };
 
