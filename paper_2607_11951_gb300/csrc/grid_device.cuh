@@ -276,6 +276,7 @@ __device__ __forceinline__ int lex_step(const T& t, int q, int lx, int b, uint32
   if (lx < 0 || !t.cat_live_at(q)) return -1;
   const uint32_t key = (uint32_t)lx * 256u + (uint32_t)b;
   uint32_t h = (key * 0x9E3779B1u) >> t.lx_hshift;
+#pragma unroll 1
   for (uint32_t i = 0; i <= t.lx_hmask; ++i) {
     const uint4 e = __ldg(&t.lx_hash[h]);
     if (e.x == key) {
@@ -294,6 +295,7 @@ __device__ __forceinline__ int lex_step(const T& t, int q, int lx, int b, uint32
 template <class T>
 __device__ __forceinline__ Bits4 lex_filter(const T& t, const Bits4 v, uint32_t cats) {
   Bits4 out = v.andnot(t.cm);
+#pragma unroll 1
   while (cats) {
     const int c = __ffs(cats) - 1;
     cats &= cats - 1;
@@ -336,6 +338,7 @@ __device__ __forceinline__ int simulate(const T& t, const uint16_t* base, int ke
   int k = keep, mm = m;
   ns = 0;
   int top = mm ? ovl[mm - 1] : base[k - 1];
+#pragma unroll 1
   for (int it = 0; it < max_chain; ++it) {
     if (top >= t.S) return 0;
     count_work(ctr, 1);
@@ -381,12 +384,14 @@ __device__ __forceinline__ Bits4 simulate_set(const T& t, const uint16_t* base, 
                                               uint32_t* ctr = nullptr) {
   Bits4 res = Bits4::zero();
   Bits4 todo = G;
+#pragma unroll 1
   for (int round = 0; round < kSetRounds && todo.any(); ++round) {
     Bits4 g = todo;
     todo = Bits4::zero();
     int k = keep, mm = m, ns = 0;
     int it = 0;
     int top = mm ? ovl[mm - 1] : base[k - 1];
+#pragma unroll 1
     for (; it < max_chain && g.any(); ++it) {
       if (top >= t.S) break;
       count_work(ctr, 1);
@@ -396,6 +401,7 @@ __device__ __forceinline__ Bits4 simulate_set(const T& t, const uint16_t* base, 
       if (!g.any()) break;
       int p = -1;
       Bits4 gp = Bits4::zero();
+#pragma unroll 1
       for (uint32_t e = t.roff(top); e < t.roff(top + 1); ++e) {
         const Bits4 x = g & t.red4(e);
         if (!x.any()) continue;
@@ -432,6 +438,7 @@ __device__ __forceinline__ Bits4 simulate_set(const T& t, const uint16_t* base, 
       return res;
     }
   }
+#pragma unroll 1
   while (todo.any()) {
     const int tau = todo.lowest();
     todo.clear_lowest();
@@ -477,6 +484,7 @@ __device__ __forceinline__ void walker_init(Walker& w, LArr ovl_store, LArr scr_
   w.base = base;
   w.keep = keep;
   w.m = min(m, cap);  // callers pass m <= cap; a larger m would only be a caller bug
+#pragma unroll 1
   for (int k = 0; k < w.m; ++k) w.ovl[k] = ovl[k];
   w.q = q;
   w.lx = lx;
@@ -493,6 +501,7 @@ __device__ __forceinline__ bool commit(Walker& w, int keep_o, int m_o, int ns, i
   if (m_o + ns + 1 > w.cap) return false;
   w.keep = keep_o;
   w.m = m_o;
+#pragma unroll 1
   for (int i = 0; i < ns; ++i) w.ovl[w.m++] = w.scr[i];
   w.ovl[w.m++] = (uint16_t)target;
   return true;
@@ -517,6 +526,7 @@ __device__ __forceinline__ bool materialize(const T& t, Walker& w, int max_chain
 // stack itself.  Returns 1 ok, 0 reject, -1 bound.
 template <class T>
 __device__ __forceinline__ int emit_set(const T& t, Walker& w, Bits4 K, int max_chain) {
+#pragma unroll 1
   while (K.any()) {
     const int tau = K.lowest();
     K.clear_lowest();
@@ -624,6 +634,7 @@ __device__ __forceinline__ Spell load_spell(const T& t, int s) {
 template <class T>
 __device__ __forceinline__ int walk_bytes(const T& t, Walker& w, const Spell& sp, int max_chain) {
   const int len = sp.len;
+#pragma unroll 1
   for (int i = 0; i < len; ++i) {
     count_work(w.ctr, 0);
     const int b = sp.at(i);
@@ -815,6 +826,7 @@ __device__ __forceinline__ int chain(const T& t, const uint16_t* win, int depth,
                                      int& keep_o, int& ns_o, int max_chain) {
   int k = depth, ns = 0, bk = depth;
   int top = win[k - 1], bv = top;  // bv = win[bk - 1]
+#pragma unroll 1
   for (int it = 0; it < max_chain; ++it) {
     if (top >= t.S) return 0;
     const int a = t.act(top * t.T1 + tau);
@@ -968,6 +980,7 @@ __device__ __forceinline__ uint16_t classify(const T& t, int q, int lx, const ui
   uint32_t pc = lx == 0 ? t.root_pc : 0u, wc = lx == 0 ? t.root_wc : 0u;
   int n = 0;
   bool first_ign = false, overflow = false;
+#pragma unroll 1
   for (int i = 0; i < len; ++i) {
     const int b = bytes[i];
     const int c = t.cls(b);
@@ -1027,6 +1040,7 @@ __device__ __forceinline__ int eval_record(const T& t, Walker& w, const uint16_t
   r.a = __ldg(reinterpret_cast<const uint4*>(rec));
   r.b = __ldg(reinterpret_cast<const uint4*>(rec) + 1);
   const int n = r.at(0);
+#pragma unroll 1
   for (int i = 0; i < n; ++i) {
     count_work(w.ctr, 3);
     const int e = emit_set(t, w, t.set4(r.at(2 + i)), max_chain);

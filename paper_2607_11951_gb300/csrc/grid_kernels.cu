@@ -575,6 +575,7 @@ __device__ __forceinline__ void advance_rest(const T& t, const T& ts, const DevC
   int status = GRID_ST_OK;
   const int mc = max_chain_of(t);
   Walker w;
+#pragma unroll 1
   for (int k = k0; k < n_steps; ++k) {
     const int tok = tokens[(size_t)b * n_steps + k];
     if (tok < 0) continue;
@@ -618,9 +619,11 @@ __device__ __forceinline__ void advance_rest(const T& t, const T& ts, const DevC
       status = GRID_ST_STACK_OVERFLOW;
       break;
     }
+#pragma unroll 1
     for (int i = 0; i < w.m; ++i) stack[w.keep + i] = w.ovl[i];
     if (w.m > 0) keep = min(keep, w.keep);
     if (use_win && w.keep + w.m <= kStackWin) {
+#pragma unroll 1
       for (int i = 0; i < w.m; ++i) win[w.keep + i] = w.ovl[i];
     } else {
       use_win = false;
@@ -854,6 +857,7 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfig
     const int nw = (t.T1 + 31) >> 5;
     uint16_t* const em = s_em[warp - 1];
     const LArr scr{s_scr[warp - 1] + lane, 32}, ovl{s_ovl2[warp - 1] + lane, 32};
+#pragma unroll 1
     for (int job = warp - 1; job < 2 * nw; job += kRowJobWarps) {
       const int cx = job < nw ? 1 : 0, w0 = cx ? job : job - nw;
       bool has = cx == 1 || q != kStart;
@@ -870,6 +874,7 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfig
         }
       }
       int tau = 32 * w0 + lane, a = 0, ko = 0, mo = 0, ns = 0;
+#pragma unroll 1
       for (;;) {
         const int kw = K.x ? 0 : (K.y ? 1 : (K.z ? 2 : 3));
         const bool run = emitting ? ((K.word(kw) >> lane) & 1u) && !ts.ign.has(32 * kw + lane)
@@ -892,6 +897,7 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfig
               bound = true;
               pick_m = 0;
             } else if (lane == l) {
+#pragma unroll 1
               for (int i = 0; i < pns; ++i) em[i] = scr[i];
               em[pns] = (uint16_t)(a - 1);
             }
@@ -922,7 +928,9 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfig
         Bits4 An = Bits4::zero();
         if (mo + ns + 1 <= kMaxOvl) {
           // the stack after the shift: base[0:ko] ++ em[0:mo] ++ scr[0:ns] ++ (a-1)
+#pragma unroll 1
           for (int i = 0; i < mo; ++i) ovl[i] = em[i];
+#pragma unroll 1
           for (int i = 0; i < ns; ++i) ovl[mo + i] = scr[i];
           ovl[mo + ns] = (uint16_t)(a - 1);
           bool over = false;
@@ -1123,6 +1131,7 @@ __device__ __forceinline__ void scan_ranges(const TabT<false>& t, RowCtx& r, con
       LexState s = s0;
       res = 1;
       ++count;
+#pragma unroll 1
       for (int i = 0; i < sp.len; ++i) {
         const int b = sp.at(i);
         const int nq = t.nxt(s.q * t.C + t.cls(b));
