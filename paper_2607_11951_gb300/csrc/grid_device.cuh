@@ -871,6 +871,26 @@ __device__ __forceinline__ int feed_live(const T& t, const Feed& f, int q, uint3
   return bound ? -1 : (ok ? 1 : 0);
 }
 
+// Shift on win: lane l's chain ended in SHIFT `a` over win[0:ko) ++ its ns
+// scratch entries.  False where a token pushes more than an overlay holds or
+// the window is full (the lane-serial feed knows what that means).
+__device__ __forceinline__ bool feed_shift(Feed& f, int a, int ko, int ns, int l, int lane) {
+  ko = __shfl_sync(0xffffffffu, ko, l);
+  ns = __shfl_sync(0xffffffffu, ns, l);
+  a = __shfl_sync(0xffffffffu, a, l);
+  const int low = min(f.low, ko), nd = ko + ns + 1;
+  if (nd - low > kMaxOvl || nd > f.cap) return false;
+  for (int i = low + lane; i < f.low; i += 32) f.undo[i] = f.win[i];
+  __syncwarp();
+  if (lane < ns) f.win[ko + lane] = f.scr[lane * 32 + l];
+  if (lane == 0) f.win[ko + ns] = (uint16_t)(a - 1);
+  __syncwarp();
+  f.low = low;
+  f.wlow = min(f.wlow, low);
+  f.depth = nd;
+  return true;
+}
+
 // Go through a batch's lists (its token k is number k0 + k).  True if
 // every token was fed; false if the feed has to go on lane-serially at token
 // f.tok, in the state at its start (the stack is put back by feed_back).
@@ -913,25 +933,64 @@ __device__ __forceinline__ bool parse_batch(const T& t, Feed& f, const LexBatch&
       }
       if (!win) continue;  // ignored
       const int l = __ffs(win) - 1;
-      ko = __shfl_sync(0xffffffffu, ko, l);
-      ns = __shfl_sync(0xffffffffu, ns, l);
-      a = __shfl_sync(0xffffffffu, a, l);
-      const int low = min(f.low, ko), nd = ko + ns + 1;
-      if (nd - low > kMaxOvl || nd > f.cap) return false;
-      for (int i = low + lane; i < f.low; i += 32) f.undo[i] = f.win[i];
-      __syncwarp();
-      if (lane < ns) f.win[ko + lane] = f.scr[lane * 32 + l];
-      if (lane == 0) f.win[ko + ns] = (uint16_t)(a - 1);
-      __syncwarp();
-      f.low = low;
-      f.wlow = min(f.wlow, low);
-      f.depth = nd;
+      if (!feed_shift(f, a, ko, ns, l, lane)) return false;
     }
     if ((f.depth + 1) * t.chain_rate + t.chain_base > max_chain &&
         feed_live(t, f, L.out[k].q, L.out[k].pc, lane, max_chain) != 1)
       return false;
   }
   return true;
+}
+
+// Feed one token of state `s` to win[0:depth), with the warp: the bytes are the
+// same in every lane, a lexeme's candidates run their chains side by side, and
+// the lexeme that is left is tested at the end.  False: for the lane-serial
+// feed, at the token's start (feed_back).
+template <class T>
+__device__ __forceinline__ bool feed_one(const T& t, Feed& f, LexState& s, const Spell& sp, int lane, int max_chain) {
+  const int len = sp.len;
+#pragma unroll 1
+  for (int i = 0; i < len; ++i) {
+    const int b = sp.at(i);
+    const int c = t.cls(b);
+    int nq = t.nxt(s.q * t.C + c);
+    if (nq == kDead) {
+      if (s.q == kStart) return false;
+      Bits4 K = cands(t, s.q, s.wc);
+      for (;;) {  // the candidates, 32 terminals at a time
+        if (!K.any()) return false;
+        const int kw = K.x ? 0 : (K.y ? 1 : (K.z ? 2 : 3));
+        const uint32_t word = K.word(kw), ig = word & t.ign.word(kw);
+        if (ig & (0u - ig) & word & (0u - word)) break;  // an ignored terminal comes first
+        int a = 0, ko = 0, ns = 0;
+        if (((word & ~ig) >> lane) & 1u) a = chain(t, f.win, f.depth, 32 * kw + lane, f.scr + lane, ko, ns, max_chain);
+        if (__any_sync(0xffffffffu, a < 0)) return false;
+        const uint32_t ok = __ballot_sync(0xffffffffu, a > 0 && a != kAccept);
+        if (!(ok | ig)) {
+          if (kw == 0) K.x = 0u;
+          else if (kw == 1) K.y = 0u;
+          else if (kw == 2) K.z = 0u;
+          else K.w = 0u;
+          continue;
+        }
+        const int l = __ffs(ok | ig) - 1;
+        if ((ok >> l) & 1u) {
+          if (!feed_shift(f, a, ko, ns, l, lane)) return false;
+        }
+        break;
+      }
+      s.q = kStart;
+      s.lx = 0;
+      s.pc = t.root_pc;
+      s.wc = t.root_wc;
+      nq = t.nxt(kStart * t.C + c);
+      if (nq == kDead) return false;
+    }
+    s.q = nq;
+    s.lx = lex_step(t, s.q, s.lx, b, s.pc, s.wc);
+    if (!live_prime(t, s.q, s.pc).any()) return false;
+  }
+  return f.depth <= t.D && feed_live(t, f, s.q, s.pc, lane, max_chain) == 1;
 }
 
 // The stack at the start of token f.tok.

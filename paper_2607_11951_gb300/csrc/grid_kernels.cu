@@ -530,10 +530,8 @@ __device__ __forceinline__ AdvRow advance_load(const T& t, const DevConfigs& cin
   return r;
 }
 
-// Whether the warp feeds the row's tokens (else all are advance_rest's).  A
-// single token is lane 0's: with one token there is little to lex side by
-// side, and setting the batch up costs a step of one expression row 0.8 us of
-// 31 (SQL rows: no difference).
+// Whether the warp feeds the row's tokens in batches (else they are
+// advance_rest's; a single token is feed_one's).
 template <class T>
 __device__ __forceinline__ bool feed_fits(const T& t, const AdvRow& r, int n_steps) {
   return n_steps > 1 && t.chain_rate > 0 && r.win && !(r.flags & 1);
@@ -561,12 +559,14 @@ __device__ __forceinline__ void feed_end(const T& ts, Feed& f, bool fed, const L
   __syncwarp();
 }
 
-// Lane 0 only: tokens k0 .. n_steps - 1, one after the other (`first`: token 0, loaded ahead).
+// Lane 0 only: tokens k0 .. n_steps - 1, one after the other (`first`: token 0,
+// loaded ahead).  Seldom reached, and a call, so that its code is not in the
+// way of the rest's.
 template <class T>
-__device__ __forceinline__ void advance_rest(const T& t, const T& ts, const DevConfigs& cout,
-                                             const int32_t* __restrict__ tokens, int k0, int n_steps,
-                                             int32_t* __restrict__ d_status, int b, uint16_t* win, AdvShared& sh,
-                                             const AdvRow& r, int keep, const LexToken& first, AdvOut& out) {
+__device__ __noinline__ void advance_rest(const T& t, const T& ts, const DevConfigs& cout,
+                                             const int32_t* __restrict__ tokens, int k0, int n_steps, int b,
+                                             uint16_t* win, AdvShared& sh, const AdvRow& r, int keep,
+                                             const LexToken& first, AdvOut& out) {
   uint16_t* stack = cout.stack + (size_t)b * t.D;
   const LArr lo{sh.lo, 1}, ls{sh.ls, 1};
   int depth = r.depth, q = r.s.q, lx = r.s.lx, flags = r.flags;
@@ -634,20 +634,36 @@ __device__ __forceinline__ void advance_rest(const T& t, const T& ts, const DevC
     pc = w.pc;
     wcat = w.wc;
   }
-  cout.depth[b] = depth;
-  cout.q[b] = q;
-  cout.lx[b] = lx;
-  cout.flags[b] = flags;
-  if (d_status) d_status[b] = status;
-  out.depth = depth;
-  out.q = q;
-  out.lx = lx;
-  out.flags = flags;
-  out.status = status;
-  out.pc = pc;
-  out.wc = wcat;
-  out.win = use_win;
-  out.keep = keep;
+  out = AdvOut{depth, q, lx, flags, status, pc, wcat, use_win, keep};
+}
+
+// One token of a row, by its warp: feed_one, else advance_rest.
+template <class T>
+__device__ __forceinline__ void advance_one(const T& t, const DevConfigs& cout, const int32_t* __restrict__ tokens,
+                                            int n_steps, int b, uint16_t* win, AdvShared& sh, AdvRow& r,
+                                            const LexToken& x, int lane, AdvOut& out) {
+  const int mc = max_chain_of(t);
+  uint16_t* stack = cout.stack + (size_t)b * t.D;
+  if (x.st == 1 && r.win && !(r.flags & 1)) {
+    Feed f = feed_begin(r, win, sh);
+    LexState s = r.s;
+    if (feed_one(t, f, s, x.sp, lane, mc)) {
+      for (int i = f.wlow + lane; i < f.depth; i += 32) stack[i] = win[i];
+      out = AdvOut{f.depth, s.q, s.lx, r.flags, GRID_ST_OK, s.pc, s.wc, true, f.wlow};
+      return;
+    }
+    feed_back(f, lane);
+  }
+  out = AdvOut{r.depth, r.s.q, r.s.lx, r.flags, GRID_ST_OK, r.s.pc, r.s.wc, r.win, r.depth};
+  if (lane == 0 && x.st != 0) advance_rest(t, t, cout, tokens, 0, n_steps, b, win, sh, r, r.depth, x, out);
+}
+
+// The configuration that the advance leaves, by lane 0.
+__device__ __forceinline__ void advance_store(const DevConfigs& cout, int b, const AdvOut& o) {
+  cout.depth[b] = o.depth;
+  cout.q[b] = o.q;
+  cout.lx[b] = o.lx;
+  cout.flags[b] = o.flags;
 }
 
 // One block per row (kRowWarps warps), plus clearing blocks after the rows.
@@ -728,19 +744,23 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfig
     AdvOut o;
     AdvShared& sh = *reinterpret_cast<AdvShared*>(s_ovl2);
     static_assert(sizeof(AdvShared) <= sizeof(s_ovl2), "the advance's shared state overlays the job warps' area");
-    int k0 = 0, keep = 0;
-    AdvRow row;
-    LexToken own;
     const int32_t* toks = adv.tokens + (size_t)b * adv.n_steps;
-    if (ADV == 1 && warp == 1) {  // the token with its spelling, beside the configuration with its stack: two chains of loads
-      own = lex_fetch(t, toks, 0, adv.n_steps, lane);
-      if (lane == 0) s_own = own;
-    }
-    if (warp == 0) {
-      if (ADV == 2) own = lex_fetch(t, toks, 0, adv.n_steps, lane);
+    AdvRow row;
+    if (ADV == 1) {
+      // the token with its spelling, and the configuration with its stack: two chains of loads on two warps
+      if (warp == 1) {
+        const LexToken own = lex_fetch(t, toks, 0, adv.n_steps, lane);
+        if (lane == 0) s_own = own;
+      } else if (warp == 0) {
+        row = advance_load(t, adv.cin, c, b, adv.copy, lane, s_stk);
+      }
+      __syncthreads();
+      if (warp == 0) advance_one(t, c, adv.tokens, adv.n_steps, b, s_stk, sh, row, s_own, lane, o);
+    } else if (warp == 0) {
+      const LexToken own = lex_fetch(t, toks, 0, adv.n_steps, lane);
       row = advance_load(t, adv.cin, c, b, adv.copy, lane, s_stk);
-      keep = row.depth;
-      if (ADV == 2 && feed_fits(t, row, adv.n_steps)) {
+      int k0 = 0, keep = row.depth;
+      if (feed_fits(t, row, adv.n_steps)) {
         Feed f = feed_begin(row, s_stk, sh);
         LexState carry = row.s;
         bool fed = true;
@@ -754,11 +774,12 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfig
         k0 = f.tok;
         keep = f.wlow;
       }
+      o = AdvOut{row.depth, row.s.q, row.s.lx, row.flags, GRID_ST_OK, row.s.pc, row.s.wc, row.win, keep};
+      if (lane == 0 && k0 < adv.n_steps)
+        advance_rest(t, ts, c, adv.tokens, k0, adv.n_steps, b, s_stk, sh, row, keep, own, o);
     }
-    if (ADV == 1) __syncthreads();
     if (threadIdx.x == 0) {
-      if (ADV == 1) own = s_own;
-      advance_rest(t, ts, c, adv.tokens, k0, adv.n_steps, nullptr, b, s_stk, sh, row, keep, own, o);
+      advance_store(c, b, o);
       s_row[0] = o.flags & 1;
       s_row[1] = o.depth;
       s_row[2] = o.q;
@@ -1793,15 +1814,29 @@ __global__ void __launch_bounds__(64, 3) k_advance(TabT<ST> t, DevConfigs cin, D
     }
   }
   if (warp != 0) return;
-  int k0 = 0, keep = row.depth;
-  if (feed_fits(t, row, n_steps)) {
-    feed_end(ts, f, fed, carry, n_steps, row, cout.stack + (size_t)b * t.D, lane, mc);
-    k0 = f.tok;
-    keep = f.wlow;
-  }
   AdvOut out;
-  out.depth = out.keep = 0;
-  if (lane == 0) advance_rest(t, ts, cout, tokens, k0, n_steps, d_status, b, s_stk, sh, row, keep, own, out);
+  if (n_steps <= 1) {
+    LexToken x;  // the row's one token is lane 0's
+    x.st = __shfl_sync(0xffffffffu, own.st, 0);
+    x.sp.len = __shfl_sync(0xffffffffu, own.sp.len, 0);
+    x.sp.head = make_uint4(__shfl_sync(0xffffffffu, own.sp.head.x, 0), __shfl_sync(0xffffffffu, own.sp.head.y, 0),
+                           __shfl_sync(0xffffffffu, own.sp.head.z, 0), __shfl_sync(0xffffffffu, own.sp.head.w, 0));
+    x.sp.all = reinterpret_cast<const uint8_t*>(__shfl_sync(0xffffffffu, (unsigned long long)own.sp.all, 0));
+    advance_one(t, cout, tokens, n_steps, b, s_stk, sh, row, x, lane, out);
+  } else {
+    int k0 = 0, keep = row.depth;
+    if (feed_fits(t, row, n_steps)) {
+      feed_end(ts, f, fed, carry, n_steps, row, cout.stack + (size_t)b * t.D, lane, mc);
+      k0 = f.tok;
+      keep = f.wlow;
+    }
+    out = AdvOut{row.depth, row.s.q, row.s.lx, row.flags, GRID_ST_OK, row.s.pc, row.s.wc, row.win, keep};
+    if (lane == 0 && k0 < n_steps) advance_rest(t, ts, cout, tokens, k0, n_steps, b, s_stk, sh, row, keep, own, out);
+  }
+  if (lane == 0) {
+    advance_store(cout, b, out);
+    d_status[b] = out.status;
+  }
   if (cout.hs) {
     __syncwarp();
     hash_nodes(t, cout.hs + (size_t)b * t.D, cout.stack + (size_t)b * t.D, __shfl_sync(0xffffffffu, out.keep, 0),
