@@ -1331,7 +1331,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) k_walk(TabT<ST> t, RowCtx*
   stage_tables(t);
   const auto& ts = t;
   pdl_wait();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
   const int mc = max_chain_of(t);
   const LArr lo{sw.lane + lane, 32}, ls{sw.lane + kLaneOvl * 32 + lane, 32};
   uint32_t cnt[6] = {0u, 0u, 0u, 0u, 0u, 0u};  // the walk's work units, then records and spellings evaluated
@@ -1508,6 +1508,93 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) k_walk(TabT<ST> t, RowCtx*
       if (cnt[k]) atomicAdd(&work[k], (unsigned long long)cnt[k]);
 }
 
+// -inf over the rejected ones of elements [e0, e1) of a row of logits, by the
+// `step` threads of which this is number `tid`; bit e of `word` (element e's
+// accept bit is bit e & 31 of word(e >> 5)).  One 256-bit access per 32-byte
+// sector of memory (8 fp32 or 16 bf16), so that every store writes a whole
+// sector and a warp's store covers 1 KB of contiguous bytes.  A sector whose
+// tokens are all rejected is written without being read; a mixed sector is
+// read, blended and written; a fully accepted sector is not touched.  Each
+// thread takes kBatch sectors at a time: their accept bits loaded
+// together, then the rejected sectors stored (they wait on nothing), then the
+// mixed sectors read together and stored, so that a thread waits on two rounds
+// of loads per batch instead of two per sector.  Where the elements start off
+// a sector boundary (SHIFTED) a sector's bits come from two words, and only
+// the elements before the first and after the last whole sector are stored one
+// by one: stored element by element throughout, 256 rows of 151,937 bf16
+// logits took 199 us, this way 23.
+constexpr int kApplyBatch = 4;
+template <typename T, bool SHIFTED, int kBatch, typename Word>
+__device__ __forceinline__ void apply_span(T* row, int e0, int e1, const Word& word, int tid, int step) {
+  constexpr int E = 32 / sizeof(T);  // elements per sector
+  constexpr uint32_t sfull = (1u << E) - 1u;
+  constexpr uint32_t fill = sizeof(T) == 4 ? 0xFF800000u : 0xFF80FF80u;  // -inf in every element of a word
+  const int o = SHIFTED ? min(e1, e0 + (int)(((32u - (uint32_t)(uintptr_t)(row + e0)) & 31u) / sizeof(T))) : e0;
+  const int nsec = (e1 - o) / E;
+  for (int s0 = tid; s0 < nsec; s0 += kBatch * step) {
+    uint32_t sb[kBatch];
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) {  // the sectors' accept bits
+      const int e = o + (s0 + u * step) * E;
+      const bool in = s0 + u * step < nsec;
+      if (SHIFTED) {
+        const uint32_t lo = in ? word(e >> 5) : 0u, hi = in ? word((e + E - 1) >> 5) : 0u;
+        sb[u] = in ? __funnelshift_r(lo, hi, e & 31) & sfull : sfull;
+      } else {
+        sb[u] = in ? (word(e >> 5) >> (e & 31)) & sfull : sfull;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) {  // rejected sectors first: written without a read
+      const int e = o + (s0 + u * step) * E;
+      if (s0 + u * step < nsec && sb[u] == 0u)
+        asm volatile("st.global.v8.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1};" ::"l"(row + e), "r"(fill) : "memory");
+    }
+    uint32_t v[kBatch][8];
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) {  // mixed sectors: read
+      const int e = o + (s0 + u * step) * E;
+      if (s0 + u * step < nsec && sb[u] != 0u && sb[u] != sfull)
+        asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=r"(v[u][0]), "=r"(v[u][1]), "=r"(v[u][2]), "=r"(v[u][3]), "=r"(v[u][4]), "=r"(v[u][5]),
+                       "=r"(v[u][6]), "=r"(v[u][7])
+                     : "l"(row + e)
+                     : "memory");
+    }
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) {  // mixed sectors: blend and store
+      if (s0 + u * step >= nsec || sb[u] == sfull || sb[u] == 0u) continue;
+      T* p = row + o + (s0 + u * step) * E;
+      uint32_t w[8];
+      if (sizeof(T) == 4) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) w[k] = ((sb[u] >> k) & 1u) ? v[u][k] : fill;
+      } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const uint32_t lo = (sb[u] >> (2 * k)) & 1u, hi = (sb[u] >> (2 * k + 1)) & 1u;
+          w[k] = (lo ? (v[u][k] & 0xFFFFu) : 0xFF80u) | (hi ? (v[u][k] & 0xFFFF0000u) : 0xFF800000u);
+        }
+      }
+      asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]),
+                   "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                   : "memory");
+    }
+  }
+  // the elements outside whole sectors, fewer than E at either end
+  if (tid < 2 * E) {
+    const int e = tid < E ? e0 + tid : o + nsec * E + tid - E;
+    if (tid < E ? e < o : e < e1) {
+      if (!((word(e >> 5) >> (e & 31)) & 1u)) {
+        if (sizeof(T) == 4)
+          reinterpret_cast<uint32_t*>(row)[e] = 0xFF800000u;
+        else
+          reinterpret_cast<uint16_t*>(row)[e] = 0xFF80u;
+      }
+    }
+  }
+}
+
 // grid = (ceil(W / kPackWords), B), kPackWords threads: thread (b, wi) makes
 // mask word wi of row b, the 32 token ids 32 wi .. 32 wi + 31 (the id tables
 // are padded to a multiple of 32 ids, so each thread reads its ids' first
@@ -1520,10 +1607,8 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) k_walk(TabT<ST> t, RowCtx*
 // with its class selections) or the walks' verdict word.  The last block of a
 // row writes its status (EMPTY_MASK for a viable row with no bit set).
 //
-// With APPLY (1 = fp32, 2 = bf16 logits) the thread also masks the logits of
-// its 32 ids (Sec. 2 masked decoding, as grid_apply_mask): a 32-byte sector
-// whose ids are all rejected is written with -inf without being read, a mixed
-// sector is read, blended and written, an accepted sector is not touched.
+// With APPLY (1 = fp32, 2 = bf16 logits) the block then masks the logits of its
+// ids (Sec. 2 masked decoding, as grid_apply_mask; apply_span).
 constexpr int kPackWords = 256;
 //
 // With FORCE (a step of grid_forced_span) the last block of a row also finds
@@ -1683,50 +1768,63 @@ __global__ void __launch_bounds__(kPackWords) k_pack(Tables t, RowCtx* __restric
       atomicMin(&s_id, 32 * wi + __ffs(m) - 1);
     }
   }
-  if (APPLY && have) {
+  if (APPLY) {
     using T = typename std::conditional<APPLY == 1, uint32_t, uint16_t>::type;
-    constexpr int E = 32 / sizeof(T);  // elements per 32-byte sector
-    constexpr int NS = 32 / E;         // sectors per mask word
-    constexpr uint32_t sfull = E == 32 ? 0xFFFFFFFFu : (1u << E) - 1u;
-    constexpr uint32_t fill = sizeof(T) == 4 ? 0xFF800000u : 0xFF80FF80u;
     T* row = reinterpret_cast<T*>(logits) + (size_t)b * stride;
-    const int V = t.V;
-    uint32_t v[NS][8];
+    if (APPLY == 2 && vec_ok) {
+      // a thread's word is two bf16 sectors of its own: written from the
+      // register (256 SQL rows: 247 us a step, 255 us through shared memory)
+      if (have) {
+        uint32_t v[2][8];
 #pragma unroll
-    for (int u = 0; u < NS; ++u) {  // mixed whole sectors: read
-      const int e0 = 32 * wi + u * E;
-      const uint32_t sb = (m >> (u * E)) & sfull;
-      if (vec_ok && e0 + E <= V && sb != 0u && sb != sfull)
-        asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=r"(v[u][0]), "=r"(v[u][1]), "=r"(v[u][2]), "=r"(v[u][3]), "=r"(v[u][4]), "=r"(v[u][5]),
-                       "=r"(v[u][6]), "=r"(v[u][7])
-                     : "l"(row + e0)
-                     : "memory");
-    }
+        for (int u = 0; u < 2; ++u) {  // mixed whole sectors: read
+          const int e = 32 * wi + 16 * u;
+          const uint32_t sb = (m >> (16 * u)) & 0xFFFFu;
+          if (e + 16 <= t.V && sb != 0u && sb != 0xFFFFu)
+            asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                         : "=r"(v[u][0]), "=r"(v[u][1]), "=r"(v[u][2]), "=r"(v[u][3]), "=r"(v[u][4]), "=r"(v[u][5]),
+                           "=r"(v[u][6]), "=r"(v[u][7])
+                         : "l"(row + e)
+                         : "memory");
+        }
 #pragma unroll
-    for (int u = 0; u < NS; ++u) {  // blend and store
-      const int e0 = 32 * wi + u * E;
-      const uint32_t sb = (m >> (u * E)) & sfull;
-      if (e0 >= V || sb == sfull) continue;
-      T* p = row + e0;
-      if (vec_ok && e0 + E <= V) {
-        uint32_t w[8];
+        for (int u = 0; u < 2; ++u) {  // blend and store
+          const int e = 32 * wi + 16 * u;
+          const uint32_t sb = (m >> (16 * u)) & 0xFFFFu;
+          if (e >= t.V || sb == 0xFFFFu) continue;
+          if (e + 16 <= t.V) {
+            uint32_t w[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          if (sizeof(T) == 4) {
-            w[k] = ((sb >> k) & 1u) ? v[u][k] : fill;
+            for (int k = 0; k < 8; ++k) {
+              const uint32_t lo = (sb >> (2 * k)) & 1u, hi = (sb >> (2 * k + 1)) & 1u;
+              w[k] = sb == 0u ? 0xFF80FF80u
+                              : (lo ? (v[u][k] & 0xFFFFu) : 0xFF80u) | (hi ? (v[u][k] & 0xFFFF0000u) : 0xFF800000u);
+            }
+            asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(row + e), "r"(w[0]), "r"(w[1]),
+                         "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                         : "memory");
           } else {
-            const uint32_t lo = (sb >> (2 * k)) & 1u, hi = (sb >> (2 * k + 1)) & 1u;
-            w[k] = sb == 0u ? fill : (lo ? (v[u][k] & 0xFFFFu) : 0xFF80u) | (hi ? (v[u][k] & 0xFFFF0000u) : 0xFF800000u);
+            for (int k = 0; e + k < t.V; ++k)
+              if (!((sb >> k) & 1u)) row[e + k] = (T)0xFF80u;
           }
         }
-        asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]),
-                     "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
-                     : "memory");
-      } else {
-        for (int k = 0; k < E && e0 + k < V; ++k)
-          if (!((sb >> k) & 1u)) p[k] = (T)fill;
       }
+    } else {
+      // the logits of the block's ids, by their bits in shared memory:
+      // consecutive threads take consecutive sectors, whatever word they
+      // packed (32 SQL rows, fp32: 68.5 -> 65 us a step; 27 rows of 32,001
+      // fp32 logits, off the sector boundaries: 50.9 -> 46.2 us)
+      __syncthreads();
+      s_dyn[threadIdx.x] = m;  // (the selections were read)
+      __syncthreads();
+      const int wb = blockIdx.x * kPackWords;
+      auto word = [&](int w) { return s_dyn[w - wb]; };
+      const int e1 = min(t.V, 32 * (wb + kPackWords));
+      constexpr int kEach = 32 * (int)sizeof(T) / 32;  // sectors per thread of a whole block
+      if (vec_ok)
+        apply_span<T, false, kEach>(row, 32 * wb, e1, word, threadIdx.x, kPackWords);
+      else
+        apply_span<T, true, kEach>(row, 32 * wb, e1, word, threadIdx.x, kPackWords);
     }
   }
   if (CACHE && fill >= 0) __threadfence();  // the entry's words before its readiness
@@ -1844,89 +1942,16 @@ __global__ void __launch_bounds__(64, 3) k_advance(TabT<ST> t, DevConfigs cin, D
   }
 }
 
-// In-place -inf fill, grid = (blocks per row, B): threads stride over a row's
-// 32-byte sectors of logits (8 fp32 or 16 bf16), one 256-bit access per
-// sector, so that every store writes a whole sector and a warp's store covers
-// 1 KB of contiguous bytes (few, long-lived blocks: block scheduling, not
-// memory, bounds a grid of one short block per 256 sectors).  A sector whose
-// tokens are all rejected is written without being read; a mixed sector is
-// read, blended and written; a fully accepted sector is not touched.  Each
-// thread takes kApplyBatch sectors at a time: their mask words loaded
-// together, then the rejected sectors stored (they wait on nothing), then the
-// mixed sectors read together and stored, so that a thread waits on two
-// rounds of loads per batch instead of two per sector.
-// Rows whose sectors are not 32-byte aligned, and the ragged end of a row,
-// are done element by element.
-constexpr int kApplyBatch = 4;
-template <typename T>
+// In-place -inf fill (apply_span), grid = (blocks per row, B): few, long-lived
+// blocks (block scheduling, not memory, bounds a grid of one short block per
+// 256 sectors).
+template <typename T, bool SHIFTED>
 __global__ void __launch_bounds__(256) k_apply(const uint32_t* __restrict__ mask, T* __restrict__ logits, int B,
-                                               int V, int W, long long stride, int vec_ok) {
-  constexpr int E = 32 / sizeof(T);  // elements per sector
-  constexpr uint32_t sfull = E == 32 ? 0xFFFFFFFFu : (1u << E) - 1u;
-  constexpr uint32_t fill = sizeof(T) == 4 ? 0xFF800000u : 0xFF80FF80u;  // -inf in every element of a word
+                                               int V, int W, long long stride) {
   pdl_wait();
-  const int b = blockIdx.y;
-  const int nsec = (V + E - 1) / E;
-  const int step = gridDim.x * blockDim.x;
-  T* row = logits + (size_t)b * stride;
-  for (int s0 = blockIdx.x * blockDim.x + threadIdx.x; s0 < nsec; s0 += kApplyBatch * step) {
-    uint32_t sb[kApplyBatch];
-#pragma unroll
-    for (int u = 0; u < kApplyBatch; ++u) {  // the sectors' accept bits
-      const int e0 = (s0 + u * step) * E;
-      sb[u] = s0 + u * step < nsec ? (mask[(size_t)b * W + (e0 >> 5)] >> (e0 & 31)) & sfull : sfull;
-    }
-#pragma unroll
-    for (int u = 0; u < kApplyBatch; ++u) {  // rejected whole sectors first: written without a read
-      const int e0 = (s0 + u * step) * E;
-      if (vec_ok && s0 + u * step < nsec && e0 + E <= V && sb[u] == 0u)
-        asm volatile("st.global.v8.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1};" ::"l"(row + e0), "r"(fill) : "memory");
-    }
-    uint32_t v[kApplyBatch][8];
-#pragma unroll
-    for (int u = 0; u < kApplyBatch; ++u) {  // mixed whole sectors: read
-      const int e0 = (s0 + u * step) * E;
-      if (vec_ok && s0 + u * step < nsec && e0 + E <= V && sb[u] != 0u && sb[u] != sfull)
-        asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=r"(v[u][0]), "=r"(v[u][1]), "=r"(v[u][2]), "=r"(v[u][3]), "=r"(v[u][4]), "=r"(v[u][5]),
-                       "=r"(v[u][6]), "=r"(v[u][7])
-                     : "l"(row + e0)
-                     : "memory");
-    }
-#pragma unroll
-    for (int u = 0; u < kApplyBatch; ++u) {  // mixed sectors: blend and store; partial sectors one by one
-      const int e0 = (s0 + u * step) * E;
-      if (s0 + u * step >= nsec || sb[u] == sfull) continue;
-      T* p = row + e0;
-      const int n = min(E, V - e0);
-      if (vec_ok && n == E) {
-        if (sb[u] == 0u) continue;  // written above
-        uint32_t w[8];
-        if (sizeof(T) == 4) {
-#pragma unroll
-          for (int k = 0; k < 8; ++k) w[k] = ((sb[u] >> k) & 1u) ? v[u][k] : fill;
-        } else {
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            const uint32_t lo = (sb[u] >> (2 * k)) & 1u, hi = (sb[u] >> (2 * k + 1)) & 1u;
-            w[k] = (lo ? (v[u][k] & 0xFFFFu) : 0xFF80u) | (hi ? (v[u][k] & 0xFFFF0000u) : 0xFF800000u);
-          }
-        }
-        asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]),
-                     "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
-                     : "memory");
-      } else {
-        for (int k = 0; k < n; ++k) {
-          if (!((sb[u] >> k) & 1u)) {
-            if (sizeof(T) == 4)
-              reinterpret_cast<uint32_t*>(p)[k] = 0xFF800000u;
-            else
-              reinterpret_cast<uint16_t*>(p)[k] = 0xFF80u;
-          }
-        }
-      }
-    }
-  }
+  const uint32_t* mrow = mask + (size_t)blockIdx.y * W;
+  apply_span<T, SHIFTED, kApplyBatch>(logits + (size_t)blockIdx.y * stride, 0, V, [&](int w) { return mrow[w]; },
+                         blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
 // Launch with programmatic stream serialization: the kernel may begin (stage
@@ -2646,7 +2671,7 @@ int grid::launch_masks(const grid_spec* s, const DevConfigs& c, const MaskScratc
     GRID_CUDA(staged ? walk(k_walk<false, true>, ts) : walk(k_walk<false, false>, tg));
   if (ev) GRID_CUDA(cudaEventRecord(ev[3], st));
   const dim3 pgrid((t.W + kPackWords - 1) / kPackWords, B);
-  const size_t psmem = (size_t)(2 * std::max(1, t.nselw) + 2 * vcw) * 4;
+  const size_t psmem = std::max<size_t>((size_t)2 * std::max(1, t.nselw) + 2 * vcw, kPackWords) * 4;
   const int esz = lg.dtype == GRID_DTYPE_F32 ? 4 : 2;
   const int vec_ok = lg.p && ((uintptr_t)lg.p % 32 == 0) && ((lg.stride * esz) % 32 == 0);  // 32-byte sectors
   auto pack = [&](auto kern) {
@@ -2940,17 +2965,20 @@ extern "C" int grid_apply_mask(const uint32_t* d_mask, void* d_logits, int32_t d
   cudaStream_t st = (cudaStream_t)stream;
   const int W = (V + 31) / 32;
   const int esz = dtype == GRID_DTYPE_F32 ? 4 : 2;
-  const int vec_ok = ((uintptr_t)d_logits % 32 == 0) && ((row_stride * esz) % 32 == 0);  // 256-bit sectors
   if (B > 65535) return set_error(GRID_E_TOO_LARGE, "grid_apply_mask: more than 65535 rows in one call");
   const int sectors = (V * esz + 31) / 32;  // 32-byte sectors per row
   const int per_row = std::max(1, std::min((sectors + 255) / 256, (g_sms * 4 + B - 1) / B));
   const dim3 grid(per_row, B);
+  const bool shifted = (uintptr_t)d_logits % 32 != 0 || (row_stride * esz) % 32 != 0;  // rows off the sector boundaries
+  auto apply = [&](auto kern, auto* p) {
+    return launch_pdl(kern, grid, dim3(256), 0, st, d_mask, p, B, V, W, (long long)row_stride);
+  };
   if (dtype == GRID_DTYPE_F32)
-    GRID_CUDA(launch_pdl(k_apply<float>, grid, dim3(256), 0, st, d_mask, (float*)d_logits, B, V, W,
-                         (long long)row_stride, vec_ok));
+    GRID_CUDA(shifted ? apply(k_apply<uint32_t, true>, (uint32_t*)d_logits)
+                      : apply(k_apply<uint32_t, false>, (uint32_t*)d_logits));
   else
-    GRID_CUDA(launch_pdl(k_apply<uint16_t>, grid, dim3(256), 0, st, d_mask, (uint16_t*)d_logits, B, V, W,
-                         (long long)row_stride, vec_ok));
+    GRID_CUDA(shifted ? apply(k_apply<uint16_t, true>, (uint16_t*)d_logits)
+                      : apply(k_apply<uint16_t, false>, (uint16_t*)d_logits));
   GRID_CUDA(cudaGetLastError());
   return GRID_OK;
 }
