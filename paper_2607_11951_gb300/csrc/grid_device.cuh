@@ -123,7 +123,6 @@ struct Tables {
   const int32_t* next_alias;   // Vp: the next larger id with the same spelling, -1 after the last
   const int32_t* first_of_byte;
   const uint8_t* first_byte_by_id;
-  const uint32_t* id_valid;    // W words: bit set for the ids with a spelling (not EOS, special or padding)
   const uint32_t* killw;       // Q * W: bit j of word (q, wi): id 32 wi + j's first byte ends a lexeme at q
   // CI tables (one per lexer state in the precomputed set; table 0 = start state)
   int ci_on;
@@ -142,7 +141,7 @@ struct Tables {
   const uint16_t* vc_first;   // class id of each verdict class's first event
   const uint32_t* vc_by_id;   // n_tbl * V: verdict class (within its table) of kClsVC spellings, or NULL
                               // when the class codes carry it (vc_inline)
-  int vc_inline;              // 1: a verdict-class id's code is ncls + kPackCodes + its class index
+  int vc_inline;              // 1: a verdict-class id's code is 32 nselw + its class index
   const uint32_t* cls_sets;   // ncls * 4: terminal set of every class (staged too where o_sets >= 0)
   const uint16_t* cls_map;    // class of every CI class id
   const uint32_t* acc_sym;    // S: the symbol entering each state (audit node hash)

@@ -78,7 +78,7 @@ constexpr int kRowJobWarps = kRowWarps - 1;  // k_row: warps 1 .. compute the al
 // (so that one bit test of the row's class selection covers CI, always and
 // never, and only verdict-class and walked tokens need a second lookup).
 constexpr int kPackCodes = 5;  // ncls + 0 always, +1 never, +2 n/a, +3 verdict class, +4 walked;
-                               // with vc_inline, ncls + 5 + v: verdict class v of the code's table
+                               // with vc_inline, 32 nselw + v: verdict class v of the code's table
 constexpr int kWalkRowsCached = 256;  // rows whose queue bounds k_walk keeps in shared memory
 constexpr int kStagedSets = 512; // classes whose terminal sets are staged with the tables, at most
 constexpr int kLaneOvl = 32;     // overlay / scratch entries per walk lane (shared memory)
@@ -202,16 +202,14 @@ __global__ void k_lex_hash(const int32_t* __restrict__ cstart, const uint8_t* __
   }
 }
 
-// Per token id: the list of each spelling's ids (aliases, in any order) and
-// the ids with a spelling (not EOS, special or padding); Vp is a multiple of 32.
+// The list of each spelling's ids (aliases, in any order); specials, EOS and
+// padding ids have no spelling.
 __global__ void k_ids(const int32_t* __restrict__ spell_of_id, int Vp, int32_t* __restrict__ id_of_spell,
-                      int32_t* __restrict__ next_alias, uint32_t* __restrict__ valid) {
+                      int32_t* __restrict__ next_alias) {
   const int id = blockIdx.x * blockDim.x + threadIdx.x;
   if (id >= Vp) return;
   const int sp = spell_of_id[id];
   next_alias[id] = sp >= 0 ? atomicExch(&id_of_spell[sp], id) : -1;
-  const uint32_t word = __ballot_sync(0xffffffffu, sp >= 0);
-  if ((id & 31) == 0) valid[id >> 5] = word;
 }
 
 // The first 16 bytes of each spelling, zero padded.
@@ -385,7 +383,7 @@ __global__ void k_permute(Tables t, const uint16_t* __restrict__ cls_sp, const u
     uint16_t code = c < kClsFirstCode ? t.cls_map[c] : c;  // the k_pack code of c
     if (c >= kClsFirstCode)
       code = (uint16_t)(t.ncls + (c == kClsAcc ? 0 : c == kClsRej ? 1 : c == kClsNA ? 2 : c == kClsVC ? 3 : 4));
-    if (c == kClsVC && t.vc_inline) code = (uint16_t)(t.ncls + kPackCodes + vc_sp[(size_t)k * t.NS + s]);
+    if (c == kClsVC && t.vc_inline) code = (uint16_t)(32 * t.nselw + vc_sp[(size_t)k * t.NS + s]);
     cls_by_id[(size_t)k * t.Vp + id] = code;
     if (vc_by_id) vc_by_id[(size_t)k * t.Vp + id] = c == kClsVC ? vc_sp[(size_t)k * t.NS + s] : 0xFFFFFFFFu;
   }
@@ -1597,15 +1595,19 @@ __device__ __forceinline__ void apply_span(T* row, int e0, int e1, const Word& w
 
 // grid = (ceil(W / kPackWords), B), kPackWords threads: thread (b, wi) makes
 // mask word wi of row b, the 32 token ids 32 wi .. 32 wi + 31 (the id tables
-// are padded to a multiple of 32 ids, so each thread reads its ids' first
-// bytes and class codes with 16-byte loads).  Per id: the first byte decides
-// the context (it ends the pending lexeme: sigma' and the start state's
-// table; otherwise sigma and the pending state's table, or the walk when the
-// state has none), the class code indexes that context's class selection (CI,
-// always and never in one bit test), and only verdict-class and walked codes
-// look further: the verdict-class bits of the row (staged in shared memory
-// with its class selections) or the walks' verdict word.  The last block of a
-// row writes its status (EMPTY_MASK for a viable row with no bit set).
+// are padded to a multiple of 32 ids, so each thread reads its ids' class
+// codes with 16-byte loads).  Per id: the first byte decides the context (it
+// ends the pending lexeme: sigma' and the start state's table; otherwise sigma
+// and the pending state's table, or the walk when the state has none), and the
+// class code is the place of the id's bit in the context's bit array, the
+// class selections followed by the verdict-class bits, which the block stages
+// in shared memory; the walks' verdicts come as a word.  Large batches are
+// bound by the instructions per id and by the four blocks that 64 registers
+// leave an SM: one look-up per id instead of three with the selects between
+// them took a step of 256 SQL rows (bf16 logits) from 251 to 234 us, of 32
+// rows from 66 to 62.5; without the bound on registers (76 to 95 of them) it
+// was 270 and 68.  The last block of a row writes its status (EMPTY_MASK for a
+// viable row with no bit set).
 //
 // With APPLY (1 = fp32, 2 = bf16 logits) the block then masks the logits of its
 // ids (Sec. 2 masked decoding, as grid_apply_mask; apply_span).
@@ -1616,87 +1618,81 @@ constexpr int kPackWords = 256;
 // exactly one bit, that id is appended to the span and is the next step's
 // token; any other row stops.  Rows that stopped before are left alone.
 template <int APPLY, bool CACHE, bool FORCE = false>
-__global__ void __launch_bounds__(kPackWords) k_pack(Tables t, RowCtx* __restrict__ ctx, const uint32_t* __restrict__ sel,
+__global__ void __launch_bounds__(kPackWords, 4) k_pack(Tables t, RowCtx* __restrict__ ctx, const uint32_t* __restrict__ sel,
                                                      const uint32_t* __restrict__ vcbits, int vcw,
                                                      const uint32_t* __restrict__ verd0,
                                                      const uint32_t* __restrict__ verd1, int words_v,
                                                      uint32_t* __restrict__ mask, int32_t* __restrict__ d_status,
                                                      void* __restrict__ logits, long long stride, int vec_ok,
                                                      CacheDev cache, ForceArgs force) {
-  extern __shared__ __align__(16) uint32_t s_dyn[];  // class selections (2 nselw) | verdict-class bits (2 vcw)
-  __shared__ int s_fl, s_tb, s_any, s_hit, s_fill, s_q, s_cnt, s_id;
+  extern __shared__ __align__(16) uint32_t s_dyn[];  // per context: class selections (nselw) | verdict-class bits (vcw)
+  __shared__ int s_any, s_cnt, s_id;
   const int b = blockIdx.y;
   const int wi = blockIdx.x * kPackWords + threadIdx.x;
   const bool have = wi < t.W;
-  const int nw = t.nselw;
-  const int code_vc = t.ncls + 3, code_walk = t.ncls + 4, code_vc0 = t.ncls + kPackCodes;
-  // spec tables only, read before the wait on the walks: which ids have a
-  // spelling, the start state's class codes
+  const int nw = t.nselw, len = nw + vcw;
+  const int code_vc = t.ncls + 3, code_walk = t.ncls + 4;
+  // spec tables only, read before the wait on the walks: the start state's class codes
   uint4 c04[4];
-  uint32_t valid = 0u;
   if (have) {
     const uint4* c = reinterpret_cast<const uint4*>(t.cls_by_id) + 4 * wi;
 #pragma unroll
     for (int k = 0; k < 4; ++k) c04[k] = c[k];
-    valid = t.id_valid[wi];
   }
-  pdl_wait();
-  const RowCtx& rc = ctx[b];
   if (threadIdx.x == 0) {
-    s_tb = rc.tbl0;
-    s_fl = (rc.emit_ok ? 1 : 0) | (rc.eos_ok ? 2 : 0) | (rc.complete ? 4 : 0) | (rc.complete == 2 ? 8 : 0);
     s_any = 0;
     if (FORCE) {
       s_cnt = 0;
       s_id = 0x7FFFFFFF;
     }
-    s_hit = CACHE ? rc.chit : -1;
-    s_fill = CACHE ? rc.cfill : -1;
-    s_q = rc.q;
   }
-  // the row's class selections and verdict-class bits, staged alongside its
-  // context (a selection k_row did not write is masked off at use)
+  pdl_wait();
+  const RowCtx& rc = ctx[b];
+  const int complete = rc.complete, tb = rc.tbl0, emit_ok = rc.emit_ok, q = rc.q;
+  const int hit = CACHE ? rc.chit : -1, fill = CACHE ? rc.cfill : -1;
+  const bool eos_ok = rc.eos_ok != 0 && !complete;
+  if (complete == 2) return;
+  // The contexts' bit arrays, indexed by class code: a context that k_row did
+  // not prepare (a completed row, sigma' without a forced emission, sigma
+  // without a table) has no bit set, so that no id asks for its context again.
   {
-    for (int i = threadIdx.x; i < 2 * nw; i += kPackWords) s_dyn[i] = sel[(size_t)b * 2 * nw + i];
+    const bool c0 = !complete && tb >= 0, c1 = !complete && emit_ok;
     const uint32_t* vb = vcbits + (size_t)b * 2 * vcw;
-    for (int i = threadIdx.x; i < 2 * vcw; i += kPackWords) s_dyn[2 * nw + i] = vb[i];
-  }
-  __syncthreads();
-  const int fl = s_fl, tb = s_tb, hit = CACHE ? s_hit : -1, fill = CACHE ? s_fill : -1;
-  if (fl & 8) return;
-  // a context that k_row did not select for (a completed row, sigma' without
-  // a forced emission, sigma without a table) selects no class
-  const uint32_t v0 = (t.ci_on && !(fl & 4) && tb >= 0) ? 1u : 0u, v1 = (t.ci_on && !(fl & 4) && (fl & 1)) ? 1u : 0u;
-  const uint32_t* sel0 = s_dyn;
-  const uint32_t* sel1 = s_dyn + nw;
-  const uint32_t* vcb0 = s_dyn + 2 * nw;
-  const uint32_t* vcb1 = s_dyn + 2 * nw + vcw;
-  uint32_t m = 0u;
-  if (have && !(fl & 4)) {
-    const uint32_t wv0 = verd0[(size_t)b * words_v + wi];
-    const uint32_t wv1 = (fl & 1) ? verd1[(size_t)b * words_v + wi] : 0u;
-    // a cache hit gives the context-independent bits; only the residue ids
-    // (verdict-class and walked) are decided here
-    uint32_t todo = valid;
-    // bit j: id 32 wi + j's first byte ends the pending lexeme (context sigma')
-    const uint32_t killw = t.killw[(size_t)s_q * t.W + wi];
-    if (CACHE && hit >= 0) {
-      m = cache.ci[(size_t)hit * t.W + wi];
-      todo = cache.sel[(size_t)hit * t.W + wi];
+    for (int i = threadIdx.x; i < len; i += kPackWords) {
+      uint32_t x0 = 0u, x1 = 0u;
+      if (i < nw) {
+        if (t.ci_on && c0) x0 = sel[(size_t)b * 2 * nw + i];
+        if (t.ci_on && c1) x1 = sel[((size_t)b * 2 + 1) * nw + i];
+      } else {
+        if (c0) x0 = vb[i - nw];
+        if (c1) x1 = vb[vcw + i - nw];
+      }
+      s_dyn[i] = x0;
+      s_dyn[len + i] = x1;
     }
-    uint32_t ci_bits = 0u, sel_bits = 0u;  // what a filling row stores
-    uint4 ct4[4];
-    if (tb >= 0 && todo) {
+  }
+  uint32_t killw = 0u, m = 0u;
+  uint4 ct4[4];
+  if (have && !complete) {
+    // bit j: id 32 wi + j's first byte ends the pending lexeme (context sigma')
+    killw = t.killw[(size_t)q * t.W + wi];
+    // the walks' verdicts (set for walked ids alone, whose codes have no bit in the arrays)
+    m = verd0[(size_t)b * words_v + wi] & ~killw;
+    if (emit_ok) m |= verd1[(size_t)b * words_v + wi] & killw;
+    if (tb >= 0) {
       const uint4* c = reinterpret_cast<const uint4*>(t.cls_by_id + (size_t)tb * t.Vp) + 4 * wi;
 #pragma unroll
       for (int k = 0; k < 4; ++k) ct4[k] = c[k];
     }
+  }
+  __syncthreads();
+  if (have && !complete) {
     const uint32_t c0w[16] = {c04[0].x, c04[0].y, c04[0].z, c04[0].w, c04[1].x, c04[1].y, c04[1].z, c04[1].w,
                               c04[2].x, c04[2].y, c04[2].z, c04[2].w, c04[3].x, c04[3].y, c04[3].z, c04[3].w};
     uint32_t ctw[16];
 #pragma unroll
     for (int k = 0; k < 16; ++k) ctw[k] = code_walk | ((uint32_t)code_walk << 16);
-    if (tb >= 0 && todo) {
+    if (tb >= 0) {
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         ctw[4 * k] = ct4[k].x;
@@ -1705,60 +1701,36 @@ __global__ void __launch_bounds__(kPackWords) k_pack(Tables t, RowCtx* __restric
         ctw[4 * k + 3] = ct4[k].w;
       }
     }
+    uint32_t dep = 0u;  // the residue: ids decided per row, in a context that exists
     if (t.vc_inline) {
-      // every id takes the same instructions (selects, no branches): its
-      // class selection bit, its verdict-class bit and its walked bit are all
-      // read (indices clamped into range) and the code picks one, so that the
-      // warp's threads never split over the kinds of their ids
-      const uint32_t ok1 = (fl & 1) ? 0xFFFFFFFFu : 0u;  // sigma' exists
 #pragma unroll
       for (int j = 0; j < 32; ++j) {
-        const uint32_t cx = (killw >> j) & 1u;
-        const int code = (int)(((cx ? c0w[j >> 1] : ctw[j >> 1]) >> ((j & 1) * 16)) & 0xFFFFu);
-        const int ci = min(code, code_vc - 1);
-        const uint32_t cbit = ((cx ? sel1 : sel0)[ci >> 5] >> (ci & 31)) & (cx ? v1 : v0);
-        const int v = max(code - code_vc0, 0);
-        const uint32_t vbit = ((cx ? vcb1 : vcb0)[v >> 5] >> (v & 31)) & 1u;
-        const uint32_t wbit = ((cx ? wv1 : wv0) >> j) & 1u;
-        const bool dep = code >= code_vc;  // verdict class or walked: decided per row
-        const bool live = !cx || ok1;      // a context k_row left out rejects its residue ids
-        const uint32_t bit = dep ? (live ? (code == code_walk ? wbit : vbit) : 0u) : cbit;
-        if (CACHE) {
-          if (dep && live)
-            sel_bits |= 1u << j;
-          else
-            ci_bits |= bit << j;
-        }
-        m |= (bit & (todo >> j)) << j;
+        const bool cx = (killw >> j) & 1u;
+        const uint32_t code = ((cx ? c0w[j >> 1] : ctw[j >> 1]) >> ((j & 1) * 16)) & 0xFFFFu;
+        if (CACHE && (int)code >= code_vc && (!cx || emit_ok)) dep |= 1u << j;
+        m |= ((s_dyn[(cx ? len : 0) + (code >> 5)] >> (code & 31)) & 1u) << j;
       }
     } else {
 #pragma unroll
       for (int j = 0; j < 32; ++j) {
-        if (!((todo >> j) & 1u)) continue;
-        const int cx = (killw >> j) & 1u;
-        const int code = (int)(((cx ? c0w[j >> 1] : ctw[j >> 1]) >> ((j & 1) * 16)) & 0xFFFFu);
-        uint32_t bit = 0u;  // codes of verdict classes and walks in a context k_row left out: rejected
-        if (code < code_vc) bit = ((cx ? sel1 : sel0)[code >> 5] >> (code & 31)) & (cx ? v1 : v0);
-        if (code >= code_vc && (!cx || (fl & 1))) {
-          if (code == code_walk) {
-            bit = ((cx ? wv1 : wv0) >> j) & 1u;
-          } else {  // the verdict class, looked up
-            const uint32_t v = t.vc_by_id[(size_t)(cx ? 0 : tb) * t.Vp + 32 * wi + j];
-            bit = ((cx ? vcb1 : vcb0)[v >> 5] >> (v & 31)) & 1u;
-          }
-          if (CACHE) sel_bits |= 1u << j;
-        } else if (CACHE) {
-          ci_bits |= bit << j;
-        }
-        m |= bit << j;
+        const bool cx = (killw >> j) & 1u;
+        uint32_t code = ((cx ? c0w[j >> 1] : ctw[j >> 1]) >> ((j & 1) * 16)) & 0xFFFFu;
+        if (CACHE && (int)code >= code_vc && (!cx || emit_ok)) dep |= 1u << j;
+        if ((int)code == code_vc)  // the verdict class, looked up
+          code = 32 * nw + t.vc_by_id[(size_t)(cx ? 0 : tb) * t.Vp + 32 * wi + j];
+        m |= ((s_dyn[(cx ? len : 0) + (code >> 5)] >> (code & 31)) & 1u) << j;
       }
     }
-    if (CACHE && fill >= 0) {
-      cache.ci[(size_t)fill * t.W + wi] = ci_bits;
-      cache.sel[(size_t)fill * t.W + wi] = sel_bits;
+    if (CACHE) {
+      if (fill >= 0) {
+        cache.ci[(size_t)fill * t.W + wi] = m & ~dep;
+        cache.sel[(size_t)fill * t.W + wi] = dep;
+      }
+      // a cache hit gives the context-independent bits; only the residue ids are decided here
+      if (hit >= 0) m = cache.ci[(size_t)hit * t.W + wi] | (m & cache.sel[(size_t)hit * t.W + wi]);
     }
     const int ej = t.eos - 32 * wi;
-    if (ej >= 0 && ej < 32 && (fl & 2)) m |= 1u << ej;  // the EOS gate is stack-dependent: never cached
+    if (ej >= 0 && ej < 32 && eos_ok) m |= 1u << ej;  // the EOS gate is stack-dependent: never cached
   }
   if (have) {
     mask[(size_t)b * t.W + wi] = m;
@@ -2286,7 +2258,6 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   const uint8_t* lx_cbyte = nullptr;
   uint4 *lx_hash = nullptr, *spell16 = nullptr;
   int32_t *id_of_spell = nullptr, *next_alias = nullptr;
-  uint32_t* id_valid = nullptr;
   Arena tmp;  // what only the specialization needs
   std::vector<std::vector<uint8_t>> keep;  // host buffers of copies in flight
   auto fail_tmp = [&](int code) {
@@ -2312,7 +2283,6 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
     up.reserve(std::max(1, t.NS), &spell16);
     up.reserve(std::max(1, t.NS), &id_of_spell);
     up.reserve(t.Vp, &next_alias);
-    up.reserve(t.W, &id_valid);
     up_tmp.add(h.lx_cstart, &lx_cstart);
     up_tmp.add(h.lx_cbyte, &lx_cbyte);
     up_tmp.add(h.lx_cnode, &lx_cnode);
@@ -2322,7 +2292,6 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   t.spell16 = spell16;
   t.id_of_spell = id_of_spell;
   t.next_alias = next_alias;
-  t.id_valid = id_valid;
   t.blob = dblob;
   t.blob_bytes = off[kSec] <= (size_t)kMaxStage ? (int)off[kSec] : 0;
   t.o_class = (int)off[0];
@@ -2359,7 +2328,7 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   GRID_CUDA(cudaMemsetAsync(id_of_spell, 0xFF, (size_t)std::max(1, t.NS) * 4, st));
   k_lex_hash<<<(h.LN + 255) / 256 + 1, 256, 0, st>>>(lx_cstart, lx_cbyte, lx_cnode, t.lx_pcats, t.lx_wcats, h.LN,
                                                     lx_hash, t.lx_hmask, t.lx_hshift);
-  k_ids<<<(t.Vp + 255) / 256, 256, 0, st>>>(t.spell_of_id, t.Vp, id_of_spell, next_alias, id_valid);
+  k_ids<<<(t.Vp + 255) / 256, 256, 0, st>>>(t.spell_of_id, t.Vp, id_of_spell, next_alias);
   k_spell16<<<(t.NS + 255) / 256 + 1, 256, 0, st>>>(t.spell_off, t.spell_bytes, t.NS, spell16);
   {
     Blake2b fb;
@@ -2491,7 +2460,7 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   // otherwise k_pack looks them up per id (the rule counts the class ids as
   // they are before equal sets share one, so that a spec's facts stay what
   // they are)
-  t.vc_inline = s->n_classes + kPackCodes + s->max_vc <= 0xFFFF ? 1 : 0;
+  t.vc_inline = s->n_classes + kPackCodes + s->max_vc <= 0xFFFF && 32 * t.nselw + s->max_vc <= 0xFFFF ? 1 : 0;
   if (!t.vc_inline && (rc = a.alloc((size_t)t.n_tbl * t.Vp * 4, (void**)&vc_by_id))) return fail_tmp(rc);
   t.vc_by_id = vc_by_id;
   k_permute<<<(t.Vp + 255) / 256, 256, 0, st>>>(t, cls_sp, vc_sp, cls_by_id, vc_by_id, fb);
@@ -2671,7 +2640,7 @@ int grid::launch_masks(const grid_spec* s, const DevConfigs& c, const MaskScratc
     GRID_CUDA(staged ? walk(k_walk<false, true>, ts) : walk(k_walk<false, false>, tg));
   if (ev) GRID_CUDA(cudaEventRecord(ev[3], st));
   const dim3 pgrid((t.W + kPackWords - 1) / kPackWords, B);
-  const size_t psmem = std::max<size_t>((size_t)2 * std::max(1, t.nselw) + 2 * vcw, kPackWords) * 4;
+  const size_t psmem = std::max<size_t>((size_t)2 * (t.nselw + vcw), kPackWords) * 4;
   const int esz = lg.dtype == GRID_DTYPE_F32 ? 4 : 2;
   const int vec_ok = lg.p && ((uintptr_t)lg.p % 32 == 0) && ((lg.stride * esz) % 32 == 0);  // 32-byte sectors
   auto pack = [&](auto kern) {
