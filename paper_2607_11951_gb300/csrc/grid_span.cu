@@ -532,7 +532,8 @@ template <bool ST>
 __global__ void __launch_bounds__(kRsvWarps * 32) k_reserve(TabT<ST> t, ReserveTables rt, DevConfigs c, ReserveArgs ra) {
   __shared__ __align__(16) uint16_t s_stk[kRsvDepth];
   __shared__ unsigned long long s_best;  // total << 32 | option of the cheapest way
-  __shared__ int s_slow;
+  __shared__ int s_slow;  // the row is reserve_serial's from the start
+  __shared__ int s_full;  // a way's search needs more entries than a warp holds
   stage_tables(t);
   const auto& ts = t;
   const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -542,6 +543,7 @@ __global__ void __launch_bounds__(kRsvWarps * 32) k_reserve(TabT<ST> t, ReserveT
   const uint16_t* gbase = c.stack + (size_t)b * t.D;
   if (threadIdx.x == 0) {
     s_best = ~0ull;
+    s_full = 0;
     s_slow = !complete && (depth > kRsvDepth || depth + kMaxOvl > t.D || t.S >= kRsvNone || rt.n_items >= kRsvNone);
   }
   if (depth <= kRsvDepth)
@@ -604,9 +606,11 @@ __global__ void __launch_bounds__(kRsvWarps * 32) k_reserve(TabT<ST> t, ReserveT
   RsvOption mine{false, 0, 0, 0, 0};  // the way that this warp looked at last
   RsvGoal goal{kInf, -1, -1, false};
   int mine_opt = -1;
-  auto look = [&](int opt) {
+  // its cost, to every lane: kInf where it leads nowhere or `goal` is full
+  auto look = [&](int opt) -> uint32_t {
     RsvOption o{false, 0, 0, 0, 0};
     mine_opt = -1;
+    goal.full = false;
     __syncwarp();
     if (lane == 0) o = build(opt);
     o.ok = __shfl_sync(0xffffffffu, (int)o.ok, 0);
@@ -614,29 +618,32 @@ __global__ void __launch_bounds__(kRsvWarps * 32) k_reserve(TabT<ST> t, ReserveT
     o.m = __shfl_sync(0xffffffffu, o.m, 0);
     o.ylen = __shfl_sync(0xffffffffu, o.ylen, 0);
     o.sep = __shfl_sync(0xffffffffu, o.sep, 0);
-    if (!o.ok) return;
+    if (!o.ok) return kInf;
     mine = o;
     mine_opt = opt;
     goal = rsv_search(ts, rt, base, o, w, lane);
-    if (goal.full) {
-      if (lane == 0) s_slow = 1;
-      return;
-    }
-    const uint32_t tot = total_of(o, goal.cost);
-    if (lane == 0 && tot < kInf) atomicMin(&s_best, ((unsigned long long)tot << 32) | (unsigned)opt);
+    return goal.full ? kInf : total_of(o, goal.cost);
   };
+  // What the warps tell each other is written between the barrier above and
+  // the one below, and read after the latter alone: s_slow is not written
+  // again, s_full and s_best are not read here.
   if (!complete && !s_slow) {
+    auto offer = [&](int opt) {
+      const uint32_t tot = look(opt);
+      if (lane == 0 && goal.full) atomicExch(&s_full, 1);
+      if (lane == 0 && tot < kInf) atomicMin(&s_best, ((unsigned long long)tot << 32) | (unsigned)opt);
+    };
     int at = 0;  // the ways in order: 0, then 1 + tau of the live terminals
-    if (warp == at++ % kRsvWarps) look(0);
+    if (warp == at++ % kRsvWarps) offer(0);
     Bits4 rest = live0;
     while (rest.any()) {
       const int tau = rest.lowest();
       rest.clear_lowest();
-      if (warp == at++ % kRsvWarps && tau < t.n_term) look(1 + tau);
+      if (warp == at++ % kRsvWarps && tau < t.n_term) offer(1 + tau);
     }
   }
   __syncthreads();
-  if (s_slow) {
+  if (s_slow || s_full) {
     if (threadIdx.x == 0) reserve_serial(t, ts, rt, c, ra, b);
     return;
   }
