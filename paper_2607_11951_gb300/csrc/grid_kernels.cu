@@ -1346,7 +1346,6 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) k_walk(TabT<ST> t, RowCtx*
   // a block's warps start on one row, so that its context, lists and A2 are in the SM's L1 (a step of 256 SQL rows: -4%)
   int row = (int)((long long)blockIdx.x * B / gridDim.x);
   if (B <= (int)gridDim.x) row = blockIdx.x % B;
-  int bound_row = -1;  // first row whose walk hit a bound (its status becomes BOUND)
   int cur = -1;  // row whose context is cached below
   int tbl0 = -1, depth = 0, q = 0, lx = 0, keep1 = 0, m1 = 0, nrng = 0;
   uint32_t pc0 = 0, wc0 = 0;
@@ -1424,7 +1423,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) k_walk(TabT<ST> t, RowCtx*
     const bool c1 = cidx >= ed && cidx < eb;
     const bool is_vc = (cidx >= ed && cidx < ea) || cidx >= eb;
     if (c1 && m1 > kLaneOvl) {  // sigma' overlay larger than a walk lane holds: flag the row
-      bound_row = bound_row < 0 ? row : bound_row;
+      if (lane == 0) atomicCAS(&r.status, GRID_ST_OK, GRID_ST_BOUND);
       continue;
     }
     const uint32_t* Ac = sw.A[c1 ? 1 : 0];
@@ -1444,7 +1443,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) k_walk(TabT<ST> t, RowCtx*
         Walker w;
         walker_init(w, lo, ls, kLaneOvl, base, ckeep, sw.ovl, cm, cq, clx, cpc, cwc, Ac, A2row, ctr);
         res = eval_record(ts, w, ts.vc_rec + (size_t)(t.vc_off[tb] + v) * kRecLen, mc);
-        if (res < 0 && bound_row < 0) bound_row = row;
+        if (res < 0) atomicCAS(&r.status, GRID_ST_OK, GRID_ST_BOUND);  // (seldom: by the lane that met it)
       }
       if (res > 0) atomicOr(&vcbits[((size_t)row * 2 + cxi) * vcw + (v >> 5)], 1u << (v & 31));
       continue;
@@ -1494,13 +1493,12 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) k_walk(TabT<ST> t, RowCtx*
         Walker w;
         walker_init(w, lo, ls, kLaneOvl, base, ckeep, sw.ovl, cm, cq, clx, cpc, cwc, Ac, A2row, ctr);
         const int res = walk_bytes(ts, w, sp, mc);
-        if (res < 0 && bound_row < 0) bound_row = row;
+        if (res < 0) atomicCAS(&r.status, GRID_ST_OK, GRID_ST_BOUND);  // (seldom: by the lane that met it)
         if (res > 0)  // the verdict of every id with this spelling, in the mask's layout
           for (int id = t.id_of_spell[sp_i]; id >= 0; id = t.next_alias[id]) atomicOr(&vb[id >> 5], 1u << (id & 31));
       }
     }
   }
-  if (lane == 0 && bound_row >= 0) atomicCAS(&ctx[bound_row].status, GRID_ST_OK, GRID_ST_BOUND);
   if (COUNT)
     for (int k = 0; k < 6; ++k)
       if (cnt[k]) atomicAdd(&work[k], (unsigned long long)cnt[k]);

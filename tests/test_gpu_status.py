@@ -125,3 +125,55 @@ def test_empty_mask_without_byte_complete_vocabulary():
     for r in range(2):
         cfg = og.config_from_ids(wl["prefixes"][r], wl["tokens"], wl["eos"])
         assert (bits[r] == np.asarray(og.mask(cfg, wl["tokens"], wl["eos"]), np.uint8)).all()
+
+
+def test_bound_of_one_walk_among_many():
+    """A token that overruns a walk's overlay among many that do not, in 1,500
+    rows (more than the walk has warps): whichever lane and warp walk it, the
+    row reports GRID_ST_BOUND and keeps every other bit; rows whose stack
+    refuses the token stay OK."""
+    from paper_2607_11951_gb300 import grid as G
+    toks = [bytes([c]) for c in ALPHA] + [b"(" * k for k in range(15, 32)] + [b"(" * k + b"a" for k in range(15, 30)]
+    toks += [b"(" * 40]
+    t40, a, lp = len(toks) - 1, toks.index(b"a"), toks.index(b"(")
+    kinds = [[], [a], [lp]]
+    wl = _expr_wl(toks, [kinds[b % 3] for b in range(1500)])
+    run = GpuRun(wl)
+    assert (run.build_configs() == 0).all()
+    og = _oracle()
+    want = [np.asarray(og.mask(og.config_from_ids(p, wl["tokens"], wl["eos"]), wl["tokens"], wl["eos"]), np.uint8)
+            for p in kinds]
+    assert [int(w[t40]) for w in want] == [1, 0, 1]
+    for w in want:
+        w[t40] = 0
+    for _ in range(3):
+        words, status = run.masks()
+        assert status.tolist() == [[G.GRID_ST_BOUND, G.GRID_ST_OK, G.GRID_ST_BOUND][b % 3] for b in range(run.B)]
+        bits = unpack(words, run.V)
+        for k in range(3):
+            assert (bits[k::3] == want[k]).all()
+
+
+def test_bound_of_the_pending_lexeme_in_many_rows():
+    """The pending lexeme's emission pushes 37 entries, more than a walk lane's
+    overlay holds and less than the advance's: every such row reports
+    GRID_ST_BOUND, also when one warp meets several of them."""
+    from paper_2607_11951_gb300 import grid as G
+    n = 36
+    text = '%token A "a"\n' + "".join('%%token X%d "x%c%c"\n' % (i, 97 + i // 6, 97 + i % 6) for i in range(n))
+    text += "%ignore WS /[ ]+/\n%start s\ns -> " + " ".join("e%d" % i for i in range(24)) + " t\n"
+    text += "t -> " + " ".join("e%d" % i for i in range(24, n)) + " A rest\n"
+    text += "".join("e%d -> %%empty\ne%d -> X%d\n" % (i, i, i) for i in range(n)) + "rest -> %empty\nrest -> rest A\n"
+    toks = [bytes([c]) for c in b"abcdefx "] + [b" a ", b" a a "] + [b"<eos>"]
+    a, blank = toks.index(b"a"), toks.index(b" ")
+    kinds = [[a], [a, blank, a]]
+    wl = dict(name="status", grammar=text, role=None, lexicons={}, tokens=toks, eos=len(toks) - 1, specials=[],
+              prefixes=[kinds[b % 2] for b in range(3000)], max_depth=4096)
+    run = GpuRun(wl)
+    assert (run.build_configs() == 0).all()
+    words, status = run.masks()
+    assert status.tolist() == [[G.GRID_ST_BOUND, G.GRID_ST_OK][b % 2] for b in range(run.B)]
+    from oracle import compile_grammar
+    og = compile_grammar(text)
+    cfg = og.config_from_ids(kinds[1], toks, wl["eos"])
+    assert (unpack(words, run.V)[1::2] == np.asarray(og.mask(cfg, toks, wl["eos"]), np.uint8)).all()
