@@ -1149,7 +1149,7 @@ __device__ __forceinline__ void scan_ranges(const TabT<false>& t, RowCtx& r, con
       const Spell sp = load_spell(t, sp_i);
       LexState s = s0;
       res = 1;
-      ++count;
+      int seen = 0;
 #pragma unroll 1
       for (int i = 0; i < sp.len; ++i) {
         const int b = sp.at(i);
@@ -1158,13 +1158,17 @@ __device__ __forceinline__ void scan_ranges(const TabT<false>& t, RowCtx& r, con
           res = 2;
           break;
         }
-        ++steps;
+        ++seen;
         s.q = nq;
         s.lx = lex_step(t, s.q, s.lx, b, s.pc, s.wc);
         if (!(live_prime(t, s.q, s.pc) & AI).any()) {
           res = 0;
           break;
         }
+      }
+      if (res != 2) {  // decided here (k_walk counts the others)
+        steps += seen;
+        ++count;
       }
       if (res == 1)
         for (int id = t.id_of_spell[sp_i]; id >= 0; id = t.next_alias[id]) atomicOr(&verd[id >> 5], 1u << (id & 31));
