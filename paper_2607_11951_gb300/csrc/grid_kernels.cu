@@ -2115,13 +2115,13 @@ static void lexeme_tables(const HostGrammar& h, std::vector<uint64_t>& ev, std::
     }
 }
 
-extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void* stream, grid_spec** out) {
-  if (!g || !v || !out) return set_error(GRID_E_INVALID_ARG, "grid_specialize: bad arguments");
-  *out = nullptr;
+// grid_specialize's work.  The caller frees what it leaves, after success and
+// after every error: what only the specialization needs is tmp's and keep's
+// (the host buffers of copies in flight); after an error, the spec too.
+static int specialize(const grid_grammar* g, const grid_vocab* v, cudaStream_t st, grid_spec* s, Arena& tmp,
+                      std::vector<std::vector<uint8_t>>& keep) {
   const HostGrammar& h = g->h;
   const HostVocab& hv = v->h;
-  cudaStream_t st = (cudaStream_t)stream;
-  auto* s = new grid_spec();
   s->g = g;
   s->v = v;
   Tables& t = s->t;
@@ -2147,11 +2147,6 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   uint32_t par[4] = {0u, 0u, 0u, 0u};
   for (int tau = 0; tau < h.n_term; ++tau) par[tau >> 5] |= 1u << (tau & 31);
   t.par = Bits4{par[0] & ~h.ignored[0], par[1] & ~h.ignored[1], par[2] & ~h.ignored[2], par[3] & ~h.ignored[3]};
-  auto fail = [&](int rc) {
-    s->mem.release();
-    delete s;
-    return rc;
-  };
   // per LALR state: the terminals that shift, and the terminals grouped by
   // the production they reduce by (for simulating a set of terminals at once)
   std::vector<uint32_t> shift_mask((size_t)h.S * 4, 0u), red_mask;
@@ -2160,8 +2155,8 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   int max_plen = 0;
   for (int pr = 0; pr < h.P; ++pr) max_plen = std::max(max_plen, (int)h.plen[pr]);
   if (h.NNT >= 1024 || max_plen >= 32)
-    return fail(set_error(GRID_E_TOO_LARGE, "grammar exceeds the packed reduce encoding (1024 nonterminals, "
-                                            "right-hand sides of 31 symbols)"));
+    return set_error(GRID_E_TOO_LARGE, "grammar exceeds the packed reduce encoding (1024 nonterminals, "
+                                       "right-hand sides of 31 symbols)");
   std::vector<int16_t> action16(h.action.size());
   for (size_t i = 0; i < h.action.size(); ++i) {
     const int a = h.action[i];
@@ -2265,13 +2260,20 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   const uint8_t* lx_cbyte = nullptr;
   uint4 *lx_hash = nullptr, *spell16 = nullptr;
   int32_t *id_of_spell = nullptr, *next_alias = nullptr;
-  Arena tmp;  // what only the specialization needs
-  std::vector<std::vector<uint8_t>> keep;  // host buffers of copies in flight
-  auto fail_tmp = [&](int code) {
+  // Copies in flight read and write this function's arrays: from here on every
+  // exit waits for the stream first.
+  auto done = [&](int code) {
     cudaStreamSynchronize(st);
-    tmp.release();
-    return fail(code);
+    return code;
   };
+#define GRID_DONE(call)                       \
+  do {                                        \
+    const int code_ = [&]() -> int {          \
+      GRID_CUDA(call);                        \
+      return GRID_OK;                         \
+    }();                                      \
+    if (code_ != GRID_OK) return done(code_); \
+  } while (0)
   {
     Upload up, up_tmp;
     up.add(blob, &dblob);
@@ -2293,7 +2295,7 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
     up_tmp.add(h.lx_cstart, &lx_cstart);
     up_tmp.add(h.lx_cbyte, &lx_cbyte);
     up_tmp.add(h.lx_cnode, &lx_cnode);
-    if ((rc = up.commit(a, st, keep)) || (rc = up_tmp.commit(tmp, st, keep))) return fail_tmp(rc);
+    if ((rc = up.commit(a, st, keep)) || (rc = up_tmp.commit(tmp, st, keep))) return done(rc);
   }
   t.lx_hash = lx_hash;
   t.spell16 = spell16;
@@ -2331,8 +2333,8 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   t.live_any = reinterpret_cast<const uint32_t*>(dblob + off[12]);
   t.cat_live = reinterpret_cast<const uint32_t*>(dblob + off[13]);
   t.tbl_of_q = reinterpret_cast<const int16_t*>(dblob + off[14]);
-  GRID_CUDA(cudaMemsetAsync(lx_hash, 0xFF, ((size_t)t.lx_hmask + 1) * 16, st));
-  GRID_CUDA(cudaMemsetAsync(id_of_spell, 0xFF, (size_t)std::max(1, t.NS) * 4, st));
+  GRID_DONE(cudaMemsetAsync(lx_hash, 0xFF, ((size_t)t.lx_hmask + 1) * 16, st));
+  GRID_DONE(cudaMemsetAsync(id_of_spell, 0xFF, (size_t)std::max(1, t.NS) * 4, st));
   k_lex_hash<<<(h.LN + 255) / 256 + 1, 256, 0, st>>>(lx_cstart, lx_cbyte, lx_cnode, t.lx_pcats, t.lx_wcats, h.LN,
                                                     lx_hash, t.lx_hmask, t.lx_hshift);
   k_ids<<<(t.Vp + 255) / 256, 256, 0, st>>>(t.spell_of_id, t.Vp, id_of_spell, next_alias);
@@ -2345,13 +2347,13 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
     fb.update(hv.fingerprint, 16);
     fb.final(s->fingerprint);
   }
-  if ((rc = set_smem_limits())) return fail(rc);
+  if ((rc = set_smem_limits())) return done(rc);
   int dev = 0;
   cudaGetDevice(&dev);
   s->device = dev;
   cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, dev);
   g_sms = s->sms;
-  // CI classification on the device (temporaries live in `tmp`)
+  // CI classification on the device
   uint16_t *cls_sp = nullptr, *key_sp = nullptr, *cls_by_id = nullptr;
   int32_t* counts_d = nullptr;  // per table: walked spellings, verdict-class spellings; then the fills of both lists
   uint32_t *vc_by_id = nullptr, *vc_sp = nullptr;
@@ -2362,25 +2364,25 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
     up.reserve((size_t)t.n_tbl * t.NS, &key_sp);
     up.reserve((size_t)t.n_tbl * t.NS, &vc_sp);
     up.reserve((size_t)t.n_tbl * 5, &counts_d);
-    if ((rc = up.commit(tmp, st, keep))) return fail_tmp(rc);
+    if ((rc = up.commit(tmp, st, keep))) return done(rc);
     up.reserve((size_t)t.n_tbl * t.Vp, &cls_by_id);
     up.reserve((size_t)t.Vp, &fb);
-    if ((rc = up.commit(a, st, keep))) return fail_tmp(rc);
+    if ((rc = up.commit(a, st, keep))) return done(rc);
   }
   t.cls_by_id = cls_by_id;
   t.first_byte_by_id = fb;
   int32_t *cd_fill = counts_d + 2 * t.n_tbl, *vc_fill = counts_d + 3 * t.n_tbl, *vc_count = counts_d + 4 * t.n_tbl;
-  GRID_CUDA(cudaMemsetAsync(counts_d, 0, (size_t)t.n_tbl * 20, st));
+  GRID_DONE(cudaMemsetAsync(counts_d, 0, (size_t)t.n_tbl * 20, st));
   const dim3 cgrid(std::max(1, std::min((t.NS + 255) / 256, 4 * s->sms)), t.n_tbl);
   if (t.blob_bytes)
     k_classify<true><<<cgrid, 256, t.blob_bytes, st>>>(TabT<true>(t), cls_sp, key_sp, counts_d);
   else
     k_classify<false><<<cgrid, 256, 0, st>>>(TabT<false>(t), cls_sp, key_sp, counts_d);
   // the reserve's tables are laid out while the device classifies
-  if ((rc = build_reserve_tables(s, st, keep))) return fail_tmp(rc);
+  if ((rc = build_reserve_tables(s, st, keep))) return done(rc);
   std::vector<int32_t> counts2(2 * t.n_tbl);
-  GRID_CUDA(cudaMemcpyAsync(counts2.data(), counts_d, t.n_tbl * 8, cudaMemcpyDeviceToHost, st));
-  GRID_CUDA(cudaStreamSynchronize(st));
+  GRID_DONE(cudaMemcpyAsync(counts2.data(), counts_d, t.n_tbl * 8, cudaMemcpyDeviceToHost, st));
+  GRID_DONE(cudaStreamSynchronize(st));
   std::vector<int32_t> counts(t.n_tbl), cdoff(t.n_tbl + 1, 0), vcbase(t.n_tbl + 1, 0);
   for (int k = 0; k < t.n_tbl; ++k) {
     counts[k] = counts2[2 * k];
@@ -2406,11 +2408,11 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
     up.reserve(nslot, &rep);
     up.reserve(nslot, &place);
     up.reserve((size_t)tab_mask + 1, &tab);
-    if ((rc = up.commit(tmp, st, keep))) return fail_tmp(rc);
+    if ((rc = up.commit(tmp, st, keep))) return done(rc);
     up.add(cdoff, &t.cd_off);
     up.reserve(cdoff.back(), &cd_list);
     up.reserve(cdoff.back(), &cd_key);
-    if ((rc = up.commit(a, st, keep))) return fail_tmp(rc);
+    if ((rc = up.commit(a, st, keep))) return done(rc);
   }
   t.cd_list = cd_list;
   t.cd_key = cd_key;
@@ -2424,11 +2426,11 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
       k_events<true><<<cgrid, 256, t.blob_bytes, st>>>(TabT<true>(t), cls_sp, vcbase_d, vc_fill, slot_tbl, slot_sp, rec16);
     else
       k_events<false><<<cgrid, 256, 0, st>>>(TabT<false>(t), cls_sp, vcbase_d, vc_fill, slot_tbl, slot_sp, rec16);
-    GRID_CUDA(cudaMemsetAsync(tab, 0xFF, ((size_t)tab_mask + 1) * 4, st));
+    GRID_DONE(cudaMemsetAsync(tab, 0xFF, ((size_t)tab_mask + 1) * 4, st));
     k_vc_merge<<<sgrid, 256, 0, st>>>(slot_tbl, slot_rec, nslot, tab, tab_mask, rep, place, vc_count);
-    GRID_CUDA(cudaMemcpyAsync(n_distinct.data(), vc_count, t.n_tbl * 4, cudaMemcpyDeviceToHost, st));
+    GRID_DONE(cudaMemcpyAsync(n_distinct.data(), vc_count, t.n_tbl * 4, cudaMemcpyDeviceToHost, st));
   }
-  GRID_CUDA(cudaStreamSynchronize(st));
+  GRID_DONE(cudaStreamSynchronize(st));
   std::vector<int32_t> vcoff(t.n_tbl + 1, 0);
   for (int k = 0; k < t.n_tbl; ++k) {
     vcoff[k + 1] = vcoff[k] + n_distinct[k];
@@ -2449,11 +2451,11 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
     up.add(vcoff, &t.vc_off);
     up.reserve(n_vc, &recs);
     up.reserve(n_vc, &firsts);
-    if ((rc = up.commit(a, st, keep))) return fail_tmp(rc);
+    if ((rc = up.commit(a, st, keep))) return done(rc);
     up.reserve(n_vc, &keys);
     up.reserve(n_vc, &src);
     up.reserve(n_vc, &rank);
-    if ((rc = up.commit(tmp, st, keep))) return fail_tmp(rc);
+    if ((rc = up.commit(tmp, st, keep))) return done(rc);
   }
   t.vc_rec = reinterpret_cast<const uint16_t*>(recs);
   t.vc_first = firsts;
@@ -2468,26 +2470,40 @@ extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void*
   // they are before equal sets share one, so that a spec's facts stay what
   // they are)
   t.vc_inline = s->n_classes + kPackCodes + s->max_vc <= 0xFFFF && 32 * t.nselw + s->max_vc <= 0xFFFF ? 1 : 0;
-  if (!t.vc_inline && (rc = a.alloc((size_t)t.n_tbl * t.Vp * 4, (void**)&vc_by_id))) return fail_tmp(rc);
+  if (!t.vc_inline && (rc = a.alloc((size_t)t.n_tbl * t.Vp * 4, (void**)&vc_by_id))) return done(rc);
   t.vc_by_id = vc_by_id;
   k_permute<<<(t.Vp + 255) / 256, 256, 0, st>>>(t, cls_sp, vc_sp, cls_by_id, vc_by_id, fb);
   {
     uint32_t* killw = nullptr;
-    if ((rc = a.alloc((size_t)t.Q * t.W * 4, (void**)&killw))) return fail_tmp(rc);
+    if ((rc = a.alloc((size_t)t.Q * t.W * 4, (void**)&killw))) return done(rc);
     k_killw<<<dim3((t.W + 255) / 256, t.Q), 256, 0, st>>>(t, killw);
     t.killw = killw;
   }
-  GRID_CUDA(cudaGetLastError());
-  GRID_CUDA(cudaStreamSynchronize(st));
-  tmp.release();
+  GRID_DONE(cudaGetLastError());
+  GRID_DONE(cudaStreamSynchronize(st));
   s->n_vc = vcoff.back();
   if ((size_t)(2 * std::max(1, t.nselw) + 2 * std::max(1, s->vcw)) * 4 > (size_t)kMaxStage)
-    return fail(set_error(GRID_E_TOO_LARGE, "grid_specialize: the class selections and verdict-class bits of one "
-                                            "row exceed the packing kernel's shared memory"));
+    return set_error(GRID_E_TOO_LARGE, "grid_specialize: the class selections and verdict-class bits of one "
+                                       "row exceed the packing kernel's shared memory");
   s->n1 = (counts[0] + kSpan - 1) / kSpan;
   s->max_cd = *std::max_element(counts.begin(), counts.end());
-  *out = s;
   return GRID_OK;
+#undef GRID_DONE
+}
+
+extern "C" int grid_specialize(const grid_grammar* g, const grid_vocab* v, void* stream, grid_spec** out) {
+  if (!g || !v || !out) return set_error(GRID_E_INVALID_ARG, "grid_specialize: bad arguments");
+  *out = nullptr;
+  auto* s = new grid_spec();
+  Arena tmp;
+  std::vector<std::vector<uint8_t>> keep;
+  const int rc = specialize(g, v, (cudaStream_t)stream, s, tmp, keep);
+  tmp.release();
+  if (rc == GRID_OK)
+    *out = s;
+  else
+    grid_spec_free(s);
+  return rc;
 }
 
 extern "C" int grid_spec_info(const grid_spec* s, int64_t out[8]) {
