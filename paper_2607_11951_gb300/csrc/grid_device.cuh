@@ -99,7 +99,6 @@ struct Tables {
   const uint32_t* live;
   const int16_t* action;
   const uint16_t* go;
-  const uint8_t* plen;
   const uint16_t* plhs;
   const uint32_t* shift_mask;  // S * 4: terminals whose action is SHIFT
   const uint32_t* red_off;     // S + 1: reduce groups of state s are red_off[s] .. red_off[s+1]

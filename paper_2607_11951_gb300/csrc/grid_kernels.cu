@@ -1316,7 +1316,10 @@ struct WalkWarp {
   uint16_t ovl[kMaxOvl];            // sigma's overlay
 };
 static_assert(sizeof(WalkWarp) % 16 == 0, "the warps' parts start on 16-byte boundaries");
-constexpr int kWalkSmem = kWalkWarps * (int)sizeof(WalkWarp);  // k_walk's dynamic shared memory beside the tables
+// k_walk's dynamic shared memory, at most: the tables, then a WalkWarp per warp (24 beside up to 99 KB of tables, 22
+// beside the largest that are staged)
+constexpr int kWalkSmem = 227 * 1024 - 5120;
+static_assert(kWalkSmem - kMaxStage >= 20 * (int)sizeof(WalkWarp), "the largest tables leave room for the warps");
 
 template <bool COUNT, bool ST>
 __global__ void __launch_bounds__(kWalkWarps * 32, 1) k_walk(TabT<ST> t, RowCtx* __restrict__ ctx,
@@ -1619,6 +1622,7 @@ __device__ __forceinline__ void apply_span(T* row, int e0, int e1, const Word& w
 // With APPLY (1 = fp32, 2 = bf16 logits) the block then masks the logits of its
 // ids (Sec. 2 masked decoding, as grid_apply_mask; apply_span).
 constexpr int kPackWords = 256;
+constexpr int kMaxPack = 96 * 1024;  // bytes of a row's bit arrays, at most
 //
 // With FORCE (a step of grid_forced_span) the last block of a row also finds
 // the row's forced token: where the step's status is OK and the mask holds
@@ -1965,7 +1969,7 @@ int grid::g_sms = 152;  // SM count of the current device, set by grid_specializ
 // spec in the process, so it is raised once to the largest staged block
 // allowed instead of to this spec's size.
 static int set_smem_limits() {
-  const int dyn = kMaxStage;
+  const int dyn = std::max(kMaxStage, kMaxPack);
   const void* kernels[] = {
       (const void*)k_classify<true>, (const void*)k_events<true>, (const void*)k_advance<true>,
       (const void*)k_row<0, true>, (const void*)k_row<1, true>, (const void*)k_row<2, true>,
@@ -1977,7 +1981,7 @@ static int set_smem_limits() {
   const void* walks[] = {(const void*)k_walk<false, true>, (const void*)k_walk<true, true>,
                          (const void*)k_walk<false, false>, (const void*)k_walk<true, false>};
   for (const void* k : walks)
-    GRID_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn + kWalkSmem));
+    GRID_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kWalkSmem));
   return GRID_OK;
 }
 
@@ -2203,8 +2207,6 @@ static int specialize(const grid_grammar* g, const grid_vocab* v, cudaStream_t s
   s->has_cats = h.n_cat > 0;
   t.ncls = (int)(sets.size() / 4);
   t.nselw = (t.ncls + kPackCodes + 31) / 32;
-  const std::vector<uint32_t> no_sets;
-  const std::vector<uint32_t>& staged_sets = t.ncls <= kStagedSets ? sets : no_sets;
   std::vector<uint32_t> cat_live((h.Q + 31) / 32, 0u);
   for (int q = 0; q < h.Q; ++q)
     for (int w = 0; w < 4; ++w)
@@ -2223,23 +2225,25 @@ static int specialize(const grid_grammar* g, const grid_vocab* v, cudaStream_t s
     }
   }
   t.n_tbl = (int)tq.size();
-  // staged block: byte classes, DFA, acc/live, ACTION, GOTO, production
-  // tables, shift masks and reduce groups, live lexemes, states
-  // with live categories, tables of states, class sets
-  constexpr int kSec = 16;
+  // staged block: byte classes, DFA, acc/live, ACTION, GOTO, left-hand
+  // sides, shift masks and reduce groups, live lexemes, states
+  // with live categories, tables of states, class sets (where they are few
+  // and there is room: the kernels find them in global memory too)
+  constexpr int kSec = 15;
   std::vector<size_t> off(kSec + 1, 0);
-  const size_t sizes[kSec] = {256, h.next.size() * 2, h.acc.size() * 4, h.live.size() * 4, h.action.size() * 2,
-                              h.go.size() * 2, h.plen.size(), h.plhs.size() * 2, shift_mask.size() * 4,
+  const size_t sizes[kSec] = {256, h.next.size() * 2, h.acc.size() * 4, h.live.size() * 4, action16.size() * 2,
+                              h.go.size() * 2, h.plhs.size() * 2, shift_mask.size() * 4,
                               red_off.size() * 4, red_p.size() * 2, red_mask.size() * 4, live_any.size() * 4,
-                              cat_live.size() * 4, tbl_of_q.size() * 2,
-                              staged_sets.size() * 4};
+                              cat_live.size() * 4, tbl_of_q.size() * 2, sets.size() * 4};
   const void* srcs[kSec] = {h.byte_class, h.next.data(), h.acc.data(), h.live.data(), action16.data(),
-                            h.go.data(), h.plen.data(), h.plhs.data(), shift_mask.data(), red_off.data(),
+                            h.go.data(), h.plhs.data(), shift_mask.data(), red_off.data(),
                             red_p.data(), red_mask.data(), live_any.data(), cat_live.data(),
-                            tbl_of_q.data(), staged_sets.data()};
+                            tbl_of_q.data(), sets.data()};
   for (int k = 0; k < kSec; ++k) off[k + 1] = align16(off[k] + sizes[k]);
+  const bool stage_sets = !sets.empty() && t.ncls <= kStagedSets && off[kSec] <= (size_t)kMaxStage;
+  if (!stage_sets) off[kSec] = off[kSec - 1];
   std::vector<uint8_t> blob(off[kSec], 0);
-  for (int k = 0; k < kSec; ++k)
+  for (int k = 0; k < (stage_sets ? kSec : kSec - 1); ++k)
     if (sizes[k]) std::memcpy(blob.data() + off[k], srcs[k], sizes[k]);
   Arena& a = s->mem;
   int rc;
@@ -2309,30 +2313,29 @@ static int specialize(const grid_grammar* g, const grid_vocab* v, cudaStream_t s
   t.o_live = (int)off[3];
   t.o_action = (int)off[4];
   t.o_go = (int)off[5];
-  t.o_lhs = (int)off[7];
-  t.o_shift = (int)off[8];
-  t.o_roff = (int)off[9];
-  t.o_rp = (int)off[10];
-  t.o_red = (int)off[11];
-  t.o_lany = (int)off[12];
-  t.o_catq = (int)off[13];
-  t.o_tblq = (int)off[14];
-  t.o_sets = staged_sets.empty() ? -1 : (int)off[15];
+  t.o_lhs = (int)off[6];
+  t.o_shift = (int)off[7];
+  t.o_roff = (int)off[8];
+  t.o_rp = (int)off[9];
+  t.o_red = (int)off[10];
+  t.o_lany = (int)off[11];
+  t.o_catq = (int)off[12];
+  t.o_tblq = (int)off[13];
+  t.o_sets = stage_sets ? (int)off[14] : -1;
   t.byte_class = dblob + off[0];
   t.next = reinterpret_cast<const uint16_t*>(dblob + off[1]);
   t.acc = reinterpret_cast<const uint32_t*>(dblob + off[2]);
   t.live = reinterpret_cast<const uint32_t*>(dblob + off[3]);
   t.action = reinterpret_cast<const int16_t*>(dblob + off[4]);
   t.go = reinterpret_cast<const uint16_t*>(dblob + off[5]);
-  t.plen = dblob + off[6];
-  t.plhs = reinterpret_cast<const uint16_t*>(dblob + off[7]);
-  t.shift_mask = reinterpret_cast<const uint32_t*>(dblob + off[8]);
-  t.red_off = reinterpret_cast<const uint32_t*>(dblob + off[9]);
-  t.red_p = reinterpret_cast<const uint16_t*>(dblob + off[10]);
-  t.red_mask = reinterpret_cast<const uint32_t*>(dblob + off[11]);
-  t.live_any = reinterpret_cast<const uint32_t*>(dblob + off[12]);
-  t.cat_live = reinterpret_cast<const uint32_t*>(dblob + off[13]);
-  t.tbl_of_q = reinterpret_cast<const int16_t*>(dblob + off[14]);
+  t.plhs = reinterpret_cast<const uint16_t*>(dblob + off[6]);
+  t.shift_mask = reinterpret_cast<const uint32_t*>(dblob + off[7]);
+  t.red_off = reinterpret_cast<const uint32_t*>(dblob + off[8]);
+  t.red_p = reinterpret_cast<const uint16_t*>(dblob + off[9]);
+  t.red_mask = reinterpret_cast<const uint32_t*>(dblob + off[10]);
+  t.live_any = reinterpret_cast<const uint32_t*>(dblob + off[11]);
+  t.cat_live = reinterpret_cast<const uint32_t*>(dblob + off[12]);
+  t.tbl_of_q = reinterpret_cast<const int16_t*>(dblob + off[13]);
   GRID_DONE(cudaMemsetAsync(lx_hash, 0xFF, ((size_t)t.lx_hmask + 1) * 16, st));
   GRID_DONE(cudaMemsetAsync(id_of_spell, 0xFF, (size_t)std::max(1, t.NS) * 4, st));
   k_lex_hash<<<(h.LN + 255) / 256 + 1, 256, 0, st>>>(lx_cstart, lx_cbyte, lx_cnode, t.lx_pcats, t.lx_wcats, h.LN,
@@ -2482,10 +2485,9 @@ static int specialize(const grid_grammar* g, const grid_vocab* v, cudaStream_t s
   GRID_DONE(cudaGetLastError());
   GRID_DONE(cudaStreamSynchronize(st));
   s->n_vc = vcoff.back();
-  if ((size_t)(2 * std::max(1, t.nselw) + 2 * std::max(1, s->vcw)) * 4 > (size_t)kMaxStage)
+  if ((size_t)(2 * std::max(1, t.nselw) + 2 * std::max(1, s->vcw)) * 4 > (size_t)kMaxPack)
     return set_error(GRID_E_TOO_LARGE, "grid_specialize: the class selections and verdict-class bits of one "
                                        "row exceed the packing kernel's shared memory");
-  s->n1 = (counts[0] + kSpan - 1) / kSpan;
   s->max_cd = *std::max_element(counts.begin(), counts.end());
   return GRID_OK;
 #undef GRID_DONE
@@ -2611,7 +2613,8 @@ extern "C" int grid_advance(const grid_spec* s, const grid_configs* in, grid_con
 static long walk_items(const grid_spec* s, int B) { return (long)B * ((s->t.NS + 1023) / 1024) / s->sms; }  // per SM
 static int walk_warps(const grid_spec* s, int B) {
   const long per_sm = walk_items(s, B);
-  return per_sm < 2 ? 4 : per_sm < 4 ? 8 : per_sm < 10 ? 12 : per_sm < 20 ? 16 : kWalkWarps;
+  const int room = (kWalkSmem - s->t.blob_bytes) / (int)sizeof(WalkWarp);
+  return per_sm < 2 ? 4 : per_sm < 4 ? 8 : per_sm < 10 ? 12 : per_sm < 20 ? 16 : std::min(kWalkWarps, room);
 }
 
 // The four kernels of one mask step on `st`; `ev` (5 events or NULL) is

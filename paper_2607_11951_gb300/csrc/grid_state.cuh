@@ -170,7 +170,11 @@ struct ForceArgs {
   int pos, max_span;
 };
 
-constexpr int kMaxStage = 96 * 1024;  // bytes of the staged tables, at most
+// Bytes of the staged tables, at most.  96 KB for the lexer's and the parser's
+// tables, and 10 KB for what goes with them (a bit per lexer state and category
+// set, at most 4 KB; two bytes and a bit per lexer state, of which 96 KB hold
+// fewer than 2,800); the class sets are staged where they leave it unfilled.
+constexpr int kMaxStage = 106 * 1024;
 
 constexpr int kMaskKernels = 4;  // k_row, k_filter, k_walk, k_pack
 
@@ -210,7 +214,6 @@ struct grid_spec {
   grid::Arena mem;
   int device = 0;
   int sms = 152;
-  int n1 = 0;  // walk chunks of the start state's CD list
   int max_cd = 0;       // longest CD list of a table
   int vcw = 0;          // words of the largest table's verdict-class bitset
   int n_vc = 0;         // verdict classes over all tables

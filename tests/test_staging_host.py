@@ -1,0 +1,63 @@
+"""Which tables are staged in shared memory, and the launches that follow, on a
+CUDA runtime without a GPU: lexer and parser tables of up to 96 KB are staged
+whatever else goes with them, and no launch asks for more shared memory than
+its kernel was allowed."""
+import ctypes
+
+import pytest
+
+from paper_2607_11951_gb300 import grid as G
+from tests import fakes
+
+SM_BYTES = 227 * 1024  # shared memory of one block, at most
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    return fakes.link(tmp_path_factory.mktemp("fake"))
+
+
+def grammar(n, cats):
+    """Statements led by n keywords, with `cats` categories of one regex."""
+    name = lambda i: "%s%s" % (chr(97 + i // 16), chr(97 + i % 16))
+    toks = "".join("%%token T%d /%s/\n" % (i, name(i)) for i in range(n))
+    toks += "".join("%%token C%d /[q-z]+/\n" % c for c in range(cats))
+    prods = "".join("stmt -> T%d T%d opt T%d T%d\n" % (i, (i * 7 + 3) % n, (i * 5 + 1) % n, (i * 3 + 2) % n)
+                    for i in range(n))
+    prods += "".join("stmt -> C%d SEMI T%d\n" % (c, c) for c in range(cats))
+    return toks + "".join("%%category C%d\n" % c for c in range(cats)) + \
+        "%token SEMI /;/\n%ignore WS /[ ]+/\n%start prog\nprog -> prog stmt\nprog -> stmt\n" + prods + \
+        "opt -> %empty\nopt -> opt2 SEMI\nopt2 -> %empty\n"
+
+
+def table_bytes(i):
+    """Lexer and parser tables without the reduce groups."""
+    Q, S, T1, N = i["dfa_states"], i["lalr_states"], i["terminals"] + 1, i["nonterminals"]
+    return 256 + 2 * Q * i["byte_classes"] + 32 * Q + 2 * S * (T1 + N) + 2 * i["productions"] + 20 * S
+
+
+@pytest.mark.parametrize("cats", [0, 7])
+def test_tables_of_96_kb_are_staged(fake, cats):
+    with fakes.use(fake) as rt:
+        toks = [bytes([b]) for b in range(256)] + [b"%d" % i for i in range(10, 2000)] + [b"<eos>"]
+        v = G.Vocab(toks, len(toks) - 1, [])
+        seen = []
+        for n in range(70, 92):
+            g = G.Grammar(grammar(n, cats), None, {"C%d" % c: [b"qr" + bytes([113 + c])] for c in range(cats)})
+            size = table_bytes(g.info())
+            rt.reset(ones=1)
+            s = G.Spec(g, v)
+            staged = s.info()["staged_bytes"]
+            seen.append((size > 94 * 1024, staged > 0))
+            assert s.info()["ci_on"] and (staged > 0 or size > 96 * 1024), (n, size)
+            c = G.Configs(s, 4096)  # enough rows for the largest blocks of the walk
+            one = ctypes.c_void_p(16)
+            assert G.lib().grid_masks(s.h, c.h, one, one, None) == G.GRID_OK
+            assert G.lib().grid_reserve(s.h, c.h, one, one, 16, one, None, 0, None, None) == G.GRID_OK
+            for name, grid, threads, smem, limit in rt.launches():
+                assert smem <= limit <= SM_BYTES, (name, smem, limit)
+                if "k_walk" in name:
+                    assert threads >= 20 * 32
+            del g, s, c
+        assert (True, True) in seen and (True, False) in seen
+        del v
