@@ -439,7 +439,7 @@ __device__ __forceinline__ void hash_nodes(const T& t, uint64_t* __restrict__ hs
 // accesses when the row stride allows them); the first 256 entries are read
 // before the depth is known.  parse_batch, over the batches that lex_batch
 // made, feeds the tokens while the stack fits the window and the grammar's
-// chains have a bound (Tables::chain_rate).  advance_rest feeds what is left
+// chains have a bound (Tables::chain_rate).  advance_serial feeds what is left
 // on lane 0 (a token that is refused, EOS, a stack beyond the window) and
 // writes the configuration it leaves, and the row's status when d_status is
 // given.
@@ -529,7 +529,7 @@ __device__ __forceinline__ AdvRow advance_load(const T& t, const DevConfigs& cin
 }
 
 // Whether the warp feeds the row's tokens in batches (else they are
-// advance_rest's; a single token is feed_one's).
+// advance_serial's; a single token is feed_one's).
 template <class T>
 __device__ __forceinline__ bool feed_fits(const T& t, const AdvRow& r, int n_steps) {
   return n_steps > 1 && t.chain_rate > 0 && r.win && !(r.flags & 1);
@@ -541,7 +541,7 @@ __device__ __forceinline__ Feed feed_begin(const AdvRow& r, uint16_t* win, AdvSh
 
 // After the last batch (`fed`: parse_batch went through all of them, `end` is
 // the lexer's state there): the test of the last token, the stack written
-// back, and the row as advance_rest goes on with it at token f.tok.
+// back, and the row as advance_serial goes on with it at token f.tok.
 template <class T>
 __device__ __forceinline__ void feed_end(const T& ts, Feed& f, bool fed, const LexState& end, int n_steps,
                                          AdvRow& r, uint16_t* stack, int lane, int max_chain) {
@@ -558,13 +558,12 @@ __device__ __forceinline__ void feed_end(const T& ts, Feed& f, bool fed, const L
 }
 
 // Lane 0 only: tokens k0 .. n_steps - 1, one after the other (`first`: token 0,
-// loaded ahead).  Seldom reached, and a call, so that its code is not in the
-// way of the rest's.
+// loaded ahead).
 template <class T>
-__device__ __noinline__ void advance_rest(const T& t, const T& ts, const DevConfigs& cout,
-                                             const int32_t* __restrict__ tokens, int k0, int n_steps, int b,
-                                             uint16_t* win, AdvShared& sh, const AdvRow& r, int keep,
-                                             const LexToken& first, AdvOut& out) {
+__device__ __forceinline__ void advance_serial(const T& t, const T& ts, const DevConfigs& cout,
+                                               const int32_t* __restrict__ tokens, int k0, int n_steps, int b,
+                                               uint16_t* win, AdvShared& sh, const AdvRow& r, int keep,
+                                               const LexToken& first, AdvOut& out) {
   uint16_t* stack = cout.stack + (size_t)b * t.D;
   const LArr lo{sh.lo, 1}, ls{sh.ls, 1};
   int depth = r.depth, q = r.s.q, lx = r.s.lx, flags = r.flags;
@@ -633,6 +632,19 @@ __device__ __noinline__ void advance_rest(const T& t, const T& ts, const DevConf
     wcat = w.wc;
   }
   out = AdvOut{depth, q, lx, flags, status, pc, wcat, use_win, keep};
+}
+
+// The same as a call, where it is seldom reached: its code is not in the way of
+// the rest's.  The call reads the tables' descriptor from a copy in local
+// memory; k_advance, where every token of a row may come this way (a grammar
+// without CI classes, a stack beyond the window), has it inline: a prompt of 400
+// tokens fed this way 1,319 us, through the call 1,610.
+template <class T>
+__device__ __noinline__ void advance_rest(const T& t, const T& ts, const DevConfigs& cout,
+                                          const int32_t* __restrict__ tokens, int k0, int n_steps, int b,
+                                          uint16_t* win, AdvShared& sh, const AdvRow& r, int keep,
+                                          const LexToken& first, AdvOut& out) {
+  advance_serial(t, ts, cout, tokens, k0, n_steps, b, win, sh, r, keep, first, out);
 }
 
 // One token of a row, by its warp: feed_one, else advance_rest.
@@ -1912,7 +1924,8 @@ __global__ void __launch_bounds__(64, 3) k_advance(TabT<ST> t, DevConfigs cin, D
       keep = f.wlow;
     }
     out = AdvOut{row.depth, row.s.q, row.s.lx, row.flags, GRID_ST_OK, row.s.pc, row.s.wc, row.win, keep};
-    if (lane == 0 && k0 < n_steps) advance_rest(t, ts, cout, tokens, k0, n_steps, b, s_stk, sh, row, keep, own, out);
+    if (lane == 0 && k0 < n_steps)
+      advance_serial(t, ts, cout, tokens, k0, n_steps, b, s_stk, sh, row, keep, own, out);
   }
   if (lane == 0) {
     advance_store(cout, b, out);
