@@ -166,7 +166,9 @@ extern __shared__ __align__(16) uint8_t smem[];
 template <bool STAGED>
 struct TabT : Tables {
   TabT() = default;
-  explicit TabT(const Tables& t) : Tables(t) {}
+  explicit TabT(const Tables& t) : Tables(t) {
+    if (!STAGED) blob_bytes = 0;
+  }
   template <typename E>
   __device__ __forceinline__ E get(const E* p, int o, int i) const {
     return STAGED ? reinterpret_cast<const E*>(smem + o)[i] : p[i];

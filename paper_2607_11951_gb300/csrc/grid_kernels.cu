@@ -451,12 +451,15 @@ __device__ __forceinline__ void hash_nodes(const T& t, uint64_t* __restrict__ hs
 // token (2,000 tokens, 32 SQL rows: 7.8 ms; 1.9 ms this way).
 constexpr int kAdvSpec = 32;  // 16-byte stack accesses issued per lane before the depth is known
 
-// What the parts share, in shared memory.
-struct AdvShared {
-  LexBatch lex;
+// What the parts share, in shared memory: of a token, of a batch.
+struct FeedShared {
   uint16_t undo[kStackWin];
   uint16_t scr[kChainNs * 32];
   uint16_t lo[kMaxOvl], ls[kMaxOvl];  // lane 0's overlay and scratch
+};
+struct AdvShared {
+  LexBatch lex;
+  FeedShared f;
 };
 
 struct AdvRow {
@@ -535,7 +538,7 @@ __device__ __forceinline__ bool feed_fits(const T& t, const AdvRow& r, int n_ste
   return n_steps > 1 && t.chain_rate > 0 && r.win && !(r.flags & 1);
 }
 
-__device__ __forceinline__ Feed feed_begin(const AdvRow& r, uint16_t* win, AdvShared& sh) {
+__device__ __forceinline__ Feed feed_begin(const AdvRow& r, uint16_t* win, FeedShared& sh) {
   return Feed{win, sh.undo, sh.scr, kStackWin, r.depth, r.depth, r.depth, 0, r.depth, false, r.s};
 }
 
@@ -562,7 +565,7 @@ __device__ __forceinline__ void feed_end(const T& ts, Feed& f, bool fed, const L
 template <class T>
 __device__ __forceinline__ void advance_serial(const T& t, const T& ts, const DevConfigs& cout,
                                                const int32_t* __restrict__ tokens, int k0, int n_steps, int b,
-                                               uint16_t* win, AdvShared& sh, const AdvRow& r, int keep,
+                                               uint16_t* win, FeedShared& sh, const AdvRow& r, int keep,
                                                const LexToken& first, AdvOut& out) {
   uint16_t* stack = cout.stack + (size_t)b * t.D;
   const LArr lo{sh.lo, 1}, ls{sh.ls, 1};
@@ -642,30 +645,34 @@ __device__ __forceinline__ void advance_serial(const T& t, const T& ts, const De
 template <class T>
 __device__ __noinline__ void advance_rest(const T& t, const T& ts, const DevConfigs& cout,
                                           const int32_t* __restrict__ tokens, int k0, int n_steps, int b,
-                                          uint16_t* win, AdvShared& sh, const AdvRow& r, int keep,
+                                          uint16_t* win, FeedShared& sh, const AdvRow& r, int keep,
                                           const LexToken& first, AdvOut& out) {
   advance_serial(t, ts, cout, tokens, k0, n_steps, b, win, sh, r, keep, first, out);
 }
 
-// One token of a row, by its warp: feed_one, else advance_rest.
+// Token k of a row, by its warp: feed_one, and `row` and `out` are the row after
+// it; else advance_rest, which feeds the tokens after it too (false; `out` is
+// lane 0's).
 template <class T>
-__device__ __forceinline__ void advance_one(const T& t, const DevConfigs& cout, const int32_t* __restrict__ tokens,
-                                            int n_steps, int b, uint16_t* win, AdvShared& sh, AdvRow& r,
+__device__ __forceinline__ bool advance_one(const T& t, const DevConfigs& cout, const int32_t* __restrict__ tokens,
+                                            int k, int n_steps, int b, uint16_t* win, FeedShared& sh, AdvRow& row,
                                             const LexToken& x, int lane, AdvOut& out) {
   const int mc = max_chain_of(t);
   uint16_t* stack = cout.stack + (size_t)b * t.D;
-  if (x.st == 1 && r.win && !(r.flags & 1)) {
-    Feed f = feed_begin(r, win, sh);
-    LexState s = r.s;
+  if (x.st == 1 && row.win && !(row.flags & 1)) {
+    Feed f = feed_begin(row, win, sh);
+    LexState s = row.s;
     if (feed_one(t, f, s, x.sp, lane, mc)) {
       for (int i = f.wlow + lane; i < f.depth; i += 32) stack[i] = win[i];
-      out = AdvOut{f.depth, s.q, s.lx, r.flags, GRID_ST_OK, s.pc, s.wc, true, f.wlow};
-      return;
+      row.depth = f.depth;
+      row.s = s;
+      out = AdvOut{f.depth, s.q, s.lx, row.flags, GRID_ST_OK, s.pc, s.wc, true, min(out.keep, f.wlow)};
+      return true;
     }
     feed_back(f, lane);
   }
-  out = AdvOut{r.depth, r.s.q, r.s.lx, r.flags, GRID_ST_OK, r.s.pc, r.s.wc, r.win, r.depth};
-  if (lane == 0 && x.st != 0) advance_rest(t, t, cout, tokens, 0, n_steps, b, win, sh, r, r.depth, x, out);
+  if (lane == 0) advance_rest(t, t, cout, tokens, k, n_steps, b, win, sh, row, out.keep, x, out);
+  return false;
 }
 
 // The configuration that the advance leaves, by lane 0.
@@ -765,13 +772,16 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfig
         row = advance_load(t, adv.cin, c, b, adv.copy, lane, s_stk);
       }
       __syncthreads();
-      if (warp == 0) advance_one(t, c, adv.tokens, adv.n_steps, b, s_stk, sh, row, s_own, lane, o);
+      if (warp == 0) {
+        o = AdvOut{row.depth, row.s.q, row.s.lx, row.flags, GRID_ST_OK, row.s.pc, row.s.wc, row.win, row.depth};
+        if (s_own.st != 0) advance_one(t, c, adv.tokens, 0, adv.n_steps, b, s_stk, sh.f, row, s_own, lane, o);
+      }
     } else if (warp == 0) {
       const LexToken own = lex_fetch(t, toks, 0, adv.n_steps, lane);
       row = advance_load(t, adv.cin, c, b, adv.copy, lane, s_stk);
       int k0 = 0, keep = row.depth;
       if (feed_fits(t, row, adv.n_steps)) {
-        Feed f = feed_begin(row, s_stk, sh);
+        Feed f = feed_begin(row, s_stk, sh.f);
         LexState carry = row.s;
         bool fed = true;
         for (int k = 0; k < adv.n_steps && fed; k = sh.lex.next) {
@@ -786,7 +796,7 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfig
       }
       o = AdvOut{row.depth, row.s.q, row.s.lx, row.flags, GRID_ST_OK, row.s.pc, row.s.wc, row.win, keep};
       if (lane == 0 && k0 < adv.n_steps)
-        advance_rest(t, ts, c, adv.tokens, k0, adv.n_steps, b, s_stk, sh, row, keep, own, o);
+        advance_rest(t, ts, c, adv.tokens, k0, adv.n_steps, b, s_stk, sh.f, row, keep, own, o);
     }
     if (threadIdx.x == 0) {
       advance_store(c, b, o);
@@ -1857,8 +1867,23 @@ __global__ void __launch_bounds__(kPackWords, 4) k_pack(Tables t, RowCtx* __rest
   }
 }
 
-// One block of two warps per row: warp 1 lexes the next batch of tokens while
-// warp 0 parses the last one.
+// What a row's advance leaves, by its warp (`out` is lane 0's).
+template <class T>
+__device__ __forceinline__ void advance_done(const T& t, const DevConfigs& cout, const AdvOut& out,
+                                             int32_t* __restrict__ d_status, int b, int lane) {
+  if (lane == 0) {
+    advance_store(cout, b, out);
+    d_status[b] = out.status;
+  }
+  if (cout.hs) {
+    __syncwarp();
+    hash_nodes(t, cout.hs + (size_t)b * t.D, cout.stack + (size_t)b * t.D, __shfl_sync(0xffffffffu, out.keep, 0),
+               __shfl_sync(0xffffffffu, out.depth, 0), lane);
+  }
+}
+
+// Several tokens per row, a block of two warps per row: warp 1 lexes the next
+// batch of tokens while warp 0 parses the last one.
 template <bool ST>
 __global__ void __launch_bounds__(64, 3) k_advance(TabT<ST> t, DevConfigs cin, DevConfigs cout,
                                                 const int32_t* __restrict__ tokens, int n_steps,
@@ -1881,7 +1906,7 @@ __global__ void __launch_bounds__(64, 3) k_advance(TabT<ST> t, DevConfigs cin, D
   own = lex_fetch(t, toks, 0, n_steps, lane);
   if (warp == 0) {
     row = advance_load(t, cin, cout, b, copy, lane, s_stk);
-    f = feed_begin(row, s_stk, sh);
+    f = feed_begin(row, s_stk, sh.f);
     if (lane == 0) {
       s_stop[0] = 0;
       s_stop[1] = feed_fits(t, row, n_steps) ? 0 : 1;
@@ -1907,35 +1932,55 @@ __global__ void __launch_bounds__(64, 3) k_advance(TabT<ST> t, DevConfigs cin, D
     }
   }
   if (warp != 0) return;
-  AdvOut out;
-  if (n_steps <= 1) {
-    LexToken x;  // the row's one token is lane 0's
-    x.st = __shfl_sync(0xffffffffu, own.st, 0);
-    x.sp.len = __shfl_sync(0xffffffffu, own.sp.len, 0);
-    x.sp.head = make_uint4(__shfl_sync(0xffffffffu, own.sp.head.x, 0), __shfl_sync(0xffffffffu, own.sp.head.y, 0),
-                           __shfl_sync(0xffffffffu, own.sp.head.z, 0), __shfl_sync(0xffffffffu, own.sp.head.w, 0));
-    x.sp.all = reinterpret_cast<const uint8_t*>(__shfl_sync(0xffffffffu, (unsigned long long)own.sp.all, 0));
-    advance_one(t, cout, tokens, n_steps, b, s_stk, sh, row, x, lane, out);
-  } else {
-    int k0 = 0, keep = row.depth;
-    if (feed_fits(t, row, n_steps)) {
-      feed_end(ts, f, fed, carry, n_steps, row, cout.stack + (size_t)b * t.D, lane, mc);
-      k0 = f.tok;
-      keep = f.wlow;
-    }
-    out = AdvOut{row.depth, row.s.q, row.s.lx, row.flags, GRID_ST_OK, row.s.pc, row.s.wc, row.win, keep};
-    if (lane == 0 && k0 < n_steps)
-      advance_serial(t, ts, cout, tokens, k0, n_steps, b, s_stk, sh, row, keep, own, out);
+  int k0 = 0, keep = row.depth;
+  if (feed_fits(t, row, n_steps)) {
+    feed_end(ts, f, fed, carry, n_steps, row, cout.stack + (size_t)b * t.D, lane, mc);
+    k0 = f.tok;
+    keep = f.wlow;
   }
-  if (lane == 0) {
-    advance_store(cout, b, out);
-    d_status[b] = out.status;
+  AdvOut out{row.depth, row.s.q, row.s.lx, row.flags, GRID_ST_OK, row.s.pc, row.s.wc, row.win, keep};
+  if (lane == 0 && k0 < n_steps)
+    advance_serial(t, ts, cout, tokens, k0, n_steps, b, s_stk, sh.f, row, keep, own, out);
+  advance_done(t, cout, out, d_status, b, lane);
+}
+
+// One token per row, or a few in large batches: a warp per row, in large batches
+// several rows in a block, so that the tables are staged once for them (one
+// token, a row a block and eight: 1,024 SQL rows 17.4 and 13.2 us, 4,096 rows
+// 43.4 and 20.4; 32 expression rows in a graph 3.3 and 3.7).
+constexpr int kOneRows = 8;  // rows of a block, at most
+constexpr int kFewTokens = 8;  // tokens of a row that k_advance_one is given, at most
+struct OneShared {
+  uint16_t win[kStackWin];
+  FeedShared f;
+};
+static_assert(sizeof(OneShared) % 16 == 0, "the rows' parts start on 16-byte boundaries");
+
+template <bool ST>
+__global__ void __launch_bounds__(kOneRows * 32) k_advance_one(TabT<ST> t, DevConfigs cin, DevConfigs cout,
+                                                               const int32_t* __restrict__ tokens, int n_steps,
+                                                               int32_t* __restrict__ d_status, int B, int copy) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  OneShared& sh = reinterpret_cast<OneShared*>(smem + t.blob_bytes)[warp];
+  stage_tables(t);
+  pdl_wait();
+  const int b = blockIdx.x * (blockDim.x >> 5) + warp;
+  if (b >= B) return;
+  const LexToken own = lex_fetch(t, tokens + (size_t)b * n_steps, 0, n_steps, lane);  // lane k: token k
+  AdvRow row = advance_load(t, cin, cout, b, copy, lane, sh.win);
+  AdvOut out{row.depth, row.s.q, row.s.lx, row.flags, GRID_ST_OK, row.s.pc, row.s.wc, row.win, row.depth};
+#pragma unroll 1
+  for (int k = 0; k < n_steps; ++k) {
+    LexToken x;
+    x.st = __shfl_sync(0xffffffffu, own.st, k);
+    if (x.st == 0) continue;
+    x.sp.len = __shfl_sync(0xffffffffu, own.sp.len, k);
+    x.sp.head = make_uint4(__shfl_sync(0xffffffffu, own.sp.head.x, k), __shfl_sync(0xffffffffu, own.sp.head.y, k),
+                           __shfl_sync(0xffffffffu, own.sp.head.z, k), __shfl_sync(0xffffffffu, own.sp.head.w, k));
+    x.sp.all = reinterpret_cast<const uint8_t*>(__shfl_sync(0xffffffffu, (unsigned long long)own.sp.all, k));
+    if (!advance_one(t, cout, tokens, k, n_steps, b, sh.win, sh.f, row, x, lane, out)) break;
   }
-  if (cout.hs) {
-    __syncwarp();
-    hash_nodes(t, cout.hs + (size_t)b * t.D, cout.stack + (size_t)b * t.D, __shfl_sync(0xffffffffu, out.keep, 0),
-               __shfl_sync(0xffffffffu, out.depth, 0), lane);
-  }
+  advance_done(t, cout, out, d_status, b, lane);
 }
 
 // In-place -inf fill (apply_span), grid = (blocks per row, B): few, long-lived
@@ -1982,9 +2027,10 @@ int grid::g_sms = 152;  // SM count of the current device, set by grid_specializ
 // spec in the process, so it is raised once to the largest staged block
 // allowed instead of to this spec's size.
 static int set_smem_limits() {
-  const int dyn = std::max(kMaxStage, kMaxPack);
+  const int dyn = std::max(kMaxStage + kOneRows * (int)sizeof(OneShared), kMaxPack);
   const void* kernels[] = {
       (const void*)k_classify<true>, (const void*)k_events<true>, (const void*)k_advance<true>,
+      (const void*)k_advance_one<true>,
       (const void*)k_row<0, true>, (const void*)k_row<1, true>, (const void*)k_row<2, true>,
       // k_pack: one row's class selections and verdict-class bits, two contexts
       (const void*)k_pack<0, false>, (const void*)k_pack<1, false>, (const void*)k_pack<2, false>,
@@ -2502,6 +2548,12 @@ static int specialize(const grid_grammar* g, const grid_vocab* v, cudaStream_t s
     return set_error(GRID_E_TOO_LARGE, "grid_specialize: the class selections and verdict-class bits of one "
                                        "row exceed the packing kernel's shared memory");
   s->max_cd = *std::max_element(counts.begin(), counts.end());
+  int per_sm = 0;
+  if (t.blob_bytes)
+    GRID_DONE(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_advance<true>, 64, t.blob_bytes));
+  else
+    GRID_DONE(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_advance<false>, 64, 0));
+  s->adv_fit = per_sm * s->sms;
   return GRID_OK;
 #undef GRID_DONE
 }
@@ -2598,10 +2650,29 @@ extern "C" int grid_configs_reset(const grid_spec* s, grid_configs* c, void* str
 
 int grid::launch_advance(const grid_spec* s, const DevConfigs& in, const DevConfigs& out, int B,
                          const int32_t* d_tokens, int32_t n_steps, int32_t* d_status, int copy, cudaStream_t st) {
-  auto advance = [&](auto kern, const auto& t) {
-    return launch_pdl(kern, dim3(B), dim3(64), t.blob_bytes, st, t, in, out, d_tokens, n_steps, d_status, B, copy);
+  const TabT<true> ts(s->t);
+  const TabT<false> tg(s->t);
+  auto launch = [&](auto kern, const auto& t, int blocks, int threads, size_t dyn) {
+    return launch_pdl(kern, dim3(blocks), dim3(threads), t.blob_bytes + dyn, st, t, in, out, d_tokens, n_steps,
+                      d_status, B, copy);
   };
-  GRID_CUDA(s->t.blob_bytes ? advance(k_advance<true>, TabT<true>(s->t)) : advance(k_advance<false>, TabT<false>(s->t)));
+  // Several tokens go to a block per row while the blocks of all rows are on the SMs at once.  In larger batches each
+  // wave of blocks would stage the tables anew: there a few tokens are fed one after the other by a warp per row (2
+  // tokens, 4,096 SQL rows: 73 us as one block per row, 27 this way), and more of them in blocks that read the tables
+  // from global memory, of which more fit (16 tokens: 255 us staged, 129; within one wave, 256 rows: 36 and 48),
+  // unless the tables are so small that staging them costs nothing (expression grammar, 16 tokens, 4,096 rows: 80 us
+  // staged, 85).
+  const bool wave = B <= s->adv_fit;
+  if (n_steps <= 1 || (n_steps <= kFewTokens && !wave)) {
+    const int rows = std::min(kOneRows, (B + s->sms - 1) / s->sms);  // of a block: one until every SM has its block
+    const size_t dyn = rows * sizeof(OneShared);
+    const int blocks = (B + rows - 1) / rows;
+    GRID_CUDA(s->t.blob_bytes ? launch(k_advance_one<true>, ts, blocks, rows * 32, dyn)
+                              : launch(k_advance_one<false>, tg, blocks, rows * 32, dyn));
+  } else {
+    const bool staged = s->t.blob_bytes > 0 && (wave || s->t.blob_bytes <= 16 * 1024);
+    GRID_CUDA(staged ? launch(k_advance<true>, ts, B, 64, 0) : launch(k_advance<false>, tg, B, 64, 0));
+  }
   GRID_CUDA(cudaGetLastError());
   return GRID_OK;
 }

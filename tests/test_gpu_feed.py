@@ -119,3 +119,50 @@ def test_feed_matches_token_by_token(name):
             assert st2[b] == want[b][0]
         ref = one.export(b)
         assert other.export(b) == ref and cfg.export(b) == ref, (b, rows[b])
+
+
+@pytest.mark.parametrize("n", [1, 2, 8, 9, 40])
+@pytest.mark.parametrize("name", ["sql", "expr", "many"])
+def test_large_batch_feeds_as_a_small_one(name, n):
+    """Rows whose blocks are not on the device at once: statuses,
+    configurations and node hashes are those of the same rows in a small
+    batch (fed as the test above checks against the oracle)."""
+    import torch
+    from paper_2607_11951_gb300 import grid as G
+    grammar, role, lexicons, tokens, eos, specials, good = _world(name)
+    rng = np.random.default_rng(n)
+    rows = []
+    for p in good * 8:
+        p = [int(x) for x in p]
+        at = int(rng.integers(0, len(p) + 1))
+        rows.append((p[:at], (p[at:] + [eos] + p[:1])[:n]))
+        rows.append((p[:at], (p[at:at + n // 2] + [int(rng.integers(0, len(tokens)))] + p[at + n // 2:])[:n]))
+        rows.append((p[:at], (p[at:at + 1] + [-1, -1] + p[at + 1:])[:n]))
+    times = 1 + 5000 // len(rows)
+    spec = G.Spec(G.Grammar(grammar, role, lexicons), G.Vocab(tokens, eos, specials))
+
+    def feed(rows):
+        B, m = len(rows), max(1, max(len(a) for a, _ in rows))
+        before, fed = np.full((B, m), -1, np.int32), np.full((B, n), -1, np.int32)
+        for b, (a, x) in enumerate(rows):
+            before[b, :len(a)] = a
+            fed[b, :len(x)] = x
+        st, cin, out = torch.zeros(B, dtype=torch.int32, device="cuda"), G.Configs(spec, B), G.Configs(spec, B)
+        for c in (cin, out):
+            G.grid_configs_enable_audit(spec.h, c.h)
+        G.grid_advance(spec, cin, cin, torch.from_numpy(before).cuda(), st)
+        assert not st.any()
+        G.grid_advance(spec, cin, out, torch.from_numpy(fed).cuda(), st)
+        records = torch.zeros((B, 80), dtype=torch.uint8, device="cuda")
+        mask, zero = torch.zeros((B, spec.W), dtype=torch.int32, device="cuda"), torch.zeros_like(st)
+        G.grid_audit_append(spec.h, out.h, mask, zero, 0, records)
+        torch.cuda.synchronize()
+        return st.cpu().numpy(), out, records.cpu().numpy()
+
+    st, out, rec = feed(rows)
+    st2, out2, rec2 = feed(rows * times)
+    assert (st2 == np.tile(st, times)).all()
+    assert (rec2 == np.tile(rec, (times, 1))).all()
+    ref = [out.export(b) for b in range(len(rows))]
+    for b in rng.integers(0, len(rows) * times, 300):
+        assert out2.export(int(b)) == ref[int(b) % len(rows)], b
