@@ -1,7 +1,8 @@
 """Which tables are staged in shared memory, and the launches that follow, on a
 CUDA runtime without a GPU: lexer and parser tables of up to 96 KB are staged
-whatever else goes with them, and no launch asks for more shared memory than
-its kernel was allowed."""
+whatever else goes with them, no launch asks for more shared memory than its
+kernel was allowed, and a batch whose spellings are all walked gets the walk's
+largest blocks."""
 import ctypes
 
 import pytest
@@ -61,3 +62,22 @@ def test_tables_of_96_kb_are_staged(fake, cats):
             del g, s, c
         assert (True, True) in seen and (True, False) in seen
         del v
+
+
+def test_walk_without_ci_classes(fake):
+    from workloads import configs
+    wl = configs.manycat(12, 21, B=1)
+    with fakes.use(fake) as rt:
+        g = G.Grammar(wl["grammar"], wl["role"], wl["lexicons"])
+        v = G.Vocab(wl["tokens"], wl["eos"], wl["specials"])
+        s = G.Spec(g, v)
+        assert not s.info()["ci_on"]
+        warps = []
+        for B in (1, 32):
+            c = G.Configs(s, B)
+            rt.reset()
+            assert G.lib().grid_masks(s.h, c.h, ctypes.c_void_p(16), ctypes.c_void_p(16), None) == G.GRID_OK
+            warps += [threads // 32 for name, _, threads, _, _ in rt.launches() if "k_walk" in name]
+            del c
+        assert warps == [8, 24]
+        del g, v, s
