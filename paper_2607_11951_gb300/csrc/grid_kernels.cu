@@ -2548,6 +2548,13 @@ static int specialize(const grid_grammar* g, const grid_vocab* v, cudaStream_t s
     return set_error(GRID_E_TOO_LARGE, "grid_specialize: the class selections and verdict-class bits of one "
                                        "row exceed the packing kernel's shared memory");
   s->max_cd = *std::max_element(counts.begin(), counts.end());
+  s->walk_items = (float)t.NS / 32;
+  if (t.ci_on) {
+    long shifts = 0;
+    for (int q = 0; q < h.S; ++q)
+      for (int tau = 0; tau < h.n_term; ++tau) shifts += h.action[(size_t)q * h.T1 + tau] > 0;
+    s->walk_items *= (float)shifts / ((float)h.S * (float)h.n_term);
+  }
   int per_sm = 0;
   if (t.blob_bytes)
     GRID_DONE(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_advance<true>, 64, t.blob_bytes));
@@ -2687,29 +2694,24 @@ extern "C" int grid_advance(const grid_spec* s, const grid_configs* in, grid_con
                         (cudaStream_t)stream);
 }
 
-// Walk items that may come up in a step, per SM: a row has about one per 1,024
-// spellings, or one per 64 where the grammar has no CI classes and every
-// spelling is walked.
-static float walk_items(const grid_spec* s, int B) {
-  const int per = s->t.ci_on ? 1024 : 64;
-  return (float)B * (float)((s->t.NS + per - 1) / per) / (float)s->sms;
-}
 // Warps per k_walk block.  A walk waits for its look-ups, so a large batch
 // wants every warp that fits (24, by shared memory and 80 registers: 256 SQL
 // rows 291 us a step, 514 us with 8 warps, 337 us with 16), a small one the
 // shortest start, and room for the next kernel's blocks beside it (one
 // expression row 24.1 us with 4 warps, 27.1 us with 24; one SQL row 38.3 and
-// 42.1).  Between them by the items that may come up; the lines are where the
-// next size is faster over batches of 1 to 128 rows of SQL, random and
-// many-category grammars of 8,000 to 152,000 tokens.  Per step with 8, 12, 16
-// and 24 warps: 8 SQL rows of 152,000 tokens 51.1, 48.0, 46.3, 47.6 us; 64 rows
-// of a random grammar, 20,000 tokens 79.4, 69.3, 65.2, 60.4 us; 16 rows without
-// CI classes 51.4, 47.5, 45.3, 44.0 us.
+// 42.1).  Between them by the walk items that may come up: a row's spellings go
+// as far as its state shifts their first terminal, the share of terminals that
+// a state shifts on average (every spelling where the grammar has no CI
+// classes).  That gives 235 items a row for 152,000 SQL tokens (counted: 196),
+// 7 for a grammar of 60 keywords (7), 46 to 60 for random grammars and 20,000
+// tokens (51 to 88).  Per step with 8, 12, 16 and 24 warps: 8 SQL rows 51.1,
+// 48.0, 46.3, 47.6 us; 64 rows of a random grammar 79.4, 69.3, 65.2, 60.4 us;
+// 16 rows without CI classes 51.4, 47.5, 45.3, 44.0 us.
 static int walk_warps(const grid_spec* s, int B) {
-  const float n = walk_items(s, B);
+  const float n = (float)B * s->walk_items / (float)s->sms;  // items per SM
   const int room = (kWalkSmem - s->t.blob_bytes) / (int)sizeof(WalkWarp);
-  if (n < (B == 1 ? 1.f : 0.5f)) return 4;
-  return n < 2.f ? 8 : n < 4.f ? 12 : n < 8.f ? 16 : std::min(kWalkWarps, room);
+  if (n < (B == 1 ? 2.f : 1.f)) return 4;
+  return n < 4.f ? 8 : n < 8.f ? 12 : n < 16.f ? 16 : std::min(kWalkWarps, room);
 }
 
 // The four kernels of one mask step on `st`; `ev` (5 events or NULL) is
@@ -2741,7 +2743,7 @@ int grid::launch_masks(const grid_spec* s, const DevConfigs& c, const MaskScratc
   // the scan of the ranges in k_filter: where the walks fill the SMs for long (256 SQL rows: 290 -> 248 us a step,
   // 128 rows 163 -> 157), not where a step waits for the longest of them (32 rows 72 -> 95 us: what is left of the
   // ranges then packs 32 long walks into a warp)
-  const bool scan = s->has_cats && m.vcap >= kScanList && walk_items(s, B) >= 100.f;
+  const bool scan = s->has_cats && m.vcap >= kScanList && (long)B * ((t.NS + 1023) / 1024) / s->sms >= 100;
   const int scan_blocks = scan ? std::min((t.NS / kRangeSpan + 256 + 7) / 8, std::max(1, 32 * s->sms / B)) : 0;
   GRID_CUDA(launch_pdl(k_filter, dim3(std::max({1, cd_blocks + vc_blocks, scan_blocks}), B, scan ? 3 : 2), dim3(256), 0,
                        st, tg, m.ctx,

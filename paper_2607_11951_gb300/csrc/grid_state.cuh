@@ -214,6 +214,7 @@ struct grid_spec {
   grid::Arena mem;
   int device = 0;
   int sms = 152;
+  float walk_items = 0;  // k_walk items that a row brings, by the grammar and the vocabulary
   int adv_fit = 0;      // rows whose blocks of k_advance are on the device at once
   int max_cd = 0;       // longest CD list of a table
   int vcw = 0;          // words of the largest table's verdict-class bitset
