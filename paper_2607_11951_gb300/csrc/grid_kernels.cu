@@ -2561,6 +2561,8 @@ static int specialize(const grid_grammar* g, const grid_vocab* v, cudaStream_t s
   else
     GRID_DONE(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_advance<false>, 64, 0));
   s->adv_fit = per_sm * s->sms;
+  GRID_DONE(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_row<1, true>, kRowWarps * 32, t.blob_bytes));
+  s->row_pair = per_sm > 1;
   return GRID_OK;
 #undef GRID_DONE
 }
@@ -2727,7 +2729,10 @@ int grid::launch_masks(const grid_spec* s, const DevConfigs& c, const MaskScratc
   if (ev) GRID_CUDA(cudaEventRecord(ev[0], st));
   const TabT<true> ts(t);  // the tables as the kernels that stage them take them, or
   const TabT<false> tg(t);  // that read a block too large to stage from global memory
-  const bool staged = t.blob_bytes > 0;
+  // Tables so large that k_row has one block on an SM are staged for batches of one row per SM alone: beyond them the
+  // blocks wait for one another's SM (tables of 96 KB, 256 rows: 54 us staged, 47 from global memory; 152 rows 36 and
+  // 38; tables of 52 KB leave two blocks, 512 rows: 149 and 160).
+  const bool staged = t.blob_bytes > 0 && (B <= s->sms || s->row_pair);
   auto row = [&](auto kern, const auto& tab) {
     return launch_pdl(kern, dim3(B + zero_blocks), dim3(kRowWarps * 32), tab.blob_bytes, st, tab, c, m.ctx, m.rng,
                       m.A2, m.sel, m.verd0, m.verd1, m.vcbits, n_vcbits, B, m.words_v, m.cache,

@@ -215,6 +215,7 @@ struct grid_spec {
   int device = 0;
   int sms = 152;
   float walk_items = 0;  // k_walk items that a row brings, by the grammar and the vocabulary
+  bool row_pair = false;  // two blocks of k_row fit an SM beside the staged tables
   int adv_fit = 0;      // rows whose blocks of k_advance are on the device at once
   int max_cd = 0;       // longest CD list of a table
   int vcw = 0;          // words of the largest table's verdict-class bitset

@@ -90,9 +90,9 @@ int cudaFuncSetAttribute(const void* f, int, int v) {
   limits[names[f]] = v;
   return kOk;
 }
-int cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t, unsigned) {
+int cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t smem, unsigned) {
   if (int e = step(kUnknown)) return e;
-  *n = 3;
+  *n = (int)(228 * 1024 / (smem + 39 * 1024));  // (as for k_row)
   return kOk;
 }
 int cudaGetSymbolAddress(void** p, const void* s) {

@@ -65,8 +65,8 @@ def test_tables_in_global_memory():
 
 
 def test_largest_staged_tables():
-    """Tables that leave the walk's largest block fewer warps: 3,200 rows of
-    which each kind's mask is the oracle's."""
+    """The largest tables that are staged, in a batch that stages them and in one
+    that reads them from global memory: every row's mask is the oracle's."""
     from oracle import compile_grammar
     from paper_2607_11951_gb300 import grid as G
     from tests.harness import GpuRun
@@ -78,14 +78,16 @@ def test_largest_staged_tables():
     eos = len(toks) - 1
     byte = {t: i for i, t in enumerate(toks)}
     kinds = [[byte[bytes([c])] for c in x] for x in (b"", b"a", b"aa ad", b"q", b"qr", b"qrq", b"qrq;", b"qrq ; aa ")]
-    run = GpuRun(dict(name="staging", grammar=text, role=None, lexicons=lexicons, tokens=toks, eos=eos, specials=[],
-                      prefixes=[kinds[b % 8] for b in range(3200)], max_depth=1024))
-    assert run.spec.info()["staged_bytes"] > 104 * 1024
     og = compile_grammar(text, None, lexicons)
     cfgs = [og.config_from_ids(p, toks, eos) for p in kinds]
-    assert all(c is not None for c in cfgs) and not run.build_configs().any()
-    words, status = run.masks()
-    assert not status.any()
-    bits = unpack(words, run.V)
-    for k, c in enumerate(cfgs):
-        assert (bits[k::8] == np.asarray(og.mask(c, toks, eos), np.uint8)).all(), kinds[k]
+    assert all(c is not None for c in cfgs)
+    for B in (152, 3200):
+        run = GpuRun(dict(name="staging", grammar=text, role=None, lexicons=lexicons, tokens=toks, eos=eos, specials=[],
+                          prefixes=[kinds[b % 8] for b in range(B)], max_depth=1024))
+        assert run.spec.info()["staged_bytes"] > 104 * 1024
+        assert not run.build_configs().any()
+        words, status = run.masks()
+        assert not status.any()
+        bits = unpack(words, run.V)
+        for k, c in enumerate(cfgs):
+            assert (bits[k::8] == np.asarray(og.mask(c, toks, eos), np.uint8)).all(), (B, kinds[k])

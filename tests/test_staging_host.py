@@ -40,7 +40,7 @@ def table_bytes(i):
 @pytest.mark.parametrize("cats", [0, 7])
 def test_tables_of_96_kb_are_staged(fake, cats):
     with fakes.use(fake) as rt:
-        toks = [bytes([b]) for b in range(256)] + [b"%d" % i for i in range(10, 2000)] + [b"<eos>"]
+        toks = [bytes([b]) for b in range(256)] + [b"%d" % i for i in range(10, 60000)] + [b"<eos>"]
         v = G.Vocab(toks, len(toks) - 1, [])
         seen = []
         for n in range(70, 92):
@@ -51,15 +51,21 @@ def test_tables_of_96_kb_are_staged(fake, cats):
             staged = s.info()["staged_bytes"]
             seen.append((size > 94 * 1024, staged > 0))
             assert s.info()["ci_on"] and (staged > 0 or size > 96 * 1024), (n, size)
-            c = G.Configs(s, 4096)  # enough rows for the largest blocks of the walk
             one = ctypes.c_void_p(16)
-            assert G.lib().grid_masks(s.h, c.h, one, one, None) == G.GRID_OK
-            assert G.lib().grid_reserve(s.h, c.h, one, one, 16, one, None, 0, None, None) == G.GRID_OK
-            for name, grid, threads, smem, limit in rt.launches():
-                assert smem <= limit <= SM_BYTES, (name, smem, limit)
-                if "k_walk" in name:
-                    assert threads >= 20 * 32
-            del g, s, c
+            for B in (152, 4096):  # rows that stage large tables, and that do not; both want the walk's largest blocks
+                c = G.Configs(s, B)
+                rt.reset()
+                assert G.lib().grid_masks(s.h, c.h, one, one, None) == G.GRID_OK
+                assert G.lib().grid_reserve(s.h, c.h, one, one, 16, one, None, 0, None, None) == G.GRID_OK
+                for name, grid, threads, smem, limit in rt.launches():
+                    assert smem <= limit <= SM_BYTES, (name, smem, limit)
+                    if "k_rowILi0E" in name or "k_walkILb0E" in name:
+                        pair = 2 * (staged + 39 * 1024) <= 228 * 1024  # two blocks of k_row on an SM
+                        assert ("0ELb1E" in name) == (staged > 0 and (B == 152 or pair)), (name, B, staged)
+                    if "k_walk" in name:
+                        assert threads >= 20 * 32
+                del c
+            del g, s
         assert (True, True) in seen and (True, False) in seen
         del v
 
