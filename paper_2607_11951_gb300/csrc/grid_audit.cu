@@ -92,6 +92,9 @@ __global__ void k_audit_init(Tables t, DevConfigs c, uint8_t* __restrict__ heads
 // audited decoding step of such rows went from 265 us to 93 us with this and
 // the deferred node hashes.
 constexpr int kAuditThreads = 128;
+constexpr int kMaxChunks = 3072;  // of a mask row (25 M tokens)
+// The id's message for n chunks, in bytes: k_audit_append's dynamic shared memory.
+constexpr int id_bytes(int n) { return ((2 + 2 * n + 15) & ~15) * 8; }
 __global__ void __launch_bounds__(kAuditThreads) k_audit_append(
     Tables t, DevConfigs c, const uint32_t* __restrict__ mask, const int32_t* __restrict__ tokens, uint32_t kind,
     uint8_t* __restrict__ heads, uint64_t* __restrict__ steps, uint8_t* __restrict__ records, long long rec_stride,
@@ -225,9 +228,8 @@ int audit_reset(const grid_spec* s, grid_configs* c, cudaStream_t st) {
 int audit_append(const grid_spec* s, grid_configs* c, const uint32_t* d_mask, const int32_t* d_tokens, uint32_t kind,
                  uint8_t* d_records, long long rec_stride, cudaStream_t st) {
   const int nch = (s->t.W + kChunkWords - 1) / kChunkWords;
-  const size_t id_bytes = (size_t)((2 + 2 * nch + 15) & ~15) * 8;
-  k_audit_append<<<c->B, kAuditThreads, id_bytes, st>>>(s->t, c->c, d_mask, d_tokens, kind, c->heads, c->steps,
-                                                              d_records, rec_stride, c->B);
+  k_audit_append<<<c->B, kAuditThreads, id_bytes(nch), st>>>(s->t, c->c, d_mask, d_tokens, kind, c->heads, c->steps,
+                                                             d_records, rec_stride, c->B);
   GRID_CUDA(cudaGetLastError());
   return GRID_OK;
 }
@@ -247,6 +249,7 @@ extern "C" int grid_configs_enable_audit(const grid_spec* s, grid_configs* c, vo
   cudaStream_t st = (cudaStream_t)stream;
   int rc = audit_reset(s, c, st);
   if (rc) return rc;
+  GRID_CUDA(cudaFuncSetAttribute(k_audit_append, cudaFuncAttributeMaxDynamicSharedMemorySize, id_bytes(kMaxChunks)));
   GRID_CUDA(cudaStreamSynchronize(st));
   return GRID_OK;
 }

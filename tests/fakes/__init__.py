@@ -9,6 +9,7 @@ import subprocess
 from paper_2607_11951_gb300 import grid as G
 
 B = importlib.import_module("paper_2607_11951_gb300.build")  # (the package has a function of this name)
+DEFAULT_SMEM = 48 * 1024  # shared memory of a block, its own and dynamic, without an attribute
 HERE = os.path.dirname(os.path.abspath(__file__))
 
 

@@ -1,8 +1,8 @@
 """Which tables are staged in shared memory, and the launches that follow, on a
 CUDA runtime without a GPU: lexer and parser tables of up to 96 KB are staged
 whatever else goes with them, no launch asks for more shared memory than its
-kernel was allowed, and a batch whose spellings are all walked gets the walk's
-largest blocks."""
+kernel was allowed, a batch whose spellings are all walked gets the walk's
+largest blocks, and a mask row's chunk digests have room up to 25 M tokens."""
 import ctypes
 
 import pytest
@@ -87,3 +87,20 @@ def test_walk_without_ci_classes(fake):
             del c
         assert warps == [8, 24]
         del g, v, s
+
+
+def test_audit_record_of_the_largest_vocabulary(fake):
+    chunks = 25_165_824 // 8192
+    with fakes.use(fake) as rt:
+        toks = [bytes([b]) for b in range(256)] + [b"<eos>"]
+        v, g = G.Vocab(toks, 256, []), G.Grammar("%token A /a/\n%ignore WS /[ ]+/\n%start s\ns -> A\n")
+        s = G.Spec(g, v)
+        c = G.Configs(s, 1)
+        one = ctypes.c_void_p(16)
+        assert G.lib().grid_configs_enable_audit(s.h, c.h, None) == G.GRID_OK
+        rt.reset()
+        assert G.lib().grid_audit_append(s.h, c.h, one, one, 0, one, None) == G.GRID_OK
+        # dynamic shared memory that the kernel may have beside its own: two words and two per chunk
+        (limit,) = [limit for name, _, _, _, limit in rt.launches() if "k_audit_append" in name]
+        assert limit != fakes.DEFAULT_SMEM and limit >= 8 * (2 + 2 * chunks)
+        del c, s, g, v
