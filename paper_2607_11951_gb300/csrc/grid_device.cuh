@@ -118,8 +118,8 @@ struct Tables {
   const uint8_t* spell_bytes;
   const uint4* spell16;  // first 16 bytes of each spelling, zero padded (one load per walk)
   const int32_t* spell_of_id;
-  const int32_t* id_of_spell;  // NS: the smallest id with each spelling
-  const int32_t* next_alias;   // Vp: the next larger id with the same spelling, -1 after the last
+  const int32_t* id_of_spell;  // NS: the first of each spelling's ids (a list in any order)
+  const int32_t* next_alias;   // Vp: the next id of the spelling's list, -1 after the last
   const int32_t* first_of_byte;
   const uint8_t* first_byte_by_id;
   const uint32_t* killw;       // Q * W: bit j of word (q, wi): id 32 wi + j's first byte ends a lexeme at q
@@ -132,7 +132,7 @@ struct Tables {
   const int32_t* tbl_q;
   const uint16_t* cls_by_id;  // n_tbl * V
   const int32_t* cd_off;      // n_tbl + 1
-  const int32_t* cd_list;     // ascending spelling indices per table
+  const int32_t* cd_list;     // spelling indices per table, in any order
   const uint16_t* cd_key;     // per cd_list entry: class of its first stack-dependent emission
   // verdict classes: table k owns records vc_off[k] .. vc_off[k+1] of vc_rec
   const int32_t* vc_off;

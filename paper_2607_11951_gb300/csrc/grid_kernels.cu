@@ -45,7 +45,7 @@
 //            from the cache entry (or stored into the entry the row claimed)
 // Decoding step (grid_advance_masks): the same kernels, k_row feeding each
 // row's tokens on warp 0 of its block before it prepares the row.
-// Parser step (grid_advance):  k_advance.   Masked logits:  k_apply.
+// Parser step (grid_advance):  k_advance, k_advance_one.   Masked logits:  k_apply.
 //
 // Every loop is bounded; hitting a bound writes GRID_ST_BOUND.  No kernel traps.
 
@@ -312,6 +312,9 @@ __global__ void k_vc_gather(const int32_t* __restrict__ slot_tbl, const Rec* __r
 
 // Each record's rank in its table: the number of smaller keys, counted over
 // the table's keys in tiles; grid (records / 256, tables, parts of the tiles).
+// Quadratic in a table's records, of which there are at most as many as
+// spellings: with 150,000 of them in the start state's table a specialization
+// takes 18.7 ms (4.2 ms with 60,000), 164 ms when the host merged and sorted them.
 __global__ void __launch_bounds__(256) k_vc_rank(const RecKey* __restrict__ key, const int32_t* __restrict__ vc_off,
                                                  int32_t* __restrict__ rank) {
   __shared__ RecKey s_key[256];
@@ -440,15 +443,13 @@ __device__ __forceinline__ void hash_nodes(const T& t, uint64_t* __restrict__ hs
 // before the depth is known.  parse_batch, over the batches that lex_batch
 // made, feeds the tokens while the stack fits the window and the grammar's
 // chains have a bound (Tables::chain_rate).  advance_serial feeds what is left
-// on lane 0 (a token that is refused, EOS, a stack beyond the window) and
-// writes the configuration it leaves, and the row's status when d_status is
-// given.
+// on lane 0 (a token that is refused, EOS, a stack beyond the window).
 //
 // A token that is fed costs the chain of its table look-ups, so nothing but
 // the stack's own steps stays serial: feeding every byte on lane 0, with the
 // token's spelling loaded when its turn came and each reduce chain run twice
 // (once for a set of terminals, once for the one that shifts), took 3.9 us a
-// token (2,000 tokens, 32 SQL rows: 7.8 ms; 1.9 ms this way).
+// token (2,000 tokens, 32 SQL rows: 7.8 ms; 1.8 ms this way).
 constexpr int kAdvSpec = 32;  // 16-byte stack accesses issued per lane before the depth is known
 
 // What the parts share, in shared memory: of a token, of a batch.
@@ -1000,7 +1001,7 @@ __global__ void __launch_bounds__(kRowWarps * 32, 2) k_row(TabT<ST> t, DevConfig
   __syncthreads();
   const int emit_ok = complete ? 0 : s_row[4], keep1 = complete ? depth : s_row[5], m1 = complete ? 0 : s_row[6];
   const Bits4 A0 = Bits4::load(s_A0), A1 = Bits4::load(s_A1);
-  // ---- phase 2: ranges (warp 0), class selections (warps 1, 2)
+  // ---- phase 2: ranges (warp 0), class selections (the other warps)
   if (!complete) {
     if (warp == 0 && ranged) {
       // continuing first-byte ranges (rows without a CI table for q).  A first
@@ -1308,9 +1309,10 @@ __device__ __forceinline__ int4 row_queue(const RowCtx& x, int scan_cap) {
 // table), the verdict classes of the start state's table under sigma' (the
 // context of tokens whose first byte ends the pending lexeme), the start
 // state's byte-walked spellings under sigma', and the verdict classes of the
-// pending lexer state's table under sigma.  Warps start at different rows and drain a
-// row's queue item by item; to find work a warp examines 32 rows at once (one
-// per lane), from its current row on, and stops when no queue has items left.
+// pending lexer state's table under sigma.  A block's warps start on one row, blocks
+// on different ones, and drain a row's queue item by item; to find work a warp
+// examines 32 rows at once (one per lane), from its current row on, and stops
+// when no queue has items left.
 // A warp keeps the current row's context (allowed sets, sigma' overlay, stack
 // mirror) until it moves to another row.
 //
@@ -1318,11 +1320,10 @@ __device__ __forceinline__ int4 row_queue(const RowCtx& x, int scan_cap) {
 // context, one per lane, each evaluated once against the row's stack; an
 // accepted record sets its bit in vcbits (cleared by k_row), which k_pack
 // reads back per token id.
-// List items (kSpan CD spellings): a spelling is walked only if the class of
-// its first stack-dependent emission is selected for the context's allowed
-// set (otherwise that emission, and so the spelling, fails) and, for sigma',
-// if its first byte ends the pending lexeme; survivors are compacted onto the
-// low lanes.  Range items (up to kRangeSpan spellings of one live first-byte
+// List items: up to kSpan spellings that k_filter kept (byte-walked ones whose
+// first stack-dependent emission can succeed and, for sigma', whose first byte
+// ends the pending lexeme; or, of a row whose ranges it scanned, those that end
+// the pending lexeme).  Range items (up to kRangeSpan spellings of one live first-byte
 // range; k_row already dropped the first-byte subtrees in which no spelling
 // can survive): the range's items interleave, lane j of item i walking
 // spelling lo + i + j * (items of the range).  Both kinds share one call of
@@ -1552,7 +1553,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) k_walk(TabT<ST> t, RowCtx*
 // a sector boundary (SHIFTED) a sector's bits come from two words, and only
 // the elements before the first and after the last whole sector are stored one
 // by one: stored element by element throughout, 256 rows of 151,937 bf16
-// logits took 199 us, this way 23.
+// logits took 199 us, this way 18.
 constexpr int kApplyBatch = 4;
 template <typename T, bool SHIFTED, int kBatch, typename Word>
 __device__ __forceinline__ void apply_span(T* row, int e0, int e1, const Word& word, int tid, int step) {

@@ -7,7 +7,7 @@
 // is left out of the later steps, whose blocks for it end at once: most rows
 // stop at the first position, and masking them anew at each of max_span
 // positions cost 480 us of nine whole steps (32 SQL rows, V = 32,000,
-// max_span 8) where this takes 140 us.
+// max_span 8) where this takes 120 us.
 
 #include <cstring>
 
@@ -527,7 +527,7 @@ __device__ RsvGoal rsv_search(const T& t, const ReserveTables& rt, const uint16_
 // One block per row (the trigger and the tokens of the cheapest way are
 // written by the warp that found it).  One thread per row, with the entries
 // and the level heads in global memory, took 1,220 us for 32 SQL rows of up
-// to 2,000 tokens; this takes 110 us.
+// to 2,000 tokens; this takes 130 us.
 template <bool ST>
 __global__ void __launch_bounds__(kRsvWarps * 32) k_reserve(TabT<ST> t, ReserveTables rt, DevConfigs c, ReserveArgs ra) {
   __shared__ __align__(16) uint16_t s_stk[kRsvDepth];

@@ -1,8 +1,8 @@
 """Feeding several tokens in one call, 32 lexed at a time: the status and the
 configuration that every row is left in, against the oracle's token-by-token
 advance and against the same tokens fed one per call.  Batch edges, gaps (-1),
-refused tokens, EOS inside and at the end, tokens that end more lexemes than a
-list holds, lexemes of more candidates than a list holds, stacks beyond the
+refused tokens, EOS inside and at the end, tokens that end several lexemes,
+lexemes of more candidates than a list holds, stacks beyond the
 shared-memory window, and chains over empty nonterminals."""
 import numpy as np
 import pytest
@@ -166,3 +166,50 @@ def test_large_batch_feeds_as_a_small_one(name, n):
     ref = [out.export(b) for b in range(len(rows))]
     for b in rng.integers(0, len(rows) * times, 300):
         assert out2.export(int(b)) == ref[int(b) % len(rows)], b
+
+
+def test_batches_cut_by_their_bytes():
+    """Tokens of 17 to 400 bytes: a batch that ends one byte below its 384
+    bytes, at them and above; tokens of exactly 384 bytes and of more (which
+    no batch holds) first, in the middle and last; spellings beyond the 16
+    bytes that are kept with them."""
+    import torch
+    from oracle import compile_grammar
+    from paper_2607_11951_gb300 import grid as G
+    by_len = {2 * k + odd: b"a+" * k + b" " * odd for k in list(range(9, 31)) + [192, 193, 200] for odd in (0, 1)}
+    tokens = [bytes([c]) for c in b"ab+*() "] + list(by_len.values()) + [b"b+" * 100 + b")", b"<eos>"]
+    eos = len(tokens) - 1
+    of = {n: tokens.index(t) for n, t in by_len.items()}
+    bad = eos - 1  # refused after 200 bytes
+    rows = []
+    for last in (23, 24, 25):  # 6 x 60 + last = 383, 384, 385 bytes
+        rows.append([of[60]] * 6 + [of[last]] + [of[41]] * 20)
+        rows.append([of[19]] * 3 + [-1] + [of[60]] * 5 + [of[last + 3]] + [of[60]] * 5 + [of[last]] * 2)
+        rows.append([of[18]] * 40 + [of[60]] * 6 + [of[last]])
+    for n in (384, 385, 386, 387, 400):
+        for at in (0, 9, 18):
+            rows.append([of[17 + 2 * (i % 9) + 1] for i in range(at)] + [of[n]] + [of[20 + i] for i in range(18 - at)])
+        rows.append([of[n], of[n], of[18], of[n]])
+    rows += [[of[60]] * 7 + [bad, of[18]], [bad], [of[385], bad], [of[18]] * 33 + [bad], [of[60], eos], [of[384], eos]]
+    og = compile_grammar(grammar_text("expr"))
+    want = [_oracle_feed(og, r, tokens, eos, []) for r in rows]
+    assert sorted({w[0] for w in want}) == [G.GRID_ST_OK, G.GRID_ST_TOKEN_NOT_ALLOWED]
+    B, n = len(rows), max(map(len, rows))
+    fed, took = np.full((B, n), -1, np.int32), np.full((B, n), -1, np.int32)
+    for b, r in enumerate(rows):
+        fed[b, :len(r)] = r
+        took[b, :len(want[b][1])] = want[b][1]
+    spec = G.Spec(G.Grammar(grammar_text("expr"), None, {}), G.Vocab(tokens, eos, []))
+    st = torch.zeros(B, dtype=torch.int32, device="cuda")
+    mask = torch.zeros((B, spec.W), dtype=torch.int32, device="cuda")
+    cfg, other, one = G.Configs(spec, B), G.Configs(spec, B), G.Configs(spec, B)
+    d = torch.from_numpy(fed).cuda()
+    G.grid_advance(spec, cfg, other, d, st)
+    assert st.cpu().tolist() == [w[0] for w in want]
+    G.grid_advance_masks(spec, cfg, cfg, d, mask, st)
+    for k in range(n):
+        G.grid_advance(spec, one, one, torch.from_numpy(np.ascontiguousarray(took[:, k:k + 1])).cuda(), st)
+        assert not st.any()
+    for b in range(B):
+        ref = one.export(b)
+        assert other.export(b) == ref and cfg.export(b) == ref, (b, rows[b])
